@@ -37,6 +37,30 @@ inline int elt_bytes(const fedattn_shape *s) { return s->dtype == FEDATTN_BF16 ?
 
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
+PrefillParams prefill_params(const fedattn_shape *s, const void *q, const void *k, const void *v, void *o, float *lse,
+                             int64_t n_q_rows, int64_t total_kv)
+{
+    PrefillParams p;
+    memset(&p, 0, sizeof(p));
+    p.q = q; p.k = k; p.v = v; p.o = o; p.lse = lse;
+    p.n_q_rows = n_q_rows; p.total_kv = total_kv;
+    p.hq = s->n_q_heads; p.hkv = s->n_kv_heads; p.d = s->head_dim;
+    p.scale = eff_scale(s); p.causal = s->causal;
+    return p;
+}
+
+// bf16 runs on the tensor cores at every head_dim; fp32 storage has no tensor-core kind that keeps its precision
+bool on_tensor_cores(const Context *c, const PrefillParams &p, int dtype)
+{
+    return dtype == FEDATTN_BF16 && p.total_kv > 0 && prefill_sm100_takes(c, p);
+}
+
+cudaError_t launch_prefill(Context *c, const PrefillParams &p, int dtype, cudaStream_t s)
+{
+    if (on_tensor_cores(c, p, dtype)) return launch_prefill_sm100(c, p, s);
+    return launch_attn_generic(generic_params(p), dtype, s, &c->launches);
+}
+
 struct DeviceGuard {
     int prev = -1;
     bool ok = true;
@@ -169,30 +193,10 @@ fedattn_status fedattn_local(fedattn_ctx *ctx, const fedattn_shape *shape, const
     if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(o)) return FEDATTN_ERR_INVALID_ARG;
     DeviceGuard g(ctx->c.device);
     if (!g.ok) return FEDATTN_ERR_CUDA;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaError_t err;
-    if (shape->dtype == FEDATTN_BF16 && shape->head_dim == 128 && prefill_sm100_supported(&ctx->c)) {
-        PrefillParams p;
-        memset(&p, 0, sizeof(p));
-        p.q = q; p.k = k; p.v = v; p.o = o; p.lse = lse;
-        p.n_q_rows = L; p.total_kv = L;
-        p.hq = shape->n_q_heads; p.hkv = shape->n_kv_heads;
-        p.scale = eff_scale(shape); p.causal = shape->causal; p.sync = 0; p.kv_head_major = 0;
-        p.kv_pos = nullptr; p.n_seg = N;
-        memcpy(p.cu, cu, sizeof(int32_t) * (N + 1));
-        err = launch_prefill_sm100(&ctx->c, p, s);
-    } else {
-        GenericParams p;
-        memset(&p, 0, sizeof(p));
-        p.q = q; p.k = k; p.v = v; p.o = o; p.lse = lse;
-        p.n_rows = L; p.hq = shape->n_q_heads; p.hkv = shape->n_kv_heads; p.d = shape->head_dim;
-        p.scale = eff_scale(shape); p.causal = shape->causal; p.mode = kLocal;
-        p.kv_tok_stride = (int64_t)shape->n_kv_heads * shape->head_dim;
-        p.kv_head_stride = shape->head_dim;
-        p.n_seg = N;
-        memcpy(p.cu, cu, sizeof(int32_t) * (N + 1));
-        err = launch_attn_generic(p, shape->dtype, s, &ctx->c.launches);
-    }
+    PrefillParams p = prefill_params(shape, q, k, v, o, lse, L, L);
+    p.n_seg = N;
+    memcpy(p.cu, cu, sizeof(int32_t) * (N + 1));
+    const cudaError_t err = launch_prefill(&ctx->c, p, shape->dtype, static_cast<cudaStream_t>(stream));
     return err == cudaSuccess ? FEDATTN_OK : FEDATTN_ERR_CUDA;
 }
 
@@ -268,42 +272,20 @@ fedattn_status fedattn_sync(fedattn_ctx *ctx, const fedattn_shape *shape, const 
     if (total_kv > 0 && (!k_agg || !v_agg || !aligned16(k_agg) || !aligned16(v_agg))) return FEDATTN_ERR_INVALID_ARG;
     DeviceGuard g(ctx->c.device);
     if (!g.ok) return FEDATTN_ERR_CUDA;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaError_t err;
-    if (shape->dtype == FEDATTN_BF16 && shape->head_dim == 128 && total_kv > 0 && prefill_sm100_supported(&ctx->c)) {
-        PrefillParams p;
-        memset(&p, 0, sizeof(p));
-        p.q = q; p.k = k_agg; p.v = v_agg; p.o = o; p.lse = lse;
-        p.n_q_rows = n_q_rows; p.total_kv = total_kv;
-        p.hq = shape->n_q_heads; p.hkv = shape->n_kv_heads;
-        p.scale = eff_scale(shape); p.causal = shape->causal; p.sync = 1; p.kv_head_major = kv_head_major;
-        p.kv_pos = kv_pos; p.n_seg = 1;
-        if (q_pos && shape->causal) {
+    PrefillParams p = prefill_params(shape, q, k_agg, v_agg, o, lse, n_q_rows, total_kv);
+    p.sync = 1; p.kv_head_major = kv_head_major; p.kv_pos = kv_pos; p.q_pos = q_pos;
+    p.n_seg = 1;
+    p.cu[0] = 0; p.cu[1] = (int32_t)n_q_rows;
+    if (on_tensor_cores(&ctx->c, p, shape->dtype) && p.d == 128) {
+        if (!shape->causal) p.q_pos = nullptr;
+        if (p.q_pos) {
             // explicit query positions: every (query, key) pair is tested on its own positions, in any order
             if (ctx->c.scratch_bytes < position_table_bytes(p.hkv, n_q_rows, total_kv)) return FEDATTN_ERR_WORKSPACE;
-            p.general = 1; p.q_pos = q_pos;
+            p.general = 1;
             p.tab = reinterpret_cast<int32_t *>(ctx->c.scratch);
         }
-        p.cu[0] = 0; p.cu[1] = (int32_t)n_q_rows;
-        err = launch_prefill_sm100(&ctx->c, p, s);
-    } else {
-        GenericParams p;
-        memset(&p, 0, sizeof(p));
-        p.q = q; p.k = k_agg; p.v = v_agg; p.o = o; p.lse = lse;
-        p.n_rows = n_q_rows; p.hq = shape->n_q_heads; p.hkv = shape->n_kv_heads; p.d = shape->head_dim;
-        p.scale = eff_scale(shape); p.causal = shape->causal; p.mode = kSync;
-        if (kv_head_major) {
-            p.kv_tok_stride = shape->head_dim;
-            p.kv_head_stride = total_kv * shape->head_dim;
-            p.kv_pos_head_stride = total_kv;
-        } else {
-            p.kv_tok_stride = (int64_t)shape->n_kv_heads * shape->head_dim;
-            p.kv_head_stride = shape->head_dim;
-            p.kv_pos_head_stride = 0;
-        }
-        p.total_kv = total_kv; p.q_pos = q_pos; p.kv_pos = kv_pos;
-        err = launch_attn_generic(p, shape->dtype, s, &ctx->c.launches);
     }
+    const cudaError_t err = launch_prefill(&ctx->c, p, shape->dtype, static_cast<cudaStream_t>(stream));
     return err == cudaSuccess ? FEDATTN_OK : FEDATTN_ERR_CUDA;
 }
 
@@ -323,38 +305,11 @@ fedattn_status fedattn_sync_remote(fedattn_ctx *ctx, const fedattn_shape *shape,
     if (total_kv > 0 && (!k_agg || !v_agg || !aligned16(k_agg) || !aligned16(v_agg))) return FEDATTN_ERR_INVALID_ARG;
     DeviceGuard g(ctx->c.device);
     if (!g.ok) return FEDATTN_ERR_CUDA;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaError_t err;
-    if (shape->dtype == FEDATTN_BF16 && shape->head_dim == 128 && total_kv > 0 && prefill_sm100_supported(&ctx->c)) {
-        PrefillParams p;
-        memset(&p, 0, sizeof(p));
-        p.q = q; p.k = k_agg; p.v = v_agg; p.o = o; p.lse = lse;
-        p.n_q_rows = L; p.total_kv = total_kv;
-        p.hq = shape->n_q_heads; p.hkv = shape->n_kv_heads;
-        p.scale = eff_scale(shape); p.causal = shape->causal; p.sync = 1; p.remote_only = 1; p.kv_head_major = kv_head_major;
-        p.kv_pos = kv_pos; p.n_seg = N;
-        memcpy(p.cu, cu, sizeof(int32_t) * (N + 1));
-        err = launch_prefill_sm100(&ctx->c, p, s);
-    } else {
-        GenericParams p;
-        memset(&p, 0, sizeof(p));
-        p.q = q; p.k = k_agg; p.v = v_agg; p.o = o; p.lse = lse;
-        p.n_rows = L; p.hq = shape->n_q_heads; p.hkv = shape->n_kv_heads; p.d = shape->head_dim;
-        p.scale = eff_scale(shape); p.causal = shape->causal; p.mode = kSync; p.remote_only = 1;
-        if (kv_head_major) {
-            p.kv_tok_stride = shape->head_dim;
-            p.kv_head_stride = total_kv * shape->head_dim;
-            p.kv_pos_head_stride = total_kv;
-        } else {
-            p.kv_tok_stride = (int64_t)shape->n_kv_heads * shape->head_dim;
-            p.kv_head_stride = shape->head_dim;
-            p.kv_pos_head_stride = 0;
-        }
-        p.total_kv = total_kv; p.kv_pos = kv_pos;
-        p.n_seg = N;
-        memcpy(p.cu, cu, sizeof(int32_t) * (N + 1));
-        err = launch_attn_generic(p, shape->dtype, s, &ctx->c.launches);
-    }
+    PrefillParams p = prefill_params(shape, q, k_agg, v_agg, o, lse, L, total_kv);
+    p.sync = 1; p.remote_only = 1; p.kv_head_major = kv_head_major; p.kv_pos = kv_pos;
+    p.n_seg = N;
+    memcpy(p.cu, cu, sizeof(int32_t) * (N + 1));
+    const cudaError_t err = launch_prefill(&ctx->c, p, shape->dtype, static_cast<cudaStream_t>(stream));
     return err == cudaSuccess ? FEDATTN_OK : FEDATTN_ERR_CUDA;
 }
 

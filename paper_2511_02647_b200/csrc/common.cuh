@@ -101,14 +101,14 @@ cudaError_t launch_gather(const PartsParams &pp, int hkv, int d, int elt_bytes, 
                           void *k_agg, void *v_agg, int32_t *kv_pos, int32_t *cu_kv, int32_t *sel_idx_out,
                           int32_t *status, int device, int sm_count, cudaStream_t s, int64_t *launches);
 
-// ---- bf16 prefill on tensor cores (tcgen05 + TMEM + TMA), head_dim 128 ------------------------
+// ---- prefill calls (local, sync, remote-only sync); bf16 runs on tensor cores (tcgen05 + TMEM + TMA) --------
 struct PrefillParams {
     const void *q, *k, *v;
     void *o;
     float *lse;
     int64_t n_q_rows;
     int64_t total_kv;             // rows of K/V (== n_q_rows for local)
-    int32_t hq, hkv;
+    int32_t hq, hkv, d;
     float scale;
     int32_t causal;
     int32_t sync;                 // 0 local, 1 sync
@@ -122,7 +122,24 @@ struct PrefillParams {
     int32_t n_seg;
     int32_t cu[kMaxP + 1];        // query segments (local: also the KV segments)
 };
+// the same call for the SIMT kernels
+inline GenericParams generic_params(const PrefillParams &p)
+{
+    GenericParams g = {};
+    g.q = p.q; g.k = p.k; g.v = p.v; g.o = p.o; g.lse = p.lse;
+    g.n_rows = p.n_q_rows; g.hq = p.hq; g.hkv = p.hkv; g.d = p.d;
+    g.scale = p.scale; g.causal = p.causal; g.mode = p.sync ? kSync : kLocal; g.remote_only = p.remote_only;
+    g.kv_tok_stride = p.kv_head_major ? p.d : (int64_t)p.hkv * p.d;
+    g.kv_head_stride = p.kv_head_major ? p.total_kv * p.d : p.d;
+    g.kv_pos_head_stride = p.kv_head_major ? p.total_kv : 0;
+    g.total_kv = p.total_kv; g.q_pos = p.q_pos; g.kv_pos = p.kv_pos;
+    g.n_seg = p.n_seg;
+    for (int i = 0; i <= p.n_seg; ++i) g.cu[i] = p.cu[i];
+    return g;
+}
 bool prefill_sm100_supported(const Context *ctx);
+// whether the tensor-core kernel takes a bf16 call (its work-item arithmetic has a limited range)
+bool prefill_sm100_takes(const Context *ctx, const PrefillParams &p);
 // scratch bytes of the per-tile position tables of a general-position sync call
 size_t position_table_bytes(int hkv, int64_t n_q_rows, int64_t total_kv);
 cudaError_t launch_prefill_sm100(Context *ctx, const PrefillParams &p, cudaStream_t s);

@@ -1,4 +1,4 @@
-// bf16 prefill attention for sm_100a: TMA-fed, tcgen05 tensor cores, accumulators in TMEM,
+// bf16 prefill attention for sm_100a (head_dim <= 128): TMA-fed, tcgen05 tensor cores, accumulators in TMEM,
 // online softmax in fp32.  Serves fedattn_local (per-participant causal attention over packed
 // segments) and fedattn_sync (queries over the aggregated KV, causal on global positions).
 //
@@ -35,6 +35,7 @@
 #include <stdlib.h>
 #include <type_traits>
 
+#include "attn_row.cuh"
 #include "common.cuh"
 
 namespace fedattn {
@@ -43,7 +44,7 @@ namespace {
 
 constexpr int kTileM = 128;          // query rows per CTA
 constexpr int kTileN = 128;          // keys per KV tile
-constexpr int kD = 128;              // head dim
+constexpr int kBoxCols = 64;          // head-dim columns of one TMA box (128-byte swizzle); a tile is 1 or 2 boxes
 // two softmax warpgroups, one per sub-tile.  (Both on the same S tile, split by columns with the row
 // maxima exchanged through shared memory, was 2-4 % slower on dense sync; four warpgroups of 32 columns
 // 20 %.)  P is handed to the MMA warp in kSplit halves of kCols keys, so that PV starts on the first.
@@ -60,11 +61,12 @@ constexpr int kSoftmaxRegs = 216, kOtherRegs = 64;
 static_assert(2 * kSoftmaxRegs + kOtherRegs <= 496 && kSoftmaxRegs % 8 == 0 && kOtherRegs % 8 == 0, "register budget");
 constexpr int kProducerWarp = 4 * kSplit, kMmaWarp = 4 * kSplit + 1;
 static_assert(kSplit == 2 || kSplit == 4, "column split");
-constexpr uint32_t kTileBytes = kTileM * kD * 2;      // 32 KB: one Q, K or V tile
-constexpr uint32_t kHalfBytes = kTileBytes / 2;       // one 64-column TMA box
+constexpr uint32_t kHalfBytes = kTileM * kBoxCols * 2;   // 16 KB: one 64-column TMA box of a Q, K or V tile
 constexpr uint32_t kStageBytes = 32 * 128;            // output staging per softmax warp: 32 rows x 64 columns
-constexpr uint32_t kSmemBytes = 6 * kTileBytes + 1024 /*alignment slack*/ + 1024 /*barriers, published items*/ +
-                                2 * kSplit * 2 * kStageBytes;
+constexpr uint32_t smem_bytes(int boxes)
+{
+    return 6 * boxes * kHalfBytes + 1024 /*alignment slack*/ + 1024 /*barriers, published items*/ + 2 * kSplit * 2 * kStageBytes;
+}
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kColS = 0, kColO = 256;   // S (and P, aliased) of sub-tile t at kColS + 128 t; O at kColO + 128 t
 // P (bf16 pairs) of keys kCols q .. kCols q + kCols - 1 sits at S column kCols q: every 32-key chunk of P
@@ -84,6 +86,8 @@ struct KernelParams {
     int32_t n_kt;                    // KV tiles: ceil(total_kv / kTileN)
     int32_t *status;
     int32_t o_tma;                   // the output may leave through TMA stores (tensor map encoded)
+    int32_t pairs;                   // exact instances: visibility is tested on explicit positions, in any order
+    GenericParams row;               // exact instances: the same call for the row routine that repairs non-finite rows
 };
 
 // Position tables of a general-position call (ints, in this order): minimum and maximum position of
@@ -359,13 +363,25 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes
     return d;
 }
 
-// Instruction descriptor, kind::f16: D fp32, A/B bf16, M = 128, N = 128.
-constexpr uint32_t kIdescBase = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
-constexpr uint32_t kIdescQK = kIdescBase;                 // A, B K-major
-constexpr uint32_t kIdescPV = kIdescBase | (1u << 16);    // B (V) MN-major
+// Instruction descriptor, kind::f16: D fp32, A/B bf16, M = 128, N columns.
+__device__ __host__ constexpr uint32_t make_idesc(uint32_t n)
+{
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((128u >> 4) << 24);
+}
+constexpr uint32_t kIdescQK = make_idesc(128);                 // A, B K-major
+constexpr uint32_t kIdescPV = make_idesc(128) | (1u << 16);    // B (V) MN-major
 
 // n / d for 0 <= n < 2^28 and 1 <= d <= 4096, with magic = ceil(2^40 / d)
 __device__ __forceinline__ int fast_div(int n, uint64_t magic) { return (int)(((uint64_t)(uint32_t)n * magic) >> 40); }
+
+// m2 ln 2 + ln l with one rounding beside the logarithm's: the product and the sum keep what they round off
+__device__ __forceinline__ float lse_exact(float m2, float l)
+{
+    const float ln2 = 0.6931471805599453f, ln2_rest = (float)(0.69314718055994530942 - (double)0.6931471805599453f);
+    const float prod = m2 * ln2, prod_rest = fmaf(m2, ln2, -prod) + m2 * ln2_rest;
+    const float lg = logf(l), sum = prod + lg, back = sum - prod;
+    return sum + (((prod - (sum - back)) + (lg - back)) + prod_rest);
+}
 
 // number of entries of the non-decreasing array pos[0..n) that are <= x
 __device__ __forceinline__ int count_le(const int32_t *pos, int n, int x)
@@ -433,10 +449,51 @@ __device__ __forceinline__ int prefix_len(const PrefillParams &p, const Item &it
     return count_le_warp(it.kvp, T, pos, lane);
 }
 
+// Explicit positions without tables (exact instances): key x is visible to a row iff pos(x) <= lo, or, when
+// two_sided, pos(x) >= hi.  lo depends on the row (explicit or implied position) or on its segment (remote-only).
+struct PairRule {
+    int lo, hi;
+    bool two_sided;
+    __device__ bool sees(int pos) const { return pos <= lo || (two_sided && pos >= hi); }
+};
+__device__ __forceinline__ PairRule pair_rule(const PrefillParams &p, const Item &it, int r)
+{
+    PairRule rule;
+    rule.two_sided = p.remote_only && !p.causal;
+    rule.hi = p.remote_only ? p.cu[it.seg + 1] : 0;
+    if (p.remote_only) rule.lo = p.cu[it.seg] - 1;
+    else {
+        const int row = it.q_row0 + min(r, it.n_valid - 1);
+        rule.lo = p.q_pos ? __ldg(p.q_pos + row) : row;
+    }
+    return rule;
+}
+// Number of KV tiles up to the last one with a key visible to some row of the item's query tile.  Walks the key
+// positions backwards, 512 at a time (sixteen coalesced loads in flight per lane); called by a converged warp.
+__device__ __forceinline__ int last_visible_tile(const KernelParams &kp, const Item &it, int lane)
+{
+    const PrefillParams &p = kp.p;
+    PairRule any = pair_rule(p, it, lane);
+    for (int r = lane + 32; r < kTileM; r += 32) any.lo = max(any.lo, pair_rule(p, it, r).lo);
+    any.lo = __reduce_max_sync(0xffffffffu, any.lo);
+    const int T = (int)p.total_kv;
+    for (int base = ((T - 1) / 512) * 512; base >= 0; base -= 512) {
+        int last = -1;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int key = base + 32 * i + lane;
+            if (key < T && any.sees(it.kvp ? __ldg(it.kvp + key) : key)) last = key;
+        }
+        last = __reduce_max_sync(0xffffffffu, last);
+        if (last >= 0) return last / kTileN + 1;
+    }
+    return 0;
+}
+
 // Called by a converged warp (all lanes get the same item).  kSpecial: the kernel instance that also
 // serves explicit positions and bidirectional remote-only attention (two key ranges); the plain instance
 // carries none of their state.  Causal remote-only attention is one more prefix mask: plain instance.
-template <bool kSpecial>
+template <bool kSpecial, bool kExact>
 __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, int lane)
 {
     const PrefillParams &p = kp.p;
@@ -469,7 +526,11 @@ __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, in
     it.kvp = p.kv_pos ? p.kv_pos + (p.kv_head_major ? (int64_t)it.kvh * p.total_kv : 0) : nullptr;
     it.kv_begin = p.sync ? 0 : p.cu[seg];
     it.t_b0 = 0; it.a = 0; it.b = 0;
-    if (kSpecial && p.general) {
+    if (kExact && kp.pairs) {
+        // tiles up to the last one that holds a key some row of the tile may see
+        it.n_tiles = last_visible_tile(kp, it, lane);
+        it.n_a = it.n_tiles;
+    } else if (kSpecial && p.general) {
         // tiles up to the last one that holds a key position <= the tile's largest query position
         const PosTables pt = pos_tables(p.tab, kp.n_qtiles, p.kv_head_major ? p.hkv : 1, kp.n_kt);
         const int32_t *suf = pt.suf_min + (p.kv_head_major ? (size_t)it.kvh * kp.n_kt : 0);
@@ -500,18 +561,29 @@ __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, in
 // Barrier phases run on: per-CTA counters of KV tiles (git) and of non-empty items (qn) give stages
 // and parities, so the producer prefetches the next item's K/V and Q while the current item's last
 // tiles and its epilogue are still in flight.
-template <bool kSpecial>
+//
+// kBoxes: 64-column boxes per tile (head_dim <= 64: one; <= 128: two).  kExact: the weights P keep 16 bits of
+// mantissa instead of 8 (two bf16 parts, two PV products), every exponential is ex2, and rows that come out
+// non-finite are redone by the row routine.  It serves the head dims below 128, whose users had fp32 weights
+// from the SIMT kernel; P's two parts take exactly the S columns that the chunk's thread has already read.
+// Its extra product makes PV as long as S again (d = 64: 4 + 2 x 8 MMAs of half width per tile); a chunk costs
+// 6 more instructions per pair of keys.  Six ragged segments of 2160 tokens in all, 16 / 4 heads of 64 channels: local
+// 2436 us (one warp per row, fp32 FMA) -> 20 us, sync 10994 -> 45 us; the error of o against fp64 is the same to
+// three digits (the rounding of the bf16 output, 1.6e-3), lse 3.5e-8 -> 5e-8 relative (half a unit of fp32).
+template <bool kSpecial, int kBoxes, bool kExact>
 __global__ void __launch_bounds__(kThreads, 1)
 prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                      const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o,
                      const __grid_constant__ KernelParams kp)
 {
     extern __shared__ uint8_t smem_raw[];
+    constexpr uint32_t kTileBytes = kBoxes * kHalfBytes;
     const PrefillParams &p = kp.p;
+    const int d = kExact ? p.d : kBoxes * kBoxCols;
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint8_t *sQ = smem;                                  // [2 sub-tiles][32 KB]
-    uint8_t *sK = smem + 2 * kTileBytes;                 // [2 stages][32 KB]
-    uint8_t *sV = smem + 4 * kTileBytes;                 // [2 stages][32 KB]
+    uint8_t *sQ = smem;                                  // [2 sub-tiles][tile]
+    uint8_t *sK = smem + 2 * kTileBytes;                 // [2 stages][tile]
+    uint8_t *sV = smem + 4 * kTileBytes;                 // [2 stages][tile]
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + 6 * kTileBytes);
     uint64_t *q_full = bars + 0, *q_empty = bars + 1;
     uint64_t *k_full = bars + 2, *k_empty = bars + 4, *v_full = bars + 6, *v_empty = bars + 8;
@@ -578,7 +650,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         for (int k = 0; k < n_rounds; ++k) {
             const int item = item_of(k);
             if (item >= n_items) continue;
-            const Item it = decode_item<kSpecial>(kp, item, lane);
+            const Item it = decode_item<kSpecial, kExact>(kp, item, lane);
             if (lane == 0) {
                 if (pn >= 2) mbar_wait_call(item_empty + (pn & 1), ((pn >> 1) - 1) & 1, abort_flag, kp.status);
                 volatile int *slot = item_pub + (pn & 1) * 16;
@@ -589,10 +661,10 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 if (it.n_tiles > 0) {
                     // this item's Q on its way into L2: the load itself has to wait for the Q buffer
                     tma_prefetch_3d(&map_q, 0, it.head0, it.q_row0);
-                    tma_prefetch_3d(&map_q, 64, it.head0, it.q_row0);
+                    if (kBoxes == 2) tma_prefetch_3d(&map_q, 64, it.head0, it.q_row0);
                     if (it.valid1) {
                         tma_prefetch_3d(&map_q, 0, it.head0 + 1, it.q_row0);
-                        tma_prefetch_3d(&map_q, 64, it.head0 + 1, it.q_row0);
+                        if (kBoxes == 2) tma_prefetch_3d(&map_q, 64, it.head0 + 1, it.q_row0);
                     }
                 }
             }
@@ -604,10 +676,10 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 item_info[(qn & 1) * 2 + 1] = it.valid1 ? 2 : 1;
                 mbar_expect_tx(q_full, it.valid1 ? 2 * kTileBytes : kTileBytes);
                 tma_load_3d(sQ, &map_q, q_full, 0, it.head0, it.q_row0);
-                tma_load_3d(sQ + kHalfBytes, &map_q, q_full, 64, it.head0, it.q_row0);
+                if (kBoxes == 2) tma_load_3d(sQ + kHalfBytes, &map_q, q_full, 64, it.head0, it.q_row0);
                 if (it.valid1) {
                     tma_load_3d(sQ + kTileBytes, &map_q, q_full, 0, it.head0 + 1, it.q_row0);
-                    tma_load_3d(sQ + kTileBytes + kHalfBytes, &map_q, q_full, 64, it.head0 + 1, it.q_row0);
+                    if (kBoxes == 2) tma_load_3d(sQ + kTileBytes + kHalfBytes, &map_q, q_full, 64, it.head0 + 1, it.q_row0);
                 }
                 for (int j = 0; j < it.n_tiles; ++j) {
                     const int gt = git + j, st = gt & 1, use = gt >> 1;
@@ -617,11 +689,11 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     TRACE(j, 7);
                     mbar_expect_tx(k_full + st, kTileBytes);
                     tma_load_3d(sK + st * kTileBytes, &map_k, k_full + st, 0, c1, c2);
-                    tma_load_3d(sK + st * kTileBytes + kHalfBytes, &map_k, k_full + st, 64, c1, c2);
+                    if (kBoxes == 2) tma_load_3d(sK + st * kTileBytes + kHalfBytes, &map_k, k_full + st, 64, c1, c2);
                     if (gt >= 2) mbar_wait_call(v_empty + st, (use - 1) & 1, abort_flag, kp.status);
                     mbar_expect_tx(v_full + st, kTileBytes);
                     tma_load_3d(sV + st * kTileBytes, &map_v, v_full + st, 0, c1, c2);
-                    tma_load_3d(sV + st * kTileBytes + kHalfBytes, &map_v, v_full + st, 64, c1, c2);
+                    if (kBoxes == 2) tma_load_3d(sV + st * kTileBytes + kHalfBytes, &map_v, v_full + st, 64, c1, c2);
                 }
             }
             __syncwarp();
@@ -652,13 +724,15 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         // stay warp-uniform; one elected lane issues the tcgen05 instructions.  Issued from inside a
         // single-lane branch the same instructions sustain only ~83 cycles per MMA instead of 64.
         const bool leader = elect_one();
+        const uint32_t idesc_pv = make_idesc((uint32_t)(d + 15) & ~15u) | (1u << 16);     // exact instances: N = head_dim
         const uint32_t aQ = smem_u32(sQ), aK = smem_u32(sK), aV = smem_u32(sV);
         const uint64_t dQ = make_desc(aQ, 16, 1024), dK = make_desc(aK, 16, 1024), dV = make_desc(aV, kHalfBytes, 1024);
         auto issue_s = [&](int t, int st) {
             if (leader) {
 #pragma unroll
-                for (int ks = 0; ks < kD / 16; ++ks) {
+                for (int ks = 0; ks < kBoxes * kBoxCols / 16; ++ks) {
                     const uint32_t off = ((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4;       // descriptor units
+                    if (!kExact || 16 * ks < d)                  // columns beyond head_dim are zero in both tiles
                     umma_ss(tmem_base + kColS + t * 128, dQ + (uint64_t)(t * (kTileBytes >> 4) + off),
                             dK + (uint64_t)(st * (kTileBytes >> 4) + off), kIdescQK, ks > 0);
                 }
@@ -699,9 +773,15 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 #pragma unroll
                             for (int kk = 0; kk < kCols / 16; ++kk) {
                                 const int ks = q * (kCols / 16) + kk;
-                                umma_ts(tmem_base + kColO + t * 128, tmem_base + kColS + t * 128 + q * kCols + kk * 8,
-                                        dV + (uint64_t)(st * (kTileBytes >> 4) + ks * (2048 >> 4)), kIdescPV,
-                                        (j > 0 || ks > 0));
+                                const uint64_t desc = dV + (uint64_t)(st * (kTileBytes >> 4) + ks * (2048 >> 4));
+                                if (kExact) {                    // chunk of 32 keys: 16 columns of high parts, 16 of low parts
+                                    const uint32_t a = tmem_base + kColS + t * 128 + 32 * (ks >> 1) + 8 * (ks & 1);
+                                    umma_ts(tmem_base + kColO + t * 128, a, desc, idesc_pv, (j > 0 || ks > 0));
+                                    umma_ts(tmem_base + kColO + t * 128, a + 16, desc, idesc_pv, 1);
+                                } else {
+                                    umma_ts(tmem_base + kColO + t * 128, tmem_base + kColS + t * 128 + q * kCols + kk * 8, desc,
+                                            kIdescPV, (j > 0 || ks > 0));
+                                }
                             }
                         }
                     }
@@ -727,7 +807,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs));      // the two idle warps of that warpgroup
         // One of them checks what the prefix-count mask relies on: key positions that never decrease
         // along the aggregated rows of a head.  The CTAs share the pairs (i, i + 1) among them.
-        if (warp == kMmaWarp + 1 && p.kv_pos && !p.general && p.sync && (p.causal || p.remote_only) && p.total_kv > 1) {
+        if (!kExact && warp == kMmaWarp + 1 && p.kv_pos && !p.general && p.sync && (p.causal || p.remote_only) && p.total_kv > 1) {
             const int64_t per = p.total_kv - 1, total = per * (p.kv_head_major ? p.hkv : 1);
             bool bad = false;
             for (int64_t i = (int64_t)blockIdx.x * 32 + lane; i < total; i += (int64_t)gridDim.x * 32) {
@@ -791,7 +871,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             const float rm = fmaxf(max3(mx[0], mx[1], mx[2]), fmaxf(max3(mx[3], mx[4], mx[5]), fmaxf(mx[6], mx[7])));
             const float t_max = rm * sl2;
             if (j == 0) {
-                m_used = (t_max == -INFINITY) ? 0.f : t_max;
+                m_used = (!kExact && t_max == -INFINITY) ? 0.f : t_max;
             } else {
                 // The exponent reference moves only when the maximum grew by more than 2^8; then what
                 // this row has accumulated so far (O in TMEM, l) is rescaled to the new reference.
@@ -801,7 +881,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     mbar_wait(o_done + t, (gt - 1) & 1, abort_flag, kp.status);   // O holds tiles 0..j-1
                     tc_fence_after();
 #pragma unroll 1
-                    for (int oc = 0; oc < 4; ++oc) {
+                    for (int oc = 0; oc < 2 * kBoxes; ++oc) {
                         uint32_t o[32];
                         FEDATTN_TMEM_LD32(tO + oc * 32, o);
                         tmem_wait_ld();
@@ -813,17 +893,19 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 }
             }
             // ---- pass 2: exponentials, row sum, P ----
-            const uint64_t negm2 = pack_f32x2(-m_used, -m_used);
+            // (exact instances: a row that has seen no key yet keeps the reference -inf, all its weights are 0)
+            const float m_ref = kExact && m_used == -INFINITY ? 0.f : m_used;
+            const uint64_t negm2 = pack_f32x2(-m_ref, -m_ref);
             uint64_t sum2[4] = {0, 0, 0, 0};
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 uint32_t *cur = c == 0 ? s0 : (c == 1 ? s1 : (c == 2 ? s2 : s3));
-                uint32_t pk[16];
+                uint32_t pk[16], pl[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
                     const uint64_t x2 = fma_f32x2(pack_f32x2(__uint_as_float(cur[2 * i]), __uint_as_float(cur[2 * i + 1])), sl2_2, negm2);
                     float p0, p1;
-                    if (!kPartial && ((kPolyMask >> (i & 7)) & 1)) {
+                    if (!kExact && !kPartial && ((kPolyMask >> (i & 7)) & 1)) {
                         exp2_poly_x2(x2, p0, p1);
                     } else {
                         float x0, x1;
@@ -832,10 +914,17 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     }
                     sum2[i & 3] = add_f32x2(sum2[i & 3], pack_f32x2(p0, p1));
                     pk[i] = pack_bf16(p0, p1);
+                    if (kExact)                                 // what the rounding left over, as a second bf16
+                        pl[i] = pack_bf16(p0 - __uint_as_float(pk[i] << 16), p1 - __uint_as_float(pk[i] & 0xffff0000u));
                 }
                 // keys 32 c .. 32 c + 31 as bf16 pairs: columns 64 (c / 2) + 16 (c % 2) .., all inside S columns
                 // that this thread has already read
-                FEDATTN_TMEM_ST16(tS + 64 * (c >> 1) + 16 * (c & 1), pk);
+                if (kExact) {
+                    FEDATTN_TMEM_ST16(tS + 32 * c, pk);
+                    FEDATTN_TMEM_ST16(tS + 32 * c + 16, pl);
+                } else {
+                    FEDATTN_TMEM_ST16(tS + 64 * (c >> 1) + 16 * (c & 1), pk);
+                }
                 if (c & 1) {                                    // a 64-key half of P is complete: PV may start on it
                     tmem_wait_st();
                     tc_fence_before();
@@ -868,20 +957,35 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             if (t == 1 && !it.valid1) continue;                 // the pair's second head does not exist
             const int n_tiles = it.n_tiles;
             const bool valid = r < it.n_valid;
-            __nv_bfloat16 *orow = reinterpret_cast<__nv_bfloat16 *>(p.o) + ((int64_t)(it.q_row0 + r) * p.hq + it.head0 + t) * kD;
+            __nv_bfloat16 *orow = reinterpret_cast<__nv_bfloat16 *>(p.o) + ((int64_t)(it.q_row0 + r) * p.hq + it.head0 + t) * d;
             float *lse_p = p.lse ? p.lse + (int64_t)(it.q_row0 + r) * p.hq + it.head0 + t : nullptr;
             if (n_tiles == 0) {                                 // nothing visible to any row of the tile
                 if (valid) {
-#pragma unroll
-                    for (int c = 0; c < kD; c += 8) *reinterpret_cast<uint4 *>(orow + c) = make_uint4(0, 0, 0, 0);
+                    for (int c = 0; c < d; c += 8) *reinterpret_cast<uint4 *>(orow + c) = make_uint4(0, 0, 0, 0);
                     if (lse_p) *lse_p = -INFINITY;
                 }
                 continue;
             }
-            const bool two_range = kSpecial && p.sync && p.remote_only && !p.causal;
+            const bool two_range = kSpecial && p.sync && p.remote_only && !p.causal;      // (pairs comes first)
             const bool general = kSpecial && p.general;
+            const bool pairs = kExact && kp.pairs;
             int c_row = 0, n_full = 0, p_row = 0;
-            if (general) {
+            PairRule mine{0, 0, false}, all{0, 0, false};       // pairs: this row's rule, and what every row of the warp sees
+            int kpos[4] = {0, 0, 0, 0};                         // pairs: positions of keys 32 c + lane of the tile at hand
+            auto load_pos = [&](int j) {
+                const int T = (int)p.total_kv;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const int key = j * kTileN + 32 * c + lane;
+                    kpos[c] = it.kvp ? __ldg(it.kvp + min(key, T - 1)) : key;
+                }
+            };
+            if (pairs) {
+                mine = pair_rule(p, it, r);
+                all = mine;
+                all.lo = __reduce_min_sync(0xffffffffu, mine.lo);
+                load_pos(0);
+            } else if (general) {
                 // every (query, key) pair on its own positions; the tiles whose keys all lie at or below the
                 // tile's smallest query position (a prefix of the walk, see PosTables) need no test
                 const PosTables pt = pos_tables(p.tab, kp.n_qtiles, p.kv_head_major ? p.hkv : 1, kp.n_kt);
@@ -918,7 +1022,25 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 // which columns of this tile the thread's row sees: everything (warp-uniform), or a mask per chunk
                 bool full;
                 uint32_t vm[4] = {0, 0, 0, 0};
-                if (two_range) {                                // keys [0, a) and [b, T)
+                if (pairs) {
+                    // column 32 c + i of the tile is key j * 128 + 32 c + i, whose position lane i holds
+                    const int k0 = j * kTileN;
+                    bool see_all = true;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) see_all = see_all && k0 + 32 * c + lane < T && all.sees(kpos[c]);
+                    full = __all_sync(0xffffffffu, see_all);
+                    if (!full) {
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            uint32_t m = 0;
+#pragma unroll 4
+                            for (int i = 0; i < 32; ++i)
+                                if (mine.sees(__shfl_sync(0xffffffffu, kpos[c], i))) m |= 1u << i;
+                            vm[c] = m & below32(T - k0 - 32 * c);
+                        }
+                    }
+                    if (j + 1 < n_tiles) load_pos(j + 1);       // lands during this tile's visit
+                } else if (two_range) {                         // keys [0, a) and [b, T)
                     const int k0 = tile_of(it, j) * kTileN;     // first key of the tile
                     full = k0 + kTileN <= it.a || (k0 >= it.b && k0 + kTileN <= T);
                     if (!full) {
@@ -960,7 +1082,22 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
             // Full warps of rows leave through shared memory and TMA stores (a warp's 32 rows x 64 columns at a
             // time); a warp with rows beyond the segment writes its valid rows directly.
-            const bool by_tma = kp.o_tma && (r | 31) < it.n_valid;
+            bool by_tma = kp.o_tma && (r | 31) < it.n_valid;
+            uint32_t bad = 0;                                   // exact instances: rows of the warp with a non-finite channel
+            if (kExact) {
+                float probe = l_run * 0.f;                      // 0 unless something is Inf or NaN
+#pragma unroll 1
+                for (int c = 0; 32 * c < d; ++c) {
+                    uint32_t o[32];
+                    FEDATTN_TMEM_LD32(tO + 32 * c, o);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int i = 0; i < 32; ++i)
+                        if (32 * c + (i & ~7) < d) probe = fmaf(__uint_as_float(o[i]), 0.f, probe);
+                }
+                bad = __ballot_sync(0xffffffffu, valid && !(probe == 0.f));
+                by_tma = by_tma && bad == 0;
+            }
             uint8_t *my_stage = stage + (size_t)warp * kStageBytes;
             if (by_tma) {
                 if (lane == 0) tma_store_wait_read();           // the previous item's last store has read the staging rows
@@ -968,10 +1105,10 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 uint32_t oa[32], ob[32];
                 FEDATTN_TMEM_LD32(tO, oa);
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
+                for (int c = 0; c < 2 * kBoxes; ++c) {
                     uint32_t *cur = (c & 1) ? ob : oa, *nxt = (c & 1) ? oa : ob;
                     tmem_wait_ld();
-                    if (c < 3) {
+                    if (c < 2 * kBoxes - 1) {
                         FEDATTN_TMEM_LD32(tO + 32 * (c + 1), nxt);
                     } else {
                         tc_fence_before();
@@ -1000,18 +1137,19 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             } else {
                 // the rare path (a warp with rows beyond the segment) is kept short rather than fast
 #pragma unroll 1
-                for (int c = 0; c < 4; ++c) {
+                for (int c = 0; c < 2 * kBoxes; ++c) {
                     uint32_t o[32];
                     FEDATTN_TMEM_LD32(tO + 32 * c, o);
                     tmem_wait_ld();
-                    if (c == 3) {
+                    if (c == 2 * kBoxes - 1) {
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(o_free + t);
                     }
-                    if (valid) {
+                    if (valid && !((bad >> lane) & 1u)) {
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
+                            if (kExact && 32 * c + 8 * u >= d) break;
                             uint32_t w[4];
 #pragma unroll
                             for (int i = 0; i < 4; ++i)
@@ -1021,7 +1159,19 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     }
                 }
             }
-            if (valid && lse_p) *lse_p = l_run > 0.f ? (m_run + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
+            if (valid && lse_p) *lse_p = !(l_run > 0.f) ? -INFINITY
+                                         : kExact ? lse_exact(m_run, l_run)
+                                                  : (m_run + log2f(l_run)) * 0.6931471805599453f;
+            if (kExact && bad) {
+                if (lane == 0) tma_store_wait_read();           // the staging rows are free again: the routine's row of Q
+                __syncwarp();
+#pragma unroll 1
+                for (uint32_t left = bad; left; left &= left - 1) {
+                    attn_row_warp<__nv_bfloat16>(kp.row, it.q_row0 + (r & ~31) + __ffs(left) - 1, it.head0 + t,
+                                                 reinterpret_cast<float *>(my_stage));
+                    __syncwarp();
+                }
+            }
             gsub += n_tiles;
         }
         if (lane == 0) tma_store_wait_read();                   // the staging rows stay alive until they are read
@@ -1143,22 +1293,33 @@ extern "C" int fedattn_debug_read_trace(long long *host, int n)
 
 bool prefill_sm100_supported(const Context *ctx) { return ctx->encode_tiled != nullptr; }
 
-// [rows, heads, 128] bf16 (token-major) or [heads, rows, 128] (head-major); boxes of 64 columns x 128 rows.
-static bool encode_map(const Context *ctx, CUtensorMap *map, const void *base, int64_t rows, int heads, bool head_major,
+// The range of fast_div: calls outside it run on the SIMT kernel where that served them before (head_dim < 128).
+bool prefill_sm100_takes(const Context *ctx, const PrefillParams &p)
+{
+    if (!prefill_sm100_supported(ctx)) return false;
+    if (p.d == 128) return true;
+    const int64_t per_tile = (int64_t)p.hkv * ((p.hq / p.hkv + 1) / 2);
+    const int64_t n_qtiles = p.n_q_rows / kTileM + p.n_seg;          // at most
+    return per_tile <= 4096 && n_qtiles * per_tile < (1LL << 28) && p.n_q_rows < 0x7fffff00LL && p.total_kv < 0x7fffff00LL;
+}
+
+// [rows, heads, d] bf16 (token-major) or [heads, rows, d] (head-major); boxes of 64 columns x 128 rows.  Columns
+// beyond d read as zero and are not written.
+static bool encode_map(const Context *ctx, CUtensorMap *map, const void *base, int64_t rows, int heads, int d, bool head_major,
                        int box_rows = kTileN)
 {
     EncodeTiledFn fn = reinterpret_cast<EncodeTiledFn>(ctx->encode_tiled);
     cuuint64_t dims[3], strides[2];
     cuuint32_t box[3], estr[3] = {1, 1, 1};
-    dims[0] = kD;
+    dims[0] = (cuuint64_t)d;
     if (head_major) {
         dims[1] = (cuuint64_t)rows; dims[2] = (cuuint64_t)heads;
-        strides[0] = kD * 2; strides[1] = (cuuint64_t)rows * kD * 2;
-        box[0] = 64; box[1] = (cuuint32_t)box_rows; box[2] = 1;
+        strides[0] = (cuuint64_t)d * 2; strides[1] = (cuuint64_t)rows * d * 2;
+        box[0] = kBoxCols; box[1] = (cuuint32_t)box_rows; box[2] = 1;
     } else {
         dims[1] = (cuuint64_t)heads; dims[2] = (cuuint64_t)rows;
-        strides[0] = kD * 2; strides[1] = (cuuint64_t)heads * kD * 2;
-        box[0] = 64; box[1] = 1; box[2] = (cuuint32_t)box_rows;
+        strides[0] = (cuuint64_t)d * 2; strides[1] = (cuuint64_t)heads * d * 2;
+        box[0] = kBoxCols; box[1] = 1; box[2] = (cuuint32_t)box_rows;
     }
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1180,10 +1341,16 @@ cudaError_t launch_wait_selftest(Context *ctx, int max_polls, cudaStream_t s)
 
 cudaError_t launch_prefill_sm100(Context *ctx, const PrefillParams &p, cudaStream_t s)
 {
-    static_assert(sizeof(KernelParams) < 3000, "kernel parameter block too large");
+    static_assert(sizeof(KernelParams) + 4 * sizeof(CUtensorMap) <= 4096, "kernel parameter block too large");
     KernelParams kp;
     kp.p = p;
     kp.status = ctx->status;
+    kp.pairs = 0;
+    if (p.d < 128) {
+        // positions in any order, as the row routine takes them, and no tables: those calls keep off the scratch
+        kp.pairs = p.sync && (p.kv_pos || p.q_pos) && (p.causal || p.remote_only);
+        kp.row = generic_params(p);
+    }
     kp.n_kt = (int32_t)((p.total_kv + kTileN - 1) / kTileN);
     int64_t n_qtiles = 0;
     for (int n = 0; n < p.n_seg; ++n) {
@@ -1216,31 +1383,35 @@ cudaError_t launch_prefill_sm100(Context *ctx, const PrefillParams &p, cudaStrea
     for (int i = 0; i < kMaxP; ++i) kp.magic_small[i] = magic(i + 1);
     const int64_t blocks = items < ctx->sm_count ? items : ctx->sm_count;     // persistent: one CTA per SM
     CUtensorMap mq, mk, mv, mo;
-    if (!encode_map(ctx, &mq, p.q, p.n_q_rows, p.hq, false) ||
-        !encode_map(ctx, &mk, p.k, p.total_kv, p.hkv, p.kv_head_major != 0) ||
-        !encode_map(ctx, &mv, p.v, p.total_kv, p.hkv, p.kv_head_major != 0))
+    if (!encode_map(ctx, &mq, p.q, p.n_q_rows, p.hq, p.d, false) ||
+        !encode_map(ctx, &mk, p.k, p.total_kv, p.hkv, p.d, p.kv_head_major != 0) ||
+        !encode_map(ctx, &mv, p.v, p.total_kv, p.hkv, p.d, p.kv_head_major != 0))
         return cudaErrorInvalidValue;
     // the output as [rows, heads, 128] in boxes of 32 rows x 64 columns; a base the encoder refuses (alignment)
     // leaves the kernel on its direct stores
-    kp.o_tma = encode_map(ctx, &mo, p.o, p.n_q_rows, p.hq, false, 32) ? 1 : 0;
+    kp.o_tma = encode_map(ctx, &mo, p.o, p.n_q_rows, p.hq, p.d, false, 32) ? 1 : 0;
     if (!kp.o_tma) mo = mq;
-    static bool attr_set[64] = {};
-    if (!attr_set[ctx->device & 63]) {
-        cudaError_t e = cudaFuncSetAttribute(prefill_sm100_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(prefill_sm100_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    // the plain instance serves local attention and sync attention under the prefix mask; explicit positions
+    // and bidirectional remote-only attention run the instance that carries their extra state; head dims below
+    // 128 run the exact instances
+    typedef void (*Kernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const KernelParams);
+    static const Kernel kernels[4] = {prefill_sm100_kernel<false, 2, false>, prefill_sm100_kernel<true, 2, false>,
+                                      prefill_sm100_kernel<true, 1, true>, prefill_sm100_kernel<true, 2, true>};
+    const int which = p.d < 128 ? (p.d <= kBoxCols ? 2 : 3) : (p.general || (p.remote_only && !p.causal)) ? 1 : 0;
+    const uint32_t smem = smem_bytes(which == 2 ? 1 : 2);
+    static bool attr_set[64][4] = {};
+    if (!attr_set[ctx->device & 63][which]) {
+        cudaError_t e = cudaFuncSetAttribute(kernels[which], cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         // the register split inside the kernel has to fit into what the launch allocates: an increase that
         // the CTA's pool cannot serve would wait for ever, so such a build is refused here
-        cudaFuncAttributes fa0, fa1;
-        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa0, prefill_sm100_kernel<false>);
-        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa1, prefill_sm100_kernel<true>);
-        if (e == cudaSuccess && (3 * fa0.numRegs < 2 * kSoftmaxRegs + kOtherRegs || 3 * fa1.numRegs < 2 * kSoftmaxRegs + kOtherRegs))
-            e = cudaErrorLaunchOutOfResources;
+        cudaFuncAttributes fa;
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernels[which]);
+        if (e == cudaSuccess && 3 * fa.numRegs < 2 * kSoftmaxRegs + kOtherRegs) e = cudaErrorLaunchOutOfResources;
         if (e != cudaSuccess) {
             if (getenv("FEDATTN_DEBUG")) fprintf(stderr, "prefill_sm100_kernel attribute: %s\n", cudaGetErrorString(e));
             return e;
         }
-        attr_set[ctx->device & 63] = true;
+        attr_set[ctx->device & 63][which] = true;
     }
     if (p.general) {
         // the per-tile position tables first (same stream): the walk and the unmasked fast path read them
@@ -1251,10 +1422,7 @@ cudaError_t launch_prefill_sm100(Context *ctx, const PrefillParams &p, cudaStrea
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    // the plain instance serves local attention and sync attention under the prefix mask; explicit positions
-    // and remote-only attention run the instance that carries their extra state
-    if (p.general || (p.remote_only && !p.causal)) prefill_sm100_kernel<true><<<(unsigned)blocks, kThreads, kSmemBytes, s>>>(mq, mk, mv, mo, kp);
-    else prefill_sm100_kernel<false><<<(unsigned)blocks, kThreads, kSmemBytes, s>>>(mq, mk, mv, mo, kp);
+    kernels[which]<<<(unsigned)blocks, kThreads, smem, s>>>(mq, mk, mv, mo, kp);
     ++ctx->launches;
     ++ctx->tc_launches;
     cudaError_t e = cudaGetLastError();

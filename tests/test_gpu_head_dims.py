@@ -1,0 +1,150 @@
+"""The prefill calls at every storage type and head_dim that the bf16 head_dim-128 kernel does not serve: bf16 with
+fewer channels (tensor cores, weights in two bf16 parts) and fp32 (tiled SIMT), against an fp64 evaluation of the
+same inputs.  The weights keep more bits than the output has, so the bf16 bound is the rounding of the output: half
+a unit in the last of 8 significant bits is at most 2^-8 |o|, plus 2^-14 for weights and sums; fp32 sums of at most
+a few hundred O(1) terms stay within 2^-24 * sqrt(terms) * a small factor, 1e-5 is generous."""
+import numpy as np
+import pytest
+import torch
+
+import fedattn_inputs as fi
+from helpers import Runner, dev, fa, host
+
+pytestmark = pytest.mark.gpu
+
+KINDS = [("bf16", 4, 2, 8), ("bf16", 3, 1, 40), ("bf16", 8, 2, 64), ("bf16", 5, 5, 72), ("bf16", 6, 2, 96), ("bf16", 2, 1, 120),
+         ("f32", 4, 4, 64), ("f32", 6, 2, 40), ("f32", 7, 1, 128), ("f32", 3, 3, 72), ("f32", 2, 2, 8)]
+
+
+def gen(seed, lens, hq, hkv, d, dtype):
+    return fi.Workload("t", seed, tuple(int(x) for x in lens), hq, hkv, d, dtype, 1.0).qkv()
+
+
+def reference(q, k, v, visible):
+    """fp64 attention; visible: [rows, keys] or [heads of K, rows, keys]; k, v: [keys, hkv, d]."""
+    rows, hq, d = q.shape
+    g = hq // k.shape[1]
+    o, lse = np.zeros((rows, hq, d)), np.full((rows, hq), -np.inf)
+    for h in range(hq):
+        vis = visible if visible.ndim == 2 else visible[h // g]
+        s = np.where(vis, q[:, h].astype(np.float64) @ k[:, h // g].astype(np.float64).T / np.sqrt(d), -np.inf)
+        some = vis.any(1)
+        m = np.where(some, s.max(1, initial=-np.inf), 0.0)
+        p = np.exp(s - m[:, None])
+        z = p.sum(1)
+        # excluded keys take no part, whatever their value rows hold
+        pv = np.array([p[i, vis[i]] @ v[vis[i], h // g].astype(np.float64) for i in range(rows)])
+        o[some, h] = pv[some] / z[some, None]
+        lse[some, h] = m[some] + np.log(z[some])
+    return o, lse
+
+
+def check(got, want, dtype, what):
+    (o, lse), (wo, wl) = got, want
+    assert np.isfinite(o).all(), what
+    tol = 2.0 ** -8 * np.abs(wo) + 2.0 ** -14 if dtype == "bf16" else 1e-5
+    assert (np.abs(o - wo) <= tol).all(), (what, np.abs(o - wo).max())
+    empty = np.isneginf(wl)
+    assert np.array_equal(np.isneginf(lse), empty), what
+    assert empty.all() or np.abs(lse[~empty] - wl[~empty]).max() <= 1e-5, what
+
+
+def owners(lens):
+    return np.repeat(np.arange(len(lens)), lens)
+
+
+@pytest.mark.parametrize("lens", [[1], [127, 1, 0, 128], [129, 300, 64], [33, 257, 5, 512]])
+@pytest.mark.parametrize("causal", [True, False])
+@pytest.mark.parametrize("dtype,hq,hkv,d", KINDS)
+def test_local_and_sync_by_row_index(dtype, hq, hkv, d, causal, lens):
+    q, k, v = gen(7, lens, hq, hkv, d, dtype)
+    L, own = sum(lens), owners(lens)
+    r = Runner(len(lens), hq, hkv, d, dtype, L, causal=causal)
+    below = np.tri(L, dtype=bool) if causal else np.ones((L, L), bool)
+    check(r.local(q, k, v, lens), reference(q, k, v, below & (own[:, None] == own)), dtype, "local")
+    check(r.sync(q, k, v), reference(q, k, v, below), dtype, "sync")
+    T = max(1, L - 3)                                             # fewer keys than queries, head-major
+    kh, vh = (np.ascontiguousarray(np.transpose(x[:T], (1, 0, 2))) for x in (k, v))
+    check(r.sync(q, kh, vh, head_major=True), reference(q, k[:T], v[:T], below[:, :T]), dtype, "sync, head-major")
+
+
+@pytest.mark.parametrize("dtype,hq,hkv,d", KINDS)
+def test_positions_in_any_order(dtype, hq, hkv, d):
+    """Key positions that go up and down, per head, with and without explicit query positions; the first tiles of
+    the walk may hold no visible key of a row whose later logits are far below zero."""
+    lens = [200, 131, 390]
+    L = sum(lens)
+    q, k, v = gen(8, lens, hq, hkv, d, dtype)
+    q = q * 3.0 if dtype == "f32" else q
+    rng = np.random.default_rng(3)
+    pos = np.stack([rng.permutation(L + 40)[:L] for _ in range(hkv)]).astype(np.int32)
+    qp = rng.permutation(L).astype(np.int32)
+    kh, vh = (np.ascontiguousarray(np.transpose(x, (1, 0, 2))) for x in (k, v))
+    r = Runner(len(lens), hq, hkv, d, dtype, L)
+    check(r.sync(q, kh, vh, kv_pos=pos, head_major=True), reference(q, k, v, pos[:, None, :] <= np.arange(L)[None, :, None]),
+          dtype, "row index against kv_pos")
+    check(r.sync(q, kh, vh, kv_pos=pos, q_pos=qp, head_major=True), reference(q, k, v, pos[:, None, :] <= qp[None, :, None]),
+          dtype, "q_pos against kv_pos")
+    check(r.sync(q, k, v, q_pos=qp), reference(q, k, v, np.arange(L)[None] <= qp[:, None]), dtype, "q_pos alone")
+    asc = np.sort(pos[0])
+    check(r.sync(q, k, v, kv_pos=asc), reference(q, k, v, asc[None] <= np.arange(L)[:, None]), dtype, "ascending kv_pos")
+
+
+@pytest.mark.parametrize("causal", [True, False])
+@pytest.mark.parametrize("dtype,hq,hkv,d", KINDS)
+def test_remote_only(dtype, hq, hkv, d, causal):
+    lens = [140, 0, 90, 260, 33]
+    L, own = sum(lens), owners(lens)
+    q, k, v = gen(9, lens, hq, hkv, d, dtype)
+    cu = np.concatenate([[0], np.cumsum(lens)])
+    m = fa()
+    r = Runner(len(lens), hq, hkv, d, dtype, L, causal=causal)
+    kept = np.sort(np.random.default_rng(4).permutation(L)[:301]).astype(np.int32)
+    for pos, what in ((kept, "ascending"), (kept[::-1].copy(), "descending"), (None, "all rows")):
+        keys = np.arange(L) if pos is None else pos
+        qd, kd, vd = dev(q, dtype), dev(k[keys], dtype), dev(v[keys], dtype)
+        o = torch.full_like(qd, float("nan"))
+        lse = torch.full((L, hq), float("nan"), device="cuda")
+        m.fedattn_sync_remote(r.ctx, r.shape, qd, cu, kd, vd, None if pos is None else torch.from_numpy(pos).cuda(), len(keys),
+                              False, o, lse)
+        assert r.poll() == 0
+        before, after = keys[None] < cu[:-1][own][:, None], keys[None] >= cu[1:][own][:, None]
+        check((host(o), host(lse)), reference(q, k[keys], v[keys], before if causal else before | after), dtype, what)
+
+
+@pytest.mark.parametrize("dtype,hq,hkv,d", KINDS)
+def test_rows_that_see_no_logit_near_zero(dtype, hq, hkv, d):
+    """A row whose first key tiles are all excluded and whose visible logits are near -300: its weights must not be
+    taken against a reference of 0."""
+    L = 400
+    q, k, v = gen(10, [L], hq, hkv, d, dtype)
+    q = np.full_like(q, 4.0)
+    k = k * 0.25 if dtype == "f32" else np.round(k * 4) / 16
+    k -= 75.0 / np.sqrt(d)
+    if dtype == "bf16":
+        k = torch.from_numpy(k).to(torch.bfloat16).float().numpy()
+    pos = np.arange(L, dtype=np.int32)[::-1].copy()               # row 0 sees the last key only
+    r = Runner(1, hq, hkv, d, dtype, L)
+    o, lse = r.sync(q, k, v, kv_pos=pos, q_pos=np.arange(L, dtype=np.int32))
+    wo, wl = reference(q, k, v, pos[None] <= np.arange(L)[:, None])
+    assert wl.max() < -200
+    assert np.abs(lse - wl).max() <= 1e-4 and np.abs(o - wo).max() <= (2e-2 if dtype == "bf16" else 1e-3)
+
+
+@pytest.mark.parametrize("dtype,hq,hkv,d", KINDS)
+def test_excluded_rows_may_hold_anything(dtype, hq, hkv, d):
+    """Inf and NaN in value rows (and NaN in key rows) that the mask excludes do not reach the output; rows that do
+    see them come out non-finite."""
+    lens = [150, 130, 100]
+    L, own = sum(lens), owners(lens)
+    q, k, v = gen(11, lens, hq, hkv, d, dtype)
+    v[140], v[149, 0, 1], k[279], v[160:170] = np.inf, np.nan, np.nan, -np.inf
+    visible = np.tri(L, dtype=bool) & (own[:, None] == own)
+    spoilt = visible[:, [140, 149, 279] + list(range(160, 170))].any(1)
+    r = Runner(len(lens), hq, hkv, d, dtype, L)
+    for (o, lse), vis in ((r.local(q, k, v, lens), visible), (r.sync(q, k, v), np.tri(L, dtype=bool))):
+        spoilt = vis[:, [140, 149, 279] + list(range(160, 170))].any(1)
+        with np.errstate(invalid="ignore"):
+            wo, wl = reference(q, k, v, vis)
+        check((o[~spoilt], lse[~spoilt]), (wo[~spoilt], wl[~spoilt]), dtype, "excluded Inf and NaN")
+        assert not np.isfinite(o[spoilt][:, 0]).all(1).any()
