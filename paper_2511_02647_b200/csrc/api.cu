@@ -58,7 +58,12 @@ bool on_tensor_cores(const Context *c, const PrefillParams &p, int dtype)
 cudaError_t launch_prefill(Context *c, const PrefillParams &p, int dtype, cudaStream_t s)
 {
     if (on_tensor_cores(c, p, dtype)) return launch_prefill_sm100(c, p, s);
-    return launch_attn_generic(generic_params(p), dtype, s, &c->launches);
+    int64_t max_kv = p.total_kv;
+    if (!p.sync) {
+        max_kv = 0;
+        for (int n = 0; n < p.n_seg; ++n) max_kv = p.cu[n + 1] - p.cu[n] > max_kv ? p.cu[n + 1] - p.cu[n] : max_kv;
+    }
+    return launch_attn_generic(generic_params(p), dtype, (int)max_kv, c->sm_count, s, &c->launches);
 }
 
 struct DeviceGuard {
@@ -366,7 +371,7 @@ fedattn_status fedattn_decode(fedattn_ctx *ctx, const fedattn_shape *shape, int3
         p.kv_tok_stride = (int64_t)shape->n_kv_heads * shape->head_dim;
         p.kv_head_stride = shape->head_dim;
         p.kv_len = kv_len; p.cache_stride = cache_stride;
-        err = launch_attn_generic(p, shape->dtype, s, &ctx->c.launches);
+        err = launch_attn_generic(p, shape->dtype, max_kv_len, ctx->c.sm_count, s, &ctx->c.launches);
     }
     return err == cudaSuccess ? FEDATTN_OK : FEDATTN_ERR_CUDA;
 }

@@ -20,8 +20,8 @@ template <> __device__ __forceinline__ void st_f<__nv_bfloat16>(__nv_bfloat16 *p
     *p = __float2bfloat16_rn(x);
 }
 
-// Called by a converged warp; q_s: d floats of shared memory of its own.
-template <typename T>
+// Called by a converged warp; q_s: d floats of shared memory of its own, which kQLoaded says hold the row of Q.
+template <typename T, bool kQLoaded = false>
 __device__ __noinline__ void attn_row_warp(const GenericParams &p, int64_t row, int h, float *q_s)
 {
     const int lane = threadIdx.x & 31;
@@ -71,7 +71,8 @@ __device__ __noinline__ void attn_row_warp(const GenericParams &p, int64_t row, 
     const int32_t *kvp = p.kv_pos ? p.kv_pos + (int64_t)kvh * p.kv_pos_head_stride : nullptr;
 
     const T *qrow = reinterpret_cast<const T *>(p.q) + (row * p.hq + h) * d;
-    for (int c = lane; c < d; c += 32) q_s[c] = ld_f(qrow + c);
+    if (!kQLoaded)
+        for (int c = lane; c < d; c += 32) q_s[c] = ld_f(qrow + c);
     __syncwarp();
 
     float m = -INFINITY, l = 0.f;

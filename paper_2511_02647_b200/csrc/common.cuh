@@ -55,7 +55,7 @@ EarlyStart early_start(int device, cudaStream_t stream, const MemRange *in, int 
 // The owner's sequence numbers are about to lose their meaning (its context is being destroyed).
 void early_start_forget(int device, const void *owner);
 
-// ---- generic SIMT attention (fp32 or bf16 storage, any head_dim <= 128) --------------------
+// ---- tiled SIMT attention (fp32 or bf16 storage, any head_dim <= 128) -----------------------
 enum GenericMode { kLocal = 0, kSync = 1, kDecodeLocal = 2, kDecodeSync = 3 };
 
 struct GenericParams {
@@ -81,7 +81,8 @@ struct GenericParams {
     int32_t cu[kMaxP + 1];        // local: segment offsets
 };
 
-cudaError_t launch_attn_generic(const GenericParams &p, int dtype, cudaStream_t s, int64_t *launches);
+// max_kv: an upper bound (decode: the caller's) on the keys of one row, which only sets how many CTAs share them
+cudaError_t launch_attn_generic(const GenericParams &p, int dtype, int max_kv, int sm_count, cudaStream_t s, int64_t *launches);
 
 // ---- aggregation -----------------------------------------------------------------------------
 struct PartsParams {
