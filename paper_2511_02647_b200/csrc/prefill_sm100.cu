@@ -80,7 +80,8 @@ struct KernelParams {
     int32_t ord_nt[kMaxP];           // their query-tile counts
     int32_t band_rank[kMaxP + 1];    // tiles ranked above band b (levels ord_nt[b+1] < lv <= ord_nt[b])
     int32_t group;                   // query heads per KV head
-    uint64_t magic_per_tile, magic_ppg, magic_small[kMaxP];   // ceil(2^40 / d) for d = per_tile, ppg, 1..kMaxP
+    int32_t straddle;                // odd groups: ranked tiles have 256 rows, the last heads of their halves form an item
+    uint64_t magic_per_tile, magic_ppk, magic_small[kMaxP];   // ceil(2^40 / d) for d = items per tile, per KV head, 1..kMaxP
     int32_t n_qtiles;                // total query tiles
     int32_t n_items;                 // query tiles x KV heads x head pairs
     int32_t n_kt;                    // KV tiles: ceil(total_kv / kTileN)
@@ -418,13 +419,17 @@ __device__ __forceinline__ int count_le_warp(const int32_t *pos, int n, int x, i
 
 }  // namespace
 
-// One unit of work: a 128-row query tile x one pair of query heads that share a KV head.
+// One unit of work: two sub-tiles of 128 query rows x one query head that share a KV head and a segment: two heads
+// of one query tile, or (odd groups) the last head of two neighbouring query tiles.  Sub-tile 1 always has work and
+// at least as many KV tiles as sub-tile 0, which may be missing (n_valid == 0).
+struct Sub {
+    int head, q_row0, n_valid, n_tiles;
+};
 struct Item {
-    int kvh, head0, q_row0, n_valid, seg, kv_begin, n_tiles;
+    int kvh, seg, kv_begin;
     // The walk visits KV tiles 0 .. n_a-1 and then t_b0, t_b0+1, ...  (n_a == n_tiles unless the allowed
     // keys are two ranges: bidirectional remote-only attention, keys [0, a) and [b, T)).
     int n_a, t_b0, a, b;
-    bool valid1;                       // the pair's second head exists (odd group size: last pair is single)
     const int32_t *kvp;                // positions of this KV head's aggregated rows (sparse sync), or null
 };
 __device__ __forceinline__ int tile_of(const Item &it, int j) { return j < it.n_a ? j : it.t_b0 + (j - it.n_a); }
@@ -432,9 +437,9 @@ __device__ __forceinline__ int tile_of(const Item &it, int j) { return j < it.n_
 // allowed-prefix length c(row): keys kv_begin .. kv_begin + c - 1 are visible to query row r of the tile.
 // Called by a converged warp with the same r in every lane (the searches are warp-cooperative).
 template <bool kSpecial>
-__device__ __forceinline__ int prefix_len(const PrefillParams &p, const Item &it, int r, int lane)
+__device__ __forceinline__ int prefix_len(const PrefillParams &p, const Item &it, const Sub &sub, int r, int lane)
 {
-    const int pos = it.q_row0 + r;
+    const int pos = sub.q_row0 + r;
     const int T = (int)p.total_kv;
     if (!p.sync) {
         const int seg_len = p.cu[it.seg + 1] - p.cu[it.seg];
@@ -456,25 +461,25 @@ struct PairRule {
     bool two_sided;
     __device__ bool sees(int pos) const { return pos <= lo || (two_sided && pos >= hi); }
 };
-__device__ __forceinline__ PairRule pair_rule(const PrefillParams &p, const Item &it, int r)
+__device__ __forceinline__ PairRule pair_rule(const PrefillParams &p, const Item &it, const Sub &sub, int r)
 {
     PairRule rule;
     rule.two_sided = p.remote_only && !p.causal;
     rule.hi = p.remote_only ? p.cu[it.seg + 1] : 0;
     if (p.remote_only) rule.lo = p.cu[it.seg] - 1;
     else {
-        const int row = it.q_row0 + min(r, it.n_valid - 1);
+        const int row = sub.q_row0 + min(r, sub.n_valid - 1);
         rule.lo = p.q_pos ? __ldg(p.q_pos + row) : row;
     }
     return rule;
 }
-// Number of KV tiles up to the last one with a key visible to some row of the item's query tile.  Walks the key
+// Number of KV tiles up to the last one with a key visible to some row of the sub-tile.  Walks the key
 // positions backwards, 512 at a time (sixteen coalesced loads in flight per lane); called by a converged warp.
-__device__ __forceinline__ int last_visible_tile(const KernelParams &kp, const Item &it, int lane)
+__device__ __forceinline__ int last_visible_tile(const KernelParams &kp, const Item &it, const Sub &sub, int lane)
 {
     const PrefillParams &p = kp.p;
-    PairRule any = pair_rule(p, it, lane);
-    for (int r = lane + 32; r < kTileM; r += 32) any.lo = max(any.lo, pair_rule(p, it, r).lo);
+    PairRule any = pair_rule(p, it, sub, lane);
+    for (int r = lane + 32; r < kTileM; r += 32) any.lo = max(any.lo, pair_rule(p, it, sub, r).lo);
     any.lo = __reduce_max_sync(0xffffffffu, any.lo);
     const int T = (int)p.total_kv;
     for (int base = ((T - 1) / 512) * 512; base >= 0; base -= 512) {
@@ -494,21 +499,18 @@ __device__ __forceinline__ int last_visible_tile(const KernelParams &kp, const I
 // serves explicit positions and bidirectional remote-only attention (two key ranges); the plain instance
 // carries none of their state.  Causal remote-only attention is one more prefix mask: plain instance.
 template <bool kSpecial, bool kExact>
-__device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, int lane)
+__device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, int lane, Sub (&sub)[2])
 {
     const PrefillParams &p = kp.p;
     Item it;
-    // divisions by launch constants go through host-computed reciprocals (kp.magic_*): this runs once
-    // per item in every role, on the softmax threads' critical path
+    // divisions by launch constants go through host-computed reciprocals (kp.magic_*)
     const int g = kp.group;
-    const int ppg = (g + 1) >> 1;                               // head pairs per KV head
-    const int per_tile = p.hkv * ppg;
+    const int ppk = kp.straddle ? g : (g + 1) >> 1;             // items per ranked tile and KV head
+    const int per_tile = p.hkv * ppk;
     const int tile_rank = fast_div(item, kp.magic_per_tile);
     const int rem = item - tile_rank * per_tile;
-    it.kvh = fast_div(rem, kp.magic_ppg);
-    const int pair = rem - it.kvh * ppg;
-    it.head0 = it.kvh * g + 2 * pair;
-    it.valid1 = 2 * pair + 1 < g;
+    it.kvh = fast_div(rem, kp.magic_ppk);
+    const int u = rem - it.kvh * ppk;
     // Heavy tiles first: query tiles are ranked by their index inside their segment, descending
     // (a causal tile's KV-tile count is that index + 1).  Level lv holds tile lv-1 of every segment
     // that has at least lv tiles.  With the segments sorted by tile count (ord_nt, descending), the
@@ -520,39 +522,72 @@ __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, in
     const int down = fast_div(in_band, kp.magic_small[b]);      // in_band / (b + 1): levels below the band's top
     const int lo = kp.ord_nt[b] - down;
     const int seg = kp.ord_seg[in_band - down * (b + 1)];
+    const int end = p.cu[seg + 1];
     it.seg = seg;
-    it.q_row0 = p.cu[seg] + (lo - 1) * kTileM;
-    it.n_valid = min(kTileM, p.cu[seg + 1] - it.q_row0);
     it.kvp = p.kv_pos ? p.kv_pos + (p.kv_head_major ? (int64_t)it.kvh * p.total_kv : 0) : nullptr;
     it.kv_begin = p.sync ? 0 : p.cu[seg];
     it.t_b0 = 0; it.a = 0; it.b = 0;
-    if (kExact && kp.pairs) {
-        // tiles up to the last one that holds a key some row of the tile may see
-        it.n_tiles = last_visible_tile(kp, it, lane);
-        it.n_a = it.n_tiles;
-    } else if (kSpecial && p.general) {
-        // tiles up to the last one that holds a key position <= the tile's largest query position
-        const PosTables pt = pos_tables(p.tab, kp.n_qtiles, p.kv_head_major ? p.hkv : 1, kp.n_kt);
-        const int32_t *suf = pt.suf_min + (p.kv_head_major ? (size_t)it.kvh * kp.n_kt : 0);
-        it.n_tiles = count_le_warp(suf, kp.n_kt, __ldg(pt.q_max + (it.q_row0 >> 7)), lane);
-        it.n_a = it.n_tiles;
-    } else if (p.sync && p.remote_only) {
+    const int row0 = p.cu[seg] + (lo - 1) * (kp.straddle ? 2 * kTileM : kTileM);
+    bool two_rows = false;
+    if (kp.straddle) {
+        // items 0 .. g-2: the head pairs of the first and of the second query tile; item g-1: both tiles' last head
+        const int half = g >> 1;
+        two_rows = u == g - 1;
+        const int second = !two_rows && u >= half ? 1 : 0;
+        const int h = two_rows ? g - 1 : 2 * (u - second * half);
+        sub[0].head = it.kvh * g + h;
+        sub[1].head = sub[0].head + (two_rows ? 0 : 1);
+        sub[0].q_row0 = row0 + second * kTileM;
+        sub[1].q_row0 = sub[0].q_row0 + (two_rows ? kTileM : 0);
+    } else {
+        sub[0].head = it.kvh * g + 2 * u;
+        sub[1].head = sub[0].head + 1;
+        sub[0].q_row0 = sub[1].q_row0 = row0;
+    }
+    sub[0].n_valid = max(0, min(kTileM, end - sub[0].q_row0));
+    sub[1].n_valid = max(0, min(kTileM, end - sub[1].q_row0));
+    if (!kp.straddle && 2 * u + 1 >= g) sub[1].n_valid = 0;     // odd group: the last pair is single
+    if (sub[1].n_valid == 0) { const Sub x = sub[0]; sub[0] = sub[1]; sub[1] = x; }
+    sub[0].n_tiles = sub[1].n_tiles = 0;
+    it.n_a = 0;
+    if (sub[1].n_valid == 0) return it;                         // no such query tile
+    if (p.sync && p.remote_only && !(kExact && kp.pairs)) {
         // keys [0, a) lie before the rows' segment; when bidirectional (special instance only), keys [b, T)
         // after it count too
         const int T = (int)p.total_kv, n_t = (T + kTileN - 1) / kTileN;
-        it.a = prefix_len<kSpecial>(p, it, 0, lane);
+        it.a = prefix_len<kSpecial>(p, it, sub[1], 0, lane);
         it.n_a = (it.a + kTileN - 1) / kTileN;
-        it.n_tiles = it.n_a;
+        sub[1].n_tiles = it.n_a;
         it.b = T;
         if (kSpecial && !p.causal) {
-            const int after = p.cu[seg + 1];
-            it.b = it.kvp ? count_le_warp(it.kvp, T, after - 1, lane) : min(after, T);
+            it.b = it.kvp ? count_le_warp(it.kvp, T, end - 1, lane) : min(end, T);
             it.t_b0 = it.b >= T ? n_t : max(it.b / kTileN, it.n_a);
-            it.n_tiles = it.n_a + (n_t - it.t_b0);
+            sub[1].n_tiles = it.n_a + (n_t - it.t_b0);
         }
+        sub[0].n_tiles = sub[0].n_valid > 0 ? sub[1].n_tiles : 0;
     } else {
-        it.n_tiles = (prefix_len<kSpecial>(p, it, it.n_valid - 1, lane) + kTileN - 1) / kTileN;
-        it.n_a = it.n_tiles;
+        // (one copy of the searches' code, walked a second time when the sub-tiles are different query tiles)
+#pragma unroll 1
+        for (int again = two_rows && sub[0].n_valid > 0 ? 1 : 0;; again = 0) {
+            const Sub x = again ? sub[0] : sub[1];
+            int n;
+            if (kExact && kp.pairs) {
+                n = last_visible_tile(kp, it, x, lane);
+            } else if (kSpecial && p.general) {
+                // tiles up to the last one that holds a key position <= the tile's largest query position
+                const PosTables pt = pos_tables(p.tab, kp.n_qtiles, p.kv_head_major ? p.hkv : 1, kp.n_kt);
+                const int32_t *suf = pt.suf_min + (p.kv_head_major ? (size_t)it.kvh * kp.n_kt : 0);
+                n = count_le_warp(suf, kp.n_kt, __ldg(pt.q_max + (x.q_row0 >> 7)), lane);
+            } else {
+                n = (prefix_len<kSpecial>(p, it, x, x.n_valid - 1, lane) + kTileN - 1) / kTileN;
+            }
+            if (again) { sub[0].n_tiles = n; continue; }
+            sub[1].n_tiles = n;
+            break;
+        }
+        if (!two_rows && sub[0].n_valid > 0) sub[0].n_tiles = sub[1].n_tiles;
+        if (sub[0].n_tiles > sub[1].n_tiles) { const Sub x = sub[0]; sub[0] = sub[1]; sub[1] = x; }
+        it.n_a = sub[1].n_tiles;
     }
     return it;
 }
@@ -592,7 +627,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 24);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars + 25);
     // what the producer tells the MMA issuer about an item, published before the item's Q load is issued
-    // and read after q_full: {KV tiles, sub-tiles}; -1 tiles = no more items.  Two slots, like the phases.
+    // and read after q_full: {KV tiles of sub-tile 1, of sub-tile 0}; -1 tiles = no more items.  Two slots, like the phases.
     volatile int *item_info = reinterpret_cast<volatile int *>(bars + 26);
     // The producer decodes every work item once and publishes it here for the softmax warps (two slots of
     // 16 ints, filled an item ahead), so that decoding is not on their path between two items.
@@ -650,38 +685,42 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         for (int k = 0; k < n_rounds; ++k) {
             const int item = item_of(k);
             if (item >= n_items) continue;
-            const Item it = decode_item<kSpecial, kExact>(kp, item, lane);
+            Sub sub[2];
+            const Item it = decode_item<kSpecial, kExact>(kp, item, lane, sub);
+            const int n_tiles = sub[1].n_tiles;
             if (lane == 0) {
                 if (pn >= 2) mbar_wait_call(item_empty + (pn & 1), ((pn >> 1) - 1) & 1, abort_flag, kp.status);
                 volatile int *slot = item_pub + (pn & 1) * 16;
-                slot[0] = it.kvh; slot[1] = it.head0; slot[2] = it.q_row0; slot[3] = it.n_valid; slot[4] = it.seg;
-                slot[5] = it.kv_begin; slot[6] = it.n_tiles; slot[7] = it.n_a; slot[8] = it.t_b0; slot[9] = it.a;
-                slot[10] = it.b; slot[11] = it.valid1 ? 1 : 0;
-                mbar_arrive(item_full + (pn & 1));
-                if (it.n_tiles > 0) {
-                    // this item's Q on its way into L2: the load itself has to wait for the Q buffer
-                    tma_prefetch_3d(&map_q, 0, it.head0, it.q_row0);
-                    if (kBoxes == 2) tma_prefetch_3d(&map_q, 64, it.head0, it.q_row0);
-                    if (it.valid1) {
-                        tma_prefetch_3d(&map_q, 0, it.head0 + 1, it.q_row0);
-                        if (kBoxes == 2) tma_prefetch_3d(&map_q, 64, it.head0 + 1, it.q_row0);
-                    }
+                slot[0] = it.kvh; slot[1] = it.seg; slot[2] = it.kv_begin; slot[3] = it.n_a; slot[4] = it.t_b0;
+                slot[5] = it.a; slot[6] = it.b;
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                    slot[8 + 4 * t] = sub[t].head; slot[9 + 4 * t] = sub[t].q_row0; slot[10 + 4 * t] = sub[t].n_valid;
+                    slot[11 + 4 * t] = sub[t].n_tiles;
                 }
+                mbar_arrive(item_full + (pn & 1));
+                // this item's Q on its way into L2: the load itself has to wait for the Q buffer
+#pragma unroll
+                for (int t = 0; t < 2; ++t)
+                    if (sub[t].n_tiles > 0) {
+                        tma_prefetch_3d(&map_q, 0, sub[t].head, sub[t].q_row0);
+                        if (kBoxes == 2) tma_prefetch_3d(&map_q, 64, sub[t].head, sub[t].q_row0);
+                    }
             }
             ++pn;
-            if (it.n_tiles == 0) continue;
+            if (n_tiles == 0) continue;
             if (lane == 0) {
                 if (qn > 0) mbar_wait_call(q_empty, (qn - 1) & 1, abort_flag, kp.status);   // previous item's S MMAs done
-                item_info[(qn & 1) * 2] = it.n_tiles;
-                item_info[(qn & 1) * 2 + 1] = it.valid1 ? 2 : 1;
-                mbar_expect_tx(q_full, it.valid1 ? 2 * kTileBytes : kTileBytes);
-                tma_load_3d(sQ, &map_q, q_full, 0, it.head0, it.q_row0);
-                if (kBoxes == 2) tma_load_3d(sQ + kHalfBytes, &map_q, q_full, 64, it.head0, it.q_row0);
-                if (it.valid1) {
-                    tma_load_3d(sQ + kTileBytes, &map_q, q_full, 0, it.head0 + 1, it.q_row0);
-                    if (kBoxes == 2) tma_load_3d(sQ + kTileBytes + kHalfBytes, &map_q, q_full, 64, it.head0 + 1, it.q_row0);
-                }
-                for (int j = 0; j < it.n_tiles; ++j) {
+                item_info[(qn & 1) * 2] = n_tiles;
+                item_info[(qn & 1) * 2 + 1] = sub[0].n_tiles;
+                mbar_expect_tx(q_full, sub[0].n_tiles > 0 ? 2 * kTileBytes : kTileBytes);
+#pragma unroll
+                for (int t = 0; t < 2; ++t)
+                    if (sub[t].n_tiles > 0) {
+                        tma_load_3d(sQ + t * kTileBytes, &map_q, q_full, 0, sub[t].head, sub[t].q_row0);
+                        if (kBoxes == 2) tma_load_3d(sQ + t * kTileBytes + kHalfBytes, &map_q, q_full, 64, sub[t].head, sub[t].q_row0);
+                    }
+                for (int j = 0; j < n_tiles; ++j) {
                     const int gt = git + j, st = gt & 1, use = gt >> 1;
                     const int row = it.kv_begin + (kSpecial ? tile_of(it, j) : j) * kTileN;
                     const int c1 = p.kv_head_major ? row : it.kvh, c2 = p.kv_head_major ? it.kvh : row;
@@ -697,7 +736,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 }
             }
             __syncwarp();
-            git += it.n_tiles;
+            git += n_tiles;
             ++qn;
         }
         if (lane == 0) {
@@ -739,19 +778,19 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             }
         };
         auto commit = [&](uint64_t *bar) { if (leader) tc_commit(bar); };
-        // git / qn count the KV tiles / items of sub-tile 0 (and of the K/V ring); git1 / qn1
-        // count only the items in which the pair's second head exists.
-        int git = 0, qn = 0, git1 = 0, qn1 = 0;
+        // git / qn count the KV tiles / items of sub-tile 1 (and of the K/V ring); git0 / qn0 those of sub-tile 0,
+        // which may be missing or end earlier.
+        int git = 0, qn = 0, git0 = 0, qn0 = 0;
         for (;;) {
             // the producer decodes the work items; this warp only learns their shape (decoding them here as
             // well does not fit into this role's 64 registers)
             if (!mbar_wait_call(q_full, qn & 1, abort_flag, kp.status)) break;
             const int n = item_info[(qn & 1) * 2];
             if (n < 0) break;
-            const int n_sub = item_info[(qn & 1) * 2 + 1];
+            const int n0 = item_info[(qn & 1) * 2 + 1];
             mbar_wait_call(k_full + (git & 1), (git >> 1) & 1, abort_flag, kp.status);
             tc_fence_after();
-            for (int t = 0; t < n_sub; ++t) {
+            for (int t = n0 > 0 ? 0 : 1; t < 2; ++t) {
                 issue_s(t, git & 1);
                 commit(s_full + t);
             }
@@ -760,9 +799,9 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             for (int j = 0; j < n; ++j) {
                 const int gt = git + j, st = gt & 1, ph = (gt >> 1) & 1;
                 const int st1 = (gt + 1) & 1, ph1 = ((gt + 1) >> 1) & 1;
-                for (int t = 0; t < n_sub; ++t) {
-                    const int gsub = (t ? git1 : git) + j, qsub = t ? qn1 : qn;
-                    if (t == 0) mbar_wait_call(v_full + st, ph, abort_flag, kp.status);
+                mbar_wait_call(v_full + st, ph, abort_flag, kp.status);
+                for (int t = j < n0 ? 0 : 1; t < 2; ++t) {
+                    const int gsub = (t ? git : git0) + j, qsub = t ? qn : qn0;
                     if (j == 0 && qsub > 0) mbar_wait_call(o_free + t, (qsub - 1) & 1, abort_flag, kp.status);
 #pragma unroll
                     for (int q = 0; q < kSplit; ++q) {
@@ -786,12 +825,12 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                         }
                     }
                     commit(o_done + t);
-                    if (t == n_sub - 1) commit(v_empty + st);
-                    if (j + 1 < n) {
-                        if (t == 0) mbar_wait_call(k_full + st1, ph1, abort_flag, kp.status);
+                    if (t == 1) commit(v_empty + st);
+                    if (j + 1 < (t ? n : n0)) {
+                        mbar_wait_call(k_full + st1, ph1, abort_flag, kp.status);   // (t = 1: mostly seen by t = 0 already)
                         issue_s(t, st1);
                         commit(s_full + t);
-                        if (t == n_sub - 1) {
+                        if (t == 1) {
                             commit(k_empty + st1);
                             if (j + 2 == n) commit(q_empty);     // last S of this item issued
                         }
@@ -801,7 +840,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             }
             git += n;
             ++qn;
-            if (n_sub == 2) { git1 += n; ++qn1; }
+            if (n0 > 0) { git0 += n0; ++qn0; }
         }
     } else if (warp >= 4 * kSplit) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs));      // the two idle warps of that warpgroup
@@ -819,7 +858,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSoftmaxRegs));
         // ================= softmax + epilogue =================
-        // Warpgroup t serves sub-tile t (query head head0 + t) on its own: thread = query row r = TMEM lane,
+        // Warpgroup t serves sub-tile t (one query head of one query tile) on its own: thread = query row r = TMEM lane,
         // all 128 key columns of the S tile, the whole row of O.  The two warpgroups never meet: no row
         // maximum or row sum has to be exchanged, and while one is in the serial part of its visit (wait,
         // TMEM load, maximum) the other computes.  A thread reads its row of S from TMEM once and keeps all
@@ -943,23 +982,24 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             const int item = item_of(k);
             if (item >= n_items) continue;
             Item it;
+            Sub sub;
             {
                 mbar_wait(item_full + (pn & 1), (pn >> 1) & 1, abort_flag, kp.status);
                 const volatile int *slot = item_pub + (pn & 1) * 16;
-                it.kvh = slot[0]; it.head0 = slot[1]; it.q_row0 = slot[2]; it.n_valid = slot[3]; it.seg = slot[4];
-                it.kv_begin = slot[5]; it.n_tiles = slot[6]; it.n_a = slot[7]; it.t_b0 = slot[8]; it.a = slot[9];
-                it.b = slot[10]; it.valid1 = slot[11] != 0;
+                it.kvh = slot[0]; it.seg = slot[1]; it.kv_begin = slot[2]; it.n_a = slot[3]; it.t_b0 = slot[4];
+                it.a = slot[5]; it.b = slot[6];
+                sub.head = slot[8 + 4 * t]; sub.q_row0 = slot[9 + 4 * t]; sub.n_valid = slot[10 + 4 * t];
+                sub.n_tiles = slot[11 + 4 * t];
                 it.kvp = p.kv_pos ? p.kv_pos + (p.kv_head_major ? (int64_t)it.kvh * p.total_kv : 0) : nullptr;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(item_empty + (pn & 1));
                 ++pn;
             }
-            if (t == 1 && !it.valid1) continue;                 // the pair's second head does not exist
-            const int n_tiles = it.n_tiles;
-            const bool valid = r < it.n_valid;
-            __nv_bfloat16 *orow = reinterpret_cast<__nv_bfloat16 *>(p.o) + ((int64_t)(it.q_row0 + r) * p.hq + it.head0 + t) * d;
-            float *lse_p = p.lse ? p.lse + (int64_t)(it.q_row0 + r) * p.hq + it.head0 + t : nullptr;
-            if (n_tiles == 0) {                                 // nothing visible to any row of the tile
+            const int n_tiles = sub.n_tiles;
+            const bool valid = r < sub.n_valid;
+            __nv_bfloat16 *orow = reinterpret_cast<__nv_bfloat16 *>(p.o) + ((int64_t)(sub.q_row0 + r) * p.hq + sub.head) * d;
+            float *lse_p = p.lse ? p.lse + (int64_t)(sub.q_row0 + r) * p.hq + sub.head : nullptr;
+            if (n_tiles == 0) {                                 // nothing visible to any row of the tile, or no rows
                 if (valid) {
                     for (int c = 0; c < d; c += 8) *reinterpret_cast<uint4 *>(orow + c) = make_uint4(0, 0, 0, 0);
                     if (lse_p) *lse_p = -INFINITY;
@@ -981,7 +1021,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 }
             };
             if (pairs) {
-                mine = pair_rule(p, it, r);
+                mine = pair_rule(p, it, sub, r);
                 all = mine;
                 all.lo = __reduce_min_sync(0xffffffffu, mine.lo);
                 load_pos(0);
@@ -990,8 +1030,8 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 // tile's smallest query position (a prefix of the walk, see PosTables) need no test
                 const PosTables pt = pos_tables(p.tab, kp.n_qtiles, p.kv_head_major ? p.hkv : 1, kp.n_kt);
                 const int32_t *pre = pt.pre_max + (p.kv_head_major ? (size_t)it.kvh * kp.n_kt : 0);
-                n_full = count_le_warp(pre, kp.n_kt, __ldg(pt.q_min + (it.q_row0 >> 7)), lane);
-                const int row = it.q_row0 + min(r, it.n_valid - 1);
+                n_full = count_le_warp(pre, kp.n_kt, __ldg(pt.q_min + (sub.q_row0 >> 7)), lane);
+                const int row = sub.q_row0 + min(r, sub.n_valid - 1);
                 p_row = p.q_pos ? __ldg(p.q_pos + row) : row;
             } else {
                 if (p.sync && p.remote_only) {
@@ -1000,7 +1040,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     // Sparse aggregate, row position = row index.  One cooperative search gives the keys
                     // visible to all of the warp's 32 consecutive rows; the next 32 keys are the only ones
                     // that can tell these rows apart (more only if positions repeat: then each lane searches).
-                    const int T = (int)p.total_kv, p0 = it.q_row0 + (r & ~31);
+                    const int T = (int)p.total_kv, p0 = sub.q_row0 + (r & ~31);
                     const int cw = count_le_warp(it.kvp, T, p0 - 1, lane);
                     const int wv = cw + lane < T ? __ldg(it.kvp + cw + lane) : INT32_MAX;
                     int cnt = 0;
@@ -1009,7 +1049,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     c_row = cw + cnt;
                     if (__shfl_sync(0xffffffffu, wv, 31) <= p0 + 31) c_row = count_le(it.kvp, T, p0 + lane);
                 } else {
-                    c_row = prefix_len<kSpecial>(p, it, r, lane);   // arithmetic only
+                    c_row = prefix_len<kSpecial>(p, it, sub, r, lane);   // arithmetic only
                 }
                 // prefix lengths do not decrease with the row, so KV tiles below the prefix of the warp's first
                 // row are unmasked for the whole warp (the choice of code path only has to be warp-uniform)
@@ -1082,7 +1122,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
             // Full warps of rows leave through shared memory and TMA stores (a warp's 32 rows x 64 columns at a
             // time); a warp with rows beyond the segment writes its valid rows directly.
-            bool by_tma = kp.o_tma && (r | 31) < it.n_valid;
+            bool by_tma = kp.o_tma && (r | 31) < sub.n_valid;
             uint32_t bad = 0;                                   // exact instances: rows of the warp with a non-finite channel
             if (kExact) {
                 float probe = l_run * 0.f;                      // 0 unless something is Inf or NaN
@@ -1131,7 +1171,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     if (c & 1) {
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         __syncwarp();
-                        if (lane == 0) tma_store_3d(&map_o, my_stage, 64 * (c >> 1), it.head0 + t, it.q_row0 + (r & ~31));
+                        if (lane == 0) tma_store_3d(&map_o, my_stage, 64 * (c >> 1), sub.head, sub.q_row0 + (r & ~31));
                     }
                 }
             } else {
@@ -1167,7 +1207,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 __syncwarp();
 #pragma unroll 1
                 for (uint32_t left = bad; left; left &= left - 1) {
-                    attn_row_warp<__nv_bfloat16>(kp.row, it.q_row0 + (r & ~31) + __ffs(left) - 1, it.head0 + t,
+                    attn_row_warp<__nv_bfloat16>(kp.row, sub.q_row0 + (r & ~31) + __ffs(left) - 1, sub.head,
                                                  reinterpret_cast<float *>(my_stage));
                     __syncwarp();
                 }
@@ -1339,6 +1379,36 @@ cudaError_t launch_wait_selftest(Context *ctx, int max_polls, cudaStream_t s)
     return cudaGetLastError();
 }
 
+// Odd groups: do pairs that straddle two query tiles end sooner than lone last heads?  A pair takes 1.14 times as
+// long per KV tile as a lone sub-tile (measured, 1 head per KV head: 37.4 against 32.7 us where every CTA has one item),
+// so lone heads win where the longest walk decides, pairs where the sum of the work does.  Measured, lone -> pairs: 8 / 8
+// heads, segments of 1000, 2000 and 3000 rows: local 59 -> 49, sync 112 -> 87 us; 24 / 8 heads: 120 -> 100, 241 -> 198 us;
+// 8 / 8 heads and six segments of 2160 rows in all: local 15.8 -> 18.4, sync 32.7 -> 37.4 us (those stay lone).
+static bool straddle_pays(const PrefillParams &p, int64_t n_qtiles, int sm_count)
+{
+    const int g = p.hq / p.hkv;
+    const double pair = 1.14, lone_tile = pair * (g / 2) + 1.0, pair_tile = pair * g / 2;    // cost per query tile and KV head
+    const double n_kt = (double)((p.total_kv + kTileN - 1) / kTileN);
+    if (p.sync && !p.remote_only && (!p.causal || p.q_pos)) {
+        // equal walks: whole rounds of items count
+        const int64_t lone = n_qtiles * p.hkv * ((g + 1) / 2), pairs = (n_qtiles + 1) / 2 * p.hkv * g;
+        return ((pairs + sm_count - 1) / sm_count) * pair <= ((lone + sm_count - 1) / sm_count) * lone_tile / ((g + 1) / 2);
+    }
+    double sum = 0, longest = 0;                                // KV tiles of all query tiles, of the longest walk
+    for (int n = 0; n < p.n_seg; ++n) {
+        const double tiles = (double)((p.cu[n + 1] - p.cu[n] + kTileM - 1) / kTileM);
+        if (tiles == 0) continue;
+        const double walk = p.remote_only ? (p.causal ? n_kt * p.cu[n] / p.n_q_rows : n_kt) : tiles;
+        sum += p.causal && !p.remote_only ? tiles * (tiles + 1) / 2 : tiles * walk;
+        longest = walk > longest ? walk : longest;
+    }
+    auto ends = [&](double per_tile, double last) {             // mean load of a CTA plus the uneven end of a static schedule
+        const double even = sum * p.hkv * per_tile / sm_count + 0.3 * last * longest;
+        return even > last * longest ? even : last * longest;
+    };
+    return ends(pair_tile, pair) <= ends(lone_tile, g > 1 ? pair : 1.0);
+}
+
 cudaError_t launch_prefill_sm100(Context *ctx, const PrefillParams &p, cudaStream_t s)
 {
     static_assert(sizeof(KernelParams) + 4 * sizeof(CUtensorMap) <= 4096, "kernel parameter block too large");
@@ -1352,11 +1422,20 @@ cudaError_t launch_prefill_sm100(Context *ctx, const PrefillParams &p, cudaStrea
         kp.row = generic_params(p);
     }
     kp.n_kt = (int32_t)((p.total_kv + kTileN - 1) / kTileN);
-    int64_t n_qtiles = 0;
+    const int g = p.hq / p.hkv;
+    int64_t n_qtiles = 0, n_ranked = 0;
+    for (int n = 0; n < p.n_seg; ++n) n_qtiles += (p.cu[n + 1] - p.cu[n] + kTileM - 1) / kTileM;
+    if (n_qtiles > 0x7fffffffLL) return cudaErrorInvalidValue;
+    kp.n_qtiles = (int32_t)n_qtiles;
+    // Odd groups leave a head over per query tile; a pair with the same head of the next query tile keeps both
+    // softmax warpgroups and the tensor pipe busy where a lone sub-tile would leave half of them idle.  (Calls beyond
+    // the range of fast_div keep lone heads.)
+    kp.straddle = (g & 1) && (int64_t)p.hkv * g <= 4096 && n_qtiles * p.hkv * g < (1LL << 28) && straddle_pays(p, n_qtiles, ctx->sm_count);
+    const int rank_rows = kp.straddle ? 2 * kTileM : kTileM, ppk = kp.straddle ? g : (g + 1) / 2;
     for (int n = 0; n < p.n_seg; ++n) {
         kp.ord_seg[n] = n;
-        kp.ord_nt[n] = (p.cu[n + 1] - p.cu[n] + kTileM - 1) / kTileM;
-        n_qtiles += kp.ord_nt[n];
+        kp.ord_nt[n] = (p.cu[n + 1] - p.cu[n] + rank_rows - 1) / rank_rows;
+        n_ranked += kp.ord_nt[n];
     }
     for (int a = 1; a < p.n_seg; ++a)          // insertion sort by tile count, descending (stable)
         for (int b = a; b > 0 && kp.ord_nt[b] > kp.ord_nt[b - 1]; --b) {
@@ -1364,22 +1443,19 @@ cudaError_t launch_prefill_sm100(Context *ctx, const PrefillParams &p, cudaStrea
             kp.ord_nt[b] = kp.ord_nt[b - 1]; kp.ord_seg[b] = kp.ord_seg[b - 1];
             kp.ord_nt[b - 1] = tn; kp.ord_seg[b - 1] = ts;
         }
-    if (n_qtiles > 0x7fffffffLL) return cudaErrorInvalidValue;
     kp.band_rank[0] = 0;
     for (int b = 0; b < p.n_seg; ++b) {
         const int64_t next = b + 1 < p.n_seg ? kp.ord_nt[b + 1] : 0;
         kp.band_rank[b + 1] = kp.band_rank[b] + (int32_t)((kp.ord_nt[b] - next) * (b + 1));
     }
-    kp.n_qtiles = (int32_t)n_qtiles;
-    const int g = p.hq / p.hkv;
-    const int64_t items = n_qtiles * p.hkv * ((g + 1) / 2);
+    const int64_t items = n_ranked * p.hkv * ppk;
     if (items == 0) return cudaSuccess;
-    if (items >= (1LL << 28) || (int64_t)p.hkv * ((g + 1) / 2) > 4096) return cudaErrorInvalidValue;   // fast_div range
+    if (items >= (1LL << 28) || (int64_t)p.hkv * ppk > 4096) return cudaErrorInvalidValue;   // fast_div range
     kp.n_items = (int32_t)items;
     auto magic = [](int64_t d) { return (uint64_t)(((1ULL << 40) + (uint64_t)d - 1) / (uint64_t)d); };
     kp.group = g;
-    kp.magic_per_tile = magic((int64_t)p.hkv * ((g + 1) / 2));
-    kp.magic_ppg = magic((g + 1) / 2);
+    kp.magic_per_tile = magic((int64_t)p.hkv * ppk);
+    kp.magic_ppk = magic(ppk);
     for (int i = 0; i < kMaxP; ++i) kp.magic_small[i] = magic(i + 1);
     const int64_t blocks = items < ctx->sm_count ? items : ctx->sm_count;     // persistent: one CTA per SM
     CUtensorMap mq, mk, mv, mo;

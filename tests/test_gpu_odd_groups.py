@@ -1,0 +1,54 @@
+"""bf16 prefill with an odd number of query heads per KV head, where the last heads of two neighbouring query tiles
+share a work item: segments around one and two tiles, tiles whose walks differ in length (also the second one's being
+the shorter), rows that see nothing; head_dim 128 and one below it."""
+import numpy as np
+import pytest
+import torch
+
+from helpers import LSE_TOL, TOL, Runner, check_close, dev, fa, host
+from test_gpu_head_dims import gen, owners, reference
+
+pytestmark = pytest.mark.gpu
+
+GROUPS = [(1, 1, 128), (3, 1, 128), (10, 2, 128), (7, 1, 128), (5, 5, 64)]
+LENS = [[1, 128, 129], [256, 257, 0, 385], [640, 100, 512]]
+
+
+def check(got, want, what):
+    check_close(got[0], want[0], TOL["bf16"], what)
+    check_close(got[1], want[1], LSE_TOL["bf16"], what + " lse")
+
+
+@pytest.mark.parametrize("lens", LENS)
+@pytest.mark.parametrize("causal", [True, False])
+@pytest.mark.parametrize("hq,hkv,d", GROUPS)
+def test_local_sync_and_remote(hq, hkv, d, causal, lens):
+    q, k, v = gen(21, lens, hq, hkv, d, "bf16")
+    L, own = sum(lens), owners(lens)
+    r = Runner(len(lens), hq, hkv, d, "bf16", L, causal=causal)
+    below = np.tri(L, dtype=bool) if causal else np.ones((L, L), bool)
+    check(r.local(q, k, v, lens), reference(q, k, v, below & (own[:, None] == own)), "local")
+    check(r.sync(q, k, v), reference(q, k, v, below), "sync")
+    # a sparse ascending aggregate whose first key lies late: the first query tile sees nothing
+    kept = np.sort(np.random.default_rng(5).permutation(np.arange(L // 3, L))[:max(1, L // 4)]).astype(np.int32)
+    check(r.sync(q, k[kept], v[kept], kv_pos=kept),
+          reference(q, k[kept], v[kept], kept[None] <= np.arange(L)[:, None] if causal else np.ones((L, len(kept)), bool)), "sparse")
+    cu = np.concatenate([[0], np.cumsum(lens)])
+    qd, kd, vd = dev(q, "bf16"), dev(k[kept], "bf16"), dev(v[kept], "bf16")
+    o, lse = torch.full_like(qd, float("nan")), torch.full((L, hq), float("nan"), device="cuda")
+    fa().fedattn_sync_remote(r.ctx, r.shape, qd, cu, kd, vd, torch.from_numpy(kept).cuda(), len(kept), False, o, lse)
+    assert r.poll() == 0
+    before, after = kept[None] < cu[:-1][own][:, None], kept[None] >= cu[1:][own][:, None]
+    check((host(o), host(lse)), reference(q, k[kept], v[kept], before if causal else before | after), "remote")
+
+
+@pytest.mark.parametrize("hq,hkv,d", GROUPS)
+def test_positions_that_fall_along_the_rows(hq, hkv, d):
+    """Query positions in falling order: the second query tile of a pair walks fewer KV tiles than the first."""
+    L = 700
+    q, k, v = gen(22, [L], hq, hkv, d, "bf16")
+    r = Runner(1, hq, hkv, d, "bf16", L)
+    qp = np.arange(L, dtype=np.int32)[::-1] - 5                   # the last rows see nothing
+    check(r.sync(q, k, v, q_pos=qp.copy()), reference(q, k, v, np.arange(L)[None] <= qp[:, None]), "falling q_pos")
+    pos = np.random.default_rng(6).permutation(L).astype(np.int32)
+    check(r.sync(q, k, v, kv_pos=pos, q_pos=qp.copy()), reference(q, k, v, pos[None] <= qp[:, None]), "falling q_pos, any kv_pos")
