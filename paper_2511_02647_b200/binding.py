@@ -111,14 +111,35 @@ def _ptr(t: Optional[torch.Tensor]):
     return t.data_ptr()
 
 
+def _ptr_array(ts):
+    """Pointers of a list of tensors (or None)."""
+    try:
+        if all([t.is_contiguous() for t in ts]):
+            return (C.c_void_p * len(ts))(*[t.data_ptr() for t in ts])
+    except AttributeError:                            # a None among them
+        pass
+    return (C.c_void_p * len(ts))(*[_ptr(t) for t in ts])
+
+
+# The current stream as an integer.  torch.cuda.current_stream() builds a Stream object first: 3.2 us of the 5.3 us
+# that marshalling a call took, against 0.3 us, where the whole C call takes 5.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream) -> int:
     if stream is None:
+        if _raw_stream is not None and _current_device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_current_device())
         return torch.cuda.current_stream().cuda_stream
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _i32_array(xs: Sequence[int]):
-    return (C.c_int32 * len(xs))(*[int(x) for x in xs])
+    try:
+        return (C.c_int32 * len(xs))(*xs)             # Python ints as they are: half the time of converting each
+    except TypeError:
+        return (C.c_int32 * len(xs))(*[int(x) for x in xs])
 
 
 def fedattn_workspace_bytes(shape: Shape, max_total_tokens: int, max_total_kv: int) -> int:
@@ -208,8 +229,7 @@ def _args_aggregate_kv(ctx, shape, mode, k_parts, v_parts, seqlens_host, k_sel_h
     n = shape.n_participants
     if len(k_parts) != n or len(v_parts) != n or len(seqlens_host) != n:
         raise ValueError("need one K part, V part and length per participant")
-    kp = (C.c_void_p * n)(*[_ptr(t) for t in k_parts])
-    vp = (C.c_void_p * n)(*[_ptr(t) for t in v_parts])
+    kp, vp = _ptr_array(k_parts), _ptr_array(v_parts)
     ks = None if k_sel_host is None else _i32_array(k_sel_host)
     return (ctx.handle, C.byref(shape), int(mode), kp, vp, _i32_array(seqlens_host), ks, _ptr(sel_idx_in), _ptr(k_agg),
             _ptr(v_agg), _ptr(kv_pos), _ptr(cu_kv), _ptr(sel_idx_out), _stream(stream))
