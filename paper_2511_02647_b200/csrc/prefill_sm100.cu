@@ -498,14 +498,14 @@ __device__ __forceinline__ int last_visible_tile(const KernelParams &kp, const I
 // Called by a converged warp (all lanes get the same item).  kSpecial: the kernel instance that also
 // serves explicit positions and bidirectional remote-only attention (two key ranges); the plain instance
 // carries none of their state.  Causal remote-only attention is one more prefix mask: plain instance.
-template <bool kSpecial, bool kExact>
+template <bool kSpecial, bool kExact, bool kHalves>
 __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, int lane, Sub (&sub)[2])
 {
     const PrefillParams &p = kp.p;
     Item it;
     // divisions by launch constants go through host-computed reciprocals (kp.magic_*)
     const int g = kp.group;
-    const int ppk = kp.straddle ? g : (g + 1) >> 1;             // items per ranked tile and KV head
+    const int ppk = kHalves || kp.straddle ? g : (g + 1) >> 1;  // items per ranked tile and KV head
     const int per_tile = p.hkv * ppk;
     const int tile_rank = fast_div(item, kp.magic_per_tile);
     const int rem = item - tile_rank * per_tile;
@@ -527,9 +527,12 @@ __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, in
     it.kvp = p.kv_pos ? p.kv_pos + (p.kv_head_major ? (int64_t)it.kvh * p.total_kv : 0) : nullptr;
     it.kv_begin = p.sync ? 0 : p.cu[seg];
     it.t_b0 = 0; it.a = 0; it.b = 0;
-    const int row0 = p.cu[seg] + (lo - 1) * (kp.straddle ? 2 * kTileM : kTileM);
+    const int row0 = p.cu[seg] + (lo - 1) * (!kHalves && kp.straddle ? 2 * kTileM : kTileM);
     bool two_rows = false;
-    if (kp.straddle) {
+    if (kHalves) {
+        sub[0].head = sub[1].head = it.kvh * g + u;
+        sub[0].q_row0 = sub[1].q_row0 = row0;
+    } else if (kp.straddle) {
         // items 0 .. g-2: the head pairs of the first and of the second query tile; item g-1: both tiles' last head
         const int half = g >> 1;
         two_rows = u == g - 1;
@@ -546,7 +549,7 @@ __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, in
     }
     sub[0].n_valid = max(0, min(kTileM, end - sub[0].q_row0));
     sub[1].n_valid = max(0, min(kTileM, end - sub[1].q_row0));
-    if (!kp.straddle && 2 * u + 1 >= g) sub[1].n_valid = 0;     // odd group: the last pair is single
+    if (!kHalves && !kp.straddle && 2 * u + 1 >= g) sub[1].n_valid = 0;     // odd group: the last pair is single
     if (sub[1].n_valid == 0) { const Sub x = sub[0]; sub[0] = sub[1]; sub[1] = x; }
     sub[0].n_tiles = sub[1].n_tiles = 0;
     it.n_a = 0;
@@ -589,6 +592,11 @@ __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, in
         if (sub[0].n_tiles > sub[1].n_tiles) { const Sub x = sub[0]; sub[0] = sub[1]; sub[1] = x; }
         it.n_a = sub[1].n_tiles;
     }
+    if (kHalves) {                                              // sub-tile 1 walks tiles 0, 2, ..., sub-tile 0 tiles 1, 3, ...
+        sub[0].n_tiles = sub[1].n_tiles >> 1;
+        sub[1].n_tiles -= sub[0].n_tiles;
+        if (sub[0].n_tiles == 0) sub[0].n_valid = 0;
+    }
     return it;
 }
 
@@ -605,7 +613,13 @@ __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, in
 // 6 more instructions per pair of keys.  Six ragged segments of 2160 tokens in all, 16 / 4 heads of 64 channels: local
 // 2436 us (one warp per row, fp32 FMA) -> 20 us, sync 10994 -> 45 us; the error of o against fp64 is the same to
 // three digits (the rounding of the bf16 output, 1.6e-3), lse 3.5e-8 -> 5e-8 relative (half a unit of fp32).
-template <bool kSpecial, int kBoxes, bool kExact>
+//
+// kHalves: both sub-tiles are the SAME query tile of one head; sub-tile 1 walks the even KV tiles and sub-tile 0 the odd
+// ones, and the epilogue merges the two partial rows (O_0 and O_1 have the same TMEM lanes, so every thread reads both;
+// maximum and sum go through shared memory).  An item takes half as long as a pair of heads over the same keys: for
+// launches whose longest walk, not their sum of work, decides.  K and V tiles then serve one product each, which
+// doubles what the CTA reads from L2.
+template <bool kSpecial, int kBoxes, bool kExact, bool kHalves>
 __global__ void __launch_bounds__(kThreads, 1)
 prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                      const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o,
@@ -686,8 +700,8 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             const int item = item_of(k);
             if (item >= n_items) continue;
             Sub sub[2];
-            const Item it = decode_item<kSpecial, kExact>(kp, item, lane, sub);
-            const int n_tiles = sub[1].n_tiles;
+            const Item it = decode_item<kSpecial, kExact, kHalves>(kp, item, lane, sub);
+            const int n_tiles = sub[1].n_tiles + (kHalves ? sub[0].n_tiles : 0);
             if (lane == 0) {
                 if (pn >= 2) mbar_wait_call(item_empty + (pn & 1), ((pn >> 1) - 1) & 1, abort_flag, kp.status);
                 volatile int *slot = item_pub + (pn & 1) * 16;
@@ -701,7 +715,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 mbar_arrive(item_full + (pn & 1));
                 // this item's Q on its way into L2: the load itself has to wait for the Q buffer
 #pragma unroll
-                for (int t = 0; t < 2; ++t)
+                for (int t = kHalves ? 1 : 0; t < 2; ++t)
                     if (sub[t].n_tiles > 0) {
                         tma_prefetch_3d(&map_q, 0, sub[t].head, sub[t].q_row0);
                         if (kBoxes == 2) tma_prefetch_3d(&map_q, 64, sub[t].head, sub[t].q_row0);
@@ -711,11 +725,11 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             if (n_tiles == 0) continue;
             if (lane == 0) {
                 if (qn > 0) mbar_wait_call(q_empty, (qn - 1) & 1, abort_flag, kp.status);   // previous item's S MMAs done
-                item_info[(qn & 1) * 2] = n_tiles;
+                item_info[(qn & 1) * 2] = sub[1].n_tiles;
                 item_info[(qn & 1) * 2 + 1] = sub[0].n_tiles;
-                mbar_expect_tx(q_full, sub[0].n_tiles > 0 ? 2 * kTileBytes : kTileBytes);
+                mbar_expect_tx(q_full, !kHalves && sub[0].n_tiles > 0 ? 2 * kTileBytes : kTileBytes);
 #pragma unroll
-                for (int t = 0; t < 2; ++t)
+                for (int t = kHalves ? 1 : 0; t < 2; ++t)       // (halves share sub-tile 1's Q)
                     if (sub[t].n_tiles > 0) {
                         tma_load_3d(sQ + t * kTileBytes, &map_q, q_full, 0, sub[t].head, sub[t].q_row0);
                         if (kBoxes == 2) tma_load_3d(sQ + t * kTileBytes + kHalfBytes, &map_q, q_full, 64, sub[t].head, sub[t].q_row0);
@@ -772,36 +786,44 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 for (int ks = 0; ks < kBoxes * kBoxCols / 16; ++ks) {
                     const uint32_t off = ((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4;       // descriptor units
                     if (!kExact || 16 * ks < d)                  // columns beyond head_dim are zero in both tiles
-                    umma_ss(tmem_base + kColS + t * 128, dQ + (uint64_t)(t * (kTileBytes >> 4) + off),
+                    umma_ss(tmem_base + kColS + t * 128, dQ + (uint64_t)((kHalves ? 1 : t) * (kTileBytes >> 4) + off),
                             dK + (uint64_t)(st * (kTileBytes >> 4) + off), kIdescQK, ks > 0);
                 }
             }
         };
         auto commit = [&](uint64_t *bar) { if (leader) tc_commit(bar); };
-        // git / qn count the KV tiles / items of sub-tile 1 (and of the K/V ring); git0 / qn0 those of sub-tile 0,
-        // which may be missing or end earlier.
-        int git = 0, qn = 0, git0 = 0, qn0 = 0;
+        // ring counts the KV tiles; git / qn the KV tiles / items of sub-tile 1, git0 / qn0 those of sub-tile 0, which
+        // may be missing or end earlier.
+        int ring = 0, git = 0, qn = 0, git0 = 0, qn0 = 0;
         for (;;) {
             // the producer decodes the work items; this warp only learns their shape (decoding them here as
             // well does not fit into this role's 64 registers)
             if (!mbar_wait_call(q_full, qn & 1, abort_flag, kp.status)) break;
-            const int n = item_info[(qn & 1) * 2];
-            if (n < 0) break;
+            const int n1 = item_info[(qn & 1) * 2];
+            if (n1 < 0) break;
             const int n0 = item_info[(qn & 1) * 2 + 1];
-            mbar_wait_call(k_full + (git & 1), (git >> 1) & 1, abort_flag, kp.status);
-            tc_fence_after();
-            for (int t = n0 > 0 ? 0 : 1; t < 2; ++t) {
-                issue_s(t, git & 1);
+            const int n = kHalves ? n0 + n1 : n1;                // KV tiles of the item
+            // halves take the sub-tiles in the order of their tiles: 1 (tile 0) first
+            for (int i = kHalves || n0 > 0 ? 0 : 1; i < 2; ++i) {
+                const int t = kHalves ? 1 - i : i, tile = kHalves ? i : 0, st = (ring + tile) & 1;
+                if (kHalves && tile >= n) break;
+                mbar_wait_call(k_full + st, ((ring + tile) >> 1) & 1, abort_flag, kp.status);
+                tc_fence_after();
+                issue_s(t, st);
                 commit(s_full + t);
+                if (kHalves || t == 1) {
+                    commit(k_empty + st);
+                    if (tile == n - 1) commit(q_empty);          // last S of this item issued
+                }
             }
-            commit(k_empty + (git & 1));
-            if (n == 1) commit(q_empty);
-            for (int j = 0; j < n; ++j) {
-                const int gt = git + j, st = gt & 1, ph = (gt >> 1) & 1;
-                const int st1 = (gt + 1) & 1, ph1 = ((gt + 1) >> 1) & 1;
-                mbar_wait_call(v_full + st, ph, abort_flag, kp.status);
-                for (int t = j < n0 ? 0 : 1; t < 2; ++t) {
+            for (int j = 0; j < n1; ++j) {
+                for (int i = kHalves || j < n0 ? 0 : 1; i < 2; ++i) {
+                    const int t = kHalves ? 1 - i : i;
+                    if (kHalves && t == 0 && j >= n0) break;
+                    const int tile = kHalves ? 2 * j + i : j;
+                    const int gt = ring + tile, st = gt & 1, ph = (gt >> 1) & 1;
                     const int gsub = (t ? git : git0) + j, qsub = t ? qn : qn0;
+                    mbar_wait_call(v_full + st, ph, abort_flag, kp.status);
                     if (j == 0 && qsub > 0) mbar_wait_call(o_free + t, (qsub - 1) & 1, abort_flag, kp.status);
 #pragma unroll
                     for (int q = 0; q < kSplit; ++q) {
@@ -825,20 +847,22 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                         }
                     }
                     commit(o_done + t);
-                    if (t == 1) commit(v_empty + st);
-                    if (j + 1 < (t ? n : n0)) {
-                        mbar_wait_call(k_full + st1, ph1, abort_flag, kp.status);   // (t = 1: mostly seen by t = 0 already)
+                    if (kHalves || t == 1) commit(v_empty + st);
+                    if (j + 1 < (t ? n1 : n0)) {
+                        const int next = tile + (kHalves ? 2 : 1), st1 = (ring + next) & 1;
+                        mbar_wait_call(k_full + st1, ((ring + next) >> 1) & 1, abort_flag, kp.status);
                         issue_s(t, st1);
                         commit(s_full + t);
-                        if (t == 1) {
+                        if (kHalves || t == 1) {
                             commit(k_empty + st1);
-                            if (j + 2 == n) commit(q_empty);     // last S of this item issued
+                            if (next == n - 1) commit(q_empty);
                         }
                     }
                     if (t == 1 && lane == 0) TRACE(j, 4);
                 }
             }
-            git += n;
+            ring += n;
+            git += n1;
             ++qn;
             if (n0 > 0) { git0 += n0; ++qn0; }
         }
@@ -983,6 +1007,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             if (item >= n_items) continue;
             Item it;
             Sub sub;
+            bool halved = false;                                // the other warpgroup walks the other KV tiles of these rows
             {
                 mbar_wait(item_full + (pn & 1), (pn >> 1) & 1, abort_flag, kp.status);
                 const volatile int *slot = item_pub + (pn & 1) * 16;
@@ -990,6 +1015,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 it.a = slot[5]; it.b = slot[6];
                 sub.head = slot[8 + 4 * t]; sub.q_row0 = slot[9 + 4 * t]; sub.n_valid = slot[10 + 4 * t];
                 sub.n_tiles = slot[11 + 4 * t];
+                halved = kHalves && slot[11] > 0;
                 it.kvp = p.kv_pos ? p.kv_pos + (p.kv_head_major ? (int64_t)it.kvh * p.total_kv : 0) : nullptr;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(item_empty + (pn & 1));
@@ -1024,7 +1050,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 mine = pair_rule(p, it, sub, r);
                 all = mine;
                 all.lo = __reduce_min_sync(0xffffffffu, mine.lo);
-                load_pos(0);
+                load_pos(kHalves ? 1 - t : 0);
             } else if (general) {
                 // every (query, key) pair on its own positions; the tiles whose keys all lie at or below the
                 // tile's smallest query position (a prefix of the walk, see PosTables) need no test
@@ -1058,13 +1084,13 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             const int T = (int)p.total_kv;
             float m_run = 0.f, l_run = 0.f;
             for (int j = 0; j < n_tiles; ++j) {
-                const int gt = gsub + j;
+                const int gt = gsub + j, tile = kHalves ? 2 * j + 1 - t : j;
                 // which columns of this tile the thread's row sees: everything (warp-uniform), or a mask per chunk
                 bool full;
                 uint32_t vm[4] = {0, 0, 0, 0};
                 if (pairs) {
                     // column 32 c + i of the tile is key j * 128 + 32 c + i, whose position lane i holds
-                    const int k0 = j * kTileN;
+                    const int k0 = tile * kTileN;
                     bool see_all = true;
 #pragma unroll
                     for (int c = 0; c < 4; ++c) see_all = see_all && k0 + 32 * c + lane < T && all.sees(kpos[c]);
@@ -1079,9 +1105,9 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                             vm[c] = m & below32(T - k0 - 32 * c);
                         }
                     }
-                    if (j + 1 < n_tiles) load_pos(j + 1);       // lands during this tile's visit
+                    if (j + 1 < n_tiles) load_pos(tile + (kHalves ? 2 : 1));        // lands during this tile's visit
                 } else if (two_range) {                         // keys [0, a) and [b, T)
-                    const int k0 = tile_of(it, j) * kTileN;     // first key of the tile
+                    const int k0 = tile_of(it, tile) * kTileN;  // first key of the tile
                     full = k0 + kTileN <= it.a || (k0 >= it.b && k0 + kTileN <= T);
                     if (!full) {
 #pragma unroll
@@ -1091,13 +1117,13 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                         }
                     }
                 } else {
-                    full = j < n_full;
+                    full = tile < n_full;
                     if (!full && general) {
                         // column i of chunk c is key cb + i: visible iff it exists and its position is not above
                         // the row's.  The address is the same in every lane: broadcast loads.
 #pragma unroll
                         for (int c = 0; c < 4; ++c) {
-                            const int cb = j * kTileN + 32 * c;
+                            const int cb = tile * kTileN + 32 * c;
                             uint32_t m = 0;
 #pragma unroll 4
                             for (int i = 0; i < 32; ++i) {
@@ -1109,7 +1135,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                         }
                     } else if (!full) {
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) vm[c] = below32(c_row - j * kTileN - 32 * c);
+                        for (int c = 0; c < 4; ++c) vm[c] = below32(c_row - tile * kTileN - 32 * c);
                     }
                 }
                 if (full) visit(std::false_type{}, j, gt, vm, m_run, l_run);
@@ -1119,7 +1145,52 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             // ---- epilogue: drain this row of O from TMEM (frees it for the next item), O / l -> bf16 -> global
             mbar_wait(o_done + t, (gsub + n_tiles - 1) & 1, abort_flag, kp.status);
             tc_fence_after();
+            // Halves: this thread and the one with the same row in the other warpgroup hold the two partials of the row.
+            // Both read both accumulators (each half of the columns; one box: sub-tile 1's warps all of them) and
+            // weigh them by w0 and w1; otherwise w = 1 / l weighs the own accumulator.
+            float w0 = 0.f, w1 = 0.f;
+            if (kHalves && halved) {
+                float2 *xch = reinterpret_cast<float2 *>(sQ);   // sub-tile 0's Q buffer is not used
+                const float m_mine = l_run == 0.f ? -INFINITY : m_run;
+                xch[t * 128 + r] = make_float2(m_mine, l_run);
+                tc_fence_before();
+                asm volatile("bar.sync 1, 256;" ::: "memory");
+                tc_fence_after();
+                const float2 other = xch[(1 - t) * 128 + r];
+                m_run = fmaxf(m_mine, other.x);
+                const float ref = m_run == -INFINITY ? 0.f : m_run, f_mine = ex2(m_mine - ref), f_other = ex2(other.x - ref);
+                l_run = l_run * f_mine + other.y * f_other;
+                const float inv_l = l_run > 0.f ? 1.f / l_run : 0.f;
+                w0 = (t == 0 ? f_mine : f_other) * inv_l;
+                w1 = (t == 0 ? f_other : f_mine) * inv_l;
+            }
             const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+            const int c_lo = kHalves && halved && kBoxes == 2 ? 2 * t : 0;                  // 32-column chunks of this thread
+            const int c_hi = kHalves && halved ? (kBoxes == 2 ? c_lo + 2 : 2 * t) : 2 * kBoxes;
+            // chunk c of the row, normalised
+            auto load_o = [&](int c, uint32_t (&o)[32]) {
+                if (kHalves && halved) {
+                    uint32_t x[32];
+                    FEDATTN_TMEM_LD32(tmem_base + lane_base + kColO + 32 * c, o);
+                    FEDATTN_TMEM_LD32(tmem_base + lane_base + kColO + 128 + 32 * c, x);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int i = 0; i < 32; ++i)
+                        o[i] = __float_as_uint(fmaf(__uint_as_float(x[i]), w1, __uint_as_float(o[i]) * w0));
+                } else {
+                    FEDATTN_TMEM_LD32(tO + 32 * c, o);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * inv);
+                }
+            };
+            // this warp has read what it needs of O: one arrival per warp lets the accumulator be overwritten
+            auto release_o = [&]() {
+                tc_fence_before();
+                if (kHalves && halved) asm volatile("bar.sync 1, 256;" ::: "memory");
+                else __syncwarp();
+                if (lane == 0) mbar_arrive(o_free + t);
+            };
             // Full warps of rows leave through shared memory and TMA stores (a warp's 32 rows x 64 columns at a
             // time); a warp with rows beyond the segment writes its valid rows directly.
             bool by_tma = kp.o_tma && (r | 31) < sub.n_valid;
@@ -1127,10 +1198,9 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             if (kExact) {
                 float probe = l_run * 0.f;                      // 0 unless something is Inf or NaN
 #pragma unroll 1
-                for (int c = 0; 32 * c < d; ++c) {
+                for (int c = c_lo; c < c_hi && 32 * c < d; ++c) {
                     uint32_t o[32];
-                    FEDATTN_TMEM_LD32(tO + 32 * c, o);
-                    tmem_wait_ld();
+                    load_o(c, o);
 #pragma unroll
                     for (int i = 0; i < 32; ++i)
                         if (32 * c + (i & ~7) < d) probe = fmaf(__uint_as_float(o[i]), 0.f, probe);
@@ -1139,7 +1209,36 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 by_tma = by_tma && bad == 0;
             }
             uint8_t *my_stage = stage + (size_t)warp * kStageBytes;
-            if (by_tma) {
+            if (kHalves && by_tma) {
+                // one box of 64 columns per warp at a time; short items, so the code stays short
+                if (lane == 0) tma_store_wait_read();
+                __syncwarp();
+#pragma unroll 1
+                for (int c = c_lo; c < c_hi; ++c) {
+                    uint32_t o[32];
+                    load_o(c, o);
+                    if (c == c_hi - 1) release_o();
+                    if (c == c_lo + 2) {                        // the first box's store has read the staging rows
+                        if (lane == 0) tma_store_wait_read();
+                        __syncwarp();
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        uint32_t w[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            w[i] = pack_bf16(__uint_as_float(o[8 * u + 2 * i]), __uint_as_float(o[8 * u + 2 * i + 1]));
+                        const int unit = 4 * (c & 1) + u;
+                        *reinterpret_cast<uint4 *>(my_stage + lane * 128 + ((unit ^ (lane & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+                    }
+                    if (c & 1) {
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) tma_store_3d(&map_o, my_stage, 64 * (c >> 1), sub.head, sub.q_row0 + (r & ~31));
+                    }
+                }
+                if (c_lo == c_hi) release_o();
+            } else if (by_tma) {
                 if (lane == 0) tma_store_wait_read();           // the previous item's last store has read the staging rows
                 __syncwarp();
                 uint32_t oa[32], ob[32];
@@ -1177,15 +1276,10 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             } else {
                 // the rare path (a warp with rows beyond the segment) is kept short rather than fast
 #pragma unroll 1
-                for (int c = 0; c < 2 * kBoxes; ++c) {
+                for (int c = c_lo; c < c_hi; ++c) {
                     uint32_t o[32];
-                    FEDATTN_TMEM_LD32(tO + 32 * c, o);
-                    tmem_wait_ld();
-                    if (c == 2 * kBoxes - 1) {
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(o_free + t);
-                    }
+                    load_o(c, o);
+                    if (c == c_hi - 1) release_o();
                     if (valid && !((bad >> lane) & 1u)) {
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
@@ -1193,11 +1287,12 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                             uint32_t w[4];
 #pragma unroll
                             for (int i = 0; i < 4; ++i)
-                                w[i] = pack_bf16(__uint_as_float(o[8 * u + 2 * i]) * inv, __uint_as_float(o[8 * u + 2 * i + 1]) * inv);
+                                w[i] = pack_bf16(__uint_as_float(o[8 * u + 2 * i]), __uint_as_float(o[8 * u + 2 * i + 1]));
                             *reinterpret_cast<uint4 *>(orow + 32 * c + 8 * u) = make_uint4(w[0], w[1], w[2], w[3]);
                         }
                     }
                 }
+                if (kHalves && c_lo == c_hi) release_o();
             }
             if (valid && lse_p) *lse_p = !(l_run > 0.f) ? -INFINITY
                                          : kExact ? lse_exact(m_run, l_run)
@@ -1379,34 +1474,78 @@ cudaError_t launch_wait_selftest(Context *ctx, int max_polls, cudaStream_t s)
     return cudaGetLastError();
 }
 
-// Odd groups: do pairs that straddle two query tiles end sooner than lone last heads?  A pair takes 1.14 times as
-// long per KV tile as a lone sub-tile (measured, 1 head per KV head: 37.4 against 32.7 us where every CTA has one item),
-// so lone heads win where the longest walk decides, pairs where the sum of the work does.  Measured, lone -> pairs: 8 / 8
-// heads, segments of 1000, 2000 and 3000 rows: local 59 -> 49, sync 112 -> 87 us; 24 / 8 heads: 120 -> 100, 241 -> 198 us;
-// 8 / 8 heads and six segments of 2160 rows in all: local 15.8 -> 18.4, sync 32.7 -> 37.4 us (those stay lone).
-static bool straddle_pays(const PrefillParams &p, int64_t n_qtiles, int sm_count)
+// How the query heads of a group and the query tiles form work items.
+enum ItemForm {
+    kPairs,       // two heads of a query tile; an odd group's last head stays alone
+    kStraddle,    // odd groups: the last head of two neighbouring query tiles forms an item too
+    kHalvesForm,  // one head, its KV tiles shared by the two sub-tiles (kernel instances kHalves)
+};
+// The form that is estimated to end first.  Unit: a lone sub-tile's time per KV tile, 1.6 us; a pair takes 1.14 times as
+// long (8 / 8 heads, 17 query tiles: lone 32.7 us, pairs 37.4), halves 0.6 per KV tile of their head (0.9 with exact
+// weights), and every item costs about 2 on top (its Q, its epilogue, the restart of the chain; halves 2.6, they merge).
+// Calls of a few items per CTA are dealt out on paper as the kernel deals them; for more items the mean load of a CTA
+// decides, and halves never pay (twice the items and twice the K and V traffic).  Measured against the estimate's second
+// choice, us: 16 / 4 heads, 700 + 500 rows: local 18.4 -> 13.9, sync 25.8 -> 18.5 (halves for pairs); 32 / 8 heads there:
+// 18.9 and 26.3 with pairs, 22.6 and 30.8 with halves; 14 / 2 heads, 2160 rows, sync: 37.9 -> 29.1 (halves for straddling
+// pairs); 24 / 8 heads, 1000 + 2000 + 3000 rows: local 120 -> 100, sync 241 -> 198 (straddling pairs for lone last heads).
+static ItemForm item_form(const PrefillParams &p, int64_t n_qtiles, int sm_count)
 {
+    constexpr int kMostSms = 256;
     const int g = p.hq / p.hkv;
-    const double pair = 1.14, lone_tile = pair * (g / 2) + 1.0, pair_tile = pair * g / 2;    // cost per query tile and KV head
-    const double n_kt = (double)((p.total_kv + kTileN - 1) / kTileN);
-    if (p.sync && !p.remote_only && (!p.causal || p.q_pos)) {
-        // equal walks: whole rounds of items count
-        const int64_t lone = n_qtiles * p.hkv * ((g + 1) / 2), pairs = (n_qtiles + 1) / 2 * p.hkv * g;
-        return ((pairs + sm_count - 1) / sm_count) * pair <= ((lone + sm_count - 1) / sm_count) * lone_tile / ((g + 1) / 2);
-    }
-    double sum = 0, longest = 0;                                // KV tiles of all query tiles, of the longest walk
-    for (int n = 0; n < p.n_seg; ++n) {
-        const double tiles = (double)((p.cu[n + 1] - p.cu[n] + kTileM - 1) / kTileM);
-        if (tiles == 0) continue;
-        const double walk = p.remote_only ? (p.causal ? n_kt * p.cu[n] / p.n_q_rows : n_kt) : tiles;
-        sum += p.causal && !p.remote_only ? tiles * (tiles + 1) / 2 : tiles * walk;
-        longest = walk > longest ? walk : longest;
-    }
-    auto ends = [&](double per_tile, double last) {             // mean load of a CTA plus the uneven end of a static schedule
-        const double even = sum * p.hkv * per_tile / sm_count + 0.3 * last * longest;
-        return even > last * longest ? even : last * longest;
+    if ((int64_t)p.hkv * g > 4096 || n_qtiles * p.hkv * g >= (1LL << 28) || sm_count > kMostSms) return kPairs;      // fast_div range
+    const float pair = 1.14f, half = p.d < 128 ? 0.9f : 0.6f, start = 2.0f, merge = 0.6f, n_kt = (float)((p.total_kv + kTileN - 1) / kTileN);
+    const bool grows = p.causal && !p.remote_only && !(p.sync && p.q_pos);
+    // KV tiles of query tile `tile` (1 ..) of a segment with `tiles` of them
+    auto walk = [&](int seg, int tile, int tiles) -> float {
+        if (p.remote_only) return p.causal ? n_kt * p.cu[seg] / p.n_q_rows : n_kt;
+        const float most = p.sync ? n_kt : (float)tiles;
+        return grows ? most * tile / tiles : most;
     };
-    return ends(pair_tile, pair) <= ends(lone_tile, g > 1 ? pair : 1.0);
+    auto tiles_of = [&](int seg) { return (p.cu[seg + 1] - p.cu[seg] + kTileM - 1) / kTileM; };
+    if (n_qtiles * p.hkv * ((g + 1) / 2) > 3 * sm_count) {
+        // Many items: straddling pairs save 0.43 of a unit per two lone KV tiles and hardly change the end.
+        return (g & 1) ? kStraddle : kPairs;
+    }
+    float load[kMostSms];
+    int longest = 0;
+    for (int n = 0; n < p.n_seg; ++n) longest = tiles_of(n) > longest ? tiles_of(n) : longest;
+    auto ends = [&](ItemForm form) -> float {
+        const int rows = form == kStraddle ? 2 : 1;             // query tiles per ranked tile
+        for (int c = 0; c < sm_count; ++c) load[c] = 0.f;
+        int c = 0, step = 1;
+        auto deal = [&](float cost) {
+            load[c] += cost;
+            c += step;
+            if (c == sm_count || c < 0) { step = -step; c += step; }
+        };
+        for (int level = (longest + rows - 1) / rows; level >= 1; --level)
+            for (int n = 0; n < p.n_seg; ++n) {
+                const int tiles = tiles_of(n), first = rows * (level - 1) + 1;
+                if (tiles < first) continue;
+                const float w = walk(n, first, tiles), w2 = rows == 2 && first < tiles ? walk(n, first + 1, tiles) : 0.f;
+                for (int h = 0; h < p.hkv; ++h) {
+                    if (form == kHalvesForm) {
+                        for (int u = 0; u < g; ++u) deal((w > 1.f ? half * w + merge : w) + start);
+                    } else {
+                        for (int u = 0; u < g / 2; ++u) deal(pair * w + start);
+                        if (rows == 2)
+                            for (int u = 0; u < g / 2; ++u) deal(w2 > 0.f ? pair * w2 + start : 0.f);
+                        if (g & 1) deal((w2 > 0.f ? pair * (w2 > w ? w2 : w) : w) + start);
+                    }
+                }
+            }
+        float most = 0.f;
+        for (int i = 0; i < sm_count; ++i) most = load[i] > most ? load[i] : most;
+        return most;
+    };
+    ItemForm best = kPairs;
+    float t = ends(kPairs);
+    if (g & 1) {
+        const float u = ends(kStraddle);
+        if (u < 0.97f * t) { t = u; best = kStraddle; }
+    }
+    if (n_qtiles * p.hq <= 3 * sm_count && ends(kHalvesForm) < 0.95f * t) best = kHalvesForm;
+    return best;
 }
 
 cudaError_t launch_prefill_sm100(Context *ctx, const PrefillParams &p, cudaStream_t s)
@@ -1427,11 +1566,10 @@ cudaError_t launch_prefill_sm100(Context *ctx, const PrefillParams &p, cudaStrea
     for (int n = 0; n < p.n_seg; ++n) n_qtiles += (p.cu[n + 1] - p.cu[n] + kTileM - 1) / kTileM;
     if (n_qtiles > 0x7fffffffLL) return cudaErrorInvalidValue;
     kp.n_qtiles = (int32_t)n_qtiles;
-    // Odd groups leave a head over per query tile; a pair with the same head of the next query tile keeps both
-    // softmax warpgroups and the tensor pipe busy where a lone sub-tile would leave half of them idle.  (Calls beyond
-    // the range of fast_div keep lone heads.)
-    kp.straddle = (g & 1) && (int64_t)p.hkv * g <= 4096 && n_qtiles * p.hkv * g < (1LL << 28) && straddle_pays(p, n_qtiles, ctx->sm_count);
-    const int rank_rows = kp.straddle ? 2 * kTileM : kTileM, ppk = kp.straddle ? g : (g + 1) / 2;
+    const ItemForm item = item_form(p, n_qtiles, ctx->sm_count);
+    const bool halves = item == kHalvesForm;
+    kp.straddle = item == kStraddle ? 1 : 0;
+    const int rank_rows = kp.straddle ? 2 * kTileM : kTileM, ppk = halves || kp.straddle ? g : (g + 1) / 2;
     for (int n = 0; n < p.n_seg; ++n) {
         kp.ord_seg[n] = n;
         kp.ord_nt[n] = (p.cu[n + 1] - p.cu[n] + rank_rows - 1) / rank_rows;
@@ -1471,11 +1609,15 @@ cudaError_t launch_prefill_sm100(Context *ctx, const PrefillParams &p, cudaStrea
     // and bidirectional remote-only attention run the instance that carries their extra state; head dims below
     // 128 run the exact instances
     typedef void (*Kernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const KernelParams);
-    static const Kernel kernels[4] = {prefill_sm100_kernel<false, 2, false>, prefill_sm100_kernel<true, 2, false>,
-                                      prefill_sm100_kernel<true, 1, true>, prefill_sm100_kernel<true, 2, true>};
-    const int which = p.d < 128 ? (p.d <= kBoxCols ? 2 : 3) : (p.general || (p.remote_only && !p.causal)) ? 1 : 0;
-    const uint32_t smem = smem_bytes(which == 2 ? 1 : 2);
-    static bool attr_set[64][4] = {};
+    static const Kernel kernels[8] = {
+        prefill_sm100_kernel<false, 2, false, false>, prefill_sm100_kernel<true, 2, false, false>,
+        prefill_sm100_kernel<true, 1, true, false>,   prefill_sm100_kernel<true, 2, true, false>,
+        prefill_sm100_kernel<false, 2, false, true>,  prefill_sm100_kernel<true, 2, false, true>,
+        prefill_sm100_kernel<true, 1, true, true>,    prefill_sm100_kernel<true, 2, true, true>};
+    const int form = p.d < 128 ? (p.d <= kBoxCols ? 2 : 3) : (p.general || (p.remote_only && !p.causal)) ? 1 : 0;
+    const int which = form + (halves ? 4 : 0);
+    const uint32_t smem = smem_bytes(form == 2 ? 1 : 2);
+    static bool attr_set[64][8] = {};
     if (!attr_set[ctx->device & 63][which]) {
         cudaError_t e = cudaFuncSetAttribute(kernels[which], cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         // the register split inside the kernel has to fit into what the launch allocates: an increase that

@@ -33,7 +33,8 @@ def reference(q, k, v, visible):
         p = np.exp(s - m[:, None])
         z = p.sum(1)
         # excluded keys take no part, whatever their value rows hold
-        pv = np.array([p[i, vis[i]] @ v[vis[i], h // g].astype(np.float64) for i in range(rows)])
+        vh = v[:, h // g].astype(np.float64)
+        pv = p @ vh if np.isfinite(vh).all() else np.array([p[i, vis[i]] @ vh[vis[i]] for i in range(rows)])
         o[some, h] = pv[some] / z[some, None]
         lse[some, h] = m[some] + np.log(z[some])
     return o, lse

@@ -1,6 +1,7 @@
-"""bf16 prefill with an odd number of query heads per KV head, where the last heads of two neighbouring query tiles
-share a work item: segments around one and two tiles, tiles whose walks differ in length (also the second one's being
-the shorter), rows that see nothing; head_dim 128 and one below it."""
+"""The forms of a work item of the bf16 prefill kernel: two heads of a query tile; the last heads of an odd group of two
+neighbouring query tiles; one head whose KV tiles two sub-tiles share (calls with few items, so all the small ones).
+Segments around one and two tiles, walks of one, two and three tiles, tiles whose walks differ in length (also the
+second one's being the shorter), rows that see nothing; head_dim 128 and one below it."""
 import numpy as np
 import pytest
 import torch
@@ -19,10 +20,12 @@ def check(got, want, what):
     check_close(got[1], want[1], LSE_TOL["bf16"], what + " lse")
 
 
-@pytest.mark.parametrize("lens", LENS)
+MANY = [(24, 8, 128), (32, 32, 128), (28, 4, 128), (32, 8, 128), (24, 8, 64)]       # enough items for the other forms
+
+
+@pytest.mark.parametrize("hq,hkv,d,lens", [(*g, n) for g in GROUPS for n in LENS] + [(*g, [300, 517, 64, 700, 129]) for g in MANY])
 @pytest.mark.parametrize("causal", [True, False])
-@pytest.mark.parametrize("hq,hkv,d", GROUPS)
-def test_local_sync_and_remote(hq, hkv, d, causal, lens):
+def test_local_sync_and_remote(hq, hkv, d, lens, causal):
     q, k, v = gen(21, lens, hq, hkv, d, "bf16")
     L, own = sum(lens), owners(lens)
     r = Runner(len(lens), hq, hkv, d, "bf16", L, causal=causal)
@@ -42,10 +45,9 @@ def test_local_sync_and_remote(hq, hkv, d, causal, lens):
     check((host(o), host(lse)), reference(q, k[kept], v[kept], before if causal else before | after), "remote")
 
 
-@pytest.mark.parametrize("hq,hkv,d", GROUPS)
-def test_positions_that_fall_along_the_rows(hq, hkv, d):
+@pytest.mark.parametrize("hq,hkv,d,L", [(*g, 700) for g in GROUPS] + [(24, 8, 128, 2000), (24, 8, 128, 2400), (32, 8, 128, 2000)])
+def test_positions_that_fall_along_the_rows(hq, hkv, d, L):
     """Query positions in falling order: the second query tile of a pair walks fewer KV tiles than the first."""
-    L = 700
     q, k, v = gen(22, [L], hq, hkv, d, "bf16")
     r = Runner(1, hq, hkv, d, "bf16", L)
     qp = np.arange(L, dtype=np.int32)[::-1] - 5                   # the last rows see nothing
