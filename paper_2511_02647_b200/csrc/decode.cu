@@ -7,7 +7,12 @@
 // swizzle (conflict-free ldmatrix).  Row max / row sum are reduced with warp shuffles inside
 // each 4-lane quad.
 //
-// Two launches per decode call, chained by programmatic dependent launch:
+// Short calls (kOneLaunchBytes, kOneLaunchTiles) are one launch: the splits of a (cache, KV head) form a cluster, and
+// the partials are merged in its shared memory.  A call of that size streams for 2-3 us, so what it costs is launches
+// (6 us of host time for two, 4 for one) and the way through the scratch: 4 x 160 keys 2.8 -> 1.4 us, 2800 shared keys
+// 6.6 -> 3.0 us, both and their merge 16.2 -> 10.7 us; four blocks over 16 x 100 keys 26 -> 13 us.
+//
+// Longer calls are two launches, chained by programmatic dependent launch:
 //   decode_stream_kernel  one CTA per (cache, KV head, split); every warp walks its key slice of the
 //                         split's tiles and leaves an unnormalised partial (m, l, o) per query row in
 //                         global scratch.  Nothing is merged here, so a CTA ends with its last tile.
@@ -25,6 +30,7 @@
 // outputs and the scratch: the launcher checks the inputs of a call against the outputs of the recent
 // calls of that kind and falls back to waiting first when they overlap (early_start.cu).  No CTA ever
 // waits on another CTA.
+#include <cooperative_groups.h>
 #include <string.h>
 
 #include "common.cuh"
@@ -41,6 +47,9 @@ constexpr int kStageBytes = 2 * kTileBytes;             // K + V
 constexpr int kPartialStride = kD + 4;                  // m, l, 2 pad, o[128]: o is 16-byte aligned
 constexpr float kRescaleThreshold = 8.0f;               // log2 units
 constexpr int kMaxSlots = 64;                           // partials per output row: splits x key slices of a CTA
+constexpr int kMaxCluster = 8;                          // splits of a one-launch call (portable cluster size)
+constexpr int64_t kOneLaunchBytes = 16 << 20;           // K and V of a one-launch call, at most
+constexpr int kOneLaunchTiles = 6;                      // and the longest walk of its CTAs
 constexpr int kMergeGroups = 4;                         // the merge kernel sums a row's partials in this many groups
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -102,7 +111,9 @@ __device__ long long g_dtrace[1024 * 8];
 // fragments are read by two warps), which halves the partials per output row.
 // Partial of output row r, slot s = split * kSlices + slice:  partial[(r * n_slots + s) * kPartialStride]
 // = { m (log2 domain, scale included), l, -, -, o[128] }, unnormalised.
-template <int kMTiles>
+// kOneLaunch: the grid's x extent is one cluster; warps leave their partials in shared memory, every CTA folds its
+// slices, and rank r of the cluster folds and writes rows r, r + n_splits, ...
+template <int kMTiles, bool kOneLaunch>
 __global__ void __launch_bounds__(128, 2)
 decode_stream_kernel(const DecodeParams p, int n_splits, int n_chunks)
 {
@@ -279,8 +290,9 @@ decode_stream_kernel(const DecodeParams p, int n_splits, int n_chunks)
 
 
     // the scratch may still be read by the merge of the previous call: the preceding grid must be complete
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    // ---- every warp leaves the partial of its key slice: nothing is merged here ----
+    // (one launch: so must it be before the outputs are written, and before this grid ends)
+    if (!kOneLaunch) asm volatile("griddepcontrol.wait;" ::: "memory");
+    // ---- every warp leaves the partial of its key slice ----
     constexpr int kRows = 16 * kMTiles;
     const int rows_here = min(kRows, rows_total - chunk * kRows);   // LOCAL stacks g rows into a 16-row tile
     const int n_slots = n_splits * kSlices, slot = split * kSlices + slice;
@@ -296,21 +308,89 @@ decode_stream_kernel(const DecodeParams p, int n_splits, int n_chunks)
     l0 += __shfl_xor_sync(0xffffffffu, l0, 1); l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
     l1 += __shfl_xor_sync(0xffffffffu, l1, 1); l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
     const int ra = mt * 16 + (lane >> 2), rb = ra + 8;          // this thread's rows inside the CTA
+    float *part = reinterpret_cast<float *>(smem);              // one launch: [slice][row], where the tiles were
+    if (kOneLaunch) __syncthreads();
     if (ra < rows_here) {
-        float *dst = p.partial + (out_row(chunk * kRows + ra) * n_slots + slot) * kPartialStride;
+        float *dst = kOneLaunch ? part + (slice * kRows + ra) * kPartialStride
+                                : p.partial + (out_row(chunk * kRows + ra) * n_slots + slot) * kPartialStride;
         if ((lane & 3) == 0) *reinterpret_cast<float2 *>(dst) = make_float2(m0, l0);
         dst += 4 + (lane & 3) * 2;
 #pragma unroll
         for (int i = 0; i < 16; ++i) *reinterpret_cast<float2 *>(dst + i * 8) = make_float2(acc[i][0], acc[i][1]);
     }
     if (rb < rows_here) {
-        float *dst = p.partial + (out_row(chunk * kRows + rb) * n_slots + slot) * kPartialStride;
+        float *dst = kOneLaunch ? part + (slice * kRows + rb) * kPartialStride
+                                : p.partial + (out_row(chunk * kRows + rb) * n_slots + slot) * kPartialStride;
         if ((lane & 3) == 0) *reinterpret_cast<float2 *>(dst) = make_float2(m1, l1);
         dst += 4 + (lane & 3) * 2;
 #pragma unroll
         for (int i = 0; i < 16; ++i) *reinterpret_cast<float2 *>(dst + i * 8) = make_float2(acc[i][2], acc[i][3]);
     }
     DTRACE(4);
+    if (!kOneLaunch) return;
+
+    // ---- fold the slices of this CTA: a warp per row, four columns per lane, into the row's first slice ----
+    namespace cg = cooperative_groups;
+    __syncthreads();
+    for (int row = warp; row < rows_here; row += 4) {
+        float *src = part + row * kPartialStride;
+        float2 ml[kSlices];
+        float mx = -INFINITY;
+#pragma unroll
+        for (int q = 0; q < kSlices; ++q) {
+            ml[q] = *reinterpret_cast<const float2 *>(src + q * kRows * kPartialStride);
+            mx = fmaxf(mx, ml[q].x);
+        }
+        const float ms = mx == -INFINITY ? 0.f : mx;
+        float z = 0.f;
+        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < kSlices; ++q) {
+            const float4 v = *reinterpret_cast<const float4 *>(src + q * kRows * kPartialStride + 4 + lane * 4);
+            const float f = ex2(ml[q].x - ms);                  // 0 for an empty partial (m = -inf)
+            z += ml[q].y * f;
+            o.x += v.x * f; o.y += v.y * f; o.z += v.z * f; o.w += v.w * f;
+        }
+        __syncwarp();                                           // every lane has read the maxima and sums
+        if (lane == 0) *reinterpret_cast<float2 *>(src) = make_float2(mx, z);
+        *reinterpret_cast<float4 *>(src + 4 + lane * 4) = o;
+    }
+    // ---- fold the CTAs of the cluster ----
+    cg::cluster_group cluster = cg::this_cluster();
+    if (n_splits > 1) cluster.sync(); else __syncthreads();
+    asm volatile("griddepcontrol.wait;" ::: "memory");          // before the first write
+    for (int row = split + n_splits * warp; row < rows_here; row += n_splits * 4) {
+        float2 ml[kMaxCluster];
+        float4 v[kMaxCluster];
+        float mx = -INFINITY;
+#pragma unroll
+        for (int q = 0; q < kMaxCluster; ++q) {
+            ml[q] = make_float2(-INFINITY, 0.f);
+            v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (q < n_splits) {
+                const float *src = (n_splits > 1 ? cluster.map_shared_rank(part, q) : part) + row * kPartialStride;
+                ml[q] = *reinterpret_cast<const float2 *>(src);
+                v[q] = *reinterpret_cast<const float4 *>(src + 4 + lane * 4);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < kMaxCluster; ++q) mx = fmaxf(mx, ml[q].x);
+        const float ms = mx == -INFINITY ? 0.f : mx;
+        float z = 0.f;
+        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < kMaxCluster; ++q) {
+            const float f = ex2(ml[q].x - ms);
+            z += ml[q].y * f;
+            o.x += v[q].x * f; o.y += v[q].y * f; o.z += v[q].z * f; o.w += v[q].w * f;
+        }
+        const float inv = z > 0.f ? 1.f / z : 0.f;
+        const size_t orow = out_row(chunk * kRows + row);
+        const uint2 w = make_uint2(pack_bf16(o.x * inv, o.y * inv), pack_bf16(o.z * inv, o.w * inv));
+        *reinterpret_cast<uint2 *>(reinterpret_cast<__nv_bfloat16 *>(p.o) + orow * kD + lane * 4) = w;
+        if (lane == 0 && p.lse) p.lse[orow] = z > 0.f ? (mx + log2f(z)) * 0.6931471805599453f : -INFINITY;
+    }
+    if (n_splits > 1) cluster.sync();                           // peers may still be reading this CTA's partials
 }
 
 // A CTA takes output rows (participant, query head) blockIdx.x, blockIdx.x + gridDim.x, ...: thread =
@@ -429,22 +509,37 @@ static cudaError_t launch_decode_split(const DecodeParams &p_in, int device, int
     if (n_splits > tiles / 2) n_splits = tiles / 2;            // at least two tiles per split
     if (n_splits > kMaxSlots / slices) n_splits = kMaxSlots / slices;
     if (n_splits < 1) n_splits = 1;
+    // One launch where the call is short and a cluster's CTAs do not walk long (16 000 keys of 2 KV heads by 16 x 7 rows:
+    // 32 splits take 12 us, 8 take 31); two CTAs per SM hold a cluster of 8 everywhere.
+    int cluster = 1;
+    while (cluster * 2 <= n_splits && cluster < kMaxCluster) cluster *= 2;
+    const bool one_launch = (int64_t)caches * p.hkv * p.max_kv_len * kD * 4 <= kOneLaunchBytes && tiles <= kOneLaunchTiles * cluster;
+    if (one_launch) n_splits = cluster;
     const int n_slots = n_splits * slices;
-    if ((size_t)p.n_part * p.hq * n_slots * kPartialStride * sizeof(float) > p.partial_bytes) return cudaErrorInvalidValue;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
+    if (!one_launch && (size_t)p.n_part * p.hq * n_slots * kPartialStride * sizeof(float) > p.partial_bytes) return cudaErrorInvalidValue;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = n_splits; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(n_splits, p.hkv, caches * n_chunks);
     cfg.blockDim = dim3(128, 1, 1);
     cfg.dynamicSmemBytes = kStages * kStageBytes;              // 96 KB
     cfg.stream = s;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = m_tiles == 1 ? cudaLaunchKernelEx(&cfg, decode_stream_kernel<1>, p, n_splits, n_chunks)
-                                 : cudaLaunchKernelEx(&cfg, decode_stream_kernel<2>, p, n_splits, n_chunks);
+    cfg.attrs = attr;
+    cfg.numAttrs = one_launch ? 2 : 1;
+    cudaError_t e;
+    if (one_launch)
+        e = m_tiles == 1 ? cudaLaunchKernelEx(&cfg, decode_stream_kernel<1, true>, p, n_splits, n_chunks)
+                         : cudaLaunchKernelEx(&cfg, decode_stream_kernel<2, true>, p, n_splits, n_chunks);
+    else
+        e = m_tiles == 1 ? cudaLaunchKernelEx(&cfg, decode_stream_kernel<1, false>, p, n_splits, n_chunks)
+                         : cudaLaunchKernelEx(&cfg, decode_stream_kernel<2, false>, p, n_splits, n_chunks);
     if (launches) ++*launches;
+    if (one_launch) return e != cudaSuccess ? e : cudaGetLastError();
+    cfg.numAttrs = 1;
     if (e != cudaSuccess) return e;
     const int n_rows = p.n_part * p.hq, rows_per_cta = (n_rows + sm_count - 1) / sm_count;
     cfg.gridDim = dim3((n_rows + rows_per_cta - 1) / rows_per_cta, 1, 1);
@@ -458,9 +553,11 @@ static cudaError_t launch_decode_split(const DecodeParams &p_in, int device, int
 static cudaError_t set_decode_smem_attr()
 {
     const int smem = kStages * kStageBytes;
-    cudaError_t e = cudaFuncSetAttribute(decode_stream_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(decode_stream_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaSuccess;
+    void (*const kernels[])(const DecodeParams, int, int) = {decode_stream_kernel<1, false>, decode_stream_kernel<2, false>,
+                                                             decode_stream_kernel<1, true>, decode_stream_kernel<2, true>};
+    for (auto k : kernels)
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     return e;
 }
 
