@@ -92,21 +92,25 @@ struct KernelParams {
 };
 
 // Position tables of a general-position call (ints, in this order): minimum and maximum position of
-// every query tile; then per KV position array (one per KV head when head-major, else one) the
-// running minimum over the tiles j, j+1, ... (suffix minimum) and the running maximum over the tiles
-// 0 .. j (prefix maximum) of the tile's key positions.  Both runs are monotone in j, so "tiles that
-// can hold a visible key" and "tiles whose keys are all visible" are prefixes found by bisection.
-// A ragged last KV tile counts as never fully visible (maximum = INT_MAX).
+// every query tile; then per KV position array (one per KV head when head-major, else one) the minimum and
+// the maximum of every KV tile's key positions.  A query tile walks the KV tiles whose minimum does not exceed its
+// largest position; those whose maximum does not exceed its smallest need no test.  A ragged last KV tile counts as
+// never fully visible (maximum = INT_MAX).
 struct PosTables {
-    const int32_t *q_min, *q_max, *suf_min, *pre_max;
+    const int32_t *q_min, *q_max, *kv_min, *kv_max;
 };
 __device__ __host__ __forceinline__ PosTables pos_tables(const int32_t *tab, int n_qtiles, int n_arrays, int n_kt)
 {
     PosTables t;
     t.q_min = tab; t.q_max = tab + n_qtiles;
-    t.suf_min = tab + 2 * (size_t)n_qtiles; t.pre_max = t.suf_min + (size_t)n_arrays * n_kt;
+    t.kv_min = tab + 2 * (size_t)n_qtiles; t.kv_max = t.kv_min + (size_t)n_arrays * n_kt;
     return t;
 }
+// Where an item's walk has tiles to skip, the producer leaves it in shared memory as a list (bit 15: the tile needs no
+// test).  Longer lists than that has room for become "every tile up to the last visible one".  (Participants that hold
+// alternate tokens of the sequence, four of 5001 rows in all, 32 / 8 heads: 955 us walking up to the last visible tile,
+// 556 us with the list; contiguous members have nothing to skip.)
+constexpr int kWalkMost = 128;
 
 #ifdef FEDATTN_TRACE
 // Debug build only: cycle stamps of one CTA's pipeline events, [tile][event].
@@ -499,7 +503,7 @@ __device__ __forceinline__ int last_visible_tile(const KernelParams &kp, const I
 // serves explicit positions and bidirectional remote-only attention (two key ranges); the plain instance
 // carries none of their state.  Causal remote-only attention is one more prefix mask: plain instance.
 template <bool kSpecial, bool kExact, bool kHalves>
-__device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, int lane, Sub (&sub)[2])
+__device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, int lane, Sub (&sub)[2], uint16_t *walk)
 {
     const PrefillParams &p = kp.p;
     Item it;
@@ -554,7 +558,35 @@ __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, in
     sub[0].n_tiles = sub[1].n_tiles = 0;
     it.n_a = 0;
     if (sub[1].n_valid == 0) return it;                         // no such query tile
-    if (p.sync && p.remote_only && !(kExact && kp.pairs)) {
+    if (kSpecial && !kExact && p.general) {
+        // both sub-tiles walk what either may see
+        const PosTables pt = pos_tables(p.tab, kp.n_qtiles, p.kv_head_major ? p.hkv : 1, kp.n_kt);
+        const size_t first = p.kv_head_major ? (size_t)it.kvh * kp.n_kt : 0;
+        int q_max = __ldg(pt.q_max + (sub[1].q_row0 >> 7)), q_min = __ldg(pt.q_min + (sub[1].q_row0 >> 7));
+        if (two_rows && sub[0].n_valid > 0) {
+            q_max = max(q_max, __ldg(pt.q_max + (sub[0].q_row0 >> 7)));
+            q_min = min(q_min, __ldg(pt.q_min + (sub[0].q_row0 >> 7)));
+        }
+        int n = 0, last = 0, run = 0;                           // visible tiles, end of the last, leading run without a test
+        bool in_run = true;
+        for (int t0 = 0; t0 < kp.n_kt; t0 += 32) {
+            const int t = min(t0 + lane, kp.n_kt - 1);
+            const bool in = t0 + lane < kp.n_kt;
+            const uint32_t seen = __ballot_sync(0xffffffffu, in && __ldg(pt.kv_min + first + t) <= q_max);
+            const uint32_t free = __ballot_sync(0xffffffffu, in && __ldg(pt.kv_max + first + t) <= q_min);
+            const int at = n + __popc(seen & ((1u << lane) - 1u));
+            if (((seen >> lane) & 1u) && at < kWalkMost) walk[at] = (uint16_t)(t | (((free >> lane) & 1u) << 15));
+            n += __popc(seen);
+            if (seen) last = t0 + 32 - __clz(seen);
+            if (in_run) run += free == 0xffffffffu ? 32 : __ffs(~free) - 1;
+            in_run = in_run && free == 0xffffffffu;
+        }
+        // nothing to skip (contiguous members), or no room for the list: a prefix of tiles, of which `run` need no test
+        it.b = n == last || n > kWalkMost || kp.n_kt > 0x7fff ? run : -1;
+        if (it.b >= 0) n = last;
+        it.n_a = sub[1].n_tiles = n;
+        sub[0].n_tiles = sub[0].n_valid > 0 ? n : 0;
+    } else if (p.sync && p.remote_only && !(kExact && kp.pairs)) {
         // keys [0, a) lie before the rows' segment; when bidirectional (special instance only), keys [b, T)
         // after it count too
         const int T = (int)p.total_kv, n_t = (T + kTileN - 1) / kTileN;
@@ -574,16 +606,8 @@ __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, in
         for (int again = two_rows && sub[0].n_valid > 0 ? 1 : 0;; again = 0) {
             const Sub x = again ? sub[0] : sub[1];
             int n;
-            if (kExact && kp.pairs) {
-                n = last_visible_tile(kp, it, x, lane);
-            } else if (kSpecial && p.general) {
-                // tiles up to the last one that holds a key position <= the tile's largest query position
-                const PosTables pt = pos_tables(p.tab, kp.n_qtiles, p.kv_head_major ? p.hkv : 1, kp.n_kt);
-                const int32_t *suf = pt.suf_min + (p.kv_head_major ? (size_t)it.kvh * kp.n_kt : 0);
-                n = count_le_warp(suf, kp.n_kt, __ldg(pt.q_max + (x.q_row0 >> 7)), lane);
-            } else {
-                n = (prefix_len<kSpecial>(p, it, x, x.n_valid - 1, lane) + kTileN - 1) / kTileN;
-            }
+            if (kExact && kp.pairs) n = last_visible_tile(kp, it, x, lane);
+            else n = (prefix_len<kSpecial>(p, it, x, x.n_valid - 1, lane) + kTileN - 1) / kTileN;
             if (again) { sub[0].n_tiles = n; continue; }
             sub[1].n_tiles = n;
             break;
@@ -647,6 +671,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     // 16 ints, filled an item ahead), so that decoding is not on their path between two items.
     uint64_t *item_full = bars + 20, *item_empty = bars + 22;
     volatile int *item_pub = reinterpret_cast<volatile int *>(bars + 32);
+    uint16_t *walks = reinterpret_cast<uint16_t *>(bars + 48);      // general: [slot][kWalkMost]
     uint8_t *stage = smem + 6 * kTileBytes + 1024;       // [softmax warp][32 rows][128 B], 128-byte swizzle
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -700,7 +725,14 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             const int item = item_of(k);
             if (item >= n_items) continue;
             Sub sub[2];
-            const Item it = decode_item<kSpecial, kExact, kHalves>(kp, item, lane, sub);
+            const bool general = kSpecial && !kExact && p.general;
+            if (general && pn >= 2) {                           // the walk goes into the slot while decoding
+                if (lane == 0) mbar_wait_call(item_empty + (pn & 1), ((pn >> 1) - 1) & 1, abort_flag, kp.status);
+                __syncwarp();
+            }
+            uint16_t *walk = walks + (pn & 1) * kWalkMost;
+            const Item it = decode_item<kSpecial, kExact, kHalves>(kp, item, lane, sub, walk);
+            __syncwarp();
             const int n_tiles = sub[1].n_tiles + (kHalves ? sub[0].n_tiles : 0);
             if (lane == 0) {
                 if (pn >= 2) mbar_wait_call(item_empty + (pn & 1), ((pn >> 1) - 1) & 1, abort_flag, kp.status);
@@ -734,9 +766,12 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                         tma_load_3d(sQ + t * kTileBytes, &map_q, q_full, 0, sub[t].head, sub[t].q_row0);
                         if (kBoxes == 2) tma_load_3d(sQ + t * kTileBytes + kHalfBytes, &map_q, q_full, 64, sub[t].head, sub[t].q_row0);
                     }
+                const bool listed = general && it.b < 0;
                 for (int j = 0; j < n_tiles; ++j) {
                     const int gt = git + j, st = gt & 1, use = gt >> 1;
-                    const int row = it.kv_begin + (kSpecial ? tile_of(it, j) : j) * kTileN;
+                    int tile = kSpecial ? tile_of(it, j) : j;
+                    if (listed) tile = walk[j] & 0x7fff;
+                    const int row = it.kv_begin + tile * kTileN;
                     const int c1 = p.kv_head_major ? row : it.kvh, c2 = p.kv_head_major ? it.kvh : row;
                     if (gt >= 2) mbar_wait_call(k_empty + st, (use - 1) & 1, abort_flag, kp.status);
                     TRACE(j, 7);
@@ -1007,6 +1042,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             if (item >= n_items) continue;
             Item it;
             Sub sub;
+            bool listed = false;                                // the walk is a list of tiles, not a prefix
             bool halved = false;                                // the other warpgroup walks the other KV tiles of these rows
             {
                 mbar_wait(item_full + (pn & 1), (pn >> 1) & 1, abort_flag, kp.status);
@@ -1018,13 +1054,17 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 halved = kHalves && slot[11] > 0;
                 it.kvp = p.kv_pos ? p.kv_pos + (p.kv_head_major ? (int64_t)it.kvh * p.total_kv : 0) : nullptr;
                 __syncwarp();
-                if (lane == 0) mbar_arrive(item_empty + (pn & 1));
+                // (a listed walk is read as it goes: the slot is given back behind it)
+                listed = kSpecial && !kExact && p.general && it.b < 0;
+                if (lane == 0 && !listed) mbar_arrive(item_empty + (pn & 1));
                 ++pn;
             }
             const int n_tiles = sub.n_tiles;
             const bool valid = r < sub.n_valid;
             __nv_bfloat16 *orow = reinterpret_cast<__nv_bfloat16 *>(p.o) + ((int64_t)(sub.q_row0 + r) * p.hq + sub.head) * d;
             float *lse_p = p.lse ? p.lse + (int64_t)(sub.q_row0 + r) * p.hq + sub.head : nullptr;
+            const bool general = kSpecial && !kExact && p.general;
+            if (n_tiles == 0 && listed && lane == 0) mbar_arrive(item_empty + ((pn - 1) & 1));
             if (n_tiles == 0) {                                 // nothing visible to any row of the tile, or no rows
                 if (valid) {
                     for (int c = 0; c < d; c += 8) *reinterpret_cast<uint4 *>(orow + c) = make_uint4(0, 0, 0, 0);
@@ -1033,7 +1073,6 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 continue;
             }
             const bool two_range = kSpecial && p.sync && p.remote_only && !p.causal;      // (pairs comes first)
-            const bool general = kSpecial && p.general;
             const bool pairs = kExact && kp.pairs;
             int c_row = 0, n_full = 0, p_row = 0;
             PairRule mine{0, 0, false}, all{0, 0, false};       // pairs: this row's rule, and what every row of the warp sees
@@ -1052,11 +1091,8 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 all.lo = __reduce_min_sync(0xffffffffu, mine.lo);
                 load_pos(kHalves ? 1 - t : 0);
             } else if (general) {
-                // every (query, key) pair on its own positions; the tiles whose keys all lie at or below the
-                // tile's smallest query position (a prefix of the walk, see PosTables) need no test
-                const PosTables pt = pos_tables(p.tab, kp.n_qtiles, p.kv_head_major ? p.hkv : 1, kp.n_kt);
-                const int32_t *pre = pt.pre_max + (p.kv_head_major ? (size_t)it.kvh * kp.n_kt : 0);
-                n_full = count_le_warp(pre, kp.n_kt, __ldg(pt.q_min + (sub.q_row0 >> 7)), lane);
+                // every (query, key) pair on its own positions
+                n_full = it.b;
                 const int row = sub.q_row0 + min(r, sub.n_valid - 1);
                 p_row = p.q_pos ? __ldg(p.q_pos + row) : row;
             } else {
@@ -1084,7 +1120,12 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             const int T = (int)p.total_kv;
             float m_run = 0.f, l_run = 0.f;
             for (int j = 0; j < n_tiles; ++j) {
-                const int gt = gsub + j, tile = kHalves ? 2 * j + 1 - t : j;
+                const int gt = gsub + j;
+                int tile = kHalves ? 2 * j + 1 - t : j, entry = 0;
+                if (listed) {
+                    entry = reinterpret_cast<const volatile uint16_t *>(walks)[((pn - 1) & 1) * kWalkMost + tile];
+                    tile = entry & 0x7fff;
+                }
                 // which columns of this tile the thread's row sees: everything (warp-uniform), or a mask per chunk
                 bool full;
                 uint32_t vm[4] = {0, 0, 0, 0};
@@ -1117,7 +1158,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                         }
                     }
                 } else {
-                    full = tile < n_full;
+                    full = listed ? (entry >> 15) != 0 : tile < n_full;
                     if (!full && general) {
                         // column i of chunk c is key cb + i: visible iff it exists and its position is not above
                         // the row's.  The address is the same in every lane: broadcast loads.
@@ -1140,6 +1181,11 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 }
                 if (full) visit(std::false_type{}, j, gt, vm, m_run, l_run);
                 else visit(std::true_type{}, j, gt, vm, m_run, l_run);
+            }
+
+            if (listed) {
+                __syncwarp();
+                if (lane == 0) mbar_arrive(item_empty + ((pn - 1) & 1));
             }
 
             // ---- epilogue: drain this row of O from TMEM (frees it for the next item), O / l -> bf16 -> global
@@ -1322,8 +1368,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 
 // ---- position tables of a general-position call -------------------------------------------------------
 // grid: one block per KV position array (n_arrays of them), then one block for the query positions.
-// A warp reduces one 128-entry tile at a time (one 16-byte load per lane when the array allows it).  The
-// KV blocks then turn the per-tile values into the running suffix minimum / prefix maximum in place.
+// A warp reduces one 128-entry tile at a time.
 constexpr int kTabThreads = 1024;
 
 __device__ __forceinline__ void tile_min_max(const int32_t *pos, int64_t n, int64_t tile, int lane, int &mn, int &mx)
@@ -1362,40 +1407,12 @@ position_tables_kernel(const int32_t *q_pos, int64_t n_q, const int32_t *kv_pos,
     }
     const int a = blockIdx.x;
     const int32_t *pos = kv_pos ? kv_pos + (size_t)a * total_kv : nullptr;
-    int32_t *suf = const_cast<int32_t *>(pt.suf_min) + (size_t)a * n_kt, *pre = const_cast<int32_t *>(pt.pre_max) + (size_t)a * n_kt;
+    int32_t *kv_min = const_cast<int32_t *>(pt.kv_min) + (size_t)a * n_kt, *kv_max = const_cast<int32_t *>(pt.kv_max) + (size_t)a * n_kt;
     for (int64_t t = warp; t < n_kt; t += n_warps) {
         int mn, mx;
         tile_min_max(pos, total_kv, t, lane, mn, mx);
         if ((t + 1) * kTileN > total_kv) mx = INT32_MAX;      // ragged tile: never fully visible
-        if (lane == 0) { suf[t] = mn; pre[t] = mx; }
-    }
-    __syncthreads();
-    if (warp == 0) {                                           // prefix maximum, 32 tiles per step
-        int carry = INT32_MIN;
-        for (int t0 = 0; t0 < n_kt; t0 += 32) {
-            int v = t0 + lane < n_kt ? pre[t0 + lane] : INT32_MIN;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int u = __shfl_up_sync(0xffffffffu, v, o);
-                if (lane >= o) v = max(v, u);
-            }
-            v = max(v, carry);
-            if (t0 + lane < n_kt) pre[t0 + lane] = v;
-            carry = __shfl_sync(0xffffffffu, v, 31);
-        }
-    } else if (warp == 1) {                                    // suffix minimum, from the last tile backwards
-        int carry = INT32_MAX;
-        for (int t0 = ((n_kt - 1) / 32) * 32; t0 >= 0; t0 -= 32) {
-            int v = t0 + lane < n_kt ? suf[t0 + lane] : INT32_MAX;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int u = __shfl_down_sync(0xffffffffu, v, o);
-                if (lane + o < 32) v = min(v, u);
-            }
-            v = min(v, carry);
-            if (t0 + lane < n_kt) suf[t0 + lane] = v;
-            carry = __shfl_sync(0xffffffffu, v, 0);
-        }
+        if (lane == 0) { kv_min[t] = mn; kv_max[t] = mx; }
     }
 }
 
@@ -1509,6 +1526,12 @@ static ItemForm item_form(const PrefillParams &p, int64_t n_qtiles, int sm_count
     float load[kMostSms];
     int longest = 0;
     for (int n = 0; n < p.n_seg; ++n) longest = tiles_of(n) > longest ? tiles_of(n) : longest;
+    if (n_qtiles * p.hq <= sm_count) {                          // an item per CTA in every form: the longest one decides
+        float w = 0.f;
+        for (int n = 0; n < p.n_seg; ++n)
+            if (tiles_of(n) > 0) w = walk(n, tiles_of(n), tiles_of(n)) > w ? walk(n, tiles_of(n), tiles_of(n)) : w;
+        return w > 1.f && half * w + merge + start < 0.95f * ((g > 1 ? pair : 1.f) * w + start) ? kHalvesForm : kPairs;
+    }
     auto ends = [&](ItemForm form) -> float {
         const int rows = form == kStraddle ? 2 : 1;             // query tiles per ranked tile
         for (int c = 0; c < sm_count; ++c) load[c] = 0.f;

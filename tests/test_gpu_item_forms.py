@@ -54,3 +54,18 @@ def test_positions_that_fall_along_the_rows(hq, hkv, d, L):
     check(r.sync(q, k, v, q_pos=qp.copy()), reference(q, k, v, np.arange(L)[None] <= qp[:, None]), "falling q_pos")
     pos = np.random.default_rng(6).permutation(L).astype(np.int32)
     check(r.sync(q, k, v, kv_pos=pos, q_pos=qp.copy()), reference(q, k, v, pos[None] <= qp[:, None]), "falling q_pos, any kv_pos")
+
+
+@pytest.mark.parametrize("T", [256 * 128, 300 * 128 + 20])
+def test_walks_that_skip_tiles_and_walks_too_long_to_list(T):
+    """Explicit positions, every other KV tile beyond what the rows see: 128 tiles are listed, 150 and more are walked up
+    to the last visible one."""
+    rows = 130
+    q, k, v = gen(23, [T], 2, 1, 128, "bf16")
+    q = q[:rows]
+    rng = np.random.default_rng(7)
+    tile, within = np.arange(T) // 128, np.arange(T) % 128
+    pos = np.where(tile % 2 == 0, (tile // 2) * 128 + within, T + tile).astype(np.int32)
+    qp = np.concatenate([[0], rng.integers(0, T // 2, rows - 2), [T - 1]]).astype(np.int32)
+    r = Runner(1, 2, 1, 128, "bf16", rows, T)
+    check(r.sync(q, k, v, kv_pos=pos, q_pos=qp), reference(q, k, v, pos[None] <= qp[:, None]), "%d keys" % T)
