@@ -126,7 +126,7 @@ constexpr int kCtasPerSm = 2;              // resident CTAs the staging rings ar
 template <int kDtype>
 __global__ void __launch_bounds__(kSelThreads)
 topk_fused_kernel(const PartsParams pp, int hkv, int vpr /* 16-byte vectors per (row, head) */,
-                  int n_stages /* buffers in every warp's staging ring, 2..4 */,
+                  int n_stages /* buffers in every warp's staging ring, 2..4 or 6 */,
                   int max_len /* longest participant: sizes the key arrays */,
                   int early /* the inputs may be read before the preceding grid of the stream is complete */,
                   long long my_seq /* this call's sequence number in its context */,
@@ -233,7 +233,8 @@ topk_fused_kernel(const PartsParams pp, int hkv, int vpr /* 16-byte vectors per 
             copy_unit(u + n_stages - 1);                       // into the buffer walked one unit ago
             if (n_stages == 2) asm volatile("cp.async.wait_group 1;" ::: "memory");
             else if (n_stages == 3) asm volatile("cp.async.wait_group 2;" ::: "memory");
-            else asm volatile("cp.async.wait_group 3;" ::: "memory");
+            else if (n_stages == 4) asm volatile("cp.async.wait_group 3;" ::: "memory");
+            else asm volatile("cp.async.wait_group 5;" ::: "memory");
             __syncwarp();
             const int g = warp + (u / n_blk) * (kSelThreads / 32), blk = u % n_blk;
             const int row = r0 + g * 32 + lane;
@@ -497,6 +498,16 @@ cudaError_t launch_topk_fused(const PartsParams &pp, int hkv, int d, int dtype, 
     int max_len = 0;
     for (int i = 0; i < pp.n; ++i) max_len = max(max_len, pp.off[i + 1] - pp.off[i]);
     if (max_len > kSelMaxLen) return cudaErrorInvalidValue;
+    // slices per (head, participant): a power of two <= 8 (one cluster), about two CTAs per SM in total, and
+    // every slice keeps at least one token per lane of the CTA (a lane walks one key row at a time)
+    const int pairs = hkv * pp.n;
+    int slices = 1;
+    while (slices * 2 <= kMaxSlices && pairs * slices * 2 <= sm_count && max_len >= kSelThreads * slices * 2) slices *= 2;
+    // A call of few CTAs (few participants, whole tokens) is bound by what one CTA does: more slices share the rows to
+    // score and to gather, down to two warps' rows each.  Six participants of 64 to 700 tokens, 8 KV heads, whole
+    // tokens: 68 -> 33 us after another kernel (with the ring below), 22.6 -> 13.6 us back to back; what is left of the
+    // former is the chain of 1024 dependent fp64 additions, 25 us.
+    while (slices * 2 <= kMaxSlices && pairs * slices * 4 <= sm_count && max_len >= 64 * slices * 2) slices *= 2;
     // Shared memory per CTA: keys (8 B) and kept rows (2 B) per token of the longest participant, then
     // the staging buffers.  As many buffers (2..4) as still let kCtasPerSm CTAs share an SM: what is in
     // flight from HBM is all but one of them.  More resident CTAs matter more than deeper rings: CTAs in
@@ -506,6 +517,9 @@ cudaError_t launch_topk_fused(const PartsParams &pp, int hkv, int d, int dtype, 
     const int per_cta = (228 * 1024) / kCtasPerSm - 1024 /*reserved per CTA*/ - 2048 /*static*/;
     int n_stages = (per_cta - fixed) / stage_bytes;
     n_stages = n_stages < 2 ? 2 : (n_stages > 4 ? 4 : n_stages);
+    // Long rows on few CTAs: the deepest ring, one CTA per SM (three calls still fit side by side; with 64 CTAs per call
+    // the deeper ring keeps later calls off the SMs: 16 x 1024 whole tokens back to back 17 -> 22 us).
+    if (pairs * slices * 3 <= sm_count && vpr >= 32 && fixed + 6 * stage_bytes <= 227 * 1024 - 2048) n_stages = 6;
     const int smem = fixed + n_stages * stage_bytes;
     static bool attr_set[64] = {};                            // the attribute is per device
     if (!attr_set[device & 63]) {
@@ -516,11 +530,6 @@ cudaError_t launch_topk_fused(const PartsParams &pp, int hkv, int d, int dtype, 
         if (e != cudaSuccess) return e;
         attr_set[device & 63] = true;
     }
-    // slices per (head, participant): a power of two <= 8 (one cluster), about two CTAs per SM in total, and
-    // every slice keeps at least one token per lane of the CTA (a lane walks one key row at a time)
-    const int pairs = hkv * pp.n;
-    int slices = 1;
-    while (slices * 2 <= kMaxSlices && pairs * slices * 2 <= sm_count && max_len >= kSelThreads * slices * 2) slices *= 2;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(hkv, pp.n, slices);
