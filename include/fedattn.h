@@ -20,7 +20,7 @@
  *     ran out, an out-of-range or unsorted index in INDEXED mode, positions in an order the call
  *     cannot handle) sets a status word in the workspace that fedattn_poll reads; the kernel still
  *     terminates and the context stays usable.  Outputs of the call that raised the status are
- *     undefined.  After FEDATTN_ERR_TIMEOUT the bf16 head_dim 128 attention calls enqueued before
+ *     undefined.  After FEDATTN_ERR_TIMEOUT the bf16 local and sync attention calls enqueued before
  *     the next fedattn_poll do no work and leave their outputs untouched (they would otherwise
  *     each wait out the same limit); poll, then repeat them.
  *   - Q, K and V must be finite.  Rows outside a query's allowed set carry weight exactly 0, but
