@@ -858,7 +858,8 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     const int tile = kHalves ? 2 * j + i : j;
                     const int gt = ring + tile, st = gt & 1, ph = (gt >> 1) & 1;
                     const int gsub = (t ? git : git0) + j, qsub = t ? qn : qn0;
-                    mbar_wait_call(v_full + st, ph, abort_flag, kp.status);
+                    // (sub-tile 1 of a shared tile: sub-tile 0 has waited for it)
+                    if (kHalves || t == 0 || j >= n0) mbar_wait_call(v_full + st, ph, abort_flag, kp.status);
                     if (j == 0 && qsub > 0) mbar_wait_call(o_free + t, (qsub - 1) & 1, abort_flag, kp.status);
 #pragma unroll
                     for (int q = 0; q < kSplit; ++q) {
@@ -885,7 +886,8 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     if (kHalves || t == 1) commit(v_empty + st);
                     if (j + 1 < (t ? n1 : n0)) {
                         const int next = tile + (kHalves ? 2 : 1), st1 = (ring + next) & 1;
-                        mbar_wait_call(k_full + st1, ((ring + next) >> 1) & 1, abort_flag, kp.status);
+                        if (kHalves || t == 0 || j + 1 >= n0)
+                            mbar_wait_call(k_full + st1, ((ring + next) >> 1) & 1, abort_flag, kp.status);
                         issue_s(t, st1);
                         commit(s_full + t);
                         if (kHalves || t == 1) {
