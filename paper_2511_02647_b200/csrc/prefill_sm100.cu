@@ -938,6 +938,8 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         // vm[c] says whether column 32 c + i is visible to this thread's row.  Masked columns become -inf and
         // every exponential goes through ex2.approx, which maps -inf to 0; in unmasked tiles a fixed subset of
         // the columns takes the polynomial so that the ex2 unit is not the bottleneck.
+        // kAnyFirst: the tile in which a row sees its first key may be any of the walk (explicit positions).
+        constexpr bool kAnyFirst = kSpecial || kExact;
         auto visit = [&](auto partial_tag, int j, int gt, const uint32_t (&vm)[4], float &m_used, float &l) {
             constexpr bool kPartial = decltype(partial_tag)::value;
             mbar_wait(s_full + t, gt & 1, abort_flag, kp.status);
@@ -971,7 +973,8 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             const float rm = fmaxf(max3(mx[0], mx[1], mx[2]), fmaxf(max3(mx[3], mx[4], mx[5]), fmaxf(mx[6], mx[7])));
             const float t_max = rm * sl2;
             if (j == 0) {
-                m_used = (!kExact && t_max == -INFINITY) ? 0.f : t_max;
+                // (a row of a prefix mask that sees nothing of its first tile sees nothing at all)
+                m_used = (!kAnyFirst && t_max == -INFINITY) ? 0.f : t_max;
             } else {
                 // The exponent reference moves only when the maximum grew by more than 2^8; then what
                 // this row has accumulated so far (O in TMEM, l) is rescaled to the new reference.
@@ -993,8 +996,8 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 }
             }
             // ---- pass 2: exponentials, row sum, P ----
-            // (exact instances: a row that has seen no key yet keeps the reference -inf, all its weights are 0)
-            const float m_ref = kExact && m_used == -INFINITY ? 0.f : m_used;
+            // (a row that has seen no key yet keeps the reference -inf, all its weights are 0)
+            const float m_ref = kAnyFirst && m_used == -INFINITY ? 0.f : m_used;
             const uint64_t negm2 = pack_f32x2(-m_ref, -m_ref);
             uint64_t sum2[4] = {0, 0, 0, 0};
 #pragma unroll

@@ -8,7 +8,7 @@ import pytest
 import torch
 
 import fedattn_inputs as fi
-from helpers import Runner, dev, fa, host
+from helpers import LSE_TOL, Runner, dev, fa, host
 
 pytestmark = pytest.mark.gpu
 
@@ -113,23 +113,49 @@ def test_remote_only(dtype, hq, hkv, d, causal):
         check((host(o), host(lse)), reference(q, k[keys], v[keys], before if causal else before | after), dtype, what)
 
 
-@pytest.mark.parametrize("dtype,hq,hkv,d", KINDS)
-def test_rows_that_see_no_logit_near_zero(dtype, hq, hkv, d):
-    """A row whose first key tiles are all excluded and whose visible logits are near -300: its weights must not be
-    taken against a reference of 0."""
-    L = 400
-    q, k, v = gen(10, [L], hq, hkv, d, dtype)
+def low_logits(seed, L, hq, hkv, d, dtype):
+    """q, k, v whose logits all lie near -300."""
+    q, k, v = gen(seed, [L], hq, hkv, d, dtype)
     q = np.full_like(q, 4.0)
     k = k * 0.25 if dtype == "f32" else np.round(k * 4) / 16
     k -= 75.0 / np.sqrt(d)
     if dtype == "bf16":
         k = torch.from_numpy(k).to(torch.bfloat16).float().numpy()
-    pos = np.arange(L, dtype=np.int32)[::-1].copy()               # row 0 sees the last key only
+    return q, k, v
+
+
+def check_low(got, want, dtype, d):
+    # head_dim 128 takes a part of its exponentials to 7.5e-5 (LSE_TOL has the bound that follows for its lse)
+    assert want[1].max() < -200
+    assert np.abs(got[1] - want[1]).max() <= (LSE_TOL["bf16"] if dtype == "bf16" and d == 128 else 1e-4)
+    assert np.abs(got[0] - want[0]).max() <= (2e-2 if dtype == "bf16" else 1e-3)
+
+
+# head_dim 128 in bf16 too: items of one head whose KV tiles two sub-tiles share, and (36 heads) of two heads
+@pytest.mark.parametrize("dtype,hq,hkv,d", KINDS + [("bf16", 8, 8, 128), ("bf16", 2, 1, 128), ("bf16", 72, 36, 128)])
+def test_rows_that_see_no_logit_near_zero(dtype, hq, hkv, d):
+    """A row whose first key tiles are all excluded and whose visible logits are near -300: its weights must not be
+    taken against a reference of 0."""
+    L = 400
+    q, k, v = low_logits(10, L, hq, hkv, d, dtype)
+    rows = np.arange(L, dtype=np.int32)
     r = Runner(1, hq, hkv, d, dtype, L)
-    o, lse = r.sync(q, k, v, kv_pos=pos, q_pos=np.arange(L, dtype=np.int32))
-    wo, wl = reference(q, k, v, pos[None] <= np.arange(L)[:, None])
-    assert wl.max() < -200
-    assert np.abs(lse - wl).max() <= 1e-4 and np.abs(o - wo).max() <= (2e-2 if dtype == "bf16" else 1e-3)
+    pos = rows[::-1].copy()                                       # row 0 sees the last key only
+    check_low(r.sync(q, k, v, kv_pos=pos, q_pos=rows), reference(q, k, v, pos[None] <= rows[:, None]), dtype, d)
+    # every row sees keys of the first tile and of the last one, but only late rows see those between
+    pos = np.concatenate([rows[:128] // 4, 300 + rows[128:256] % 64, 280 + rows[256:384] % 64, rows[384:] - 384]).astype(np.int32)
+    check_low(r.sync(q, k, v, kv_pos=pos, q_pos=rows), reference(q, k, v, pos[None] <= rows[:, None]), dtype, d)
+
+
+@pytest.mark.parametrize("dtype,hq,hkv,d", [("bf16", 8, 8, 128), ("bf16", 32, 8, 128), ("bf16", 6, 2, 96)])
+def test_interleaved_members_with_low_logits(dtype, hq, hkv, d):
+    """Two members that hold alternate tokens of the sequence: a query tile sees a stretch of each member's KV tiles,
+    and its rows differ in the last one of either."""
+    L = 2000
+    q, k, v = low_logits(12, L, hq, hkv, d, dtype)
+    pos = np.concatenate([np.arange(0, L, 2), np.arange(1, L, 2)]).astype(np.int32)
+    r = Runner(2, hq, hkv, d, dtype, L)
+    check_low(r.sync(q, k, v, kv_pos=pos, q_pos=pos), reference(q, k, v, pos[None] <= pos[:, None]), dtype, d)
 
 
 @pytest.mark.parametrize("dtype,hq,hkv,d", KINDS)
