@@ -670,6 +670,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     // The producer decodes every work item once and publishes it here for the softmax warps (two slots of
     // 16 ints, filled an item ahead), so that decoding is not on their path between two items.
     uint64_t *item_full = bars + 20, *item_empty = bars + 22;
+    uint64_t *halves_met = bars + 28;                    // halves: both warpgroups have left their partials' (m, l)
     volatile int *item_pub = reinterpret_cast<volatile int *>(bars + 32);
     uint16_t *walks = reinterpret_cast<uint16_t *>(bars + 48);      // general: [slot][kWalkMost]
     uint8_t *stage = smem + 6 * kTileBytes + 1024;       // [softmax warp][32 rows][128 B], 128-byte swizzle
@@ -688,10 +689,12 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         mbar_init(q_full, 1); mbar_init(q_empty, 1);
         for (int i = 0; i < 2; ++i) {
             mbar_init(k_full + i, 1); mbar_init(k_empty + i, 1); mbar_init(v_full + i, 1); mbar_init(v_empty + i, 1);
-            mbar_init(s_full + i, 1); mbar_init(o_done + i, 1); mbar_init(o_free + i, 4);
+            mbar_init(s_full + i, 1); mbar_init(o_done + i, 1);
+            mbar_init(o_free + i, kHalves ? 8 : 4);             // (halves: every warp reads both accumulators)
             for (int q = 0; q < kSplit; ++q) mbar_init(p_full + kSplit * i + q, 4);
             mbar_init(item_full + i, 1); mbar_init(item_empty + i, 2 * kSplit * 2);
         }
+        mbar_init(halves_met, 8);
         *abort_flag = (*reinterpret_cast<volatile int32_t *>(kp.status) == FEDATTN_ERR_TIMEOUT) ? 1 : 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -721,21 +724,25 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&map_v) : "memory");
         }
         int git = 0, qn = 0, pn = 0;
+        // After a wait that ran out nothing is published or loaded any more: a slot may still be read, a buffer still be
+        // written.  (All lanes get lane 0's answer.)
+        auto slot_free = [&]() -> bool {
+            bool ok = true;
+            if (lane == 0 && pn >= 2) ok = mbar_wait_call(item_empty + (pn & 1), ((pn >> 1) - 1) & 1, abort_flag, kp.status);
+            return __shfl_sync(0xffffffffu, ok, 0);
+        };
         for (int k = 0; k < n_rounds; ++k) {
             const int item = item_of(k);
             if (item >= n_items) continue;
             Sub sub[2];
             const bool general = kSpecial && !kExact && p.general;
-            if (general && pn >= 2) {                           // the walk goes into the slot while decoding
-                if (lane == 0) mbar_wait_call(item_empty + (pn & 1), ((pn >> 1) - 1) & 1, abort_flag, kp.status);
-                __syncwarp();
-            }
+            if (general && !slot_free()) break;                 // the walk goes into the slot while decoding
             uint16_t *walk = walks + (pn & 1) * kWalkMost;
             const Item it = decode_item<kSpecial, kExact, kHalves>(kp, item, lane, sub, walk);
             __syncwarp();
             const int n_tiles = sub[1].n_tiles + (kHalves ? sub[0].n_tiles : 0);
+            if (!general && !slot_free()) break;
             if (lane == 0) {
-                if (pn >= 2) mbar_wait_call(item_empty + (pn & 1), ((pn >> 1) - 1) & 1, abort_flag, kp.status);
                 volatile int *slot = item_pub + (pn & 1) * 16;
                 slot[0] = it.kvh; slot[1] = it.seg; slot[2] = it.kv_begin; slot[3] = it.n_a; slot[4] = it.t_b0;
                 slot[5] = it.a; slot[6] = it.b;
@@ -755,8 +762,10 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             }
             ++pn;
             if (n_tiles == 0) continue;
-            if (lane == 0) {
-                if (qn > 0) mbar_wait_call(q_empty, (qn - 1) & 1, abort_flag, kp.status);   // previous item's S MMAs done
+            int issued = 0;                                     // lane 0: KV tiles of the item on their way
+            bool q_free = true;
+            if (lane == 0 && qn > 0) q_free = mbar_wait_call(q_empty, (qn - 1) & 1, abort_flag, kp.status);   // previous item's S MMAs done
+            if (lane == 0 && q_free) {
                 item_info[(qn & 1) * 2] = sub[1].n_tiles;
                 item_info[(qn & 1) * 2 + 1] = sub[0].n_tiles;
                 mbar_expect_tx(q_full, !kHalves && sub[0].n_tiles > 0 ? 2 * kTileBytes : kTileBytes);
@@ -773,20 +782,22 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     if (listed) tile = walk[j] & 0x7fff;
                     const int row = it.kv_begin + tile * kTileN;
                     const int c1 = p.kv_head_major ? row : it.kvh, c2 = p.kv_head_major ? it.kvh : row;
-                    if (gt >= 2) mbar_wait_call(k_empty + st, (use - 1) & 1, abort_flag, kp.status);
+                    if (gt >= 2 && !mbar_wait_call(k_empty + st, (use - 1) & 1, abort_flag, kp.status)) break;
+                    issued = j + 1;
                     TRACE(j, 7);
                     mbar_expect_tx(k_full + st, kTileBytes);
                     tma_load_3d(sK + st * kTileBytes, &map_k, k_full + st, 0, c1, c2);
                     if (kBoxes == 2) tma_load_3d(sK + st * kTileBytes + kHalfBytes, &map_k, k_full + st, 64, c1, c2);
-                    if (gt >= 2) mbar_wait_call(v_empty + st, (use - 1) & 1, abort_flag, kp.status);
+                    if (gt >= 2 && !mbar_wait_call(v_empty + st, (use - 1) & 1, abort_flag, kp.status)) break;
                     mbar_expect_tx(v_full + st, kTileBytes);
                     tma_load_3d(sV + st * kTileBytes, &map_v, v_full + st, 0, c1, c2);
                     if (kBoxes == 2) tma_load_3d(sV + st * kTileBytes + kHalfBytes, &map_v, v_full + st, 64, c1, c2);
                 }
             }
-            __syncwarp();
-            git += n_tiles;
-            ++qn;
+            issued = __shfl_sync(0xffffffffu, issued, 0);
+            git += issued;
+            qn += __shfl_sync(0xffffffffu, (int)q_free, 0);
+            if (issued < n_tiles) break;
         }
         if (lane == 0) {
             // end marker for the MMA issuer, in the slot and phase the next item would have used
@@ -1042,6 +1053,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         };
 
         int pn = 0;                                             // items read from the producer's slots
+        int n_met = 0;                                          // halves: items merged so far
         for (int k = 0; k < n_rounds; ++k) {
             const int item = item_of(k);
             if (item >= n_items) continue;
@@ -1050,7 +1062,8 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             bool listed = false;                                // the walk is a list of tiles, not a prefix
             bool halved = false;                                // the other warpgroup walks the other KV tiles of these rows
             {
-                mbar_wait(item_full + (pn & 1), (pn >> 1) & 1, abort_flag, kp.status);
+                const bool ok = mbar_wait(item_full + (pn & 1), (pn >> 1) & 1, abort_flag, kp.status);
+                if (!__all_sync(0xffffffffu, ok)) break;        // nothing is published any more
                 const volatile int *slot = item_pub + (pn & 1) * 16;
                 it.kvh = slot[0]; it.seg = slot[1]; it.kv_begin = slot[2]; it.n_a = slot[3]; it.t_b0 = slot[4];
                 it.a = slot[5]; it.b = slot[6];
@@ -1201,12 +1214,17 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             // weigh them by w0 and w1; otherwise w = 1 / l weighs the own accumulator.
             float w0 = 0.f, w1 = 0.f;
             if (kHalves && halved) {
-                float2 *xch = reinterpret_cast<float2 *>(sQ);   // sub-tile 0's Q buffer is not used
+                // (sub-tile 0's Q buffer is not used; two slots: a warp that is an item ahead finds the other one, and it
+                // gets no further before every warp has arrived there, behind its reads of this one)
+                float2 *xch = reinterpret_cast<float2 *>(sQ) + (n_met & 1) * 256;
                 const float m_mine = l_run == 0.f ? -INFINITY : m_run;
                 xch[t * 128 + r] = make_float2(m_mine, l_run);
                 tc_fence_before();
-                asm volatile("bar.sync 1, 256;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(halves_met);
+                mbar_wait(halves_met, n_met & 1, abort_flag, kp.status);
                 tc_fence_after();
+                ++n_met;
                 const float2 other = xch[(1 - t) * 128 + r];
                 m_run = fmaxf(m_mine, other.x);
                 const float ref = m_run == -INFINITY ? 0.f : m_run, f_mine = ex2(m_mine - ref), f_other = ex2(other.x - ref);
@@ -1235,12 +1253,15 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * inv);
                 }
             };
-            // this warp has read what it needs of O: one arrival per warp lets the accumulator be overwritten
+            // this warp has read what it needs of O: one arrival per warp lets the accumulator be overwritten (halves: of
+            // both, or, where the other warpgroup has no part in the item, its share too)
             auto release_o = [&]() {
                 tc_fence_before();
-                if (kHalves && halved) asm volatile("bar.sync 1, 256;" ::: "memory");
-                else __syncwarp();
-                if (lane == 0) mbar_arrive(o_free + t);
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(o_free + t);
+                    if (kHalves) mbar_arrive(o_free + (halved ? 1 - t : t));
+                }
             };
             // Full warps of rows leave through shared memory and TMA stores (a warp's 32 rows x 64 columns at a
             // time); a warp with rows beyond the segment writes its valid rows directly.
