@@ -1225,13 +1225,14 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 mbar_wait(halves_met, n_met & 1, abort_flag, kp.status);
                 tc_fence_after();
                 ++n_met;
-                const float2 other = xch[(1 - t) * 128 + r];
-                m_run = fmaxf(m_mine, other.x);
-                const float ref = m_run == -INFINITY ? 0.f : m_run, f_mine = ex2(m_mine - ref), f_other = ex2(other.x - ref);
-                l_run = l_run * f_mine + other.y * f_other;
+                // both warpgroups add in the same order: they hold the same row sum to the last bit
+                const float2 ml0 = xch[r], ml1 = xch[128 + r];
+                m_run = fmaxf(ml0.x, ml1.x);
+                const float ref = m_run == -INFINITY ? 0.f : m_run, f0 = ex2(ml0.x - ref), f1 = ex2(ml1.x - ref);
+                l_run = ml0.y * f0 + ml1.y * f1;
                 const float inv_l = l_run > 0.f ? 1.f / l_run : 0.f;
-                w0 = (t == 0 ? f_mine : f_other) * inv_l;
-                w1 = (t == 0 ? f_other : f_mine) * inv_l;
+                w0 = f0 * inv_l;
+                w1 = f1 * inv_l;
             }
             const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
             const int c_lo = kHalves && halved && kBoxes == 2 ? 2 * t : 0;                  // 32-column chunks of this thread
@@ -1366,9 +1367,9 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 }
                 if (kHalves && c_lo == c_hi) release_o();
             }
-            if (valid && lse_p) *lse_p = !(l_run > 0.f) ? -INFINITY
-                                         : kExact ? lse_exact(m_run, l_run)
-                                                  : (m_run + log2f(l_run)) * 0.6931471805599453f;
+            // (halves: sub-tile 1's warpgroup, which has a part in every item, writes it)
+            if (valid && lse_p && !(kHalves && halved && t == 0))
+                *lse_p = !(l_run > 0.f) ? -INFINITY : kExact ? lse_exact(m_run, l_run) : (m_run + log2f(l_run)) * 0.6931471805599453f;
             if (kExact && bad) {
                 if (lane == 0) tma_store_wait_read();           // the staging rows are free again: the routine's row of Q
                 __syncwarp();

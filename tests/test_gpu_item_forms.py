@@ -69,3 +69,23 @@ def test_walks_that_skip_tiles_and_walks_too_long_to_list(T):
     qp = np.concatenate([[0], rng.integers(0, T // 2, rows - 2), [T - 1]]).astype(np.int32)
     r = Runner(1, 2, 1, 128, "bf16", rows, T)
     check(r.sync(q, k, v, kv_pos=pos, q_pos=qp), reference(q, k, v, pos[None] <= qp[:, None]), "%d keys" % T)
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(16, 4, 128), (8, 8, 128), (16, 4, 64), (16, 4, 96)])
+def test_repeated_calls_agree_to_the_bit(hq, hkv, d):
+    """Calls whose items are shared by two warpgroups: every output has one writer."""
+    lens = [700, 500]
+    L, T = sum(lens), 400
+    cu = np.concatenate([[0], np.cumsum(lens)])
+    q, k, v = (dev(x, "bf16") for x in gen(24, lens, hq, hkv, d, "bf16"))
+    pos = torch.arange(0, L, 3, dtype=torch.int32, device="cuda")
+    r = Runner(2, hq, hkv, d, "bf16", L)
+    seen = None
+    for _ in range(20):
+        o, lse = [torch.full_like(q, float("nan")) for _ in range(3)], [torch.full((L, hq), float("nan"), device="cuda") for _ in range(3)]
+        fa().fedattn_local(r.ctx, r.shape, q, k, v, cu, o[0], lse[0])
+        fa().fedattn_sync(r.ctx, r.shape, q, None, k, v, None, L, False, o[1], lse[1])
+        fa().fedattn_sync_remote(r.ctx, r.shape, q, cu, k[:T], v[:T], pos, T, False, o[2], lse[2])
+        assert r.poll() == 0
+        seen = seen or (o, lse)
+        assert all(torch.equal(a, b) for a, b in zip(o + lse, seen[0] + seen[1]))
