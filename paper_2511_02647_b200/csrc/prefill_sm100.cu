@@ -1270,8 +1270,9 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             uint32_t bad = 0;                                   // exact instances: rows of the warp with a non-finite channel
             if (kExact) {
                 float probe = l_run * 0.f;                      // 0 unless something is Inf or NaN
+                // (halves: all columns, so that both warpgroups find the same rows)
 #pragma unroll 1
-                for (int c = c_lo; c < c_hi && 32 * c < d; ++c) {
+                for (int c = 0; c < 2 * kBoxes && 32 * c < d; ++c) {
                     uint32_t o[32];
                     load_o(c, o);
 #pragma unroll
@@ -1368,9 +1369,9 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 if (kHalves && c_lo == c_hi) release_o();
             }
             // (halves: sub-tile 1's warpgroup, which has a part in every item, writes it)
-            if (valid && lse_p && !(kHalves && halved && t == 0))
+            if (valid && lse_p && !(kHalves && halved && t == 0) && !((bad >> lane) & 1u))
                 *lse_p = !(l_run > 0.f) ? -INFINITY : kExact ? lse_exact(m_run, l_run) : (m_run + log2f(l_run)) * 0.6931471805599453f;
-            if (kExact && bad) {
+            if (kExact && bad && !(kHalves && halved && t == 0)) {      // (one warpgroup redoes them, neither stores them)
                 if (lane == 0) tma_store_wait_read();           // the staging rows are free again: the routine's row of Q
                 __syncwarp();
 #pragma unroll 1

@@ -7,7 +7,7 @@ import pytest
 import torch
 
 from helpers import LSE_TOL, TOL, Runner, check_close, dev, fa, host
-from test_gpu_head_dims import gen, owners, reference
+from test_gpu_head_dims import check as check_rows, gen, owners, reference
 
 pytestmark = pytest.mark.gpu
 
@@ -89,3 +89,25 @@ def test_repeated_calls_agree_to_the_bit(hq, hkv, d):
         assert r.poll() == 0
         seen = seen or (o, lse)
         assert all(torch.equal(a, b) for a, b in zip(o + lse, seen[0] + seen[1]))
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(16, 4, 96), (3, 3, 120), (16, 4, 64), (8, 8, 72)])
+def test_one_warpgroup_redoes_a_row(hq, hkv, d):
+    """Items shared by two warpgroups, each of which writes half of the columns: a value that is not finite in one
+    channel of an excluded row, below and above column 64, leaves every row that does not see it as it is."""
+    lens = [700, 500]
+    L, own = sum(lens), owners(lens)
+    q, k, v = gen(25, lens, hq, hkv, d, "bf16")
+    v[690, :, 3], v[1190, 0, d - 5] = np.inf, np.nan
+    visible = np.tri(L, dtype=bool) & (own[:, None] == own)
+    spoilt = visible[:, [690, 1190]].any(1)
+    r = Runner(2, hq, hkv, d, "bf16", L)
+    with np.errstate(invalid="ignore"):
+        want = reference(q, k, v, visible)
+    seen = None
+    for _ in range(10):
+        o, lse = r.local(q, k, v, lens)
+        check_rows((o[~spoilt], lse[~spoilt]), (want[0][~spoilt], want[1][~spoilt]), "bf16", "excluded")
+        assert np.abs(lse - want[1]).max() <= 1e-5 and not np.isfinite(o[690:700, :, 3]).any() and not np.isfinite(o[1190:, 0, d - 5]).any()
+        seen = seen or (o, lse)
+        assert np.array_equal(o, seen[0], equal_nan=True) and np.array_equal(lse, seen[1])
