@@ -104,6 +104,7 @@ attn_tiled_kernel(const __grid_constant__ GenericParams p, const __grid_constant
     constexpr int kM = L::kM, kThreads = L::kThreads, kKeys = L::kKeys;
     constexpr int kJ = kKeyWarps > 1 ? 1 : 4;                                // keys of a tile per thread
     constexpr int kC = kDP / 16;                                             // output columns per thread: 4 tk + 64 cc + 0..3
+    // Keys, rows and positions are ints up to 2^31 - 1: no sum below passes the last key.
     extern __shared__ __align__(16) uint8_t smem[];
     float *sQ = reinterpret_cast<float *>(smem), *sP = reinterpret_cast<float *>(smem + L::kOffP);
     T *sKV = reinterpret_cast<T *>(smem + L::kOffKv);                        // [stage][K, V]
@@ -150,14 +151,14 @@ attn_tiled_kernel(const __grid_constant__ GenericParams p, const __grid_constant
     constexpr int kVec = 16 / (int)sizeof(T), kRowVecs = kDP / kVec, kStep = kThreads / kRowVecs;
     const int ld_r = tid / kRowVecs, ld_c = (tid % kRowVecs) * kVec;
     auto load_tile = [&](T *dst, const T *src, int t) {
-        const int k0 = kv_lo + t * kKeys + ld_r;
+        const int left = kv_hi - kv_lo - t * kKeys - ld_r;                   // this thread's rows: ld_r + kStep i, while below `left`
         if (ld_c < d) {                                                      // head_dim is a multiple of 8
-            const T *from = src + (int64_t)k0 * p.kv_tok_stride + ld_c;
+            const T *from = src + ((int64_t)kv_lo + (int64_t)t * kKeys + ld_r) * p.kv_tok_stride + ld_c;
             uint32_t to = (uint32_t)__cvta_generic_to_shared(dst + ld_r * L::kKvPitch + ld_c);
             const int64_t step = (int64_t)kStep * p.kv_tok_stride;
 #pragma unroll 4
             for (int i = 0; i < kKeys / kStep; ++i, from += step, to += kStep * L::kKvPitch * (int)sizeof(T)) {
-                const bool ok = k0 + i * kStep < kv_hi;                      // rows past the end read as zero
+                const bool ok = i * kStep < left;                            // rows past the end read as zero
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(ok ? from : src), "r"(ok ? 16 : 0) : "memory");
             }
         }
@@ -165,7 +166,7 @@ attn_tiled_kernel(const __grid_constant__ GenericParams p, const __grid_constant
     };
     // the first K and V tile are on their way while Q and the rows' bounds are set up (a walk that turns out shorter
     // does not use them)
-    const int n_kt_most = kv_hi > kv_lo ? (kv_hi - kv_lo + kKeys - 1) / kKeys : 0;
+    const int n_kt_most = kv_hi > kv_lo ? (kv_hi - kv_lo - 1) / kKeys + 1 : 0;
     constexpr int kKvElts = L::kKvBytes / (int)sizeof(T);
     const int stages = plan.stages;
 #pragma unroll 1
@@ -212,8 +213,8 @@ attn_tiled_kernel(const __grid_constant__ GenericParams p, const __grid_constant
                 int last = -1;
 #pragma unroll
                 for (int i = 0; i < 1024 / kThreads; ++i) {
-                    const int key = base + i * kThreads + tid;
-                    if (key < kv_hi) {
+                    if (i * kThreads + tid < kv_hi - base) {
+                        const int key = base + i * kThreads + tid;
                         const int pos = __ldg(kvp + key);
                         if (pos <= lo_max || (two_sided && pos >= hi)) last = key;
                     }
@@ -229,7 +230,7 @@ attn_tiled_kernel(const __grid_constant__ GenericParams p, const __grid_constant
         }
     }
 
-    const int n_kt = kv_hi > kv_lo ? (kv_hi - kv_lo + kKeys - 1) / kKeys : 0;
+    const int n_kt = kv_hi > kv_lo ? (kv_hi - kv_lo - 1) / kKeys + 1 : 0;
     float m[kR], l[kR];
     uint64_t acc[kR / 2][kC];                                                // rows (2 i, 2 i + 1)
 #pragma unroll
@@ -251,14 +252,14 @@ attn_tiled_kernel(const __grid_constant__ GenericParams p, const __grid_constant
     auto load_pos = [&](int t) {
 #pragma unroll
         for (int j = 0; j < kJ; ++j) {
-            const int key = kv_lo + t * kKeys + key_l + 16 * j;
-            pos[j] = kvp && by_pos ? __ldg(kvp + min(key, kv_hi - 1)) : key;
+            const int key = min(key_l + 16 * j, kv_hi - 1 - kv_lo - t * kKeys) + kv_lo + t * kKeys;     // (past the end: the last one)
+            pos[j] = kvp && by_pos ? __ldg(kvp + key) : key;
         }
     };
     if (rank < n_kt) load_pos(rank);
 #pragma unroll 1
     for (int t = rank; t < n_kt; t += plan.splits) {
-        const int k0 = kv_lo + t * kKeys;
+        const int k0 = kv_lo + t * kKeys, left = kv_hi - k0;                 // keys from the tile's first to the last
         const int next = t + stages * plan.splits;                           // the tile that takes this one's place
         T *sK = sKV + 2 * slot * kKvElts, *sV = sK + kKvElts;
         slot = slot + 1 == stages ? 0 : slot + 1;
@@ -291,7 +292,7 @@ attn_tiled_kernel(const __grid_constant__ GenericParams p, const __grid_constant
         if (next < n_kt) load_tile(sK, K, next);
         else asm volatile("cp.async.commit_group;" ::: "memory");
         // ---- mask, online softmax (16 lanes share a row), P transposed to shared memory ----
-        const bool all_seen = !(kvp && by_pos) && !two_sided && k0 + kKeys <= kv_hi && k0 + kKeys - 1 <= lo_min;
+        const bool all_seen = !(kvp && by_pos) && !two_sided && kKeys <= left && k0 + kKeys - 1 <= lo_min;
         float al[kR];
 #pragma unroll
         for (int i = 0; i < kR; ++i) {
@@ -300,7 +301,7 @@ attn_tiled_kernel(const __grid_constant__ GenericParams p, const __grid_constant
             for (int j = 0; j < kJ; ++j) {
                 const float2 v = unpack2(s2[i][j]);
                 s[j] = (v.x + v.y) * p.scale;
-                if (!all_seen && !(k0 + key_l + 16 * j < kv_hi && (pos[j] <= lo[i] || (two_sided && pos[j] >= hi && my_row0 + i < n_rows))))
+                if (!all_seen && !(key_l + 16 * j < left && (pos[j] <= lo[i] || (two_sided && pos[j] >= hi && my_row0 + i < n_rows))))
                     s[j] = -INFINITY;
                 mx = fmaxf(mx, s[j]);
             }

@@ -175,3 +175,33 @@ def test_excluded_rows_may_hold_anything(dtype, hq, hkv, d):
             wo, wl = reference(q, k, v, vis)
         check((o[~spoilt], lse[~spoilt]), (wo[~spoilt], wl[~spoilt]), dtype, "excluded Inf and NaN")
         assert not np.isfinite(o[spoilt][:, 0]).all(1).any()
+
+
+@pytest.mark.parametrize("positions", [False, True])
+def test_as_many_keys_as_an_int_counts(positions):
+    """2^31 - 1 keys of one head of 8 channels (34 GB, K and V in one buffer): the last tile ends where 32-bit sums would
+    wrap.  All keys are zero but the last 1000, whose logits are large enough to decide the output."""
+    T, d, tail = 2 ** 31 - 1, 8, 1000
+    if torch.cuda.mem_get_info()[0] < 60 << 30:
+        pytest.skip("needs 60 GB of free device memory")
+    rng = np.random.default_rng(13)
+    last = torch.from_numpy(rng.standard_normal((tail, d))).to(torch.bfloat16)
+    q = torch.from_numpy(16.0 + rng.standard_normal((2, 1, d))).to(torch.bfloat16)
+    kv = torch.zeros((T, 1, d), dtype=torch.bfloat16, device="cuda")
+    kv[T - tail:, 0] = last.cuda()
+    seen = np.ones((2, tail), bool)
+    pos = None
+    if positions:
+        pos = torch.zeros(T, dtype=torch.int32, device="cuda")
+        pos[T - tail:] = torch.arange(tail, dtype=torch.int32, device="cuda")
+        seen = np.arange(tail)[None] <= np.array([500, tail])[:, None]
+    m = fa()
+    r = Runner(1, 1, 1, d, "bf16", 2, 1)
+    qp = torch.tensor([500, tail] if positions else [T, T], dtype=torch.int32, device="cuda")
+    o, lse = torch.full((2, 1, d), float("nan"), dtype=torch.bfloat16, device="cuda"), torch.full((2, 1), float("nan"), device="cuda")
+    m.fedattn_sync(r.ctx, r.shape, q.cuda(), qp, kv, kv, pos, T, False, o, lse)
+    assert r.poll() == 0
+    s = np.where(seen, host(q)[:, 0] @ host(last).T / np.sqrt(d), -np.inf)
+    z = np.exp(s).sum(1) + (T - tail)
+    wo = (np.exp(s) @ host(last) / z[:, None])[:, None]
+    check((host(o), host(lse)), (wo, np.log(z)[:, None]), "bf16", "2^31 - 1 keys")
