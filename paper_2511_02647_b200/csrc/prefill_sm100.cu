@@ -47,9 +47,8 @@ constexpr int kTileN = 128;          // keys per KV tile
 constexpr int kBoxCols = 64;          // head-dim columns of one TMA box (128-byte swizzle); a tile is 1 or 2 boxes
 // two softmax warpgroups, one per sub-tile.  (Both on the same S tile, split by columns with the row
 // maxima exchanged through shared memory, was 2-4 % slower on dense sync; four warpgroups of 32 columns
-// 20 %.)  P is handed to the MMA warp in kSplit halves of kCols keys, so that PV starts on the first.
+// 20 %.)  P is handed to the MMA warp in kSplit halves, so that PV starts on the first.
 constexpr int kSplit = 2;
-constexpr int kCols = kTileN / kSplit;
 constexpr int kSoftmaxThreads = 128 * kSplit;
 constexpr int kThreads = kSoftmaxThreads + 128;  // then a warpgroup holding the TMA producer warp and the MMA issuer warp
 // Registers move from that warpgroup to the softmax warpgroups once the roles split (setmaxnreg):
@@ -67,9 +66,12 @@ constexpr uint32_t smem_bytes(int boxes)
 {
     return 6 * boxes * kHalfBytes + 1024 /*alignment slack*/ + 1024 /*barriers, published items*/ + 2 * kSplit * 2 * kStageBytes;
 }
+// Keys per KV tile of an instance: weights in three bf16 parts take 3 x 16 columns of TMEM per 32 keys where S had 32; one
+// box (head_dim <= 64) has the third part beside O, whose upper 64 columns are free, two boxes have room for 64 keys only.
+__host__ __device__ constexpr int tile_keys(bool exact, int boxes) { return exact && boxes == 2 ? 64 : kTileN; }
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kColS = 0, kColO = 256;   // S (and P, aliased) of sub-tile t at kColS + 128 t; O at kColO + 128 t
-// P (bf16 pairs) of keys kCols q .. kCols q + kCols - 1 sits at S column kCols q: every 32-key chunk of P
+// P (bf16 pairs) of keys 64 q .. 64 q + 63 sits at S column 64 q: every 32-key chunk of P
 // lands in S columns that its thread has already read
 constexpr uint32_t kWaitLimit = 1u << 20;
 constexpr float kRescaleThreshold = 8.0f;
@@ -88,6 +90,7 @@ struct KernelParams {
     int32_t *status;
     int32_t o_tma;                   // the output may leave through TMA stores (tensor map encoded)
     int32_t pairs;                   // exact instances: visibility is tested on explicit positions, in any order
+    float sl2;                       // exact instances: logits to base 2 per unit of S
     GenericParams row;               // exact instances: the same call for the row routine that repairs non-finite rows
 };
 
@@ -373,7 +376,6 @@ __device__ __host__ constexpr uint32_t make_idesc(uint32_t n)
 {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((128u >> 4) << 24);
 }
-constexpr uint32_t kIdescQK = make_idesc(128);                 // A, B K-major
 constexpr uint32_t kIdescPV = make_idesc(128) | (1u << 16);    // B (V) MN-major
 
 // n / d for 0 <= n < 2^28 and 1 <= d <= 4096, with magic = ceil(2^40 / d)
@@ -479,6 +481,7 @@ __device__ __forceinline__ PairRule pair_rule(const PrefillParams &p, const Item
 }
 // Number of KV tiles up to the last one with a key visible to some row of the sub-tile.  Walks the key
 // positions backwards, 512 at a time (sixteen coalesced loads in flight per lane); called by a converged warp.
+template <int kKeys>
 __device__ __forceinline__ int last_visible_tile(const KernelParams &kp, const Item &it, const Sub &sub, int lane)
 {
     const PrefillParams &p = kp.p;
@@ -494,7 +497,7 @@ __device__ __forceinline__ int last_visible_tile(const KernelParams &kp, const I
             if (key < T && any.sees(it.kvp ? __ldg(it.kvp + key) : key)) last = key;
         }
         last = __reduce_max_sync(0xffffffffu, last);
-        if (last >= 0) return last / kTileN + 1;
+        if (last >= 0) return last / kKeys + 1;
     }
     return 0;
 }
@@ -502,7 +505,7 @@ __device__ __forceinline__ int last_visible_tile(const KernelParams &kp, const I
 // Called by a converged warp (all lanes get the same item).  kSpecial: the kernel instance that also
 // serves explicit positions and bidirectional remote-only attention (two key ranges); the plain instance
 // carries none of their state.  Causal remote-only attention is one more prefix mask: plain instance.
-template <bool kSpecial, bool kExact, bool kHalves>
+template <bool kSpecial, bool kExact, bool kHalves, int kKeys>
 __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, int lane, Sub (&sub)[2], uint16_t *walk)
 {
     const PrefillParams &p = kp.p;
@@ -589,14 +592,14 @@ __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, in
     } else if (p.sync && p.remote_only && !(kExact && kp.pairs)) {
         // keys [0, a) lie before the rows' segment; when bidirectional (special instance only), keys [b, T)
         // after it count too
-        const int T = (int)p.total_kv, n_t = (T + kTileN - 1) / kTileN;
+        const int T = (int)p.total_kv, n_t = (T + kKeys - 1) / kKeys;
         it.a = prefix_len<kSpecial>(p, it, sub[1], 0, lane);
-        it.n_a = (it.a + kTileN - 1) / kTileN;
+        it.n_a = (it.a + kKeys - 1) / kKeys;
         sub[1].n_tiles = it.n_a;
         it.b = T;
         if (kSpecial && !p.causal) {
             it.b = it.kvp ? count_le_warp(it.kvp, T, end - 1, lane) : min(end, T);
-            it.t_b0 = it.b >= T ? n_t : max(it.b / kTileN, it.n_a);
+            it.t_b0 = it.b >= T ? n_t : max(it.b / kKeys, it.n_a);
             sub[1].n_tiles = it.n_a + (n_t - it.t_b0);
         }
         sub[0].n_tiles = sub[0].n_valid > 0 ? sub[1].n_tiles : 0;
@@ -606,8 +609,8 @@ __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, in
         for (int again = two_rows && sub[0].n_valid > 0 ? 1 : 0;; again = 0) {
             const Sub x = again ? sub[0] : sub[1];
             int n;
-            if (kExact && kp.pairs) n = last_visible_tile(kp, it, x, lane);
-            else n = (prefix_len<kSpecial>(p, it, x, x.n_valid - 1, lane) + kTileN - 1) / kTileN;
+            if (kExact && kp.pairs) n = last_visible_tile<kKeys>(kp, it, x, lane);
+            else n = (prefix_len<kSpecial>(p, it, x, x.n_valid - 1, lane) + kKeys - 1) / kKeys;
             if (again) { sub[0].n_tiles = n; continue; }
             sub[1].n_tiles = n;
             break;
@@ -629,14 +632,13 @@ __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, in
 // and parities, so the producer prefetches the next item's K/V and Q while the current item's last
 // tiles and its epilogue are still in flight.
 //
-// kBoxes: 64-column boxes per tile (head_dim <= 64: one; <= 128: two).  kExact: the weights P keep 16 bits of
-// mantissa instead of 8 (two bf16 parts, two PV products), every exponential is ex2, and rows that come out
-// non-finite are redone by the row routine.  It serves the head dims below 128, whose users had fp32 weights
-// from the SIMT kernel; P's two parts take exactly the S columns that the chunk's thread has already read.
-// Its extra product makes PV as long as S again (d = 64: 4 + 2 x 8 MMAs of half width per tile); a chunk costs
-// 6 more instructions per pair of keys.  Six ragged segments of 2160 tokens in all, 16 / 4 heads of 64 channels: local
-// 2436 us (one warp per row, fp32 FMA) -> 20 us, sync 10994 -> 45 us; the error of o against fp64 is the same to
-// three digits (the rounding of the bf16 output, 1.6e-3), lse 3.5e-8 -> 5e-8 relative (half a unit of fp32).
+// kBoxes: 64-column boxes per tile (head_dim <= 64: one; <= 128: two).  kExact: the weights P keep their 24 bits (three
+// bf16 parts, three PV products), every exponential is ex2, and rows that come out non-finite are redone by the row
+// routine.  It serves the head dims below 128, whose users had fp32 weights from the SIMT kernel.  Bound by the PV
+// products (d = 64: 4 + 3 x 8 MMAs per tile, the latter of N = 64 and no faster than of N = 128): two parts, 16 bits, take
+// 20.7 and 47.1 us, three 24.7 and 55.9 for the local and the sync call of six ragged segments of 2160 tokens, 16 / 4 heads of 64
+// channels (2436 and 10994 us with one warp per row, fp32 FMA).  The error of o against fp64 is that of fp32 weights (the
+// rounding of the bf16 output, 1.587459e-3 there; 1.587460e-3 with two parts), lse 3.2e-8 -> 2.9e-8 relative.
 //
 // kHalves: both sub-tiles are the SAME query tile of one head; sub-tile 1 walks the even KV tiles and sub-tile 0 the odd
 // ones, and the epilogue merges the two partial rows (O_0 and O_1 have the same TMEM lanes, so every thread reads both;
@@ -650,14 +652,18 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                      const __grid_constant__ KernelParams kp)
 {
     extern __shared__ uint8_t smem_raw[];
-    constexpr uint32_t kTileBytes = kBoxes * kHalfBytes;
+    constexpr uint32_t kTileBytes = kBoxes * kHalfBytes;                            // a Q tile
+    constexpr int kKeys = tile_keys(kExact, kBoxes), kChunks = kKeys / 32;         // keys of a KV tile, in chunks of 32
+    constexpr int kPartKeys = kKeys / kSplit;                                      // keys of a half of P
+    constexpr uint32_t kColP3 = (kBoxes == 1 ? kColO : kColS) + 64;                // exact instances: third parts of sub-tile 0's P
+    constexpr uint32_t kKvBox = kKeys * kBoxCols * 2, kKvBytes = kBoxes * kKvBox;  // a K or V tile
     const PrefillParams &p = kp.p;
     const int d = kExact ? p.d : kBoxes * kBoxCols;
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t *sQ = smem;                                  // [2 sub-tiles][tile]
     uint8_t *sK = smem + 2 * kTileBytes;                 // [2 stages][tile]
-    uint8_t *sV = smem + 4 * kTileBytes;                 // [2 stages][tile]
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + 6 * kTileBytes);
+    uint8_t *sV = sK + 2 * kKvBytes;                     // [2 stages][tile]
+    uint64_t *bars = reinterpret_cast<uint64_t *>(sV + 2 * kKvBytes);
     uint64_t *q_full = bars + 0, *q_empty = bars + 1;
     uint64_t *k_full = bars + 2, *k_empty = bars + 4, *v_full = bars + 6, *v_empty = bars + 8;
     uint64_t *s_full = bars + 10, *o_done = bars + 12, *o_free = bars + 14;
@@ -673,7 +679,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     uint64_t *halves_met = bars + 28;                    // halves: both warpgroups have left their partials' (m, l)
     volatile int *item_pub = reinterpret_cast<volatile int *>(bars + 32);
     uint16_t *walks = reinterpret_cast<uint16_t *>(bars + 48);      // general: [slot][kWalkMost]
-    uint8_t *stage = smem + 6 * kTileBytes + 1024;       // [softmax warp][32 rows][128 B], 128-byte swizzle
+    uint8_t *stage = sV + 2 * kKvBytes + 1024;           // [softmax warp][32 rows][128 B], 128-byte swizzle
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int n_items = kp.n_items;
@@ -738,7 +744,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             const bool general = kSpecial && !kExact && p.general;
             if (general && !slot_free()) break;                 // the walk goes into the slot while decoding
             uint16_t *walk = walks + (pn & 1) * kWalkMost;
-            const Item it = decode_item<kSpecial, kExact, kHalves>(kp, item, lane, sub, walk);
+            const Item it = decode_item<kSpecial, kExact, kHalves, kKeys>(kp, item, lane, sub, walk);
             __syncwarp();
             const int n_tiles = sub[1].n_tiles + (kHalves ? sub[0].n_tiles : 0);
             if (!general && !slot_free()) break;
@@ -780,18 +786,18 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     const int gt = git + j, st = gt & 1, use = gt >> 1;
                     int tile = kSpecial ? tile_of(it, j) : j;
                     if (listed) tile = walk[j] & 0x7fff;
-                    const int row = it.kv_begin + tile * kTileN;
+                    const int row = it.kv_begin + tile * kKeys;
                     const int c1 = p.kv_head_major ? row : it.kvh, c2 = p.kv_head_major ? it.kvh : row;
                     if (gt >= 2 && !mbar_wait_call(k_empty + st, (use - 1) & 1, abort_flag, kp.status)) break;
                     issued = j + 1;
                     TRACE(j, 7);
-                    mbar_expect_tx(k_full + st, kTileBytes);
-                    tma_load_3d(sK + st * kTileBytes, &map_k, k_full + st, 0, c1, c2);
-                    if (kBoxes == 2) tma_load_3d(sK + st * kTileBytes + kHalfBytes, &map_k, k_full + st, 64, c1, c2);
+                    mbar_expect_tx(k_full + st, kKvBytes);
+                    tma_load_3d(sK + st * kKvBytes, &map_k, k_full + st, 0, c1, c2);
+                    if (kBoxes == 2) tma_load_3d(sK + st * kKvBytes + kKvBox, &map_k, k_full + st, 64, c1, c2);
                     if (gt >= 2 && !mbar_wait_call(v_empty + st, (use - 1) & 1, abort_flag, kp.status)) break;
-                    mbar_expect_tx(v_full + st, kTileBytes);
-                    tma_load_3d(sV + st * kTileBytes, &map_v, v_full + st, 0, c1, c2);
-                    if (kBoxes == 2) tma_load_3d(sV + st * kTileBytes + kHalfBytes, &map_v, v_full + st, 64, c1, c2);
+                    mbar_expect_tx(v_full + st, kKvBytes);
+                    tma_load_3d(sV + st * kKvBytes, &map_v, v_full + st, 0, c1, c2);
+                    if (kBoxes == 2) tma_load_3d(sV + st * kKvBytes + kKvBox, &map_v, v_full + st, 64, c1, c2);
                 }
             }
             issued = __shfl_sync(0xffffffffu, issued, 0);
@@ -825,15 +831,15 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         const bool leader = elect_one();
         const uint32_t idesc_pv = make_idesc((uint32_t)(d + 15) & ~15u) | (1u << 16);     // exact instances: N = head_dim
         const uint32_t aQ = smem_u32(sQ), aK = smem_u32(sK), aV = smem_u32(sV);
-        const uint64_t dQ = make_desc(aQ, 16, 1024), dK = make_desc(aK, 16, 1024), dV = make_desc(aV, kHalfBytes, 1024);
+        const uint64_t dQ = make_desc(aQ, 16, 1024), dK = make_desc(aK, 16, 1024), dV = make_desc(aV, kKvBox, 1024);
         auto issue_s = [&](int t, int st) {
             if (leader) {
 #pragma unroll
                 for (int ks = 0; ks < kBoxes * kBoxCols / 16; ++ks) {
-                    const uint32_t off = ((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4;       // descriptor units
+                    const uint32_t off_q = ((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4, off_k = ((ks >> 2) * kKvBox + (ks & 3) * 32) >> 4;
                     if (!kExact || 16 * ks < d)                  // columns beyond head_dim are zero in both tiles
-                    umma_ss(tmem_base + kColS + t * 128, dQ + (uint64_t)((kHalves ? 1 : t) * (kTileBytes >> 4) + off),
-                            dK + (uint64_t)(st * (kTileBytes >> 4) + off), kIdescQK, ks > 0);
+                    umma_ss(tmem_base + kColS + t * 128, dQ + (uint64_t)((kHalves ? 1 : t) * (kTileBytes >> 4) + off_q),
+                            dK + (uint64_t)(st * (kKvBytes >> 4) + off_k), make_idesc(kKeys), ks > 0);
                 }
             }
         };
@@ -879,15 +885,17 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                         tc_fence_after();
                         if (leader) {
 #pragma unroll
-                            for (int kk = 0; kk < kCols / 16; ++kk) {
-                                const int ks = q * (kCols / 16) + kk;
-                                const uint64_t desc = dV + (uint64_t)(st * (kTileBytes >> 4) + ks * (2048 >> 4));
-                                if (kExact) {                    // chunk of 32 keys: 16 columns of high parts, 16 of low parts
+                            for (int kk = 0; kk < kPartKeys / 16; ++kk) {
+                                const int ks = q * (kPartKeys / 16) + kk;
+                                const uint64_t desc = dV + (uint64_t)(st * (kKvBytes >> 4) + ks * (2048 >> 4));
+                                if (kExact) {                    // chunk of 32 keys: 16 columns each of the first, second, third parts
                                     const uint32_t a = tmem_base + kColS + t * 128 + 32 * (ks >> 1) + 8 * (ks & 1);
+                                    const uint32_t a3 = tmem_base + kColP3 + t * 128 + 16 * (ks >> 1) + 8 * (ks & 1);
                                     umma_ts(tmem_base + kColO + t * 128, a, desc, idesc_pv, (j > 0 || ks > 0));
                                     umma_ts(tmem_base + kColO + t * 128, a + 16, desc, idesc_pv, 1);
+                                    umma_ts(tmem_base + kColO + t * 128, a3, desc, idesc_pv, 1);
                                 } else {
-                                    umma_ts(tmem_base + kColO + t * 128, tmem_base + kColS + t * 128 + q * kCols + kk * 8, desc,
+                                    umma_ts(tmem_base + kColO + t * 128, tmem_base + kColS + t * 128 + q * kPartKeys + kk * 8, desc,
                                             kIdescPV, (j > 0 || ks > 0));
                                 }
                             }
@@ -940,7 +948,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t tS = tmem_base + lane_base + kColS + t * 128;   // fp32 S; bf16 P of keys 64q.. at column 64q
         const uint32_t tO = tmem_base + lane_base + kColO + t * 128;
-        const float sl2 = p.scale * 1.4426950408889634f;
+        const float sl2 = kExact ? kp.sl2 : p.scale * 1.4426950408889634f;
         const uint64_t sl2_2 = pack_f32x2(sl2, sl2);
         int gsub = 0;                                           // KV tiles this sub-tile has been through
         auto below32 = [](int n) -> uint32_t { return n <= 0 ? 0u : (n >= 32 ? 0xffffffffu : (1u << n) - 1u); };
@@ -964,10 +972,12 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             FEDATTN_TMEM_LD32(tS, s0);
             FEDATTN_TMEM_LD32(tS + 32, s1);
             tmem_wait_ld();
-            FEDATTN_TMEM_LD32(tS + 64, s2);
-            FEDATTN_TMEM_LD32(tS + 96, s3);
+            if (kChunks == 4) {
+                FEDATTN_TMEM_LD32(tS + 64, s2);
+                FEDATTN_TMEM_LD32(tS + 96, s3);
+            }
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
+            for (int c = 0; c < kChunks; ++c) {
                 uint32_t *cur = c == 0 ? s0 : (c == 1 ? s1 : (c == 2 ? s2 : s3));
                 if (c == 2) tmem_wait_ld();
                 if (kPartial) {
@@ -1012,9 +1022,23 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             const uint64_t negm2 = pack_f32x2(-m_ref, -m_ref);
             uint64_t sum2[4] = {0, 0, 0, 0};
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
+            for (int c = 0; c < kChunks; ++c) {
                 uint32_t *cur = c == 0 ? s0 : (c == 1 ? s1 : (c == 2 ? s2 : s3));
-                uint32_t pk[16], pl[16];
+                uint32_t pk[16];
+                // Exact instances: the leading 8 bits of the values in cur as bf16 pairs; what is left stays in cur.  Three
+                // times that is a weight's 24 bits.
+                auto take_part = [&](bool last) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        pk[i] = __byte_perm(cur[2 * i], cur[2 * i + 1], 0x7632);
+                        if (last) continue;
+                        const uint64_t top = pack_f32x2(__uint_as_float(cur[2 * i] & 0xffff0000u), __uint_as_float(cur[2 * i + 1] & 0xffff0000u));
+                        float r0, r1;
+                        unpack_f32x2(fma_f32x2(top, pack_f32x2(-1.f, -1.f), pack_f32x2(__uint_as_float(cur[2 * i]), __uint_as_float(cur[2 * i + 1]))), r0, r1);
+                        cur[2 * i] = __float_as_uint(r0);
+                        cur[2 * i + 1] = __float_as_uint(r1);
+                    }
+                };
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
                     const uint64_t x2 = fma_f32x2(pack_f32x2(__uint_as_float(cur[2 * i]), __uint_as_float(cur[2 * i + 1])), sl2_2, negm2);
@@ -1027,23 +1051,26 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                         p0 = ex2(x0); p1 = ex2(x1);
                     }
                     sum2[i & 3] = add_f32x2(sum2[i & 3], pack_f32x2(p0, p1));
-                    pk[i] = pack_bf16(p0, p1);
-                    if (kExact)                                 // what the rounding left over, as a second bf16
-                        pl[i] = pack_bf16(p0 - __uint_as_float(pk[i] << 16), p1 - __uint_as_float(pk[i] & 0xffff0000u));
+                    if (kExact) { cur[2 * i] = __float_as_uint(p0); cur[2 * i + 1] = __float_as_uint(p1); }
+                    else pk[i] = pack_bf16(p0, p1);
                 }
                 // keys 32 c .. 32 c + 31 as bf16 pairs: columns 64 (c / 2) + 16 (c % 2) .., all inside S columns
                 // that this thread has already read
                 if (kExact) {
+                    take_part(false);
                     FEDATTN_TMEM_ST16(tS + 32 * c, pk);
-                    FEDATTN_TMEM_ST16(tS + 32 * c + 16, pl);
+                    take_part(false);
+                    FEDATTN_TMEM_ST16(tS + 32 * c + 16, pk);
+                    take_part(true);
+                    FEDATTN_TMEM_ST16(tmem_base + lane_base + kColP3 + t * 128 + 16 * c, pk);
                 } else {
                     FEDATTN_TMEM_ST16(tS + 64 * (c >> 1) + 16 * (c & 1), pk);
                 }
-                if (c & 1) {                                    // a 64-key half of P is complete: PV may start on it
+                if ((32 * c + 32) % kPartKeys == 0) {           // a half of P is complete: PV may start on it
                     tmem_wait_st();
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(p_full + kSplit * t + (c >> 1));      // one arrival per warp
+                    if (lane == 0) mbar_arrive(p_full + kSplit * t + 32 * c / kPartKeys);       // one arrival per warp
                 }
             }
             float r0, r1;
@@ -1098,8 +1125,8 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             auto load_pos = [&](int j) {
                 const int T = (int)p.total_kv;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const int key = j * kTileN + 32 * c + lane;
+                for (int c = 0; c < kChunks; ++c) {
+                    const int key = j * kKeys + 32 * c + lane;
                     kpos[c] = it.kvp ? __ldg(it.kvp + min(key, T - 1)) : key;
                 }
             };
@@ -1133,7 +1160,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 }
                 // prefix lengths do not decrease with the row, so KV tiles below the prefix of the warp's first
                 // row are unmasked for the whole warp (the choice of code path only has to be warp-uniform)
-                n_full = __shfl_sync(0xffffffffu, c_row, 0) / kTileN;
+                n_full = __shfl_sync(0xffffffffu, c_row, 0) / kKeys;
             }
             const int T = (int)p.total_kv;
             float m_run = 0.f, l_run = 0.f;
@@ -1148,15 +1175,15 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 bool full;
                 uint32_t vm[4] = {0, 0, 0, 0};
                 if (pairs) {
-                    // column 32 c + i of the tile is key j * 128 + 32 c + i, whose position lane i holds
-                    const int k0 = tile * kTileN;
+                    // column 32 c + i of the tile is its key 32 c + i, whose position lane i holds
+                    const int k0 = tile * kKeys;
                     bool see_all = true;
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) see_all = see_all && k0 + 32 * c + lane < T && all.sees(kpos[c]);
+                    for (int c = 0; c < kChunks; ++c) see_all = see_all && k0 + 32 * c + lane < T && all.sees(kpos[c]);
                     full = __all_sync(0xffffffffu, see_all);
                     if (!full) {
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
+                        for (int c = 0; c < kChunks; ++c) {
                             uint32_t m = 0;
 #pragma unroll 4
                             for (int i = 0; i < 32; ++i)
@@ -1166,11 +1193,11 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     }
                     if (j + 1 < n_tiles) load_pos(tile + (kHalves ? 2 : 1));        // lands during this tile's visit
                 } else if (two_range) {                         // keys [0, a) and [b, T)
-                    const int k0 = tile_of(it, tile) * kTileN;  // first key of the tile
-                    full = k0 + kTileN <= it.a || (k0 >= it.b && k0 + kTileN <= T);
+                    const int k0 = tile_of(it, tile) * kKeys;   // first key of the tile
+                    full = k0 + kKeys <= it.a || (k0 >= it.b && k0 + kKeys <= T);
                     if (!full) {
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
+                        for (int c = 0; c < kChunks; ++c) {
                             const int cb = k0 + 32 * c;
                             vm[c] = below32(it.a - cb) | (below32(T - cb) & ~below32(it.b - cb));
                         }
@@ -1181,8 +1208,8 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                         // column i of chunk c is key cb + i: visible iff it exists and its position is not above
                         // the row's.  The address is the same in every lane: broadcast loads.
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            const int cb = tile * kTileN + 32 * c;
+                        for (int c = 0; c < kChunks; ++c) {
+                            const int cb = tile * kKeys + 32 * c;
                             uint32_t m = 0;
 #pragma unroll 4
                             for (int i = 0; i < 32; ++i) {
@@ -1194,7 +1221,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                         }
                     } else if (!full) {
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) vm[c] = below32(c_row - tile * kTileN - 32 * c);
+                        for (int c = 0; c < kChunks; ++c) vm[c] = below32(c_row - tile * kKeys - 32 * c);
                     }
                 }
                 if (full) visit(std::false_type{}, j, gt, vm, m_run, l_run);
@@ -1610,6 +1637,13 @@ cudaError_t launch_prefill_sm100(Context *ctx, const PrefillParams &p, cudaStrea
         // positions in any order, as the row routine takes them, and no tables: those calls keep off the scratch
         kp.pairs = p.sync && (p.kv_pos || p.q_pos) && (p.causal || p.remote_only);
         kp.row = generic_params(p);
+        // The tensor core cuts off what a sum has below its last place, after each step of 16 channels: a logit comes out
+        // smaller by kCutOff of itself for the last step and proportionally less for the ones before.  (lse of N(0, 1)
+        // inputs, error against fp64, mean and rms in 1e-7: head_dim 64 -1.0 and 1.9 without the factor, -0.3 and 1.6
+        // with it; 96: -1.5 and 2.3, -0.5 and 1.8; 120: -1.8 and 2.5, 0.3 and 1.6; fp32 FMA chains: rms 1.8.)
+        constexpr double kCutOff = 3e-8;
+        const int steps = (p.d + 15) / 16;
+        kp.sl2 = (float)((double)p.scale * 1.4426950408889634 * (1.0 + kCutOff * (steps + 1) / 2));
     }
     kp.n_kt = (int32_t)((p.total_kv + kTileN - 1) / kTileN);
     const int g = p.hq / p.hkv;
@@ -1647,10 +1681,11 @@ cudaError_t launch_prefill_sm100(Context *ctx, const PrefillParams &p, cudaStrea
     kp.magic_ppk = magic(ppk);
     for (int i = 0; i < kMaxP; ++i) kp.magic_small[i] = magic(i + 1);
     const int64_t blocks = items < ctx->sm_count ? items : ctx->sm_count;     // persistent: one CTA per SM
+    const int boxes = p.d <= kBoxCols ? 1 : 2;
     CUtensorMap mq, mk, mv, mo;
     if (!encode_map(ctx, &mq, p.q, p.n_q_rows, p.hq, p.d, false) ||
-        !encode_map(ctx, &mk, p.k, p.total_kv, p.hkv, p.d, p.kv_head_major != 0) ||
-        !encode_map(ctx, &mv, p.v, p.total_kv, p.hkv, p.d, p.kv_head_major != 0))
+        !encode_map(ctx, &mk, p.k, p.total_kv, p.hkv, p.d, p.kv_head_major != 0, tile_keys(p.d < 128, boxes)) ||
+        !encode_map(ctx, &mv, p.v, p.total_kv, p.hkv, p.d, p.kv_head_major != 0, tile_keys(p.d < 128, boxes)))
         return cudaErrorInvalidValue;
     // the output as [rows, heads, 128] in boxes of 32 rows x 64 columns; a base the encoder refuses (alignment)
     // leaves the kernel on its direct stores
@@ -1665,9 +1700,9 @@ cudaError_t launch_prefill_sm100(Context *ctx, const PrefillParams &p, cudaStrea
         prefill_sm100_kernel<true, 1, true, false>,   prefill_sm100_kernel<true, 2, true, false>,
         prefill_sm100_kernel<false, 2, false, true>,  prefill_sm100_kernel<true, 2, false, true>,
         prefill_sm100_kernel<true, 1, true, true>,    prefill_sm100_kernel<true, 2, true, true>};
-    const int form = p.d < 128 ? (p.d <= kBoxCols ? 2 : 3) : (p.general || (p.remote_only && !p.causal)) ? 1 : 0;
+    const int form = p.d < 128 ? 1 + boxes : (p.general || (p.remote_only && !p.causal)) ? 1 : 0;
     const int which = form + (halves ? 4 : 0);
-    const uint32_t smem = smem_bytes(form == 2 ? 1 : 2);
+    const uint32_t smem = smem_bytes(boxes);
     static bool attr_set[64][8] = {};
     if (!attr_set[ctx->device & 63][which]) {
         cudaError_t e = cudaFuncSetAttribute(kernels[which], cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
