@@ -1233,6 +1233,10 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 if (lane == 0) mbar_arrive(item_empty + ((pn - 1) & 1));
             }
 
+            // The first key a row sees weighs 1 but for the rounding of its reference.  Where a unit of the reference is
+            // worth more than its weight (logits beyond 2^24) the row is one for the routine below.
+            if (kExact && m_run != -INFINITY && !(l_run >= 0.25f)) l_run = __int_as_float(0x7fc00000);       // NaN
+
             // ---- epilogue: drain this row of O from TMEM (frees it for the next item), O / l -> bf16 -> global
             mbar_wait(o_done + t, (gsub + n_tiles - 1) & 1, abort_flag, kp.status);
             tc_fence_after();

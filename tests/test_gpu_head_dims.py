@@ -206,6 +206,22 @@ def test_lse_has_no_bias(hq, hkv, d, L):
     assert abs(err.mean()) <= 9e-8 and err.std() <= 2.5e-7
 
 
+@pytest.mark.parametrize("lens", [[400], [300, 517, 129]])
+@pytest.mark.parametrize("dtype,hq,hkv,d", [("bf16", 8, 2, 64), ("bf16", 6, 2, 96), ("bf16", 32, 32, 40), ("f32", 4, 4, 64)])
+def test_logits_whose_last_place_exceeds_one(dtype, hq, hkv, d, lens):
+    """Logits around 10^12, a unit of which is 2^16: a row's largest logit takes it all, and its weight must not depend on
+    how the reference was rounded."""
+    L, own = sum(lens), owners(lens)
+    q, k, v = gen(16, lens, hq, hkv, d, dtype)
+    q, k = q * 2.0 ** 20, k * 2.0 ** 20
+    r = Runner(len(lens), hq, hkv, d, dtype, L)
+    visible = np.tri(L, dtype=bool)
+    for (o, lse), vis in ((r.local(q, k, v, lens), visible & (own[:, None] == own)), (r.sync(q, k, v), visible)):
+        wo, wl = reference(q, k, v, vis)
+        # a logit is a sum of d terms around 2^40 / sqrt(d) that may cancel: d / 2 roundings of up to 2^-24 of sqrt(d) 2^40
+        assert np.abs(o - wo).max() <= 1e-6 and np.abs(lse - wl).max() <= d / 2 * 2.0 ** -24 * np.sqrt(d) * 2.0 ** 40
+
+
 @pytest.mark.parametrize("positions", [False, True])
 def test_as_many_keys_as_an_int_counts(positions):
     """2^31 - 1 keys of one head of 8 channels (34 GB, K and V in one buffer): the last tile ends where 32-bit sums would
