@@ -17,6 +17,15 @@ constexpr int kMaxP = FEDATTN_MAX_PARTICIPANTS;
 // Upper bound on spin iterations of any in-kernel wait before it gives up.
 constexpr uint32_t kSpinLimit = 1u << 22;
 
+// m2 ln 2 + ln l with one rounding beside the logarithm's: the product and the sum keep what they round off
+__device__ __forceinline__ float lse_exact(float m2, float l)
+{
+    const float ln2 = 0.6931471805599453f, ln2_rest = (float)(0.69314718055994530942 - (double)0.6931471805599453f);
+    const float prod = m2 * ln2, prod_rest = fmaf(m2, ln2, -prod) + m2 * ln2_rest;
+    const float lg = logf(l), sum = prod + lg, back = sum - prod;
+    return sum + (((prod - (sum - back)) + (lg - back)) + prod_rest);
+}
+
 struct Context {
     int device;
     int sm_count;

@@ -381,15 +381,6 @@ constexpr uint32_t kIdescPV = make_idesc(128) | (1u << 16);    // B (V) MN-major
 // n / d for 0 <= n < 2^28 and 1 <= d <= 4096, with magic = ceil(2^40 / d)
 __device__ __forceinline__ int fast_div(int n, uint64_t magic) { return (int)(((uint64_t)(uint32_t)n * magic) >> 40); }
 
-// m2 ln 2 + ln l with one rounding beside the logarithm's: the product and the sum keep what they round off
-__device__ __forceinline__ float lse_exact(float m2, float l)
-{
-    const float ln2 = 0.6931471805599453f, ln2_rest = (float)(0.69314718055994530942 - (double)0.6931471805599453f);
-    const float prod = m2 * ln2, prod_rest = fmaf(m2, ln2, -prod) + m2 * ln2_rest;
-    const float lg = logf(l), sum = prod + lg, back = sum - prod;
-    return sum + (((prod - (sum - back)) + (lg - back)) + prod_rest);
-}
-
 // number of entries of the non-decreasing array pos[0..n) that are <= x
 __device__ __forceinline__ int count_le(const int32_t *pos, int n, int x)
 {
