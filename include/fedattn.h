@@ -228,8 +228,10 @@ fedattn_status fedattn_merge(fedattn_ctx *ctx, const fedattn_shape *shape, int64
  *   FEDATTN_DECODE_SYNC   every participant reads rows 0..kv_len[0]-1 of one shared cache
  *                         [T,Hkv,d]; kv_len dev int32 [1]; cache_stride_participant ignored.
  *   q, o dev [N,Hq,d]; lse dev float [N,Hq] or NULL; max_kv_len >= every kv_len (host; sizes the
- *   split-KV grid).  kv_len = 0 gives o = 0, lse = -inf.  Uses the workspace for split-KV partials.
- *   Two launches per call (stream, then merge), chained by programmatic dependent launch. */
+ *   split-KV grid).  kv_len = 0 gives o = 0, lse = -inf.  Uses the workspace for split-KV partials
+ *   (bf16, head_dim 128).
+ *   bf16 with head_dim 128: short calls are one launch, longer ones two (stream, then merge), chained by
+ *   programmatic dependent launch.  Other types and head dims: one launch. */
 typedef enum { FEDATTN_DECODE_LOCAL = 0, FEDATTN_DECODE_SYNC = 1 } fedattn_decode_mode;
 
 fedattn_status fedattn_decode(fedattn_ctx *ctx, const fedattn_shape *shape, int32_t mode,

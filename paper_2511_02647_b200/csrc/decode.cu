@@ -10,7 +10,7 @@
 // Short calls (kOneLaunchBytes, kOneLaunchTiles) are one launch: the splits of a (cache, KV head) form a cluster, and
 // the partials are merged in its shared memory.  A call of that size streams for 2-3 us, so what it costs is launches
 // (6 us of host time for two, 4 for one) and the way through the scratch: 4 x 160 keys 2.8 -> 1.4 us, 2800 shared keys
-// 6.6 -> 3.0 us, both and their merge 16.2 -> 10.7 us; four blocks over 16 x 100 keys 26 -> 13 us.
+// 6.6 -> 3.0 us, both and their merge 18.4 -> 12.4 us; four blocks over 16 x 100 keys 26 -> 13 us.
 //
 // Longer calls are two launches, chained by programmatic dependent launch:
 //   decode_stream_kernel  one CTA per (cache, KV head, split); every warp walks its key slice of the
@@ -28,8 +28,9 @@
 // call i are hidden behind the next call's streaming.  Reading before the wait is sound because the
 // only grids that release dependents early are this library's own, and they write nothing but their
 // outputs and the scratch: the launcher checks the inputs of a call against the outputs of the recent
-// calls of that kind and falls back to waiting first when they overlap (early_start.cu).  No CTA ever
-// waits on another CTA.
+// calls of that kind and falls back to waiting first when they overlap (early_start.cu).  A CTA waits for no CTA of
+// another grid but through griddepcontrol.wait; those of a one-launch call wait for the CTAs of their own cluster, which
+// are scheduled together and take nothing from later grids, so an early start cannot hold them up.
 #include <cooperative_groups.h>
 #include <string.h>
 

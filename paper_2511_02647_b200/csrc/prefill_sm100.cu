@@ -2,9 +2,10 @@
 // online softmax in fp32.  Serves fedattn_local (per-participant causal attention over packed
 // segments) and fedattn_sync (queries over the aggregated KV, causal on global positions).
 //
-// Persistent kernel, one CTA per SM.  A work item is one 128-row query tile of a PAIR of query heads
-// that share a KV head (two "sub-tiles"); the CTA walks the key/value tiles the rows may see, and
-// tiles that the segment descriptors or the causal mask rule out are never loaded.  Items are sorted
+// Persistent kernel, one CTA per SM.  A work item is two "sub-tiles" of 128 query rows x one query head that share a
+// KV head: two heads of a query tile; the last heads of an odd group in two neighbouring query tiles ("straddle"); or
+// one head of one query tile, whose KV tiles the sub-tiles share ("halves").  Each sub-tile walks the key/value tiles
+// its rows may see; tiles that the segment descriptors or the causal mask rule out are never loaded.  Items are sorted
 // by cost and dealt to the CTAs in snake order.
 //
 // Per KV tile j and sub-tile t:
@@ -19,7 +20,8 @@
 //
 // Warp roles: warps 0-3 softmax/epilogue of sub-tile 0, warps 4-7 of sub-tile 1: thread = query row =
 // TMEM lane, all 128 key columns of the S tile (read from TMEM once, held in registers for the row
-// maximum and then the exponentials) and the whole row of O; nothing is exchanged between threads.  Warp 8
+// maximum and then the exponentials) and the whole row of O; nothing is exchanged between threads (halves: the two
+// partials of a row meet in the epilogue).  Warp 8
 // TMA producer (+ TMEM allocation), warp 9 MMA issuer (the whole warp walks the loop, one elected lane
 // issues); warp 10 checks the order of the key positions, warp 11 only fills that warpgroup, which
 // hands most of its registers to the softmax warpgroups (setmaxnreg works on whole warpgroups).
@@ -85,7 +87,7 @@ struct KernelParams {
     int32_t straddle;                // odd groups: ranked tiles have 256 rows, the last heads of their halves form an item
     uint64_t magic_per_tile, magic_ppk, magic_small[kMaxP];   // ceil(2^40 / d) for d = items per tile, per KV head, 1..kMaxP
     int32_t n_qtiles;                // total query tiles
-    int32_t n_items;                 // query tiles x KV heads x head pairs
+    int32_t n_items;                 // ranked tiles x KV heads x items of one KV head
     int32_t n_kt;                    // KV tiles: ceil(total_kv / kTileN)
     int32_t *status;
     int32_t o_tma;                   // the output may leave through TMA stores (tensor map encoded)
@@ -433,7 +435,6 @@ __device__ __forceinline__ int tile_of(const Item &it, int j) { return j < it.n_
 
 // allowed-prefix length c(row): keys kv_begin .. kv_begin + c - 1 are visible to query row r of the tile.
 // Called by a converged warp with the same r in every lane (the searches are warp-cooperative).
-template <bool kSpecial>
 __device__ __forceinline__ int prefix_len(const PrefillParams &p, const Item &it, const Sub &sub, int r, int lane)
 {
     const int pos = sub.q_row0 + r;
@@ -584,7 +585,7 @@ __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, in
         // keys [0, a) lie before the rows' segment; when bidirectional (special instance only), keys [b, T)
         // after it count too
         const int T = (int)p.total_kv, n_t = (T + kKeys - 1) / kKeys;
-        it.a = prefix_len<kSpecial>(p, it, sub[1], 0, lane);
+        it.a = prefix_len(p, it, sub[1], 0, lane);
         it.n_a = (it.a + kKeys - 1) / kKeys;
         sub[1].n_tiles = it.n_a;
         it.b = T;
@@ -601,7 +602,7 @@ __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, in
             const Sub x = again ? sub[0] : sub[1];
             int n;
             if (kExact && kp.pairs) n = last_visible_tile<kKeys>(kp, it, x, lane);
-            else n = (prefix_len<kSpecial>(p, it, x, x.n_valid - 1, lane) + kKeys - 1) / kKeys;
+            else n = (prefix_len(p, it, x, x.n_valid - 1, lane) + kKeys - 1) / kKeys;
             if (again) { sub[0].n_tiles = n; continue; }
             sub[1].n_tiles = n;
             break;
@@ -625,10 +626,10 @@ __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, in
 //
 // kBoxes: 64-column boxes per tile (head_dim <= 64: one; <= 128: two).  kExact: the weights P keep their 24 bits (three
 // bf16 parts, three PV products), every exponential is ex2, and rows that come out non-finite are redone by the row
-// routine.  It serves the head dims below 128, whose users had fp32 weights from the SIMT kernel.  Bound by the PV
-// products (d = 64: 4 + 3 x 8 MMAs per tile, the latter of N = 64 and no faster than of N = 128): two parts, 16 bits, take
-// 20.7 and 47.1 us, three 24.7 and 55.9 for the local and the sync call of six ragged segments of 2160 tokens, 16 / 4 heads of 64
-// channels (2436 and 10994 us with one warp per row, fp32 FMA).  The error of o against fp64 is that of fp32 weights (the
+// routine.  It serves the head dims below 128, whose users had fp32 weights from the SIMT kernel.  Bound by the chain
+// softmax -> PV -> S, which carries the products (d = 64: 4 + 3 x 8 MMAs per tile, the latter of N = 64, no faster than of
+// N = 128): two parts, 16 bits, take 20.7 and 47.1 us, three 24.7 and 55.9 for the local and the sync call of six ragged
+// segments of 2160 tokens, 16 / 4 heads of 64 channels (2436 and 10994 us with one warp per row, fp32 FMA).  The error of o against fp64 is that of fp32 weights (the
 // rounding of the bf16 output, 1.587459e-3 there; 1.587460e-3 with two parts), lse 3.2e-8 -> 2.9e-8 relative.
 //
 // kHalves: both sub-tiles are the SAME query tile of one head; sub-tile 1 walks the even KV tiles and sub-tile 0 the odd
@@ -930,10 +931,10 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSoftmaxRegs));
         // ================= softmax + epilogue =================
         // Warpgroup t serves sub-tile t (one query head of one query tile) on its own: thread = query row r = TMEM lane,
-        // all 128 key columns of the S tile, the whole row of O.  The two warpgroups never meet: no row
-        // maximum or row sum has to be exchanged, and while one is in the serial part of its visit (wait,
-        // TMEM load, maximum) the other computes.  A thread reads its row of S from TMEM once and keeps all
-        // 128 values in registers for both walks (maximum, then exponentials).
+        // all key columns of the S tile, the whole row of O.  During the walk the two warpgroups never meet (those of a
+        // halved item do in the epilogue): no row maximum or row sum has to be exchanged, and while one is in the
+        // serial part of its visit (wait, TMEM load, maximum) the other computes.  A thread reads its row of S from TMEM once and keeps
+        // its values in registers for both walks (maximum, then exponentials).
         const int t = warp >> 2;                                // sub-tile of this warpgroup
         const int r = tid & 127;                                // query row = TMEM lane
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
@@ -1147,7 +1148,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     c_row = cw + cnt;
                     if (__shfl_sync(0xffffffffu, wv, 31) <= p0 + 31) c_row = count_le(it.kvp, T, p0 + lane);
                 } else {
-                    c_row = prefix_len<kSpecial>(p, it, sub, r, lane);   // arithmetic only
+                    c_row = prefix_len(p, it, sub, r, lane);   // arithmetic only
                 }
                 // prefix lengths do not decrease with the row, so KV tiles below the prefix of the warp's first
                 // row are unmasked for the whole warp (the choice of code path only has to be warp-uniform)
@@ -1682,7 +1683,7 @@ cudaError_t launch_prefill_sm100(Context *ctx, const PrefillParams &p, cudaStrea
         !encode_map(ctx, &mk, p.k, p.total_kv, p.hkv, p.d, p.kv_head_major != 0, tile_keys(p.d < 128, boxes)) ||
         !encode_map(ctx, &mv, p.v, p.total_kv, p.hkv, p.d, p.kv_head_major != 0, tile_keys(p.d < 128, boxes)))
         return cudaErrorInvalidValue;
-    // the output as [rows, heads, 128] in boxes of 32 rows x 64 columns; a base the encoder refuses (alignment)
+    // the output as [rows, heads, head_dim] in boxes of 32 rows x 64 columns; a base the encoder refuses (alignment)
     // leaves the kernel on its direct stores
     kp.o_tma = encode_map(ctx, &mo, p.o, p.n_q_rows, p.hq, p.d, false, 32) ? 1 : 0;
     if (!kp.o_tma) mo = mq;
