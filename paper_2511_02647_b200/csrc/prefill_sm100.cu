@@ -1549,8 +1549,12 @@ enum ItemForm {
     kHalvesForm,  // one head, its KV tiles shared by the two sub-tiles (kernel instances kHalves)
 };
 // The form that is estimated to end first.  Unit: a lone sub-tile's time per KV tile, 1.6 us; a pair takes 1.14 times as
-// long (8 / 8 heads, 17 query tiles: lone 32.7 us, pairs 37.4), halves 0.6 per KV tile of their head (0.9 with exact
-// weights), and every item costs about 2 on top (its Q, its epilogue, the restart of the chain; halves 2.6, they merge).
+// long (8 / 8 heads, 17 query tiles: lone 32.7 us, pairs 37.4), halves 0.6 per KV tile of their head, and every item costs
+// about 2 on top (its Q, its epilogue, the restart of the chain; halves 2.6, they merge).  With exact weights, and an item
+// per CTA, the unit is 3.2 us per 128 keys, a pair takes 1.05, halves 0.65 and an item 1 on top (halves 1.4): 4 / 4 heads
+// of 64, two segments of 500 rows: 16.6 -> 14.5 and 31.1 -> 24.7 us (halves for pairs).  Several items per CTA gain less,
+// halves 0.9: 16 / 4 heads of 64, six segments of 2160 rows, sync 55.5 -> 51.5 us in a loop, but a round that runs its local
+// call as pairs fetches the other instance's code for it, and takes 85.3 us with pairs and 87.4 with halves.
 // Calls of a few items per CTA are dealt out on paper as the kernel deals them; for more items the mean load of a CTA
 // decides, and halves never pay (twice the items and twice the K and V traffic).  Measured against the estimate's second
 // choice, us: 16 / 4 heads, 700 + 500 rows: local 18.4 -> 13.9, sync 25.8 -> 18.5 (halves for pairs); 32 / 8 heads there:
@@ -1561,7 +1565,10 @@ static ItemForm item_form(const PrefillParams &p, int64_t n_qtiles, int sm_count
     constexpr int kMostSms = 256;
     const int g = p.hq / p.hkv;
     if ((int64_t)p.hkv * g > 4096 || n_qtiles * p.hkv * g >= (1LL << 28) || sm_count > kMostSms) return kPairs;      // fast_div range
-    const float pair = 1.14f, half = p.d < 128 ? 0.9f : 0.6f, start = 2.0f, merge = 0.6f, n_kt = (float)((p.total_kv + kTileN - 1) / kTileN);
+    const bool alone = n_qtiles * p.hq <= sm_count;             // an item per CTA in every form
+    const bool narrow = p.d < 128 && alone;
+    const float pair = narrow ? 1.05f : 1.14f, half = narrow ? 0.65f : (p.d < 128 ? 0.9f : 0.6f);
+    const float start = narrow ? 1.0f : 2.0f, merge = narrow ? 0.4f : 0.6f, n_kt = (float)((p.total_kv + kTileN - 1) / kTileN);
     const bool grows = p.causal && !p.remote_only && !(p.sync && p.q_pos);
     // KV tiles of query tile `tile` (1 ..) of a segment with `tiles` of them
     auto walk = [&](int seg, int tile, int tiles) -> float {
@@ -1577,7 +1584,7 @@ static ItemForm item_form(const PrefillParams &p, int64_t n_qtiles, int sm_count
     float load[kMostSms];
     int longest = 0;
     for (int n = 0; n < p.n_seg; ++n) longest = tiles_of(n) > longest ? tiles_of(n) : longest;
-    if (n_qtiles * p.hq <= sm_count) {                          // an item per CTA in every form: the longest one decides
+    if (alone) {                                                // the longest item decides
         float w = 0.f;
         for (int n = 0; n < p.n_seg; ++n)
             if (tiles_of(n) > 0) w = walk(n, tiles_of(n), tiles_of(n)) > w ? walk(n, tiles_of(n), tiles_of(n)) : w;
