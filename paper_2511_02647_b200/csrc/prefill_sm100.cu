@@ -47,27 +47,30 @@ namespace {
 constexpr int kTileM = 128;          // query rows per CTA
 constexpr int kTileN = 128;          // keys per KV tile
 constexpr int kBoxCols = 64;          // head-dim columns of one TMA box (128-byte swizzle); a tile is 1 or 2 boxes
-constexpr int kSoftmaxWarps = 16;     // four warpgroups: sub-tile x half of the keys (and of the output channels)
-constexpr int kThreads = 32 * kSoftmaxWarps + 128;  // then a warpgroup holding the TMA producer warp and the MMA issuer warp
+// two softmax warpgroups, one per sub-tile.  (Both on the same S tile, split by columns with the row
+// maxima exchanged through shared memory, was 2-4 % slower on dense sync; four warpgroups of 32 columns
+// 20 %.)  P is handed to the MMA warp in kSplit halves, so that PV starts on the first.
+constexpr int kSplit = 2;
+constexpr int kSoftmaxThreads = 128 * kSplit;
+constexpr int kThreads = kSoftmaxThreads + 128;  // then a warpgroup holding the TMA producer warp and the MMA issuer warp
 // Registers move from that warpgroup to the softmax warpgroups once the roles split (setmaxnreg):
-// 640 threads start with 96 each, and that allocation (5 x 96 = 480 registers per lane slot of a
+// 384 threads start with 168 each, and that allocation (3 x 168 = 504 registers per lane slot of a
 // scheduler) is the pool the increases draw from.  setmaxnreg.inc waits, without limit, until the pool
-// can give what it asks for, so the split must fit into it: 4 x kSoftmaxRegs + kOtherRegs <= 480.
-constexpr int kSoftmaxRegs = 104, kOtherRegs = 64, kLaunchRegs = 96;
-static_assert(4 * kSoftmaxRegs + kOtherRegs <= 5 * kLaunchRegs && kSoftmaxRegs % 8 == 0 && kOtherRegs % 8 == 0, "register budget");
-constexpr int kProducerWarp = kSoftmaxWarps, kMmaWarp = kSoftmaxWarps + 1;
-constexpr uint32_t kBoxBytes = kTileM * kBoxCols * 2;    // 16 KB: one 64-column TMA box of a Q tile
-constexpr uint32_t kBarrierBytes = 1024;              // barriers, published items, walks
+// can give what it asks for, so the split must fit into it: 2 x kSoftmaxRegs + kOtherRegs <= 504; it
+// keeps 8 spare.  (A 200 / 112 split asks for 512 per lane slot and never came back from the increase.)
+constexpr int kSoftmaxRegs = 216, kOtherRegs = 64;
+static_assert(2 * kSoftmaxRegs + kOtherRegs <= 496 && kSoftmaxRegs % 8 == 0 && kOtherRegs % 8 == 0, "register budget");
+constexpr int kProducerWarp = 4 * kSplit, kMmaWarp = 4 * kSplit + 1;
+static_assert(kSplit == 2 || kSplit == 4, "column split");
+constexpr uint32_t kHalfBytes = kTileM * kBoxCols * 2;   // 16 KB: one 64-column TMA box of a Q, K or V tile
+constexpr uint32_t kStageBytes = 32 * 128;            // output staging per softmax warp: 32 rows x 64 columns
+constexpr uint32_t smem_bytes(int boxes)
+{
+    return 6 * boxes * kHalfBytes + 1024 /*alignment slack*/ + 1024 /*barriers, published items*/ + 2 * kSplit * 2 * kStageBytes;
+}
 // Keys per KV tile of an instance: weights in three bf16 parts take 3 x 16 columns of TMEM per 32 keys where S had 32; one
 // box (head_dim <= 64) has the third part beside O, whose upper 64 columns are free, two boxes have room for 64 keys only.
 __host__ __device__ constexpr int tile_keys(bool exact, int boxes) { return exact && boxes == 2 ? 64 : kTileN; }
-// Stages of the ring of K and V tiles: three of 32 KB beside two items' Q, four where the tiles are smaller.
-__host__ __device__ constexpr int kv_stages(bool exact, int boxes) { return exact ? 4 : 3; }
-constexpr uint32_t smem_bytes(bool exact, int boxes)
-{
-    return 4 * boxes * kBoxBytes + kv_stages(exact, boxes) * boxes * tile_keys(exact, boxes) * kBoxCols * 2 + kBarrierBytes + 4 * kTileM * 4;
-}
-static_assert(smem_bytes(false, 2) <= 227 * 1024, "shared memory");
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kColS = 0, kColO = 256;   // S (and P, aliased) of sub-tile t at kColS + 128 t; O at kColO + 128 t
 // P (bf16 pairs) of keys 64 q .. 64 q + 63 sits at S column 64 q: every 32-key chunk of P
@@ -113,6 +116,14 @@ __device__ __host__ __forceinline__ PosTables pos_tables(const int32_t *tab, int
 // alternate tokens of the sequence, four of 5001 rows in all, 32 / 8 heads: 955 us walking up to the last visible tile,
 // 556 us with the list; contiguous members have nothing to skip.)
 constexpr int kWalkMost = 128;
+
+#ifdef FEDATTN_TRACE
+// Debug build only: cycle stamps of one CTA's pipeline events, [tile][event].
+__device__ long long g_trace[64 * 8];
+#define TRACE(j, e) do { if (k == 0 && blockIdx.x == gridDim.x / 2 && (j) < 64) g_trace[(j) * 8 + (e)] = clock64(); } while (0)
+#else
+#define TRACE(j, e) do { } while (0)
+#endif
 
 // ---- PTX wrappers ---------------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -186,6 +197,12 @@ __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, u
                  " [%0], [%1, {%3, %4, %5}], [%2];"
                  ::"r"(smem_u32(dst)), "l"((uint64_t)map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2)
                  : "memory");
+}
+
+__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap *map, int c0, int c1, int c2)
+{
+    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];"
+                 ::"l"((uint64_t)map), "r"(c0), "r"(c1), "r"(c2) : "memory");
 }
 
 // [32 rows x 64 columns] from shared memory (128-byte swizzle) to the output, one bulk group per call
@@ -603,8 +620,8 @@ __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, in
 }
 
 // Persistent kernel: one CTA per SM walks the work items item = blockIdx.x, blockIdx.x + gridDim.x, ...
-// Barrier phases run on: per-CTA counters of loaded tiles, of KV tiles and of non-empty items (qn) give stages
-// and parities, so the producer loads the next item's Q (into the other slot) and K/V while the current item's last
+// Barrier phases run on: per-CTA counters of KV tiles (git) and of non-empty items (qn) give stages
+// and parities, so the producer prefetches the next item's K/V and Q while the current item's last
 // tiles and its epilogue are still in flight.
 //
 // kBoxes: 64-column boxes per tile (head_dim <= 64: one; <= 128: two).  kExact: the weights P keep their 24 bits (three
@@ -626,36 +643,35 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                      const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o,
                      const __grid_constant__ KernelParams kp)
 {
-    extern __shared__ __align__(1024) uint8_t smem[];
-    constexpr uint32_t kTileBytes = kBoxes * kBoxBytes;                             // a Q tile
-    constexpr int kKeys = tile_keys(kExact, kBoxes);                                // keys of a KV tile
-    constexpr int kMyKeys = kKeys / 2, kParts = kMyKeys / 32;                       // a thread's share: its keys, in chunks of 32
-    constexpr int kStages = kv_stages(kExact, kBoxes);                              // K and V tiles on their way or in use
+    extern __shared__ uint8_t smem_raw[];
+    constexpr uint32_t kTileBytes = kBoxes * kHalfBytes;                            // a Q tile
+    constexpr int kKeys = tile_keys(kExact, kBoxes), kChunks = kKeys / 32;         // keys of a KV tile, in chunks of 32
+    constexpr int kPartKeys = kKeys / kSplit;                                      // keys of a half of P
     constexpr uint32_t kColP3 = (kBoxes == 1 ? kColO : kColS) + 64;                // exact instances: third parts of sub-tile 0's P
     constexpr uint32_t kKvBox = kKeys * kBoxCols * 2, kKvBytes = kBoxes * kKvBox;  // a K or V tile
     const PrefillParams &p = kp.p;
     const int d = kExact ? p.d : kBoxes * kBoxCols;
-    uint8_t *sQ = smem;                                  // [2 slots][2 sub-tiles][tile]; an item's output is staged in its dead Q
-    uint8_t *sKV = smem + 4 * kTileBytes;                // [kStages][tile], K and V in the order of their use
-    uint64_t *bars = reinterpret_cast<uint64_t *>(sKV + kStages * kKvBytes);
-    uint64_t *q_full = bars + 0, *q_empty = bars + 2;    // [slot]
-    uint64_t *kv_full = bars + 4, *kv_empty = bars + 10; // [stage], at most 6
-    uint64_t *s_full = bars + 16, *o_done = bars + 18, *o_free = bars + 20;
-    uint64_t *p_full = bars + 22;                        // [sub-tile][part]
-    // The producer decodes every work item once and publishes it here for the softmax warps (two slots of
-    // 16 ints, filled an item ahead), so that decoding is not on their path between two items.
-    uint64_t *item_full = bars + 26, *item_empty = bars + 28;
-    uint64_t *row_met = bars + 30;                       // [sub-tile][32 rows]: the two warps of these rows have left a value
-    uint64_t *halves_met = bars + 38;                    // halves: all warps have left their partials' (m, l)
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 39);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(bars + 40);
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t *sQ = smem;                                  // [2 sub-tiles][tile]
+    uint8_t *sK = smem + 2 * kTileBytes;                 // [2 stages][tile]
+    uint8_t *sV = sK + 2 * kKvBytes;                     // [2 stages][tile]
+    uint64_t *bars = reinterpret_cast<uint64_t *>(sV + 2 * kKvBytes);
+    uint64_t *q_full = bars + 0, *q_empty = bars + 1;
+    uint64_t *k_full = bars + 2, *k_empty = bars + 4, *v_full = bars + 6, *v_empty = bars + 8;
+    uint64_t *s_full = bars + 10, *o_done = bars + 12, *o_free = bars + 14;
+    uint64_t *p_full = bars + 16;                        // [sub-tile][column part]
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 24);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(bars + 25);
     // what the producer tells the MMA issuer about an item, published before the item's Q load is issued
     // and read after q_full: {KV tiles of sub-tile 1, of sub-tile 0}; -1 tiles = no more items.  Two slots, like the phases.
-    volatile int *item_info = reinterpret_cast<volatile int *>(bars + 41);
-    volatile int *item_pub = reinterpret_cast<volatile int *>(bars + 44);
-    uint16_t *walks = reinterpret_cast<uint16_t *>(bars + 60);      // general: [slot][kWalkMost]
-    static_assert(60 * 8 + 2 * kWalkMost * 2 <= kBarrierBytes, "barrier area");
-    float *row_val = reinterpret_cast<float *>(reinterpret_cast<uint8_t *>(bars) + kBarrierBytes);    // [sub-tile][half][row]
+    volatile int *item_info = reinterpret_cast<volatile int *>(bars + 26);
+    // The producer decodes every work item once and publishes it here for the softmax warps (two slots of
+    // 16 ints, filled an item ahead), so that decoding is not on their path between two items.
+    uint64_t *item_full = bars + 20, *item_empty = bars + 22;
+    uint64_t *halves_met = bars + 28;                    // halves: both warpgroups have left their partials' (m, l)
+    volatile int *item_pub = reinterpret_cast<volatile int *>(bars + 32);
+    uint16_t *walks = reinterpret_cast<uint16_t *>(bars + 48);      // general: [slot][kWalkMost]
+    uint8_t *stage = sV + 2 * kKvBytes + 1024;           // [softmax warp][32 rows][128 B], 128-byte swizzle
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int n_items = kp.n_items;
@@ -668,16 +684,15 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 
     // ---- setup ------------------------------------------------------------------------------------
     if (tid == 0) {
+        mbar_init(q_full, 1); mbar_init(q_empty, 1);
         for (int i = 0; i < 2; ++i) {
-            mbar_init(q_full + i, 1); mbar_init(q_empty + i, kSoftmaxWarps);
+            mbar_init(k_full + i, 1); mbar_init(k_empty + i, 1); mbar_init(v_full + i, 1); mbar_init(v_empty + i, 1);
             mbar_init(s_full + i, 1); mbar_init(o_done + i, 1);
-            mbar_init(o_free + i, kHalves ? kSoftmaxWarps : kSoftmaxWarps / 2);     // (halves: every warp reads both accumulators)
-            for (int q = 0; q < 2; ++q) mbar_init(p_full + 2 * i + q, kSoftmaxWarps / 2);
-            mbar_init(item_full + i, 1); mbar_init(item_empty + i, kSoftmaxWarps);
+            mbar_init(o_free + i, kHalves ? 8 : 4);             // (halves: every warp reads both accumulators)
+            for (int q = 0; q < kSplit; ++q) mbar_init(p_full + kSplit * i + q, 4);
+            mbar_init(item_full + i, 1); mbar_init(item_empty + i, 2 * kSplit * 2);
         }
-        for (int i = 0; i < kStages; ++i) { mbar_init(kv_full + i, 1); mbar_init(kv_empty + i, 1); }
-        for (int i = 0; i < 8; ++i) mbar_init(row_met + i, 2);
-        mbar_init(halves_met, kSoftmaxWarps);
+        mbar_init(halves_met, 8);
         *abort_flag = (*reinterpret_cast<volatile int32_t *>(kp.status) == FEDATTN_ERR_TIMEOUT) ? 1 : 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -706,7 +721,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&map_k) : "memory");
             asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&map_v) : "memory");
         }
-        int loads = 0, st = 0, laps = 0, qn = 0, pn = 0;        // tiles loaded, the next one's stage, times round the ring
+        int git = 0, qn = 0, pn = 0;
         // After a wait that ran out nothing is published or loaded any more: a slot may still be read, a buffer still be
         // written.  (All lanes get lane 0's answer.)
         auto slot_free = [&]() -> bool {
@@ -735,206 +750,171 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     slot[11 + 4 * t] = sub[t].n_tiles;
                 }
                 mbar_arrive(item_full + (pn & 1));
+                // this item's Q on its way into L2: the load itself has to wait for the Q buffer
+#pragma unroll
+                for (int t = kHalves ? 1 : 0; t < 2; ++t)
+                    if (sub[t].n_tiles > 0) {
+                        tma_prefetch_3d(&map_q, 0, sub[t].head, sub[t].q_row0);
+                        if (kBoxes == 2) tma_prefetch_3d(&map_q, 64, sub[t].head, sub[t].q_row0);
+                    }
             }
             ++pn;
             if (n_tiles == 0) continue;
-            int issued = 0;                                     // lane 0: tiles of the item on their way
+            int issued = 0;                                     // lane 0: KV tiles of the item on their way
             bool q_free = true;
-            uint8_t *q_slot = sQ + (qn & 1) * 2 * kTileBytes;
-            // the item before the previous one: its output has left the slot
-            if (lane == 0 && qn >= 2) q_free = mbar_wait_call(q_empty + (qn & 1), ((qn >> 1) - 1) & 1, abort_flag, kp.status);
+            if (lane == 0 && qn > 0) q_free = mbar_wait_call(q_empty, (qn - 1) & 1, abort_flag, kp.status);   // previous item's S MMAs done
             if (lane == 0 && q_free) {
-                uint64_t *full = q_full + (qn & 1);
                 item_info[(qn & 1) * 2] = sub[1].n_tiles;
                 item_info[(qn & 1) * 2 + 1] = sub[0].n_tiles;
-                mbar_expect_tx(full, !kHalves && sub[0].n_tiles > 0 ? 2 * kTileBytes : kTileBytes);
+                mbar_expect_tx(q_full, !kHalves && sub[0].n_tiles > 0 ? 2 * kTileBytes : kTileBytes);
 #pragma unroll
                 for (int t = kHalves ? 1 : 0; t < 2; ++t)       // (halves share sub-tile 1's Q)
                     if (sub[t].n_tiles > 0) {
-                        tma_load_3d(q_slot + t * kTileBytes, &map_q, full, 0, sub[t].head, sub[t].q_row0);
-                        if (kBoxes == 2) tma_load_3d(q_slot + t * kTileBytes + kBoxBytes, &map_q, full, 64, sub[t].head, sub[t].q_row0);
+                        tma_load_3d(sQ + t * kTileBytes, &map_q, q_full, 0, sub[t].head, sub[t].q_row0);
+                        if (kBoxes == 2) tma_load_3d(sQ + t * kTileBytes + kHalfBytes, &map_q, q_full, 64, sub[t].head, sub[t].q_row0);
                     }
                 const bool listed = general && it.b < 0;
-                for (int c = 0; c < 2 * n_tiles; ++c) {
-                    // in the order of their use: K0 V0 K1 V1 ..., halves K0 K1 V0 K2 V1 ... K V V
-                    int j = c >> 1;
-                    bool is_v = c & 1;
-                    if (kHalves && c > 0) {
-                        is_v = !is_v || c == 2 * n_tiles - 1;
-                        j = !is_v ? j + 1 : ((c & 1) ? j : j - 1);
-                    }
+                for (int j = 0; j < n_tiles; ++j) {
+                    const int gt = git + j, st = gt & 1, use = gt >> 1;
                     int tile = kSpecial ? tile_of(it, j) : j;
                     if (listed) tile = walk[j] & 0x7fff;
                     const int row = it.kv_begin + tile * kKeys;
                     const int c1 = p.kv_head_major ? row : it.kvh, c2 = p.kv_head_major ? it.kvh : row;
-                    if (laps > 0 && !mbar_wait_call(kv_empty + st, (laps - 1) & 1, abort_flag, kp.status)) break;
-                    issued = c + 1;
-                    const CUtensorMap *map = is_v ? &map_v : &map_k;
-                    mbar_expect_tx(kv_full + st, kKvBytes);
-                    tma_load_3d(sKV + st * kKvBytes, map, kv_full + st, 0, c1, c2);
-                    if (kBoxes == 2) tma_load_3d(sKV + st * kKvBytes + kKvBox, map, kv_full + st, 64, c1, c2);
-                    if (++st == kStages) { st = 0; ++laps; }
+                    if (gt >= 2 && !mbar_wait_call(k_empty + st, (use - 1) & 1, abort_flag, kp.status)) break;
+                    issued = j + 1;
+                    TRACE(j, 7);
+                    mbar_expect_tx(k_full + st, kKvBytes);
+                    tma_load_3d(sK + st * kKvBytes, &map_k, k_full + st, 0, c1, c2);
+                    if (kBoxes == 2) tma_load_3d(sK + st * kKvBytes + kKvBox, &map_k, k_full + st, 64, c1, c2);
+                    if (gt >= 2 && !mbar_wait_call(v_empty + st, (use - 1) & 1, abort_flag, kp.status)) break;
+                    mbar_expect_tx(v_full + st, kKvBytes);
+                    tma_load_3d(sV + st * kKvBytes, &map_v, v_full + st, 0, c1, c2);
+                    if (kBoxes == 2) tma_load_3d(sV + st * kKvBytes + kKvBox, &map_v, v_full + st, 64, c1, c2);
                 }
             }
             issued = __shfl_sync(0xffffffffu, issued, 0);
-            loads += issued;
+            git += issued;
             qn += __shfl_sync(0xffffffffu, (int)q_free, 0);
-            if (issued < 2 * n_tiles) break;
+            if (issued < n_tiles) break;
         }
         if (lane == 0) {
             // end marker for the MMA issuer, in the slot and phase the next item would have used
-            if (qn >= 2) mbar_wait_call(q_empty + (qn & 1), ((qn >> 1) - 1) & 1, abort_flag, kp.status);
+            if (qn > 0) mbar_wait_call(q_empty, (qn - 1) & 1, abort_flag, kp.status);
             item_info[(qn & 1) * 2] = -1;
-            mbar_arrive(q_full + (qn & 1));
+            mbar_arrive(q_full);
             if (*abort_flag) {
                 // give the copies still in flight a bounded chance to land before the CTA retires
-                for (int i = max(0, loads - kStages); i < loads; ++i)
-                    for (uint32_t w = 0; w < 4096 && !mbar_try_wait(kv_full + i % kStages, (i / kStages) & 1); ++w) {}
-                for (int i = max(0, qn - 2); i < qn; ++i)
-                    for (uint32_t w = 0; w < 4096 && !mbar_try_wait(q_full + (i & 1), (i >> 1) & 1); ++w) {}
+                for (int gt = max(0, git - 2); gt < git; ++gt) {
+                    for (uint32_t w = 0; w < 4096 && !mbar_try_wait(k_full + (gt & 1), (gt >> 1) & 1); ++w) {}
+                    for (uint32_t w = 0; w < 4096 && !mbar_try_wait(v_full + (gt & 1), (gt >> 1) & 1); ++w) {}
+                }
+                if (qn > 0)
+                    for (uint32_t w = 0; w < 4096 && !mbar_try_wait(q_full, (qn - 1) & 1); ++w) {}
             }
         }
     } else if (warp == kMmaWarp) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs));
         // ================= MMA issuer =================
         // Issue order per item  S0(0) S1(0) | PV0(0) S0(1) | PV1(0) S1(1) | PV0(1) S0(2) | ...  : while one
-        // sub-tile's softmax runs, the tensor pipe works on the other sub-tile.  Behind a sub-tile's last PV comes its
-        // first S of the next item, if that item's Q and K are there already.
+        // sub-tile's softmax runs, the tensor pipe works on the other sub-tile.
         // The whole warp walks the loop (waits included) so that control flow and operand descriptors
         // stay warp-uniform; one elected lane issues the tcgen05 instructions.  Issued from inside a
         // single-lane branch the same instructions sustain only ~83 cycles per MMA instead of 64.
         const bool leader = elect_one();
         const uint32_t idesc_pv = make_idesc((uint32_t)(d + 15) & ~15u) | (1u << 16);     // exact instances: N = head_dim
-        const uint32_t aQ = smem_u32(sQ), aKV = smem_u32(sKV);
-        const uint64_t dQ = make_desc(aQ, 16, 1024), dK = make_desc(aKV, 16, 1024), dV = make_desc(aKV, kKvBox, 1024);
-        auto issue_s = [&](int t, int st, int item) {
+        const uint32_t aQ = smem_u32(sQ), aK = smem_u32(sK), aV = smem_u32(sV);
+        const uint64_t dQ = make_desc(aQ, 16, 1024), dK = make_desc(aK, 16, 1024), dV = make_desc(aV, kKvBox, 1024);
+        auto issue_s = [&](int t, int st) {
             if (leader) {
-                const uint64_t q = dQ + (uint64_t)((2 * (item & 1) + (kHalves ? 1 : t)) * (kTileBytes >> 4));
 #pragma unroll
                 for (int ks = 0; ks < kBoxes * kBoxCols / 16; ++ks) {
-                    const uint32_t off_q = ((ks >> 2) * kBoxBytes + (ks & 3) * 32) >> 4, off_k = ((ks >> 2) * kKvBox + (ks & 3) * 32) >> 4;
+                    const uint32_t off_q = ((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4, off_k = ((ks >> 2) * kKvBox + (ks & 3) * 32) >> 4;
                     if (!kExact || 16 * ks < d)                  // columns beyond head_dim are zero in both tiles
-                    umma_ss(tmem_base + kColS + t * 128, q + off_q, dK + (uint64_t)(st * (kKvBytes >> 4) + off_k), make_idesc(kKeys), ks > 0);
-                }
-            }
-        };
-        // O_t (+)= P_t V: the chunks of 32 keys in the order in which the two warps of a row finish them
-        auto issue_pv = [&](int t, int st, uint32_t parity, bool first) {
-#pragma unroll
-            for (int q = 0; q < kParts; ++q) {
-                mbar_wait_call(p_full + 2 * t + q, parity, abort_flag, kp.status);
-                tc_fence_after();
-                if (leader) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int c = kParts * (i >> 1) + q, ks = 2 * c + (i & 1);          // chunk of 32 keys, 16 of them
-                        const uint64_t desc = dV + (uint64_t)(st * (kKvBytes >> 4) + ks * (2048 >> 4));
-                        const uint32_t acc = !first || q + i > 0, o = tmem_base + kColO + t * 128;
-                        if (kExact) {                            // 16 columns each of the first, second, third parts of a chunk
-                            const uint32_t a = tmem_base + kColS + t * 128 + 32 * c + 8 * (i & 1);
-                            const uint32_t a3 = tmem_base + kColP3 + t * 128 + 16 * c + 8 * (i & 1);
-                            umma_ts(o, a, desc, idesc_pv, acc);
-                            umma_ts(o, a + 16, desc, idesc_pv, 1);
-                            umma_ts(o, a3, desc, idesc_pv, 1);
-                        } else {
-                            umma_ts(o, tmem_base + kColS + t * 128 + 64 * (i >> 1) + 16 * q + 8 * (i & 1), desc, kIdescPV, acc);
-                        }
-                    }
+                    umma_ss(tmem_base + kColS + t * 128, dQ + (uint64_t)((kHalves ? 1 : t) * (kTileBytes >> 4) + off_q),
+                            dK + (uint64_t)(st * (kKvBytes >> 4) + off_k), make_idesc(kKeys), ks > 0);
                 }
             }
         };
         auto commit = [&](uint64_t *bar) { if (leader) tc_commit(bar); };
-        // k_st, k_ph: stage and phase of the ring's next tile; git / qn count the KV tiles / items of sub-tile 1,
-        // git0 / qn0 those of sub-tile 0, which may be missing or end earlier.
-        int k_st = 0, qn = 0, git = 0, git0 = 0, qn0 = 0;
-        uint32_t k_ph = 0;
-        auto advance = [&](int &st, uint32_t &ph) { if (++st == kStages) { st = 0; ph ^= 1; } };
-        int next1 = 0, next0 = 0, started = 0;                  // the next item's tiles, its sub-tiles whose first S is issued
-        bool have = false;                                      // the next item is known
+        // ring counts the KV tiles; git / qn the KV tiles / items of sub-tile 1, git0 / qn0 those of sub-tile 0, which
+        // may be missing or end earlier.
+        int ring = 0, git = 0, qn = 0, git0 = 0, qn0 = 0;
         for (;;) {
             // the producer decodes the work items; this warp only learns their shape (decoding them here as
             // well does not fit into this role's 64 registers)
-            if (!have) {
-                if (!mbar_wait_call(q_full + (qn & 1), (qn >> 1) & 1, abort_flag, kp.status)) break;
-                next1 = item_info[(qn & 1) * 2];
-                next0 = item_info[(qn & 1) * 2 + 1];
-            }
-            have = false;
-            const int n1 = next1, n0 = next0;
+            if (!mbar_wait_call(q_full, qn & 1, abort_flag, kp.status)) break;
+            const int n1 = item_info[(qn & 1) * 2];
             if (n1 < 0) break;
-            if constexpr (kHalves) {
-                // sub-tile 1 (tile 0) first; every tile serves one product
-                auto use = [&](auto products) {
-                    mbar_wait_call(kv_full + k_st, k_ph, abort_flag, kp.status);
-                    tc_fence_after();
-                    products();
-                    commit(kv_empty + k_st);
-                    advance(k_st, k_ph);
-                };
-                const int n = n0 + n1;
-                for (int tile = 0; tile < min(n, 2); ++tile) use([&]() { issue_s(1 - tile, k_st, qn); commit(s_full + 1 - tile); });
-                for (int tile = 0; tile < n; ++tile) {
-                    const int t = 1 - (tile & 1), j = tile >> 1;
-                    use([&]() {
-                        if (j == 0 && (t ? qn : qn0) > 0) mbar_wait_call(o_free + t, ((t ? qn : qn0) - 1) & 1, abort_flag, kp.status);
-                        issue_pv(t, k_st, ((t ? git : git0) + j) & 1, j == 0);
-                        commit(o_done + t);
-                    });
-                    if (tile + 2 < n) use([&]() { issue_s(t, k_st, qn); commit(s_full + t); });
+            const int n0 = item_info[(qn & 1) * 2 + 1];
+            const int n = kHalves ? n0 + n1 : n1;                // KV tiles of the item
+            // halves take the sub-tiles in the order of their tiles: 1 (tile 0) first
+            for (int i = kHalves || n0 > 0 ? 0 : 1; i < 2; ++i) {
+                const int t = kHalves ? 1 - i : i, tile = kHalves ? i : 0, st = (ring + tile) & 1;
+                if (kHalves && tile >= n) break;
+                mbar_wait_call(k_full + st, ((ring + tile) >> 1) & 1, abort_flag, kp.status);
+                tc_fence_after();
+                issue_s(t, st);
+                commit(s_full + t);
+                if (kHalves || t == 1) {
+                    commit(k_empty + st);
+                    if (tile == n - 1) commit(q_empty);          // last S of this item issued
                 }
-            } else {
-                if (!started) {                                  // (a started sub-tile's K may have left the ring already)
-                    mbar_wait_call(kv_full + k_st, k_ph, abort_flag, kp.status);
-                    tc_fence_after();
-                    if (n0 > 0) { issue_s(0, k_st, qn); commit(s_full + 0); }
-                }
-                if (!(started & 2)) { issue_s(1, k_st, qn); commit(s_full + 1); commit(kv_empty + k_st); }
-                started = 0;
-                advance(k_st, k_ph);
-                for (int j = 0; j < n1; ++j) {
-                    const int v_st = k_st;                       // V of tile j, then K of tile j + 1 or of the next item
-                    const uint32_t v_ph = k_ph;
-                    advance(k_st, k_ph);
-                    for (int t = j < n0 ? 0 : 1; t < 2; ++t) {
-                        const int gsub = (t ? git : git0) + j, qsub = t ? qn : qn0;
-                        const bool first = t == 0 || j >= n0;    // (sub-tile 1 of a shared tile: sub-tile 0 has waited for it)
-                        if (first) mbar_wait_call(kv_full + v_st, v_ph, abort_flag, kp.status);
-                        if (j == 0 && qsub > 0) mbar_wait_call(o_free + t, (qsub - 1) & 1, abort_flag, kp.status);
-                        issue_pv(t, v_st, gsub & 1, j == 0);
-                        commit(o_done + t);
-                        if (t == 1) commit(kv_empty + v_st);
-                        if (j + 1 < (t ? n1 : n0)) {
-                            if (first || j + 1 >= n0) mbar_wait_call(kv_full + k_st, k_ph, abort_flag, kp.status);
-                            tc_fence_after();
-                            issue_s(t, k_st, qn);
-                            commit(s_full + t);
-                            if (t == 1) commit(kv_empty + k_st);
-                        } else if (j + 1 == n1) {
-                            // the next item's first S of this sub-tile, if nothing has to be waited for
-                            const int nx = qn + 1;
-                            if (!have && __all_sync(0xffffffffu, mbar_test_wait(q_full + (nx & 1), (nx >> 1) & 1))) {
-                                have = true;
-                                next1 = item_info[(nx & 1) * 2];
-                                next0 = item_info[(nx & 1) * 2 + 1];
-                            }
-                            if (have && next1 > 0 && (t == 0 ? next0 > 0 : next0 == 0 || started == 1) &&
-                                __all_sync(0xffffffffu, mbar_test_wait(kv_full + k_st, k_ph))) {
-                                tc_fence_after();
-                                issue_s(t, k_st, nx);
-                                commit(s_full + t);
-                                if (t == 1) commit(kv_empty + k_st);
-                                started |= 1 << t;
+            }
+            for (int j = 0; j < n1; ++j) {
+                for (int i = kHalves || j < n0 ? 0 : 1; i < 2; ++i) {
+                    const int t = kHalves ? 1 - i : i;
+                    if (kHalves && t == 0 && j >= n0) break;
+                    const int tile = kHalves ? 2 * j + i : j;
+                    const int gt = ring + tile, st = gt & 1, ph = (gt >> 1) & 1;
+                    const int gsub = (t ? git : git0) + j, qsub = t ? qn : qn0;
+                    // (sub-tile 1 of a shared tile: sub-tile 0 has waited for it)
+                    if (kHalves || t == 0 || j >= n0) mbar_wait_call(v_full + st, ph, abort_flag, kp.status);
+                    if (j == 0 && qsub > 0) mbar_wait_call(o_free + t, (qsub - 1) & 1, abort_flag, kp.status);
+#pragma unroll
+                    for (int q = 0; q < kSplit; ++q) {
+                        mbar_wait_call(p_full + kSplit * t + q, gsub & 1, abort_flag, kp.status);
+                        if (lane == 0 && q == 0) TRACE(j, 2 + t);
+                        tc_fence_after();
+                        if (leader) {
+#pragma unroll
+                            for (int kk = 0; kk < kPartKeys / 16; ++kk) {
+                                const int ks = q * (kPartKeys / 16) + kk;
+                                const uint64_t desc = dV + (uint64_t)(st * (kKvBytes >> 4) + ks * (2048 >> 4));
+                                if (kExact) {                    // chunk of 32 keys: 16 columns each of the first, second, third parts
+                                    const uint32_t a = tmem_base + kColS + t * 128 + 32 * (ks >> 1) + 8 * (ks & 1);
+                                    const uint32_t a3 = tmem_base + kColP3 + t * 128 + 16 * (ks >> 1) + 8 * (ks & 1);
+                                    umma_ts(tmem_base + kColO + t * 128, a, desc, idesc_pv, (j > 0 || ks > 0));
+                                    umma_ts(tmem_base + kColO + t * 128, a + 16, desc, idesc_pv, 1);
+                                    umma_ts(tmem_base + kColO + t * 128, a3, desc, idesc_pv, 1);
+                                } else {
+                                    umma_ts(tmem_base + kColO + t * 128, tmem_base + kColS + t * 128 + q * kPartKeys + kk * 8, desc,
+                                            kIdescPV, (j > 0 || ks > 0));
+                                }
                             }
                         }
                     }
-                    if (j + 1 < n1) advance(k_st, k_ph);
+                    commit(o_done + t);
+                    if (kHalves || t == 1) commit(v_empty + st);
+                    if (j + 1 < (t ? n1 : n0)) {
+                        const int next = tile + (kHalves ? 2 : 1), st1 = (ring + next) & 1;
+                        if (kHalves || t == 0 || j + 1 >= n0)
+                            mbar_wait_call(k_full + st1, ((ring + next) >> 1) & 1, abort_flag, kp.status);
+                        issue_s(t, st1);
+                        commit(s_full + t);
+                        if (kHalves || t == 1) {
+                            commit(k_empty + st1);
+                            if (next == n - 1) commit(q_empty);
+                        }
+                    }
+                    if (t == 1 && lane == 0) TRACE(j, 4);
                 }
             }
+            ring += n;
             git += n1;
             ++qn;
             if (n0 > 0) { git0 += n0; ++qn0; }
         }
-    } else if (warp >= kSoftmaxWarps) {
+    } else if (warp >= 4 * kSplit) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs));      // the two idle warps of that warpgroup
         // One of them checks what the prefix-count mask relies on: key positions that never decrease
         // along the aggregated rows of a head.  The CTAs share the pairs (i, i + 1) among them.
@@ -950,76 +930,67 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSoftmaxRegs));
         // ================= softmax + epilogue =================
-        // Two warpgroups serve a sub-tile (one query head of one query tile): thread = query row r = TMEM lane; warpgroup
-        // h has the keys kMyKeys h .. of every tile and half of the row's output channels.  The two warps of a row
-        // (same scheduler, same TMEM lanes) meet once per tile, to exchange their row maxima.
-        const int t = warp >> 3, h = (warp >> 2) & 1;           // sub-tile and half of this warpgroup
+        // Warpgroup t serves sub-tile t (one query head of one query tile) on its own: thread = query row r = TMEM lane,
+        // all key columns of the S tile, the whole row of O.  During the walk the two warpgroups never meet (those of a
+        // halved item do in the epilogue): no row maximum or row sum has to be exchanged, and while one is in the
+        // serial part of its visit (wait, TMEM load, maximum) the other computes.  A thread reads its row of S from TMEM once and keeps
+        // its values in registers for both walks (maximum, then exponentials).
+        const int t = warp >> 2;                                // sub-tile of this warpgroup
         const int r = tid & 127;                                // query row = TMEM lane
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        const uint32_t tS = tmem_base + lane_base + kColS + t * 128 + kMyKeys * h;     // fp32 S; bf16 P over it
-        const uint32_t tP3 = tmem_base + lane_base + kColP3 + t * 128 + 16 * kParts * h;
+        const uint32_t tS = tmem_base + lane_base + kColS + t * 128;   // fp32 S; bf16 P of keys 64q.. at column 64q
         const uint32_t tO = tmem_base + lane_base + kColO + t * 128;
-        float *val_mine = row_val + (2 * t + h) * 128 + r;
-        const float *val_other = row_val + (2 * t + 1 - h) * 128 + r;
-        uint64_t *met = row_met + 4 * t + (warp & 3);
         const float sl2 = kExact ? kp.sl2 : p.scale * 1.4426950408889634f;
         const uint64_t sl2_2 = pack_f32x2(sl2, sl2);
         int gsub = 0;                                           // KV tiles this sub-tile has been through
-        int n_row_met = 0, n_halves_met = 0;                    // phases of `met`, of `halves_met` so far
         auto below32 = [](int n) -> uint32_t { return n <= 0 ? 0u : (n >= 32 ? 0xffffffffu : (1u << n) - 1u); };
-        // the value that the other warp of these rows left
-        auto exchange = [&](float mine) -> float {
-            *val_mine = mine;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(met);
-            mbar_wait(met, n_row_met & 1, abort_flag, kp.status);
-            ++n_row_met;
-            return *val_other;
-        };
 
-        // One visit = the softmax of this warpgroup's half of one S tile.  kPartial: some row of the warp has masked columns;
-        // bit i of vm[c] says whether column 32 c + i of the half is visible to this thread's row.  Masked columns become -inf and
+        // One visit = the softmax of one S tile.  kPartial: some row of the tile has masked columns; bit i of
+        // vm[c] says whether column 32 c + i is visible to this thread's row.  Masked columns become -inf and
         // every exponential goes through ex2.approx, which maps -inf to 0; in unmasked tiles a fixed subset of
         // the columns takes the polynomial so that the ex2 unit is not the bottleneck.
         // kAnyFirst: the tile in which a row sees its first key may be any of the walk (explicit positions).
         constexpr bool kAnyFirst = kSpecial || kExact;
-        auto visit = [&](auto partial_tag, int j, int gt, const uint32_t (&vm)[2], float &m_used, float &l) {
+        auto visit = [&](auto partial_tag, int j, int gt, const uint32_t (&vm)[4], float &m_used, float &l) {
             constexpr bool kPartial = decltype(partial_tag)::value;
             mbar_wait(s_full + t, gt & 1, abort_flag, kp.status);
+            if (tid == 0) TRACE(j, t ? 5 : 0);
             tc_fence_after();
-            // this half of the row of S in registers: read from TMEM once, used for the maximum and the exponentials
-            uint32_t s0[32], s1[32];
-            float mx[4];
+            // the whole row of S in registers: read from TMEM once, used for the maximum and the exponentials
+            uint32_t s0[32], s1[32], s2[32], s3[32];
+            float mx[8];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) mx[i] = -INFINITY;
+            for (int i = 0; i < 8; ++i) mx[i] = -INFINITY;
             FEDATTN_TMEM_LD32(tS, s0);
+            FEDATTN_TMEM_LD32(tS + 32, s1);
             tmem_wait_ld();
-            if (kParts == 2) FEDATTN_TMEM_LD32(tS + 32, s1);
+            if (kChunks == 4) {
+                FEDATTN_TMEM_LD32(tS + 64, s2);
+                FEDATTN_TMEM_LD32(tS + 96, s3);
+            }
 #pragma unroll
-            for (int c = 0; c < kParts; ++c) {
-                uint32_t *cur = c == 0 ? s0 : s1;
-                if (c == 1) tmem_wait_ld();
+            for (int c = 0; c < kChunks; ++c) {
+                uint32_t *cur = c == 0 ? s0 : (c == 1 ? s1 : (c == 2 ? s2 : s3));
+                if (c == 2) tmem_wait_ld();
                 if (kPartial) {
 #pragma unroll
                     for (int i = 0; i < 32; ++i)
                         if (!((vm[c] >> i) & 1u)) cur[i] = 0xff800000u;          // -inf
                 }
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    mx[i & 3] = max3(mx[i & 3], __uint_as_float(cur[2 * i]), __uint_as_float(cur[2 * i + 1]));
+                for (int i = 0; i < 8; ++i) {
+                    mx[i] = max3(mx[i], __uint_as_float(cur[2 * i]), __uint_as_float(cur[2 * i + 1]));
+                    mx[i] = max3(mx[i], __uint_as_float(cur[16 + 2 * i]), __uint_as_float(cur[16 + 2 * i + 1]));
+                }
             }
-            // (the other warp has read what this one left before an item's first tile; later it has behind its weights of the
-            // tile before, without which there is no S)
-            if (j == 0 && n_row_met > 0) mbar_wait(met, (n_row_met - 1) & 1, abort_flag, kp.status);
-            const float half_max = max3(mx[0], mx[1], fmaxf(mx[2], mx[3]));
-            const float t_max = fmaxf(half_max, exchange(half_max)) * sl2;
+            const float rm = fmaxf(max3(mx[0], mx[1], mx[2]), fmaxf(max3(mx[3], mx[4], mx[5]), fmaxf(mx[6], mx[7])));
+            const float t_max = rm * sl2;
             if (j == 0) {
                 // (a row of a prefix mask that sees nothing of its first tile sees nothing at all)
                 m_used = (!kAnyFirst && t_max == -INFINITY) ? 0.f : t_max;
             } else {
                 // The exponent reference moves only when the maximum grew by more than 2^8; then what
-                // this row has accumulated so far (O in TMEM, l) is rescaled to the new reference: each warp's half of it.
-                // (PV starts behind the weights of both warps.)
+                // this row has accumulated so far (O in TMEM, l) is rescaled to the new reference.
                 const bool need = t_max > m_used + kRescaleThreshold;
                 if (__any_sync(0xffffffffu, need)) {
                     const float alpha = need ? ex2(m_used - t_max) : 1.f;
@@ -1027,12 +998,12 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     tc_fence_after();
 #pragma unroll 1
                     for (int oc = 0; oc < 2 * kBoxes; ++oc) {
-                        uint32_t o[16];
-                        FEDATTN_TMEM_LD16(tO + 32 * kBoxes * h + oc * 16, o);
+                        uint32_t o[32];
+                        FEDATTN_TMEM_LD32(tO + oc * 32, o);
                         tmem_wait_ld();
 #pragma unroll
-                        for (int c = 0; c < 16; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * alpha);
-                        FEDATTN_TMEM_ST16(tO + 32 * kBoxes * h + oc * 16, o);
+                        for (int c = 0; c < 32; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * alpha);
+                        FEDATTN_TMEM_ST32(tO + oc * 32, o);
                     }
                     if (need) { l *= alpha; m_used = t_max; }
                 }
@@ -1041,10 +1012,10 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             // (a row that has seen no key yet keeps the reference -inf, all its weights are 0)
             const float m_ref = kAnyFirst && m_used == -INFINITY ? 0.f : m_used;
             const uint64_t negm2 = pack_f32x2(-m_ref, -m_ref);
-            uint64_t sum2[2] = {0, 0};
+            uint64_t sum2[4] = {0, 0, 0, 0};
 #pragma unroll
-            for (int c = 0; c < kParts; ++c) {
-                uint32_t *cur = c == 0 ? s0 : s1;
+            for (int c = 0; c < kChunks; ++c) {
+                uint32_t *cur = c == 0 ? s0 : (c == 1 ? s1 : (c == 2 ? s2 : s3));
                 uint32_t pk[16];
                 // Exact instances: the leading 8 bits of the values in cur as bf16 pairs; what is left stays in cur.  Three
                 // times that is a weight's 24 bits.
@@ -1071,47 +1042,44 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                         unpack_f32x2(x2, x0, x1);
                         p0 = ex2(x0); p1 = ex2(x1);
                     }
-                    sum2[i & 1] = add_f32x2(sum2[i & 1], pack_f32x2(p0, p1));
+                    sum2[i & 3] = add_f32x2(sum2[i & 3], pack_f32x2(p0, p1));
                     if (kExact) { cur[2 * i] = __float_as_uint(p0); cur[2 * i + 1] = __float_as_uint(p1); }
                     else pk[i] = pack_bf16(p0, p1);
                 }
-                // bf16 pairs of the chunk's 32 keys, inside S columns that this thread has already read
+                // keys 32 c .. 32 c + 31 as bf16 pairs: columns 64 (c / 2) + 16 (c % 2) .., all inside S columns
+                // that this thread has already read
                 if (kExact) {
                     take_part(false);
                     FEDATTN_TMEM_ST16(tS + 32 * c, pk);
                     take_part(false);
                     FEDATTN_TMEM_ST16(tS + 32 * c + 16, pk);
                     take_part(true);
-                    FEDATTN_TMEM_ST16(tP3 + 16 * c, pk);
+                    FEDATTN_TMEM_ST16(tmem_base + lane_base + kColP3 + t * 128 + 16 * c, pk);
                 } else {
-                    FEDATTN_TMEM_ST16(tS + 16 * c, pk);
+                    FEDATTN_TMEM_ST16(tS + 64 * (c >> 1) + 16 * (c & 1), pk);
                 }
-                tmem_wait_st();                                 // PV may start on the chunks c of both halves
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(p_full + 2 * t + c);         // one arrival per warp
+                if ((32 * c + 32) % kPartKeys == 0) {           // a half of P is complete: PV may start on it
+                    tmem_wait_st();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(p_full + kSplit * t + 32 * c / kPartKeys);       // one arrival per warp
+                }
             }
             float r0, r1;
-            unpack_f32x2(add_f32x2(sum2[0], sum2[1]), r0, r1);
+            unpack_f32x2(add_f32x2(add_f32x2(sum2[0], sum2[1]), add_f32x2(sum2[2], sum2[3])), r0, r1);
             l += r0 + r1;
+            if (tid == 0) TRACE(j, t ? 6 : 1);
         };
 
-        int pn = 0, qn = 0;                                     // items read from the producer's slots, non-empty ones
-        bool staged = false;                                    // the Q slot of item qn - 1 is still to be given back
-        auto give_q_back = [&]() {
-            if (staged && lane == 0) {
-                tma_store_wait_read();                          // the output has left it
-                mbar_arrive(q_empty + ((qn - 1) & 1));
-            }
-            staged = false;
-        };
+        int pn = 0;                                             // items read from the producer's slots
+        int n_met = 0;                                          // halves: items merged so far
         for (int k = 0; k < n_rounds; ++k) {
             const int item = item_of(k);
             if (item >= n_items) continue;
             Item it;
             Sub sub;
             bool listed = false;                                // the walk is a list of tiles, not a prefix
-            bool halved = false;                                // the other sub-tile's warps walk the other KV tiles of these rows
+            bool halved = false;                                // the other warpgroup walks the other KV tiles of these rows
             {
                 const bool ok = mbar_wait(item_full + (pn & 1), (pn >> 1) & 1, abort_flag, kp.status);
                 if (!__all_sync(0xffffffffu, ok)) break;        // nothing is published any more
@@ -1122,27 +1090,22 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 sub.n_tiles = slot[11 + 4 * t];
                 halved = kHalves && slot[11] > 0;
                 it.kvp = p.kv_pos ? p.kv_pos + (p.kv_head_major ? (int64_t)it.kvh * p.total_kv : 0) : nullptr;
-                const bool loaded = slot[15] > 0;               // the item has a Q slot
                 __syncwarp();
                 // (a listed walk is read as it goes: the slot is given back behind it)
                 listed = kSpecial && !kExact && p.general && it.b < 0;
                 if (lane == 0 && !listed) mbar_arrive(item_empty + (pn & 1));
                 ++pn;
-                if (sub.n_tiles == 0) {                         // no part in it
-                    give_q_back();
-                    if (loaded && lane == 0) mbar_arrive(q_empty + (qn & 1));
-                    qn += loaded;
-                }
             }
             const int n_tiles = sub.n_tiles;
             const bool valid = r < sub.n_valid;
+            __nv_bfloat16 *orow = reinterpret_cast<__nv_bfloat16 *>(p.o) + ((int64_t)(sub.q_row0 + r) * p.hq + sub.head) * d;
+            float *lse_p = p.lse ? p.lse + (int64_t)(sub.q_row0 + r) * p.hq + sub.head : nullptr;
             const bool general = kSpecial && !kExact && p.general;
             if (n_tiles == 0 && listed && lane == 0) mbar_arrive(item_empty + ((pn - 1) & 1));
             if (n_tiles == 0) {                                 // nothing visible to any row of the tile, or no rows
                 if (valid) {
-                    __nv_bfloat16 *orow = reinterpret_cast<__nv_bfloat16 *>(p.o) + ((int64_t)(sub.q_row0 + r) * p.hq + sub.head) * d;
-                    for (int c = 8 * h; c < d; c += 16) *reinterpret_cast<uint4 *>(orow + c) = make_uint4(0, 0, 0, 0);
-                    if (p.lse && h == 0) p.lse[(int64_t)(sub.q_row0 + r) * p.hq + sub.head] = -INFINITY;
+                    for (int c = 0; c < d; c += 8) *reinterpret_cast<uint4 *>(orow + c) = make_uint4(0, 0, 0, 0);
+                    if (lse_p) *lse_p = -INFINITY;
                 }
                 continue;
             }
@@ -1150,12 +1113,12 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             const bool pairs = kExact && kp.pairs;
             int c_row = 0, n_full = 0, p_row = 0;
             PairRule mine{0, 0, false}, all{0, 0, false};       // pairs: this row's rule, and what every row of the warp sees
-            int kpos[2] = {0, 0};                               // pairs: positions of keys 32 c + lane of the half tile at hand
+            int kpos[4] = {0, 0, 0, 0};                         // pairs: positions of keys 32 c + lane of the tile at hand
             auto load_pos = [&](int j) {
                 const int T = (int)p.total_kv;
 #pragma unroll
-                for (int c = 0; c < kParts; ++c) {
-                    const int key = j * kKeys + kMyKeys * h + 32 * c + lane;
+                for (int c = 0; c < kChunks; ++c) {
+                    const int key = j * kKeys + 32 * c + lane;
                     kpos[c] = it.kvp ? __ldg(it.kvp + min(key, T - 1)) : key;
                 }
             };
@@ -1189,8 +1152,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 }
                 // prefix lengths do not decrease with the row, so KV tiles below the prefix of the warp's first
                 // row are unmasked for the whole warp (the choice of code path only has to be warp-uniform)
-                const int beyond = __shfl_sync(0xffffffffu, c_row, 0) - kMyKeys * (h + 1);
-                n_full = beyond < 0 ? 0 : beyond / kKeys + 1;   // tiles whose half of this warp lies in that prefix
+                n_full = __shfl_sync(0xffffffffu, c_row, 0) / kKeys;
             }
             const int T = (int)p.total_kv;
             float m_run = 0.f, l_run = 0.f;
@@ -1201,19 +1163,19 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     entry = reinterpret_cast<const volatile uint16_t *>(walks)[((pn - 1) & 1) * kWalkMost + tile];
                     tile = entry & 0x7fff;
                 }
-                // which of its columns of this tile the thread's row sees: everything (warp-uniform), or a mask per chunk
+                // which columns of this tile the thread's row sees: everything (warp-uniform), or a mask per chunk
                 bool full;
-                uint32_t vm[2] = {0, 0};
+                uint32_t vm[4] = {0, 0, 0, 0};
                 if (pairs) {
-                    // column 32 c + i of the half is its key 32 c + i, whose position lane i holds
-                    const int k0 = tile * kKeys + kMyKeys * h;
+                    // column 32 c + i of the tile is its key 32 c + i, whose position lane i holds
+                    const int k0 = tile * kKeys;
                     bool see_all = true;
 #pragma unroll
-                    for (int c = 0; c < kParts; ++c) see_all = see_all && k0 + 32 * c + lane < T && all.sees(kpos[c]);
+                    for (int c = 0; c < kChunks; ++c) see_all = see_all && k0 + 32 * c + lane < T && all.sees(kpos[c]);
                     full = __all_sync(0xffffffffu, see_all);
                     if (!full) {
 #pragma unroll
-                        for (int c = 0; c < kParts; ++c) {
+                        for (int c = 0; c < kChunks; ++c) {
                             uint32_t m = 0;
 #pragma unroll 4
                             for (int i = 0; i < 32; ++i)
@@ -1223,11 +1185,11 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     }
                     if (j + 1 < n_tiles) load_pos(tile + (kHalves ? 2 : 1));        // lands during this tile's visit
                 } else if (two_range) {                         // keys [0, a) and [b, T)
-                    const int k0 = tile_of(it, tile) * kKeys + kMyKeys * h;         // the half's first key
-                    full = k0 + kMyKeys <= it.a || (k0 >= it.b && k0 + kMyKeys <= T);
+                    const int k0 = tile_of(it, tile) * kKeys;   // first key of the tile
+                    full = k0 + kKeys <= it.a || (k0 >= it.b && k0 + kKeys <= T);
                     if (!full) {
 #pragma unroll
-                        for (int c = 0; c < kParts; ++c) {
+                        for (int c = 0; c < kChunks; ++c) {
                             const int cb = k0 + 32 * c;
                             vm[c] = below32(it.a - cb) | (below32(T - cb) & ~below32(it.b - cb));
                         }
@@ -1238,8 +1200,8 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                         // column i of chunk c is key cb + i: visible iff it exists and its position is not above
                         // the row's.  The address is the same in every lane: broadcast loads.
 #pragma unroll
-                        for (int c = 0; c < kParts; ++c) {
-                            const int cb = tile * kKeys + kMyKeys * h + 32 * c;
+                        for (int c = 0; c < kChunks; ++c) {
+                            const int cb = tile * kKeys + 32 * c;
                             uint32_t m = 0;
 #pragma unroll 4
                             for (int i = 0; i < 32; ++i) {
@@ -1251,12 +1213,11 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                         }
                     } else if (!full) {
 #pragma unroll
-                        for (int c = 0; c < kParts; ++c) vm[c] = below32(c_row - tile * kKeys - kMyKeys * h - 32 * c);
+                        for (int c = 0; c < kChunks; ++c) vm[c] = below32(c_row - tile * kKeys - 32 * c);
                     }
                 }
                 if (full) visit(std::false_type{}, j, gt, vm, m_run, l_run);
                 else visit(std::true_type{}, j, gt, vm, m_run, l_run);
-                if (j == 0) give_q_back();
             }
 
             if (listed) {
@@ -1266,53 +1227,39 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 
             // The first key a row sees weighs 1 but for the rounding of its reference.  Where a unit of the reference is
             // worth more than its weight (logits beyond 2^24) the row is one for the routine below.
-            auto sound = [](float m, float l) { return m != -INFINITY && !(l >= 0.25f) ? __int_as_float(0x7fc00000) /* NaN */ : l; };
+            if (kExact && m_run != -INFINITY && !(l_run >= 0.25f)) l_run = __int_as_float(0x7fc00000);       // NaN
 
             // ---- epilogue: drain this row of O from TMEM (frees it for the next item), O / l -> bf16 -> global
             mbar_wait(o_done + t, (gsub + n_tiles - 1) & 1, abort_flag, kp.status);
             tc_fence_after();
-            // The item's Q is dead: its slot takes the output.  A warp stages kOutCols columns of its 32 rows at a time
-            // (halves, one box: 32 columns in 64-byte rows, so that every warp has boxes of its own).
-            constexpr int kOutCols = kHalves || kBoxes == 1 ? 32 : 64;
-            uint8_t *q_slot = sQ + (qn & 1) * 2 * kTileBytes;
-            uint8_t *my_stage = q_slot + t * kTileBytes + (4 * h + (warp & 3)) * (kTileBytes / 8);
-            // Halves: the four threads of a row hold its two partials.  They read both accumulators (a quarter of the columns
-            // each; one box: sub-tile 1's warps a half) and weigh them by w0 and w1; otherwise w = 1 / l weighs the own one.
+            // Halves: this thread and the one with the same row in the other warpgroup hold the two partials of the row.
+            // Both read both accumulators (each half of the columns; one box: sub-tile 1's warps all of them) and
+            // weigh them by w0 and w1; otherwise w = 1 / l weighs the own accumulator.
             float w0 = 0.f, w1 = 0.f;
             if (kHalves && halved) {
-                // (sub-tile 0's Q is not used, its half of the slot has room behind what a warp stages)
-                float *xch = reinterpret_cast<float *>(q_slot + (warp & 3) * (kTileBytes / 8) + kTileBytes / 16) + 8 * lane;
-                if (h == 0) xch[t] = m_run;
-                xch[2 + 2 * t + h] = l_run;
+                // (sub-tile 0's Q buffer is not used; two slots: a warp that is an item ahead finds the other one, and it
+                // gets no further before every warp has arrived there, behind its reads of this one)
+                float2 *xch = reinterpret_cast<float2 *>(sQ) + (n_met & 1) * 256;
+                const float m_mine = l_run == 0.f ? -INFINITY : m_run;
+                xch[t * 128 + r] = make_float2(m_mine, l_run);
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(halves_met);
-                mbar_wait(halves_met, n_halves_met & 1, abort_flag, kp.status);
+                mbar_wait(halves_met, n_met & 1, abort_flag, kp.status);
                 tc_fence_after();
-                ++n_halves_met;
-                // all warps add in the same order: they hold the same row sum to the last bit
-                float l0 = xch[2] + xch[3], l1 = xch[4] + xch[5];
-                if (kExact) { l0 = sound(xch[0], l0); l1 = sound(xch[1], l1); }
-                const float m0 = l0 == 0.f ? -INFINITY : xch[0], m1 = l1 == 0.f ? -INFINITY : xch[1];
-                m_run = fmaxf(m0, m1);
-                const float ref = m_run == -INFINITY ? 0.f : m_run, f0 = ex2(m0 - ref), f1 = ex2(m1 - ref);
-                l_run = l0 * f0 + l1 * f1;
+                ++n_met;
+                // both warpgroups add in the same order: they hold the same row sum to the last bit
+                const float2 ml0 = xch[r], ml1 = xch[128 + r];
+                m_run = fmaxf(ml0.x, ml1.x);
+                const float ref = m_run == -INFINITY ? 0.f : m_run, f0 = ex2(ml0.x - ref), f1 = ex2(ml1.x - ref);
+                l_run = ml0.y * f0 + ml1.y * f1;
                 const float inv_l = l_run > 0.f ? 1.f / l_run : 0.f;
                 w0 = f0 * inv_l;
                 w1 = f1 * inv_l;
-            } else {
-                // the sums of the row's halves (the maxima of the last tile have been read: its PV is done)
-                const float other = exchange(l_run);
-                l_run += other;
-                if (kExact) l_run = sound(m_run, l_run);
-                __syncwarp();
-                if (lane == 0) mbar_arrive(met);                // read: waited for before the next value is left
-                ++n_row_met;
             }
             const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
-            // 32-column chunks of this thread
-            const int c_lo = kHalves && halved ? (kBoxes == 2 ? 2 * t + h : h) : kBoxes * h;
-            const int c_hi = kHalves && halved ? (kBoxes == 2 || t == 1 ? c_lo + 1 : c_lo) : c_lo + kBoxes;
+            const int c_lo = kHalves && halved && kBoxes == 2 ? 2 * t : 0;                  // 32-column chunks of this thread
+            const int c_hi = kHalves && halved ? (kBoxes == 2 ? c_lo + 2 : 2 * t) : 2 * kBoxes;
             // chunk c of the row, normalised
             auto load_o = [&](int c, uint32_t (&o)[32]) {
                 if (kHalves && halved) {
@@ -1331,7 +1278,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 }
             };
             // this warp has read what it needs of O: one arrival per warp lets the accumulator be overwritten (halves: of
-            // both, or, where the other sub-tile has no part in the item, its share too)
+            // both, or, where the other warpgroup has no part in the item, its share too)
             auto release_o = [&]() {
                 tc_fence_before();
                 __syncwarp();
@@ -1340,13 +1287,13 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     if (kHalves) mbar_arrive(o_free + (halved ? 1 - t : t));
                 }
             };
-            // Full warps of rows leave through shared memory and TMA stores; a warp with rows beyond the segment writes its
-            // valid rows directly.
+            // Full warps of rows leave through shared memory and TMA stores (a warp's 32 rows x 64 columns at a
+            // time); a warp with rows beyond the segment writes its valid rows directly.
             bool by_tma = kp.o_tma && (r | 31) < sub.n_valid;
             uint32_t bad = 0;                                   // exact instances: rows of the warp with a non-finite channel
             if (kExact) {
                 float probe = l_run * 0.f;                      // 0 unless something is Inf or NaN
-                // (all columns, so that all warps of a row find the same)
+                // (halves: all columns, so that both warpgroups find the same rows)
 #pragma unroll 1
                 for (int c = 0; c < 2 * kBoxes && 32 * c < d; ++c) {
                     uint32_t o[32];
@@ -1358,36 +1305,71 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 bad = __ballot_sync(0xffffffffu, valid && !(probe == 0.f));
                 by_tma = by_tma && bad == 0;
             }
-            auto pack4 = [](const uint32_t (&o)[32], int u) -> uint4 {
-                uint32_t w[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) w[i] = pack_bf16(__uint_as_float(o[8 * u + 2 * i]), __uint_as_float(o[8 * u + 2 * i + 1]));
-                return make_uint4(w[0], w[1], w[2], w[3]);
-            };
-            if (by_tma) {
-                const int row0 = sub.q_row0 + (r & ~31);
-#pragma unroll
-                for (int i = 0; i < kBoxes; ++i) {
-                    const int c = c_lo + i;
-                    if (kHalves && c >= c_hi) break;
+            uint8_t *my_stage = stage + (size_t)warp * kStageBytes;
+            if (kHalves && by_tma) {
+                // one box of 64 columns per warp at a time; short items, so the code stays short
+                if (lane == 0) tma_store_wait_read();
+                __syncwarp();
+#pragma unroll 1
+                for (int c = c_lo; c < c_hi; ++c) {
                     uint32_t o[32];
                     load_o(c, o);
-                    if (kHalves ? c == c_hi - 1 : i == kBoxes - 1) release_o();
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {               // 16-byte units of the row's staged bytes, swizzled
-                        if (kOutCols == 64) *reinterpret_cast<uint4 *>(my_stage + lane * 128 + (((4 * (i & 1) + u) ^ (lane & 7)) << 4)) = pack4(o, u);
-                        else *reinterpret_cast<uint4 *>(my_stage + i * 2048 + lane * 64 + ((u ^ ((lane >> 1) & 3)) << 4)) = pack4(o, u);
+                    if (c == c_hi - 1) release_o();
+                    if (c == c_lo + 2) {                        // the first box's store has read the staging rows
+                        if (lane == 0) tma_store_wait_read();
+                        __syncwarp();
                     }
-                    if (kOutCols == 32 || i == kBoxes - 1) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        uint32_t w[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            w[i] = pack_bf16(__uint_as_float(o[8 * u + 2 * i]), __uint_as_float(o[8 * u + 2 * i + 1]));
+                        const int unit = 4 * (c & 1) + u;
+                        *reinterpret_cast<uint4 *>(my_stage + lane * 128 + ((unit ^ (lane & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+                    }
+                    if (c & 1) {
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         __syncwarp();
-                        if (lane == 0) {
-                            if (kOutCols == 64) tma_store_3d(&map_o, my_stage, 64 * h, sub.head, row0);
-                            else if (32 * c < d) tma_store_3d(&map_o, my_stage + i * 2048, 32 * c, sub.head, row0);
-                        }
+                        if (lane == 0) tma_store_3d(&map_o, my_stage, 64 * (c >> 1), sub.head, sub.q_row0 + (r & ~31));
                     }
                 }
-                if (kHalves && c_lo == c_hi) release_o();
+                if (c_lo == c_hi) release_o();
+            } else if (by_tma) {
+                if (lane == 0) tma_store_wait_read();           // the previous item's last store has read the staging rows
+                __syncwarp();
+                uint32_t oa[32], ob[32];
+                FEDATTN_TMEM_LD32(tO, oa);
+#pragma unroll
+                for (int c = 0; c < 2 * kBoxes; ++c) {
+                    uint32_t *cur = (c & 1) ? ob : oa, *nxt = (c & 1) ? oa : ob;
+                    tmem_wait_ld();
+                    if (c < 2 * kBoxes - 1) {
+                        FEDATTN_TMEM_LD32(tO + 32 * (c + 1), nxt);
+                    } else {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(o_free + t); // one arrival per warp: O_t may be overwritten
+                    }
+                    if (c == 2) {                               // the first half's store has read the staging rows
+                        if (lane == 0) tma_store_wait_read();
+                        __syncwarp();
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {               // 16-byte unit 4 (c & 1) + u of the row's 128 staged bytes
+                        uint32_t w[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            w[i] = pack_bf16(__uint_as_float(cur[8 * u + 2 * i]) * inv, __uint_as_float(cur[8 * u + 2 * i + 1]) * inv);
+                        const int unit = 4 * (c & 1) + u;
+                        *reinterpret_cast<uint4 *>(my_stage + lane * 128 + ((unit ^ (lane & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+                    }
+                    if (c & 1) {
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) tma_store_3d(&map_o, my_stage, 64 * (c >> 1), sub.head, sub.q_row0 + (r & ~31));
+                    }
+                }
             } else {
                 // the rare path (a warp with rows beyond the segment) is kept short rather than fast
 #pragma unroll 1
@@ -1396,22 +1378,25 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     load_o(c, o);
                     if (c == c_hi - 1) release_o();
                     if (valid && !((bad >> lane) & 1u)) {
-                        __nv_bfloat16 *orow = reinterpret_cast<__nv_bfloat16 *>(p.o) + ((int64_t)(sub.q_row0 + r) * p.hq + sub.head) * d;
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
                             if (kExact && 32 * c + 8 * u >= d) break;
-                            *reinterpret_cast<uint4 *>(orow + 32 * c + 8 * u) = pack4(o, u);
+                            uint32_t w[4];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+                                w[i] = pack_bf16(__uint_as_float(o[8 * u + 2 * i]), __uint_as_float(o[8 * u + 2 * i + 1]));
+                            *reinterpret_cast<uint4 *>(orow + 32 * c + 8 * u) = make_uint4(w[0], w[1], w[2], w[3]);
                         }
                     }
                 }
                 if (kHalves && c_lo == c_hi) release_o();
             }
-            // (one of the row's threads writes it; halves: of sub-tile 1, which has a part in every item)
-            const bool writer = h == 0 && !(kHalves && halved && t == 0);
-            if (valid && p.lse && writer && !((bad >> lane) & 1u))
-                p.lse[(int64_t)(sub.q_row0 + r) * p.hq + sub.head] =
-                    !(l_run > 0.f) ? -INFINITY : kExact ? lse_exact(m_run, l_run) : (m_run + log2f(l_run)) * 0.6931471805599453f;
-            if (kExact && bad && writer) {                      // (one warp redoes them, none stores them)
+            // (halves: sub-tile 1's warpgroup, which has a part in every item, writes it)
+            if (valid && lse_p && !(kHalves && halved && t == 0) && !((bad >> lane) & 1u))
+                *lse_p = !(l_run > 0.f) ? -INFINITY : kExact ? lse_exact(m_run, l_run) : (m_run + log2f(l_run)) * 0.6931471805599453f;
+            if (kExact && bad && !(kHalves && halved && t == 0)) {      // (one warpgroup redoes them, neither stores them)
+                if (lane == 0) tma_store_wait_read();           // the staging rows are free again: the routine's row of Q
+                __syncwarp();
 #pragma unroll 1
                 for (uint32_t left = bad; left; left &= left - 1) {
                     attn_row_warp<__nv_bfloat16>(kp.row, sub.q_row0 + (r & ~31) + __ffs(left) - 1, sub.head,
@@ -1419,13 +1404,6 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     __syncwarp();
                 }
             }
-            if (kHalves || kExact) {
-                // values left in the slot without a store behind them: the next load comes after them
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                __syncwarp();
-            }
-            staged = true;
-            ++qn;
             gsub += n_tiles;
         }
         if (lane == 0) tma_store_wait_read();                   // the staging rows stay alive until they are read
@@ -1509,6 +1487,13 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+#ifdef FEDATTN_TRACE
+extern "C" int fedattn_debug_read_trace(long long *host, int n)
+{
+    return (int)cudaMemcpyFromSymbol(host, g_trace, sizeof(long long) * n);
+}
+#endif
+
 bool prefill_sm100_supported(const Context *ctx) { return ctx->encode_tiled != nullptr; }
 
 // The range of fast_div: calls outside it run on the SIMT kernel where that served them before (head_dim < 128).
@@ -1524,7 +1509,7 @@ bool prefill_sm100_takes(const Context *ctx, const PrefillParams &p)
 // [rows, heads, d] bf16 (token-major) or [heads, rows, d] (head-major); boxes of 64 columns x 128 rows.  Columns
 // beyond d read as zero and are not written.
 static bool encode_map(const Context *ctx, CUtensorMap *map, const void *base, int64_t rows, int heads, int d, bool head_major,
-                       int box_rows = kTileN, int box_cols = kBoxCols)
+                       int box_rows = kTileN)
 {
     EncodeTiledFn fn = reinterpret_cast<EncodeTiledFn>(ctx->encode_tiled);
     cuuint64_t dims[3], strides[2];
@@ -1533,14 +1518,14 @@ static bool encode_map(const Context *ctx, CUtensorMap *map, const void *base, i
     if (head_major) {
         dims[1] = (cuuint64_t)rows; dims[2] = (cuuint64_t)heads;
         strides[0] = (cuuint64_t)d * 2; strides[1] = (cuuint64_t)rows * d * 2;
-        box[0] = (cuuint32_t)box_cols; box[1] = (cuuint32_t)box_rows; box[2] = 1;
+        box[0] = kBoxCols; box[1] = (cuuint32_t)box_rows; box[2] = 1;
     } else {
         dims[1] = (cuuint64_t)heads; dims[2] = (cuuint64_t)rows;
         strides[0] = (cuuint64_t)d * 2; strides[1] = (cuuint64_t)heads * d * 2;
-        box[0] = (cuuint32_t)box_cols; box[1] = 1; box[2] = (cuuint32_t)box_rows;
+        box[0] = kBoxCols; box[1] = 1; box[2] = (cuuint32_t)box_rows;
     }
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, box_cols == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -1707,7 +1692,7 @@ cudaError_t launch_prefill_sm100(Context *ctx, const PrefillParams &p, cudaStrea
         return cudaErrorInvalidValue;
     // the output as [rows, heads, head_dim] in boxes of 32 rows x 64 columns; a base the encoder refuses (alignment)
     // leaves the kernel on its direct stores
-    kp.o_tma = encode_map(ctx, &mo, p.o, p.n_q_rows, p.hq, p.d, false, 32, halves || boxes == 1 ? 32 : 64) ? 1 : 0;
+    kp.o_tma = encode_map(ctx, &mo, p.o, p.n_q_rows, p.hq, p.d, false, 32) ? 1 : 0;
     if (!kp.o_tma) mo = mq;
     // the plain instance serves local attention and sync attention under the prefix mask; explicit positions
     // and bidirectional remote-only attention run the instance that carries their extra state; head dims below
@@ -1720,7 +1705,7 @@ cudaError_t launch_prefill_sm100(Context *ctx, const PrefillParams &p, cudaStrea
         prefill_sm100_kernel<true, 1, true, true>,    prefill_sm100_kernel<true, 2, true, true>};
     const int form = p.d < 128 ? 1 + boxes : (p.general || (p.remote_only && !p.causal)) ? 1 : 0;
     const int which = form + (halves ? 4 : 0);
-    const uint32_t smem = smem_bytes(p.d < 128, boxes);
+    const uint32_t smem = smem_bytes(boxes);
     static bool attr_set[64][8] = {};
     if (!attr_set[ctx->device & 63][which]) {
         cudaError_t e = cudaFuncSetAttribute(kernels[which], cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -1728,7 +1713,7 @@ cudaError_t launch_prefill_sm100(Context *ctx, const PrefillParams &p, cudaStrea
         // the CTA's pool cannot serve would wait for ever, so such a build is refused here
         cudaFuncAttributes fa;
         if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernels[which]);
-        if (e == cudaSuccess && 5 * fa.numRegs < 4 * kSoftmaxRegs + kOtherRegs) e = cudaErrorLaunchOutOfResources;
+        if (e == cudaSuccess && 3 * fa.numRegs < 2 * kSoftmaxRegs + kOtherRegs) e = cudaErrorLaunchOutOfResources;
         if (e != cudaSuccess) {
             if (getenv("FEDATTN_DEBUG")) fprintf(stderr, "prefill_sm100_kernel attribute: %s\n", cudaGetErrorString(e));
             return e;
