@@ -39,6 +39,7 @@ __global__ void __launch_bounds__(256)
 concat_kernel(const PartsParams pp, int64_t row_vecs, int64_t total_vecs, uint4 *k_agg, uint4 *v_agg,
               int32_t *kv_pos, int32_t *cu_kv)
 {
+    grid_wait();
     const bool is_v = blockIdx.y != 0;
     uint4 *dst = is_v ? v_agg : k_agg;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -78,10 +79,10 @@ cudaError_t launch_concat(const PartsParams &pp, int hkv, int d, int elt_bytes, 
     const int64_t cap = (int64_t)sm_count * 8;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    concat_kernel<<<dim3((unsigned)blocks, 2), 256, 0, s>>>(pp, row_vecs, total, (uint4 *)k_agg, (uint4 *)v_agg,
-                                                            kv_pos, cu_kv);
+    WaitFirstLaunch l(dim3((unsigned)blocks, 2), dim3(256), 0, s);
+    const cudaError_t e = cudaLaunchKernelEx(&l.cfg, concat_kernel, pp, row_vecs, total, (uint4 *)k_agg, (uint4 *)v_agg, kv_pos, cu_kv);
     ++*launches;
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // ---- key-norm scores -----------------------------------------------------------------------------

@@ -134,6 +134,7 @@ attn_tiled_kernel(const __grid_constant__ GenericParams p, const __grid_constant
     const bool two_sided = by_pos && p.remote_only && !p.causal;
     const int hi = two_sided ? p.cu[seg + 1] : 0;
     int kv_lo = 0, kv_hi;
+    grid_wait();                                                             // nothing is read or written before
     if (p.mode == kLocal) {
         kv_lo = p.cu[seg];
         kv_hi = p.causal ? kv_lo + token_of(n_rows - 1) + 1 : p.cu[seg + 1];
@@ -453,18 +454,11 @@ cudaError_t launch_variant(const GenericParams &p, TiledPlan plan, int sm_count,
         attr_set[dev & 63] = e == cudaSuccess;
     }
     if (e != cudaSuccess) return e;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = plan.splits; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3((unsigned)((int64_t)plan.n_tiles * p.hkv * plan.splits), 1, 1);
-    cfg.blockDim = dim3(L::kThreads, 1, 1);
-    cfg.dynamicSmemBytes = L::bytes(plan.stages);
-    cfg.stream = s;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, attn_tiled_kernel<T, kR, kDP, kKeyWarps>, p, plan);
+    WaitFirstLaunch l(dim3((unsigned)((int64_t)plan.n_tiles * p.hkv * plan.splits)), dim3(L::kThreads), L::bytes(plan.stages), s);
+    l.attr[1].id = cudaLaunchAttributeClusterDimension;
+    l.attr[1].val.clusterDim.x = plan.splits; l.attr[1].val.clusterDim.y = 1; l.attr[1].val.clusterDim.z = 1;
+    l.cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&l.cfg, attn_tiled_kernel<T, kR, kDP, kKeyWarps>, p, plan);
 }
 
 // M = 8, 16 (keys over warps), 32 (rows over warps; four CTAs of 64 channels share an SM.  64 rows at 8 per thread

@@ -39,6 +39,7 @@ __global__ void __launch_bounds__(256)
 merge_kernel(int64_t n_items /* rows * hq * d / 8 */, int d8, const T *o_a, const float *lse_a, const T *o_b,
              const float *lse_b, T *o, float *lse)
 {
+    grid_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_items; i += stride) {
         const int64_t rh = i / d8;                              // (row, head)
@@ -66,14 +67,15 @@ cudaError_t launch_merge(int dtype, int64_t n_rows, int hq, int d, const void *o
     if (n_items == 0) return cudaSuccess;
     int64_t blocks = (n_items + 255) / 256;
     if (blocks > (int64_t)sm_count * 16) blocks = (int64_t)sm_count * 16;
-    if (dtype == FEDATTN_BF16)
-        merge_kernel<__nv_bfloat16><<<(unsigned)blocks, 256, 0, s>>>(n_items, d / 8, (const __nv_bfloat16 *)o_a, lse_a,
-                                                                     (const __nv_bfloat16 *)o_b, lse_b, (__nv_bfloat16 *)o, lse);
-    else
-        merge_kernel<float><<<(unsigned)blocks, 256, 0, s>>>(n_items, d / 8, (const float *)o_a, lse_a, (const float *)o_b, lse_b,
-                                                             (float *)o, lse);
+    WaitFirstLaunch l(dim3((unsigned)blocks), dim3(256), 0, s);
+    typedef __nv_bfloat16 bf;
+    const cudaError_t e =
+        dtype == FEDATTN_BF16
+            ? cudaLaunchKernelEx(&l.cfg, merge_kernel<bf>, n_items, d / 8, (const bf *)o_a, lse_a, (const bf *)o_b, lse_b, (bf *)o, lse)
+            : cudaLaunchKernelEx(&l.cfg, merge_kernel<float>, n_items, d / 8, (const float *)o_a, lse_a, (const float *)o_b, lse_b,
+                                 (float *)o, lse);
     ++*launches;
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace fedattn
