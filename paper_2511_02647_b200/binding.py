@@ -3,6 +3,8 @@ supply device memory and the current CUDA stream."""
 from __future__ import annotations
 
 import ctypes as C
+import importlib.machinery
+import importlib.util
 import os
 from typing import Optional, Sequence
 
@@ -46,6 +48,18 @@ def library_path() -> str:
     return _LIB_PATH
 
 
+def _load_marshal():
+    """The native marshalling module (csrc/marshal.cpp), built beside the library."""
+    name, path = "_fedattn_marshal", os.path.join(_PKG, "lib", "_fedattn_marshal.so")
+    if not os.path.exists(path):
+        raise ImportError("FedAttn marshalling module missing: %s (run `python paper_2511_02647_b200/build.py` "
+                          "or __graft_entry__.build()); there is no fallback path" % path)
+    loader = importlib.machinery.ExtensionFileLoader(name, path)
+    module = importlib.util.module_from_spec(importlib.util.spec_from_loader(name, loader))
+    loader.exec_module(module)
+    return module
+
+
 def _load():
     if not os.path.exists(_LIB_PATH):
         raise ImportError("FedAttn CUDA library missing: %s (run `python paper_2511_02647_b200/build.py` "
@@ -69,14 +83,13 @@ def _load():
     lib.fedattn_selftest_wait_timeout.restype = C.c_int
     lib.fedattn_selftest_wait_timeout.argtypes = [vp, i32, vp]
     lib.fedattn_local.restype = C.c_int
-    lib.fedattn_local.argtypes = [vp, C.POINTER(Shape), vp, vp, vp, C.POINTER(i32), vp, vp, vp]
+    lib.fedattn_local.argtypes = [vp, C.POINTER(Shape), vp, vp, vp, vp, vp, vp, vp]
     lib.fedattn_aggregate_kv.restype = C.c_int
-    lib.fedattn_aggregate_kv.argtypes = [vp, C.POINTER(Shape), i32, C.POINTER(vp), C.POINTER(vp),
-                                         C.POINTER(i32), C.POINTER(i32), vp, vp, vp, vp, vp, vp, vp]
+    lib.fedattn_aggregate_kv.argtypes = [vp, C.POINTER(Shape), i32, vp, vp, vp, vp, vp, vp, vp, vp, vp, vp, vp]
     lib.fedattn_sync.restype = C.c_int
     lib.fedattn_sync.argtypes = [vp, C.POINTER(Shape), vp, i64, vp, vp, vp, vp, i64, i32, vp, vp, vp]
     lib.fedattn_sync_remote.restype = C.c_int
-    lib.fedattn_sync_remote.argtypes = [vp, C.POINTER(Shape), vp, C.POINTER(i32), vp, vp, vp, i64, i32, vp, vp, vp]
+    lib.fedattn_sync_remote.argtypes = [vp, C.POINTER(Shape), vp, vp, vp, vp, vp, i64, i32, vp, vp, vp]
     lib.fedattn_merge.restype = C.c_int
     lib.fedattn_merge.argtypes = [vp, C.POINTER(Shape), i64, vp, vp, vp, vp, vp, vp, vp]
     lib.fedattn_decode.restype = C.c_int
@@ -87,6 +100,7 @@ def _load():
 
 
 _lib = _load()
+_marshal = _load_marshal()
 
 
 def exported_symbols():
@@ -103,9 +117,14 @@ def _check(code: int, where: str):
         raise FedAttnError(code, where)
 
 
+# Arrays travel as bytes objects that hold the C array (parameters declared void *), which the argument tuple keeps
+# alive; what the native module does not take (it answers None) goes through ctypes below.
 def _ptr(t: Optional[torch.Tensor]):
     if t is None:
         return None
+    p = _marshal.pointer(t)
+    if p is not None:
+        return p
     if not t.is_contiguous():
         raise ValueError("tensor must be contiguous")
     return t.data_ptr()
@@ -113,12 +132,8 @@ def _ptr(t: Optional[torch.Tensor]):
 
 def _ptr_array(ts):
     """Pointers of a list of tensors (or None)."""
-    try:
-        if all([t.is_contiguous() for t in ts]):
-            return (C.c_void_p * len(ts))(*[t.data_ptr() for t in ts])
-    except AttributeError:                            # a None among them
-        pass
-    return (C.c_void_p * len(ts))(*[_ptr(t) for t in ts])
+    packed = _marshal.pointers(ts)
+    return packed if packed is not None else (C.c_void_p * len(ts))(*[_ptr(t) for t in ts])
 
 
 # The current stream as an integer.  torch.cuda.current_stream() builds a Stream object first: 3.2 us of the 5.3 us
@@ -136,10 +151,8 @@ def _stream(stream) -> int:
 
 
 def _i32_array(xs: Sequence[int]):
-    try:
-        return (C.c_int32 * len(xs))(*xs)             # Python ints as they are: half the time of converting each
-    except TypeError:
-        return (C.c_int32 * len(xs))(*[int(x) for x in xs])
+    packed = _marshal.int32s(xs)
+    return packed if packed is not None else (C.c_int32 * len(xs))(*[int(x) for x in xs])
 
 
 def fedattn_workspace_bytes(shape: Shape, max_total_tokens: int, max_total_kv: int) -> int:
@@ -208,9 +221,9 @@ class PreparedCall:
 
 
 def _args_local(ctx, shape, q, k, v, cu_seqlens_host, o, lse, stream):
-    cu = _i32_array(cu_seqlens_host)
-    if len(cu) != shape.n_participants + 1:
+    if len(cu_seqlens_host) != shape.n_participants + 1:
         raise ValueError("cu_seqlens must have N+1 entries")
+    cu = _i32_array(cu_seqlens_host)
     return (ctx.handle, C.byref(shape), _ptr(q), _ptr(k), _ptr(v), cu, _ptr(o), _ptr(lse), _stream(stream))
 
 
@@ -271,9 +284,9 @@ def prepare_sync(ctx: Context, shape: Shape, q, q_pos, k_agg, v_agg, kv_pos, tot
 
 
 def _args_sync_remote(ctx, shape, q, cu_seqlens_host, k_agg, v_agg, kv_pos, total_kv, kv_head_major, o, lse, stream):
-    cu = _i32_array(cu_seqlens_host)
-    if len(cu) != shape.n_participants + 1:
+    if len(cu_seqlens_host) != shape.n_participants + 1:
         raise ValueError("cu_seqlens must have N+1 entries")
+    cu = _i32_array(cu_seqlens_host)
     return (ctx.handle, C.byref(shape), _ptr(q), cu, _ptr(k_agg), _ptr(v_agg), _ptr(kv_pos), int(total_kv),
             int(bool(kv_head_major)), _ptr(o), _ptr(lse), _stream(stream))
 

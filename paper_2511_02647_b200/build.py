@@ -11,6 +11,8 @@ _ROOT = os.path.dirname(_PKG)
 CSRC = os.path.join(_PKG, "csrc")
 LIB_DIR = os.path.join(_PKG, "lib")
 LIB_PATH = os.path.join(LIB_DIR, "libfedattn.so")
+MARSHAL_SRC = os.path.join(CSRC, "marshal.cpp")
+MARSHAL_PATH = os.path.join(LIB_DIR, "_fedattn_marshal.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC"]
@@ -28,11 +30,30 @@ def _stale() -> bool:
     return any(os.path.getmtime(p) > t for p in deps)
 
 
+def build_marshal(force: bool = False) -> str:
+    """Compile the binding's native marshalling module (a CPython extension against torch's headers)."""
+    if not force and os.path.exists(MARSHAL_PATH) and os.path.getmtime(MARSHAL_PATH) >= os.path.getmtime(MARSHAL_SRC):
+        return MARSHAL_PATH
+    import sysconfig
+    import torch
+    inc = os.path.join(os.path.dirname(torch.__file__), "include")
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    tmp = MARSHAL_PATH + ".tmp%d" % os.getpid()
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC",
+                           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+                           "-I", sysconfig.get_paths()["include"], "-I", inc,
+                           "-I", os.path.join(inc, "torch", "csrc", "api", "include"), MARSHAL_SRC, "-o", tmp,
+                           "-L", lib, "-ltorch_python", "-ltorch_cpu", "-lc10"])
+    os.replace(tmp, MARSHAL_PATH)
+    return MARSHAL_PATH
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu under csrc/ into lib/libfedattn.so (no-op when up to date)."""
+    """Compile every .cu under csrc/ into lib/libfedattn.so, and the marshalling module (no-op when up to date)."""
+    os.makedirs(LIB_DIR, exist_ok=True)
+    build_marshal(force)
     if not force and not _stale():
         return LIB_PATH
-    os.makedirs(LIB_DIR, exist_ok=True)
     objs = []
     procs = []
     for src in _sources():

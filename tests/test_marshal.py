@@ -1,0 +1,43 @@
+"""Argument arrays of the binding: what the native module packs, and what it leaves to the general path."""
+import ctypes as C
+import struct
+
+import numpy as np
+import pytest
+import torch
+
+import paper_2511_02647_b200.binding as b
+
+
+def words(x, fmt):
+    raw = x if isinstance(x, bytes) else bytes(x)
+    return list(struct.unpack("%d%s" % (len(raw) // struct.calcsize(fmt), fmt), raw))
+
+
+@pytest.mark.parametrize("n", [0, 1, 2, 64])
+@pytest.mark.parametrize("kind", [list, tuple])
+def test_pointers(n, kind):
+    ts = kind(torch.empty(3, 4)[i % 3:] for i in range(n))
+    assert words(b._ptr_array(ts), "Q") == [t.data_ptr() for t in ts]
+
+
+def test_pointers_of_what_is_not_a_plain_tensor():
+    t, par = torch.empty(2, 2), torch.nn.Parameter(torch.empty(3))
+    assert words(b._ptr_array([None, t, par]), "Q") == [0, t.data_ptr(), par.data_ptr()]
+    assert b._ptr(None) is None and b._ptr(t) == t.data_ptr() and b._ptr(par) == par.data_ptr() and b._ptr(torch.empty(0)) == 0
+    for bad in (torch.empty(2, 3).t(), torch.empty(4)[::2]):
+        with pytest.raises(ValueError):
+            b._ptr(bad)
+        with pytest.raises(ValueError):
+            b._ptr_array([t, bad])
+    with pytest.raises(AttributeError):
+        b._ptr_array([t, 3])
+
+
+@pytest.mark.parametrize("xs", [[], [0], (1, -1, 2 ** 31 - 1, -2 ** 31), np.arange(5), [np.int64(7), 3], range(4), [True, 2], [2.0, 3]])
+def test_int32s(xs):
+    assert words(b._i32_array(xs), "i") == [int(x) for x in xs]
+
+
+def test_int32s_beyond_32_bits_wrap_as_ctypes_does():
+    assert words(b._i32_array([2 ** 32 + 5, 1]), "i") == words(bytes((C.c_int32 * 2)(2 ** 32 + 5, 1)), "i")
