@@ -63,6 +63,7 @@ cudaError_t launch_prefill(Context *c, const PrefillParams &p, int dtype, cudaSt
         max_kv = 0;
         for (int n = 0; n < p.n_seg; ++n) max_kv = p.cu[n + 1] - p.cu[n] > max_kv ? p.cu[n + 1] - p.cu[n] : max_kv;
     }
+    c->released = false;
     return launch_attn_generic(generic_params(p), dtype, (int)max_kv, c->sm_count, s, &c->launches);
 }
 
@@ -134,6 +135,7 @@ fedattn_status fedattn_create(fedattn_ctx **out, int device, void *workspace, si
     c.tc_launches = 0;
     c.agg_seq = 0;
     c.agg_key = ~0ull;
+    c.released = false;
     c.encode_tiled = nullptr;
     if (prop.major == 10) {
         void *fn = nullptr;
@@ -246,6 +248,7 @@ fedattn_status fedattn_aggregate_kv(fedattn_ctx *ctx, const fedattn_shape *shape
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int hkv = shape->n_kv_heads, d = shape->head_dim, eb = elt_bytes(shape);
     cudaError_t err = cudaSuccess;
+    ctx->c.released = mode != FEDATTN_AGG_CONCAT;
     if (mode == FEDATTN_AGG_CONCAT) {
         err = launch_concat(pp, hkv, d, eb, k_agg, v_agg, kv_pos, cu_kv, s, ctx->c.sm_count, &ctx->c.launches);
         return err == cudaSuccess ? FEDATTN_OK : FEDATTN_ERR_CUDA;
@@ -328,6 +331,7 @@ fedattn_status fedattn_merge(fedattn_ctx *ctx, const fedattn_shape *shape, int64
     if (!aligned16(o_a) || !aligned16(o_b) || !aligned16(o)) return FEDATTN_ERR_INVALID_ARG;
     DeviceGuard g(ctx->c.device);
     if (!g.ok) return FEDATTN_ERR_CUDA;
+    ctx->c.released = false;
     cudaError_t err = launch_merge(shape->dtype, n_rows, shape->n_q_heads, shape->head_dim, o_a, lse_a, o_b, lse_b, o, lse,
                                    ctx->c.sm_count, static_cast<cudaStream_t>(stream), &ctx->c.launches);
     return err == cudaSuccess ? FEDATTN_OK : FEDATTN_ERR_CUDA;
@@ -351,7 +355,8 @@ fedattn_status fedattn_decode(fedattn_ctx *ctx, const fedattn_shape *shape, int3
     cudaError_t err;
     const int N = shape->n_participants;
     const size_t need = decode_scratch_bytes(N, shape->n_q_heads, shape->head_dim, ctx->c.sm_count);
-    if (shape->dtype == FEDATTN_BF16 && shape->head_dim == 128 && need > 0) {
+    ctx->c.released = shape->dtype == FEDATTN_BF16 && shape->head_dim == 128 && need > 0;
+    if (ctx->c.released) {
         if (ctx->c.scratch_bytes < need) return FEDATTN_ERR_WORKSPACE;
         DecodeParams p;
         memset(&p, 0, sizeof(p));

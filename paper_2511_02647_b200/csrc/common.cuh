@@ -39,6 +39,7 @@ struct Context {
     int64_t tc_launches;   // launches of the tcgen05 attention kernel among them
     int64_t agg_seq;       // sequence number of the latest sparse aggregation call
     uint64_t agg_key;      // key of the stream that call ran on (early-start bookkeeping)
+    bool released;         // the latest call releases its dependents early (selection, gather, bf16 decode)
     void *encode_tiled;    // cuTensorMapEncodeTiled entry point (driver), or nullptr
 };
 

@@ -682,6 +682,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         return k * (int)gridDim.x + c;
     };
 
+    grid_wait();                                        // nothing is read or written before
     // ---- setup ------------------------------------------------------------------------------------
     if (tid == 0) {
         mbar_init(q_full, 1); mbar_init(q_empty, 1);
@@ -1729,10 +1730,18 @@ cudaError_t launch_prefill_sm100(Context *ctx, const PrefillParams &p, cudaStrea
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    kernels[which]<<<(unsigned)blocks, kThreads, smem, s>>>(mq, mk, mv, mo, kp);
+    // Set up while the preceding grid ends, but behind a call of this context that releases its dependents early launched as
+    // usual: there the CTAs would take whatever SMs that grid leaves one by one (sparse sync behind its selection 569 us, 577
+    // set up early; bidirectional local + remote behind theirs 115.5, 117.0).  Elsewhere the early set-up gains: ragged round
+    // with 64 channels 84.3 -> 80.2, local of 4 x 2048 154.2 -> 152.5, dense sync 523.8 -> 518.5.  (The barriers and the TMEM
+    // set up before the wait: 79.5, 155.7, 533.7.)
+    WaitFirstLaunch l(dim3((unsigned)blocks), dim3(kThreads), smem, s);
+    if (ctx->released) l.cfg.numAttrs = 0;
+    ctx->released = false;
+    cudaError_t e = cudaLaunchKernelEx(&l.cfg, kernels[which], mq, mk, mv, mo, kp);
     ++ctx->launches;
     ++ctx->tc_launches;
-    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess && getenv("FEDATTN_DEBUG")) fprintf(stderr, "prefill_sm100_kernel launch: %s\n", cudaGetErrorString(e));
     return e;
 }
