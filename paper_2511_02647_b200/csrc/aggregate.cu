@@ -630,6 +630,9 @@ cudaError_t launch_gather(const PartsParams &pp, int hkv, int d, int elt_bytes, 
     const int64_t vpr = (int64_t)d * elt_bytes / 16;
     const int64_t T = pp.cu_kv[pp.n];
     const int64_t total = (int64_t)hkv * T * vpr;
+    // Nothing to write: no grid.  (A grid of which no thread waits would end before its predecessor, and what waits for it
+    // in turn could overtake that one.  Otherwise thread 0 waits, in its first step or before it writes cu_kv.)
+    if (T == 0 && !cu_kv) return cudaSuccess;
     // the whole grid is resident at once (the next grid of the stream starts when every CTA of this one has)
     int64_t blocks = (total + 256 * kGatherBatch - 1) / (256 * kGatherBatch);
     if (blocks > (int64_t)sm_count * 3) blocks = (int64_t)sm_count * 3;

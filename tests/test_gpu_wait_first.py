@@ -79,3 +79,39 @@ def test_sequences_without_synchronisation(dtype, d, hq, hkv, seed):
     for mode in ("free", "graph"):
         for a, b in zip(run(dtype, d, hq, hkv, seed, mode), want):
             assert torch.equal(a, b), mode
+
+
+def test_empty_selection_lets_nothing_overtake_a_decode():
+    """A grid of which no thread waits would end before the decode in front of it, and the merge behind would read the
+    decode's output too soon: an empty indexed selection without cu_kv launches nothing."""
+    m, N, L, hq, hkv, d = fa(), 8, 4096, 32, 8, 128
+    shape = m.Shape(N, hq, hkv, d, m.BF16)
+    ctx = m.Context(shape, N * L, N * L)
+    g = torch.Generator(device="cuda").manual_seed(6)
+    q, k, v = (torch.randn(s, generator=g, device="cuda").to(torch.bfloat16) for s in ((N, hq, d), (N * L, hkv, d), (N * L, hkv, d)))
+    parts, lens = list(k.split(L)), torch.full((N,), L, dtype=torch.int32, device="cuda")
+    none = torch.zeros(0, dtype=torch.int32, device="cuda")
+
+    def rounds(synchronised):
+        res = []
+        for i in range(6):
+            o, lse, out = torch.zeros_like(q), torch.zeros(N, hq, device="cuda"), torch.zeros_like(q)
+            for c in (lambda: m.fedattn_decode(ctx, shape, m.DECODE_LOCAL, q * (i + 1), k, v, L * hkv * d, lens, L, o, lse),
+                      lambda: m.fedattn_aggregate_kv(ctx, shape, m.AGG_INDEXED, parts, parts, [L] * N, [0] * N, none),
+                      lambda: m.fedattn_merge(ctx, shape, N, o, lse, o, lse, out)):
+                c()
+                if synchronised:
+                    torch.cuda.synchronize()
+            res.append(out)
+        torch.cuda.synchronize()
+        return res
+
+    before = ctx.launch_count()
+    m.fedattn_aggregate_kv(ctx, shape, m.AGG_INDEXED, parts, parts, [L] * N, [0] * N, none)
+    assert ctx.launch_count() == before
+    cu_kv = torch.full((N + 1,), -1, dtype=torch.int32, device="cuda")
+    m.fedattn_aggregate_kv(ctx, shape, m.AGG_INDEXED, parts, parts, [L] * N, [0] * N, none, None, None, None, cu_kv)
+    assert ctx.launch_count() == before + 1 and not cu_kv.any()
+    for a, b in zip(rounds(False), rounds(True)):
+        assert torch.equal(a, b)
+    assert ctx.poll() == 0
