@@ -475,10 +475,8 @@ cudaError_t launch_topk_fused(const PartsParams &pp, int hkv, int d, int dtype, 
     int64_t *launches = &ctx->launches;
     if (pp.cu_kv[pp.n] == 0 && !cu_kv) return cudaSuccess;
     const int elt = dtype == FEDATTN_BF16 ? 2 : 4;
-    int early;
+    EarlyStart es;
     long long *done_seq = reinterpret_cast<long long *>(ctx->workspace + kDoneSeqOffset);
-    long long my_seq = 0;
-    int64_t need_seq = 0;
     {
         const size_t row_bytes = (size_t)hkv * d * elt;
         const size_t T = (size_t)pp.cu_kv[pp.n];
@@ -490,11 +488,10 @@ cudaError_t launch_topk_fused(const PartsParams &pp, int hkv, int d, int dtype, 
         }
         const MemRange out[5] = {{k_agg, T * row_bytes}, {v_agg, T * row_bytes}, {kv_pos, kv_pos ? T * hkv * 4 : 0},
                                  {cu_kv, cu_kv ? (size_t)(pp.n + 1) * 4 : 0}, {sel_idx_out, sel_idx_out ? T * hkv * 4 : 0}};
-        const EarlyStart es = early_start(device, s, in, 2 * pp.n, out, 5, true, done_seq, &ctx->agg_seq, &ctx->agg_key);
-        early = es.early ? 1 : 0;
-        my_seq = es.seq;
-        need_seq = es.need_seq;
+        es = early_start(device, s, in, 2 * pp.n, out, 5, true, done_seq, &ctx->agg_seq, &ctx->agg_key);
     }
+    const int early = es.early ? 1 : 0;
+    const long long my_seq = es.seq, need_seq = es.need_seq;
     const int vpr = d * elt / 16;
     int max_len = 0;
     for (int i = 0; i < pp.n; ++i) max_len = max(max_len, pp.off[i + 1] - pp.off[i]);
@@ -546,9 +543,10 @@ cudaError_t launch_topk_fused(const PartsParams &pp, int hkv, int d, int dtype, 
     cfg.numAttrs = 2;
     cudaError_t e = dtype == FEDATTN_BF16
                         ? cudaLaunchKernelEx(&cfg, topk_fused_kernel<FEDATTN_BF16>, pp, hkv, vpr, n_stages, max_len, early, my_seq,
-                                             (long long)need_seq, done_seq, (uint4 *)k_agg, (uint4 *)v_agg, kv_pos, cu_kv, sel_idx_out)
+                                             need_seq, done_seq, (uint4 *)k_agg, (uint4 *)v_agg, kv_pos, cu_kv, sel_idx_out)
                         : cudaLaunchKernelEx(&cfg, topk_fused_kernel<FEDATTN_F32>, pp, hkv, vpr, n_stages, max_len, early, my_seq,
-                                             (long long)need_seq, done_seq, (uint4 *)k_agg, (uint4 *)v_agg, kv_pos, cu_kv, sel_idx_out);
+                                             need_seq, done_seq, (uint4 *)k_agg, (uint4 *)v_agg, kv_pos, cu_kv, sel_idx_out);
+    early_start_end(es);
     ++*launches;
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -637,7 +635,7 @@ cudaError_t launch_gather(const PartsParams &pp, int hkv, int d, int elt_bytes, 
     int64_t blocks = (total + 256 * kGatherBatch - 1) / (256 * kGatherBatch);
     if (blocks > (int64_t)sm_count * 3) blocks = (int64_t)sm_count * 3;
     if (blocks < 1) blocks = 1;
-    int early;
+    EarlyStart es;
     {
         const size_t row_bytes = (size_t)hkv * d * elt_bytes;
         MemRange in[2 * kMaxP + 1];
@@ -650,7 +648,7 @@ cudaError_t launch_gather(const PartsParams &pp, int hkv, int d, int elt_bytes, 
         const MemRange out[5] = {{k_agg, (size_t)T * row_bytes}, {v_agg, (size_t)T * row_bytes}, {kv_pos, kv_pos ? (size_t)T * hkv * 4 : 0},
                                  {cu_kv, cu_kv ? (size_t)(pp.n + 1) * 4 : 0},
                                  {sel_idx_out, (sel_idx_out && sel_idx_out != sel_idx) ? (size_t)T * hkv * 4 : 0}};
-        early = early_start(device, s, in, 2 * pp.n + 1, out, 5).early ? 1 : 0;
+        es = early_start(device, s, in, 2 * pp.n + 1, out, 5);
     }
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
@@ -663,7 +661,8 @@ cudaError_t launch_gather(const PartsParams &pp, int hkv, int d, int elt_bytes, 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, gather_kernel, pp, hkv, vpr, sel_idx, (uint4 *)k_agg, (uint4 *)v_agg, kv_pos, cu_kv,
-                                             sel_idx_out, status, early);
+                                             sel_idx_out, status, es.early ? 1 : 0);
+    early_start_end(es);
     ++*launches;
     return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -3,6 +3,7 @@
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -53,6 +54,9 @@ struct EarlyStart {
     int64_t seq;         // this call's sequence number in its context (0: none, publish nothing)
     int64_t need_seq;    // the context's latest recorded call that reads or writes one of `out` (0: none;
                          // INT64_MAX: one that cannot be named, wait before the first write)
+    int device;
+    cudaStream_t stream;
+    bool capturing;
 };
 // Records `in` (read) and `out` (written) as buffers that grids of this call may still be using when
 // later grids of `stream` start, and decides how the call may start.  writes_before_wait: the call's
@@ -63,6 +67,8 @@ struct EarlyStart {
 EarlyStart early_start(int device, cudaStream_t stream, const MemRange *in, int n_in, const MemRange *out, int n_out,
                        bool writes_before_wait = false, const void *owner = nullptr, int64_t *seq_counter = nullptr,
                        uint64_t *owner_key = nullptr);
+// Behind the call's last launch: while the stream is being captured, notes the node that launch became.
+void early_start_end(const EarlyStart &r);
 // The owner's sequence numbers are about to lose their meaning (its context is being destroyed).
 void early_start_forget(int device, const void *owner);
 

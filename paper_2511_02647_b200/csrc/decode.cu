@@ -489,6 +489,7 @@ static cudaError_t launch_decode_split(const DecodeParams &p_in, int device, int
                                        int64_t *launches)
 {
     DecodeParams p = p_in;
+    EarlyStart es;
     {
         // may the stream kernel read its inputs before the preceding grid of the stream is complete?
         const size_t row_bytes = (size_t)p.hkv * kD * 2, qo_bytes = (size_t)p.n_part * p.hq * kD * 2;
@@ -497,7 +498,8 @@ static cudaError_t launch_decode_split(const DecodeParams &p_in, int device, int
         const MemRange in[4] = {{p.q, qo_bytes}, {p.k, cache_bytes}, {p.v, cache_bytes},
                                 {p.kv_len, (p.sync ? 1 : p.n_part) * sizeof(int32_t)}};
         const MemRange out[2] = {{p.o, qo_bytes}, {p.lse, p.lse ? (size_t)p.n_part * p.hq * sizeof(float) : 0}};
-        p.early = early_start(device, s, in, 4, out, 2).early ? 1 : 0;
+        es = early_start(device, s, in, 4, out, 2);
+        p.early = es.early ? 1 : 0;
     }
     const int g = p.hq / p.hkv;
     p.g_shift = -1;
@@ -543,7 +545,10 @@ static cudaError_t launch_decode_split(const DecodeParams &p_in, int device, int
         e = m_tiles == 1 ? cudaLaunchKernelEx(&cfg, decode_stream_kernel<1, false>, p, n_splits, n_chunks)
                          : cudaLaunchKernelEx(&cfg, decode_stream_kernel<2, false>, p, n_splits, n_chunks);
     if (launches) ++*launches;
-    if (one_launch) return e != cudaSuccess ? e : cudaGetLastError();
+    if (one_launch) {
+        early_start_end(es);
+        return e != cudaSuccess ? e : cudaGetLastError();
+    }
     cfg.numAttrs = 1;
     if (e != cudaSuccess) return e;
     const int n_rows = p.n_part * p.hq, rows_per_cta = (n_rows + sm_count - 1) / sm_count;
@@ -551,6 +556,7 @@ static cudaError_t launch_decode_split(const DecodeParams &p_in, int device, int
     cfg.blockDim = dim3(kMergeGroups * (kD / 4), 1, 1);
     cfg.dynamicSmemBytes = 0;
     e = cudaLaunchKernelEx(&cfg, decode_merge_kernel, p, n_slots, n_rows);
+    early_start_end(es);
     if (launches) ++*launches;
     return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -28,7 +28,11 @@
 //   * While a stream is being captured the calls are recorded under the capture's own key, carry no
 //     sequence number and publish nothing: the values baked into a captured launch must hold for every
 //     replay, so a captured call whose outputs overlap an earlier captured call's buffers always waits
-//     before it writes (need_seq = INT64_MAX) but may still read early.
+//     before it writes (need_seq = INT64_MAX) but may still read early.  There an event does not complete a
+//     grid: a launch of this kind gets a programmatic edge from every kernel that the stream then depends on,
+//     also from those of other streams of the capture, whose buffers its record does not hold.  So a captured
+//     call waits first unless the stream's one dependency is the last kernel of its latest recorded call.
+//     (Behind any other kernel waiting costs nothing: what releases nothing early has ended by then.)
 #include <memory>
 #include <mutex>
 
@@ -43,6 +47,7 @@ constexpr int kSlots = 8;          // streams (or captures) remembered per devic
 struct Slot {
     uint64_t key = 0, last_use = 0;
     int n = 0;
+    cudaGraphNode_t node = nullptr;    // captured: the last kernel of the latest call
     uintptr_t lo[kRecord], hi[kRecord];
     const void *owner[kRecord];    // whose sequence numbers `seq` counts in (a context's done word), or null
     int64_t seq[kRecord];          // the owner's latest call that touches this range
@@ -61,30 +66,57 @@ struct Range {
     uint8_t rd;
 };
 
+struct Capture {
+    bool active = false;
+    unsigned long long id = 0;
+    cudaGraphNode_t node = nullptr;    // what the stream's next node will depend on, when it is one node
+};
+Capture capture_of(cudaStream_t stream)
+{
+    Capture c;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamGetCaptureInfo(stream, &st, &c.id) != cudaSuccess) {
+        cudaGetLastError();
+        return c;
+    }
+    c.active = st != cudaStreamCaptureStatusNone;
+    if (c.active) {
+        cudaGraph_t graph;
+        const cudaGraphNode_t *deps = nullptr;
+        const cudaGraphEdgeData *edges = nullptr;
+        size_t n = 0;
+        if (cudaStreamGetCaptureInfo_v3(stream, &st, &c.id, &graph, &deps, &edges, &n) != cudaSuccess) cudaGetLastError();
+        else if (n == 1) c.node = deps[0];
+    }
+    return c;
+}
+uint64_t key_of(cudaStream_t stream, const Capture &c)
+{
+    const uint64_t s = (uint64_t)(uintptr_t)stream;
+    return c.active ? ((s * 0x9E3779B97F4A7C15ull) ^ (c.id << 1)) | 1ull : s << 1;
+}
+Slot *find_slot(DeviceRecord *dev, uint64_t key)
+{
+    for (int i = 0; i < dev->n_slots; ++i)
+        if (dev->slot[i].key == key) return &dev->slot[i];
+    return nullptr;
+}
+
 }  // namespace
 
 EarlyStart early_start(int device, cudaStream_t stream, const MemRange *in, int n_in, const MemRange *out, int n_out,
                        bool writes_before_wait, const void *owner, int64_t *seq_counter, uint64_t *owner_key)
 {
-    EarlyStart r{false, 0, 0};
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    unsigned long long cap_id = 0;
-    if (cudaStreamGetCaptureInfo(stream, &cap, &cap_id) != cudaSuccess) {
-        cudaGetLastError();
-        cap = cudaStreamCaptureStatusNone;
-    }
-    const bool capturing = cap != cudaStreamCaptureStatusNone;
-    const uint64_t key = capturing ? (((uint64_t)(uintptr_t)stream * 0x9E3779B97F4A7C15ull) ^ (cap_id << 1)) | 1ull
-                                   : (uint64_t)(uintptr_t)stream << 1;
-    if (capturing) owner = nullptr;
+    const Capture cap = capture_of(stream);
+    const uint64_t key = key_of(stream, cap);
+    EarlyStart r{false, 0, 0, device, stream, cap.active};
+    if (cap.active) owner = nullptr;
 
     std::lock_guard<std::mutex> lock(g_record_mutex);
     std::unique_ptr<DeviceRecord> &dev = g_record[device & 63];
     if (!dev) dev.reset(new DeviceRecord);
     bool wait_first = false;
-    Slot *sl = nullptr;
-    for (int i = 0; i < dev->n_slots; ++i)
-        if (dev->slot[i].key == key) sl = &dev->slot[i];
+    Slot *sl = find_slot(dev.get(), key);
     if (!sl) {                                                    // nothing is known about this stream
         if (dev->n_slots < kSlots) sl = &dev->slot[dev->n_slots++];
         else {
@@ -94,8 +126,11 @@ EarlyStart early_start(int device, cudaStream_t stream, const MemRange *in, int 
         }
         sl->key = key;
         sl->n = 0;
+        sl->node = nullptr;
         wait_first = true;
     }
+    if (cap.active && (!sl->node || cap.node != sl->node)) wait_first = true;
+    sl->node = nullptr;                                           // until early_start_end
     sl->last_use = ++dev->clock;
     if (owner && owner_key && *owner_key != key) {                // the context has moved to this stream
         for (int i = 0; i < dev->n_slots; ++i)
@@ -144,7 +179,7 @@ EarlyStart early_start(int device, cudaStream_t stream, const MemRange *in, int 
         n_new += match[i] < 0;
     }
     if (unknown) {
-        if (capturing) need = INT64_MAX;
+        if (cap.active) need = INT64_MAX;
         else wait_first = true;
     }
     if (sl->n + n_new > kRecord) wait_first = true;
@@ -161,6 +196,15 @@ EarlyStart early_start(int device, cudaStream_t stream, const MemRange *in, int 
     r.early = !wait_first;
     r.need_seq = need;
     return r;
+}
+
+void early_start_end(const EarlyStart &r)
+{
+    if (!r.capturing) return;
+    const Capture cap = capture_of(r.stream);
+    std::lock_guard<std::mutex> lock(g_record_mutex);
+    DeviceRecord *dev = g_record[r.device & 63].get();
+    if (Slot *sl = dev ? find_slot(dev, key_of(r.stream, cap)) : nullptr) sl->node = cap.node;
 }
 
 void early_start_forget(int device, const void *owner)

@@ -115,3 +115,43 @@ def test_empty_selection_lets_nothing_overtake_a_decode():
     for a, b in zip(rounds(False), rounds(True)):
         assert torch.equal(a, b)
     assert ctx.poll() == 0
+
+
+def test_captured_branches_that_join():
+    """A graph of two branches: one selects, the other decodes, joins it and gathers by what it selected.  The gather's
+    launch gets a programmatic edge from the other branch's selection too."""
+    m, N, L, K, hq, hkv, d = fa(), 16, 1024, 256, 8, 4, 128
+    shape = m.Shape(N, hq, hkv, d, m.BF16)
+    ctx, ctx2 = m.Context(shape, N * L, N * L), m.Context(shape, N * L, N * L)
+    g = torch.Generator(device="cuda").manual_seed(7)
+    q, k, v, w = (torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)
+                  for s in ((N, hq, d), (N * L, hkv, d), (N * L, hkv, d), (N * L, hkv, d)))
+    lens, rows = torch.full((N,), 64, dtype=torch.int32, device="cuda"), torch.arange(K, dtype=torch.int32, device="cuda").repeat(hkv, N)
+    ks, vs, kg, vg = (torch.zeros(hkv, N * K, d, dtype=torch.bfloat16, device="cuda") for _ in range(4))
+    sel, o = rows.clone(), torch.zeros_like(q)
+
+    def branches(one, two):
+        m.fedattn_decode(ctx2, shape, m.DECODE_LOCAL, q, k, v, L * hkv * d, lens, 64, o, stream=two)
+        m.fedattn_aggregate_kv(ctx, shape, m.AGG_TOPK_KNORM, list(k.split(L)), list(v.split(L)), [L] * N, [K] * N, None, ks, vs, None, None,
+                               sel, stream=one)
+        two.wait_stream(one)
+        m.fedattn_aggregate_kv(ctx2, shape, m.AGG_INDEXED, list(w.split(L)), list(v.split(L)), [L] * N, [K] * N, sel, kg, vg, None, None,
+                               None, stream=two)
+
+    one, two, graph = torch.cuda.Stream(), torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    branches(one, two)
+    torch.cuda.synchronize()
+    want = [x.clone() for x in (ks, vs, kg, vg, sel, o)]
+    with torch.cuda.graph(graph, stream=one):
+        two.wait_stream(one)
+        branches(one, two)
+        one.wait_stream(two)
+    for _ in range(10):
+        for x in (ks, vs, kg, vg, o):
+            x.zero_()
+        sel.copy_(rows)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert ctx.poll() == 0 and ctx2.poll() == 0
+        for a, b in zip((ks, vs, kg, vg, sel, o), want):
+            assert torch.equal(a, b)
