@@ -495,7 +495,7 @@ cudaError_t launch_topk_fused(const PartsParams &pp, int hkv, int d, int dtype, 
     const int vpr = d * elt / 16;
     int max_len = 0;
     for (int i = 0; i < pp.n; ++i) max_len = max(max_len, pp.off[i + 1] - pp.off[i]);
-    if (max_len > kSelMaxLen) return cudaErrorInvalidValue;
+    if (max_len > kSelMaxLen) return early_start_end(es, cudaErrorInvalidValue);
     // slices per (head, participant): a power of two <= 8 (one cluster), about two CTAs per SM in total, and
     // every slice keeps at least one token per lane of the CTA (a lane walks one key row at a time)
     const int pairs = hkv * pp.n;
@@ -525,7 +525,7 @@ cudaError_t launch_topk_fused(const PartsParams &pp, int hkv, int d, int dtype, 
         cudaError_t e = cudaFuncSetAttribute(topk_fused_kernel<FEDATTN_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(topk_fused_kernel<FEDATTN_F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess) return early_start_end(es, e);
         attr_set[device & 63] = true;
     }
     cudaLaunchConfig_t cfg;
@@ -546,9 +546,8 @@ cudaError_t launch_topk_fused(const PartsParams &pp, int hkv, int d, int dtype, 
                                              need_seq, done_seq, (uint4 *)k_agg, (uint4 *)v_agg, kv_pos, cu_kv, sel_idx_out)
                         : cudaLaunchKernelEx(&cfg, topk_fused_kernel<FEDATTN_F32>, pp, hkv, vpr, n_stages, max_len, early, my_seq,
                                              need_seq, done_seq, (uint4 *)k_agg, (uint4 *)v_agg, kv_pos, cu_kv, sel_idx_out);
-    early_start_end(es);
     ++*launches;
-    return e != cudaSuccess ? e : cudaGetLastError();
+    return early_start_end(es, e != cudaSuccess ? e : cudaGetLastError());
 }
 
 // ---- indexed gather ------------------------------------------------------------------------------
@@ -662,9 +661,8 @@ cudaError_t launch_gather(const PartsParams &pp, int hkv, int d, int elt_bytes, 
     cfg.numAttrs = 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, gather_kernel, pp, hkv, vpr, sel_idx, (uint4 *)k_agg, (uint4 *)v_agg, kv_pos, cu_kv,
                                              sel_idx_out, status, es.early ? 1 : 0);
-    early_start_end(es);
     ++*launches;
-    return e != cudaSuccess ? e : cudaGetLastError();
+    return early_start_end(es, e != cudaSuccess ? e : cudaGetLastError());
 }
 
 }  // namespace fedattn

@@ -67,8 +67,9 @@ struct EarlyStart {
 EarlyStart early_start(int device, cudaStream_t stream, const MemRange *in, int n_in, const MemRange *out, int n_out,
                        bool writes_before_wait = false, const void *owner = nullptr, int64_t *seq_counter = nullptr,
                        uint64_t *owner_key = nullptr);
-// Behind the call's last launch: while the stream is being captured, notes the node that launch became.
-void early_start_end(const EarlyStart &r);
+// Behind the call's last launch, or where it ends without one; returns e.  A call that was not launched leaves no record of
+// the grids before it behind.  While the stream is being captured, notes the node that the last launch became.
+cudaError_t early_start_end(const EarlyStart &r, cudaError_t e);
 // The owner's sequence numbers are about to lose their meaning (its context is being destroyed).
 void early_start_forget(int device, const void *owner);
 

@@ -523,7 +523,8 @@ static cudaError_t launch_decode_split(const DecodeParams &p_in, int device, int
     const bool one_launch = (int64_t)caches * p.hkv * p.max_kv_len * kD * 4 <= kOneLaunchBytes && tiles <= kOneLaunchTiles * cluster;
     if (one_launch) n_splits = cluster;
     const int n_slots = n_splits * slices;
-    if (!one_launch && (size_t)p.n_part * p.hq * n_slots * kPartialStride * sizeof(float) > p.partial_bytes) return cudaErrorInvalidValue;
+    if (!one_launch && (size_t)p.n_part * p.hq * n_slots * kPartialStride * sizeof(float) > p.partial_bytes)
+        return early_start_end(es, cudaErrorInvalidValue);
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -545,20 +546,16 @@ static cudaError_t launch_decode_split(const DecodeParams &p_in, int device, int
         e = m_tiles == 1 ? cudaLaunchKernelEx(&cfg, decode_stream_kernel<1, false>, p, n_splits, n_chunks)
                          : cudaLaunchKernelEx(&cfg, decode_stream_kernel<2, false>, p, n_splits, n_chunks);
     if (launches) ++*launches;
-    if (one_launch) {
-        early_start_end(es);
-        return e != cudaSuccess ? e : cudaGetLastError();
-    }
+    if (one_launch) return early_start_end(es, e != cudaSuccess ? e : cudaGetLastError());
     cfg.numAttrs = 1;
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) return early_start_end(es, e);
     const int n_rows = p.n_part * p.hq, rows_per_cta = (n_rows + sm_count - 1) / sm_count;
     cfg.gridDim = dim3((n_rows + rows_per_cta - 1) / rows_per_cta, 1, 1);
     cfg.blockDim = dim3(kMergeGroups * (kD / 4), 1, 1);
     cfg.dynamicSmemBytes = 0;
     e = cudaLaunchKernelEx(&cfg, decode_merge_kernel, p, n_slots, n_rows);
-    early_start_end(es);
     if (launches) ++*launches;
-    return e != cudaSuccess ? e : cudaGetLastError();
+    return early_start_end(es, e != cudaSuccess ? e : cudaGetLastError());
 }
 
 static cudaError_t set_decode_smem_attr()

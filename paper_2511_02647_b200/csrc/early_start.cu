@@ -198,13 +198,20 @@ EarlyStart early_start(int device, cudaStream_t stream, const MemRange *in, int 
     return r;
 }
 
-void early_start_end(const EarlyStart &r)
+cudaError_t early_start_end(const EarlyStart &r, cudaError_t e)
 {
-    if (!r.capturing) return;
+    if (e != cudaSuccess) {
+        // the record says that this call ran, and when it was to wait first, that nothing before it is left
+        std::lock_guard<std::mutex> lock(g_record_mutex);
+        if (DeviceRecord *dev = g_record[r.device & 63].get()) dev->n_slots = 0;
+        return e;
+    }
+    if (!r.capturing) return e;
     const Capture cap = capture_of(r.stream);
     std::lock_guard<std::mutex> lock(g_record_mutex);
     DeviceRecord *dev = g_record[r.device & 63].get();
     if (Slot *sl = dev ? find_slot(dev, key_of(r.stream, cap)) : nullptr) sl->node = cap.node;
+    return e;
 }
 
 void early_start_forget(int device, const void *owner)

@@ -44,7 +44,7 @@ extern "C" int start(size_t stream, size_t in, size_t out)
     g_es = early_start(0, (cudaStream_t)stream, &i, 1, &o, 1);
     return g_es.early;
 }
-extern "C" void end() { early_start_end(g_es); }
+extern "C" int end(int e) { return early_start_end(g_es, (cudaError_t)e); }
 """
 
 
@@ -83,7 +83,7 @@ def test_captured_calls_of_one_stream(lib):
         lib.set_capture(7, 1 if dep else 0, dep, 0)
         early = lib.start(s, i, o)
         lib.set_capture(7, 1, node, 0)
-        lib.end()
+        lib.end(0)
         return early
 
     assert call(0, 0xa, 0x1000, 0x2000) == 0
@@ -99,15 +99,15 @@ def test_captured_call_behind_another_branch_waits_first(lib, deps):
     lib.set_capture(7, 0, 0, 0)
     assert lib.start(two, 0x1000, 0x2000) == 0
     lib.set_capture(7, 1, 0xa, 0)
-    lib.end()
+    lib.end(0)
     lib.set_capture(7, 0, 0, 0)
     assert lib.start(one, 0x3000, 0x8000) == 0
     lib.set_capture(7, 1, 0xb, 0)
-    lib.end()
+    lib.end(0)
     lib.set_capture(7, len(deps), *(deps + (0, 0))[:2])
     assert lib.start(two, 0x8000, 0x9000) == 0
     lib.set_capture(7, 1, 0xc, 0)
-    lib.end()
+    lib.end(0)
     assert lib.start(two, 0x3000, 0xb000) == 1                   # behind the call that waited
 
 
@@ -116,3 +116,18 @@ def test_captured_call_whose_node_is_unknown_is_followed_by_one_that_waits(lib):
     lib.set_capture(7, 0, 0, 0)
     lib.start(s, 0x1000, 0x2000)                                 # (its launch failed: no end)
     assert lib.start(s, 0x3000, 0x4000) == 0
+
+
+@pytest.mark.parametrize("capture", [0, 7])
+def test_call_that_was_not_launched_vouches_for_nothing(lib, capture):
+    """The call behind it must not start early on the word of a call that was to wait and never ran."""
+    s = 0x100
+    lib.set_capture(capture, 0, 0, 0)
+    lib.start(s, 0x1000, 0x2000)
+    lib.set_capture(capture, 1, 0xa, 0)
+    assert lib.end(0) == 0
+    assert lib.start(s, 0x2000, 0x3000) == 0                     # is to wait for the first call; its launch fails
+    assert lib.end(700) == 700
+    assert lib.start(s, 0x2000, 0x4000) == 0                     # the first call may still be writing
+    assert lib.end(0) == 0
+    assert lib.start(s, 0x5000, 0x6000) == 1
