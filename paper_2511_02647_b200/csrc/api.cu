@@ -69,14 +69,15 @@ cudaError_t launch_prefill(Context *c, const PrefillParams &p, int dtype, cudaSt
 
 struct DeviceGuard {
     int prev = -1;
-    bool ok = true;
+    cudaError_t err;
     explicit DeviceGuard(int dev)
     {
-        if (cudaGetDevice(&prev) != cudaSuccess) { ok = false; return; }
-        if (prev != dev && cudaSetDevice(dev) != cudaSuccess) ok = false;
+        err = cudaGetDevice(&prev);
+        if (err != cudaSuccess) { prev = -1; return; }
+        if (prev != dev) err = cudaSetDevice(dev);
         if (prev == dev) prev = -1;
     }
-    ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
+    ~DeviceGuard() { if (prev >= 0) status_of(cudaSetDevice(prev)); }
 };
 
 }  // namespace
@@ -116,11 +117,14 @@ fedattn_status fedattn_create(fedattn_ctx **out, int device, void *workspace, si
     if (!workspace || workspace_bytes < kStatusBytes || (reinterpret_cast<uintptr_t>(workspace) & 255))
         return FEDATTN_ERR_WORKSPACE;
     int count = 0;
-    if (cudaGetDeviceCount(&count) != cudaSuccess || device < 0 || device >= count) return FEDATTN_ERR_CUDA;
+    cudaError_t err = cudaGetDeviceCount(&count);
+    if (err != cudaSuccess) return status_of(err);
+    if (device < 0 || device >= count) return FEDATTN_ERR_CUDA;
     DeviceGuard g(device);
-    if (!g.ok) return FEDATTN_ERR_CUDA;
+    if (g.err != cudaSuccess) return status_of(g.err);
     cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return FEDATTN_ERR_CUDA;
+    err = cudaGetDeviceProperties(&prop, device);
+    if (err != cudaSuccess) return status_of(err);
     fedattn_ctx *ctx = new (std::nothrow) fedattn_ctx();
     if (!ctx) return FEDATTN_ERR_CUDA;
     Context &c = ctx->c;
@@ -140,13 +144,15 @@ fedattn_status fedattn_create(fedattn_ctx **out, int device, void *workspace, si
     if (prop.major == 10) {
         void *fn = nullptr;
         cudaDriverEntryPointQueryResult qres;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) == cudaSuccess &&
+        if (status_of(cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres)) == FEDATTN_OK &&
             qres == cudaDriverEntryPointSuccess)
             c.encode_tiled = fn;
     }
-    if (cudaMemset(workspace, 0, kStatusBytes) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
+    err = cudaMemset(workspace, 0, kStatusBytes);
+    if (err == cudaSuccess) err = cudaDeviceSynchronize();
+    if (err != cudaSuccess) {
         delete ctx;
-        return FEDATTN_ERR_CUDA;
+        return status_of(err);
     }
     *out = ctx;
     return FEDATTN_OK;
@@ -167,22 +173,21 @@ fedattn_status fedattn_selftest_wait_timeout(fedattn_ctx *ctx, int32_t max_polls
     if (!ctx || max_polls < 1 || max_polls > 65536) return FEDATTN_ERR_INVALID_ARG;
     if (!prefill_sm100_supported(&ctx->c)) return FEDATTN_ERR_UNSUPPORTED;
     DeviceGuard g(ctx->c.device);
-    if (!g.ok) return FEDATTN_ERR_CUDA;
-    return launch_wait_selftest(&ctx->c, max_polls, static_cast<cudaStream_t>(stream)) == cudaSuccess ? FEDATTN_OK
-                                                                                                       : FEDATTN_ERR_CUDA;
+    if (g.err != cudaSuccess) return status_of(g.err);
+    return status_of(launch_wait_selftest(&ctx->c, max_polls, static_cast<cudaStream_t>(stream)));
 }
 
 fedattn_status fedattn_poll(fedattn_ctx *ctx, fedattn_stream stream)
 {
     if (!ctx) return FEDATTN_ERR_INVALID_ARG;
     DeviceGuard g(ctx->c.device);
-    if (!g.ok) return FEDATTN_ERR_CUDA;
+    if (g.err != cudaSuccess) return status_of(g.err);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     int32_t word = 0;
-    if (cudaStreamSynchronize(s) != cudaSuccess) return FEDATTN_ERR_CUDA;
-    if (cudaMemcpy(&word, ctx->c.status, sizeof(word), cudaMemcpyDeviceToHost) != cudaSuccess)
-        return FEDATTN_ERR_CUDA;
-    if (word != 0 && cudaMemset(ctx->c.status, 0, sizeof(word)) != cudaSuccess) return FEDATTN_ERR_CUDA;
+    cudaError_t err = cudaStreamSynchronize(s);
+    if (err == cudaSuccess) err = cudaMemcpy(&word, ctx->c.status, sizeof(word), cudaMemcpyDeviceToHost);
+    if (err == cudaSuccess && word != 0) err = cudaMemset(ctx->c.status, 0, sizeof(word));
+    if (err != cudaSuccess) return status_of(err);
     return static_cast<fedattn_status>(word);
 }
 
@@ -199,12 +204,12 @@ fedattn_status fedattn_local(fedattn_ctx *ctx, const fedattn_shape *shape, const
     if (!q || !k || !v || !o) return FEDATTN_ERR_INVALID_ARG;
     if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(o)) return FEDATTN_ERR_INVALID_ARG;
     DeviceGuard g(ctx->c.device);
-    if (!g.ok) return FEDATTN_ERR_CUDA;
+    if (g.err != cudaSuccess) return status_of(g.err);
     PrefillParams p = prefill_params(shape, q, k, v, o, lse, L, L);
     p.n_seg = N;
     memcpy(p.cu, cu, sizeof(int32_t) * (N + 1));
     const cudaError_t err = launch_prefill(&ctx->c, p, shape->dtype, static_cast<cudaStream_t>(stream));
-    return err == cudaSuccess ? FEDATTN_OK : FEDATTN_ERR_CUDA;
+    return status_of(err);
 }
 
 fedattn_status fedattn_aggregate_kv(fedattn_ctx *ctx, const fedattn_shape *shape, int32_t mode,
@@ -244,28 +249,28 @@ fedattn_status fedattn_aggregate_kv(fedattn_ctx *ctx, const fedattn_shape *shape
         for (int n = 0; n < N; ++n)
             if (seqlens[n] > 4096) return FEDATTN_ERR_UNSUPPORTED;
     DeviceGuard g(ctx->c.device);
-    if (!g.ok) return FEDATTN_ERR_CUDA;
+    if (g.err != cudaSuccess) return status_of(g.err);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int hkv = shape->n_kv_heads, d = shape->head_dim, eb = elt_bytes(shape);
     cudaError_t err = cudaSuccess;
     ctx->c.released = mode != FEDATTN_AGG_CONCAT;
     if (mode == FEDATTN_AGG_CONCAT) {
         err = launch_concat(pp, hkv, d, eb, k_agg, v_agg, kv_pos, cu_kv, s, ctx->c.sm_count, &ctx->c.launches);
-        return err == cudaSuccess ? FEDATTN_OK : FEDATTN_ERR_CUDA;
+        return status_of(err);
     }
     if (mode == FEDATTN_AGG_TOPK_KNORM) {
         err = launch_topk_fused(pp, hkv, d, shape->dtype, k_agg, v_agg, kv_pos, cu_kv, sel_idx_out, &ctx->c, s);
-        return err == cudaSuccess ? FEDATTN_OK : FEDATTN_ERR_CUDA;
+        return status_of(err);
     }
     if (mode == FEDATTN_AGG_TOPK_TOKEN) {
         // the per-head kernel on the token row viewed as one head of Hkv * d channels: token-major output
         err = launch_topk_fused(pp, 1, hkv * d, shape->dtype, k_agg, v_agg, kv_pos, cu_kv, sel_idx_out, &ctx->c, s);
-        return err == cudaSuccess ? FEDATTN_OK : FEDATTN_ERR_CUDA;
+        return status_of(err);
     }
     const int32_t *sel = sel_idx_in;
     err = launch_gather(pp, hkv, d, eb, sel, k_agg, v_agg, kv_pos, cu_kv, sel_idx_out, ctx->c.status, ctx->c.device, ctx->c.sm_count, s,
                         &ctx->c.launches);
-    return err == cudaSuccess ? FEDATTN_OK : FEDATTN_ERR_CUDA;
+    return status_of(err);
 }
 
 fedattn_status fedattn_sync(fedattn_ctx *ctx, const fedattn_shape *shape, const void *q, int64_t n_q_rows,
@@ -279,7 +284,7 @@ fedattn_status fedattn_sync(fedattn_ctx *ctx, const fedattn_shape *shape, const 
     if (!q || !o || !aligned16(q) || !aligned16(o)) return FEDATTN_ERR_INVALID_ARG;
     if (total_kv > 0 && (!k_agg || !v_agg || !aligned16(k_agg) || !aligned16(v_agg))) return FEDATTN_ERR_INVALID_ARG;
     DeviceGuard g(ctx->c.device);
-    if (!g.ok) return FEDATTN_ERR_CUDA;
+    if (g.err != cudaSuccess) return status_of(g.err);
     PrefillParams p = prefill_params(shape, q, k_agg, v_agg, o, lse, n_q_rows, total_kv);
     p.sync = 1; p.kv_head_major = kv_head_major; p.kv_pos = kv_pos; p.q_pos = q_pos;
     p.n_seg = 1;
@@ -294,7 +299,7 @@ fedattn_status fedattn_sync(fedattn_ctx *ctx, const fedattn_shape *shape, const 
         }
     }
     const cudaError_t err = launch_prefill(&ctx->c, p, shape->dtype, static_cast<cudaStream_t>(stream));
-    return err == cudaSuccess ? FEDATTN_OK : FEDATTN_ERR_CUDA;
+    return status_of(err);
 }
 
 fedattn_status fedattn_sync_remote(fedattn_ctx *ctx, const fedattn_shape *shape, const void *q, const int32_t *cu,
@@ -312,13 +317,13 @@ fedattn_status fedattn_sync_remote(fedattn_ctx *ctx, const fedattn_shape *shape,
     if (!q || !o || !aligned16(q) || !aligned16(o)) return FEDATTN_ERR_INVALID_ARG;
     if (total_kv > 0 && (!k_agg || !v_agg || !aligned16(k_agg) || !aligned16(v_agg))) return FEDATTN_ERR_INVALID_ARG;
     DeviceGuard g(ctx->c.device);
-    if (!g.ok) return FEDATTN_ERR_CUDA;
+    if (g.err != cudaSuccess) return status_of(g.err);
     PrefillParams p = prefill_params(shape, q, k_agg, v_agg, o, lse, L, total_kv);
     p.sync = 1; p.remote_only = 1; p.kv_head_major = kv_head_major; p.kv_pos = kv_pos;
     p.n_seg = N;
     memcpy(p.cu, cu, sizeof(int32_t) * (N + 1));
     const cudaError_t err = launch_prefill(&ctx->c, p, shape->dtype, static_cast<cudaStream_t>(stream));
-    return err == cudaSuccess ? FEDATTN_OK : FEDATTN_ERR_CUDA;
+    return status_of(err);
 }
 
 fedattn_status fedattn_merge(fedattn_ctx *ctx, const fedattn_shape *shape, int64_t n_rows, const void *o_a,
@@ -330,11 +335,11 @@ fedattn_status fedattn_merge(fedattn_ctx *ctx, const fedattn_shape *shape, int64
     if (!o_a || !o_b || !lse_a || !lse_b || !o) return FEDATTN_ERR_INVALID_ARG;
     if (!aligned16(o_a) || !aligned16(o_b) || !aligned16(o)) return FEDATTN_ERR_INVALID_ARG;
     DeviceGuard g(ctx->c.device);
-    if (!g.ok) return FEDATTN_ERR_CUDA;
+    if (g.err != cudaSuccess) return status_of(g.err);
     ctx->c.released = false;
     cudaError_t err = launch_merge(shape->dtype, n_rows, shape->n_q_heads, shape->head_dim, o_a, lse_a, o_b, lse_b, o, lse,
                                    ctx->c.sm_count, static_cast<cudaStream_t>(stream), &ctx->c.launches);
-    return err == cudaSuccess ? FEDATTN_OK : FEDATTN_ERR_CUDA;
+    return status_of(err);
 }
 
 fedattn_status fedattn_decode(fedattn_ctx *ctx, const fedattn_shape *shape, int32_t mode, const void *q,
@@ -350,7 +355,7 @@ fedattn_status fedattn_decode(fedattn_ctx *ctx, const fedattn_shape *shape, int3
     if (!aligned16(q) || !aligned16(o)) return FEDATTN_ERR_INVALID_ARG;
     if (mode == FEDATTN_DECODE_LOCAL && (cache_stride * elt_bytes(shape)) % 16 != 0) return FEDATTN_ERR_INVALID_ARG;
     DeviceGuard g(ctx->c.device);
-    if (!g.ok) return FEDATTN_ERR_CUDA;
+    if (g.err != cudaSuccess) return status_of(g.err);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     cudaError_t err;
     const int N = shape->n_participants;
@@ -378,7 +383,7 @@ fedattn_status fedattn_decode(fedattn_ctx *ctx, const fedattn_shape *shape, int3
         p.kv_len = kv_len; p.cache_stride = cache_stride;
         err = launch_attn_generic(p, shape->dtype, max_kv_len, ctx->c.sm_count, s, &ctx->c.launches);
     }
-    return err == cudaSuccess ? FEDATTN_OK : FEDATTN_ERR_CUDA;
+    return status_of(err);
 }
 
 }  // extern "C"

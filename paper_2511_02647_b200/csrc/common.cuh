@@ -28,6 +28,15 @@ __device__ __forceinline__ float lse_exact(float m2, float l)
     return sum + (((prod - (sum - back)) + (lg - back)) + prod_rest);
 }
 
+// How an entry point answers a runtime call.  The runtime keeps a failed call's error until it is taken; left there, the
+// next call's own check would report it although its work was enqueued.
+inline fedattn_status status_of(cudaError_t e)
+{
+    if (e == cudaSuccess) return FEDATTN_OK;
+    cudaGetLastError();
+    return FEDATTN_ERR_CUDA;
+}
+
 struct Context {
     int device;
     int sm_count;

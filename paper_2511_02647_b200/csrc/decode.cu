@@ -625,15 +625,18 @@ extern "C" fedattn_status fedattn_decode_noalloc(const fedattn_shape *shape, int
     if (!(shape->scale >= 0.f)) return FEDATTN_ERR_INVALID_ARG;
 
     int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return FEDATTN_ERR_CUDA;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess) return status_of(err);
+    if (dev < 0 || dev >= 64) return FEDATTN_ERR_CUDA;
     if (!g_decode_scratch_ptr[dev]) {
         // first call on this device: resolve the array's device address and the SM count
         float *ptr = nullptr;
-        if (cudaGetSymbolAddress((void **)&ptr, g_decode_scratch) != cudaSuccess || !ptr) return FEDATTN_ERR_CUDA;
         int sms = 0;
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-            return FEDATTN_ERR_CUDA;
-        if (set_decode_smem_attr() != cudaSuccess) return FEDATTN_ERR_CUDA;
+        err = cudaGetSymbolAddress((void **)&ptr, g_decode_scratch);
+        if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (err == cudaSuccess) err = set_decode_smem_attr();
+        if (err != cudaSuccess) return status_of(err);
+        if (!ptr || sms < 1) return FEDATTN_ERR_CUDA;
         g_decode_sm_count[dev] = sms;
         g_decode_scratch_ptr[dev] = ptr;
     }
@@ -649,7 +652,5 @@ extern "C" fedattn_status fedattn_decode_noalloc(const fedattn_shape *shape, int
     p.partial_bytes = kStaticScratchFloats * sizeof(float);
 
     // same kernels and grid rule as the workspace-backed call
-    if (launch_decode_split(p, dev, g_decode_sm_count[dev], static_cast<cudaStream_t>(stream), nullptr) != cudaSuccess)
-        return FEDATTN_ERR_CUDA;
-    return FEDATTN_OK;
+    return status_of(launch_decode_split(p, dev, g_decode_sm_count[dev], static_cast<cudaStream_t>(stream), nullptr));
 }
