@@ -55,7 +55,7 @@ def built(tmp_path_factory):
     cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
     src, so = tmp_path / "stand_in.cpp", tmp_path / "early.so"
     src.write_text(STAND_IN)
-    subprocess.check_call(["g++", "-O1", "-std=c++17", "-w", "-shared", "-fPIC", "-I", CSRC, "-I", os.path.join(ROOT, "include"), "-I", cuda,
+    subprocess.check_call(["g++", "-O1", "-std=c++17", "-w", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", CSRC, "-I", os.path.join(ROOT, "include"), "-I", cuda,
                            "-x", "c++", str(src), os.path.join(CSRC, "early_start.cu"), "-o", str(so)])
     return so
 
