@@ -25,7 +25,7 @@ __device__ __forceinline__ int find_segment(const int32_t *pre, int n, int32_t x
 __device__ __forceinline__ uint4 ld_stream(const uint4 *p)
 {
     uint4 r;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
     return r;
 }
@@ -584,11 +584,11 @@ gather_kernel(const PartsParams pp, int hkv, int64_t vpr /* 16-byte vectors per 
             const int h = (int)(rowid / T);
             const int32_t t = (int32_t)(rowid - (int64_t)h * T);
             const int n = find_segment(pp.cu_kv, pp.n, t);
-            const int32_t j = __ldg(sel_idx + rowid);
+            const int32_t j = ld_int(sel_idx + rowid);
             const int32_t len = pp.off[n + 1] - pp.off[n];
             // in range, and strictly above its predecessor inside the same (head, participant) block: the
             // aggregate's positions must come out ascending, which the attention over it relies on
-            if (j < 0 || j >= len || (t > pp.cu_kv[n] && __ldg(sel_idx + rowid - 1) >= j)) {
+            if (j < 0 || j >= len || (t > pp.cu_kv[n] && ld_int(sel_idx + rowid - 1) >= j)) {
                 bad |= vi == 0;
                 if (j < 0 || j >= len) continue;
             }

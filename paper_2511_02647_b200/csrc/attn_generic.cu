@@ -184,7 +184,7 @@ attn_tiled_kernel(const __grid_constant__ GenericParams p, const __grid_constant
         int lo = INT_MAX;
         if (r >= n_rows) lo = INT_MIN;                                       // no such row
         else if (p.mode == kLocal && p.causal) lo = row;
-        else if (by_pos) lo = p.remote_only ? p.cu[seg] - 1 : (p.q_pos ? __ldg(p.q_pos + row) : row);
+        else if (by_pos) lo = p.remote_only ? p.cu[seg] - 1 : (p.q_pos ? ld_int(p.q_pos + row) : row);
         s_lo[r] = lo;
         s_bad[r] = 0;
     }
@@ -216,7 +216,7 @@ attn_tiled_kernel(const __grid_constant__ GenericParams p, const __grid_constant
                 for (int i = 0; i < 1024 / kThreads; ++i) {
                     if (i * kThreads + tid < kv_hi - base) {
                         const int key = base + i * kThreads + tid;
-                        const int pos = __ldg(kvp + key);
+                        const int pos = ld_int(kvp + key);
                         if (pos <= lo_max || (two_sided && pos >= hi)) last = key;
                     }
                 }
@@ -254,7 +254,7 @@ attn_tiled_kernel(const __grid_constant__ GenericParams p, const __grid_constant
 #pragma unroll
         for (int j = 0; j < kJ; ++j) {
             const int key = min(key_l + 16 * j, kv_hi - 1 - kv_lo - t * kKeys) + kv_lo + t * kKeys;     // (past the end: the last one)
-            pos[j] = kvp && by_pos ? __ldg(kvp + key) : key;
+            pos[j] = kvp && by_pos ? ld_int(kvp + key) : key;
         }
     };
     if (rank < n_kt) load_pos(rank);

@@ -10,7 +10,7 @@
 namespace fedattn {
 
 template <typename T> __device__ __forceinline__ float ld_f(const T *p);
-template <> __device__ __forceinline__ float ld_f<float>(const float *p) { return __ldg(p); }
+template <> __device__ __forceinline__ float ld_f<float>(const float *p) { return __int_as_float(ld_int(reinterpret_cast<const int32_t *>(p))); }
 template <> __device__ __forceinline__ float ld_f<__nv_bfloat16>(const __nv_bfloat16 *p) {
     return __bfloat162float(*p);
 }

@@ -92,6 +92,20 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
     return r;
 }
 
+// the stream kernel's partials, past L1 (volatile: behind the wait for that kernel)
+__device__ __forceinline__ float2 ld_partial2(const float *p)
+{
+    float2 v;
+    asm volatile("ld.global.cg.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 ld_partial4(const float *p)
+{
+    float4 v;
+    asm volatile("ld.global.cg.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+
 // byte offset of 16-byte chunk `chunk` (0..15) of key row `row` inside a swizzled [64][128] bf16 tile
 __device__ __forceinline__ uint32_t swz(int row, int chunk) { return (uint32_t)(row * 256 + ((chunk ^ (row & 7)) << 4)); }
 
@@ -423,8 +437,8 @@ decode_merge_kernel(const DecodeParams p, int n_slots, int n_rows)
 #pragma unroll
         for (int k = 0; k < 4; ++k)
             if (k0 + k < s1) {
-                ml[k] = __ldcg(reinterpret_cast<const float2 *>(src + (size_t)(k0 + k) * kPartialStride));
-                v[k] = __ldcg(reinterpret_cast<const float4 *>(src + (size_t)(k0 + k) * kPartialStride + 4 + c4 * 4));
+                ml[k] = ld_partial2(src + (size_t)(k0 + k) * kPartialStride);
+                v[k] = ld_partial4(src + (size_t)(k0 + k) * kPartialStride + 4 + c4 * 4);
             }
         float mn = mm;
 #pragma unroll

@@ -389,7 +389,7 @@ __device__ __forceinline__ int count_le(const int32_t *pos, int n, int x)
     int lo = 0, hi = n;
     while (lo < hi) {
         const int mid = (lo + hi) >> 1;
-        if (__ldg(pos + mid) <= x) lo = mid + 1; else hi = mid;
+        if (ld_int(pos + mid) <= x) lo = mid + 1; else hi = mid;
     }
     return lo;
 }
@@ -403,12 +403,12 @@ __device__ __forceinline__ int count_le_warp(const int32_t *pos, int n, int x, i
     while (hi > lo) {
         const int width = hi - lo;
         if (width <= 32) {
-            const bool le = lane < width && __ldg(pos + lo + lane) <= x;
+            const bool le = lane < width && ld_int(pos + lo + lane) <= x;
             return lo + __popc(__ballot_sync(0xffffffffu, le));  // the entries <= x are a prefix
         }
         const int stride = (width + 31) >> 5;
         const int probe = min(lo + (lane + 1) * stride - 1, hi - 1);
-        const int k = __popc(__ballot_sync(0xffffffffu, __ldg(pos + probe) <= x));
+        const int k = __popc(__ballot_sync(0xffffffffu, ld_int(pos + probe) <= x));
         if (k == 32) return hi;                                 // even the last entry is <= x
         hi = min(lo + (k + 1) * stride - 1, hi - 1);            // entry `hi` is > x: the count is at most hi
         lo = lo + k * stride;
@@ -467,7 +467,7 @@ __device__ __forceinline__ PairRule pair_rule(const PrefillParams &p, const Item
     if (p.remote_only) rule.lo = p.cu[it.seg] - 1;
     else {
         const int row = sub.q_row0 + min(r, sub.n_valid - 1);
-        rule.lo = p.q_pos ? __ldg(p.q_pos + row) : row;
+        rule.lo = p.q_pos ? ld_int(p.q_pos + row) : row;
     }
     return rule;
 }
@@ -486,7 +486,7 @@ __device__ __forceinline__ int last_visible_tile(const KernelParams &kp, const I
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             const int key = base + 32 * i + lane;
-            if (key < T && any.sees(it.kvp ? __ldg(it.kvp + key) : key)) last = key;
+            if (key < T && any.sees(it.kvp ? ld_int(it.kvp + key) : key)) last = key;
         }
         last = __reduce_max_sync(0xffffffffu, last);
         if (last >= 0) return last / kKeys + 1;
@@ -557,18 +557,18 @@ __device__ __forceinline__ Item decode_item(const KernelParams &kp, int item, in
         // both sub-tiles walk what either may see
         const PosTables pt = pos_tables(p.tab, kp.n_qtiles, p.kv_head_major ? p.hkv : 1, kp.n_kt);
         const size_t first = p.kv_head_major ? (size_t)it.kvh * kp.n_kt : 0;
-        int q_max = __ldg(pt.q_max + (sub[1].q_row0 >> 7)), q_min = __ldg(pt.q_min + (sub[1].q_row0 >> 7));
+        int q_max = ld_int(pt.q_max + (sub[1].q_row0 >> 7)), q_min = ld_int(pt.q_min + (sub[1].q_row0 >> 7));
         if (two_rows && sub[0].n_valid > 0) {
-            q_max = max(q_max, __ldg(pt.q_max + (sub[0].q_row0 >> 7)));
-            q_min = min(q_min, __ldg(pt.q_min + (sub[0].q_row0 >> 7)));
+            q_max = max(q_max, ld_int(pt.q_max + (sub[0].q_row0 >> 7)));
+            q_min = min(q_min, ld_int(pt.q_min + (sub[0].q_row0 >> 7)));
         }
         int n = 0, last = 0, run = 0;                           // visible tiles, end of the last, leading run without a test
         bool in_run = true;
         for (int t0 = 0; t0 < kp.n_kt; t0 += 32) {
             const int t = min(t0 + lane, kp.n_kt - 1);
             const bool in = t0 + lane < kp.n_kt;
-            const uint32_t seen = __ballot_sync(0xffffffffu, in && __ldg(pt.kv_min + first + t) <= q_max);
-            const uint32_t free = __ballot_sync(0xffffffffu, in && __ldg(pt.kv_max + first + t) <= q_min);
+            const uint32_t seen = __ballot_sync(0xffffffffu, in && ld_int(pt.kv_min + first + t) <= q_max);
+            const uint32_t free = __ballot_sync(0xffffffffu, in && ld_int(pt.kv_max + first + t) <= q_min);
             const int at = n + __popc(seen & ((1u << lane) - 1u));
             if (((seen >> lane) & 1u) && at < kWalkMost) walk[at] = (uint16_t)(t | (((free >> lane) & 1u) << 15));
             n += __popc(seen);
@@ -924,7 +924,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             bool bad = false;
             for (int64_t i = (int64_t)blockIdx.x * 32 + lane; i < total; i += (int64_t)gridDim.x * 32) {
                 const int64_t a = i / per, e = a * p.total_kv + (i - a * per);
-                bad |= __ldg(p.kv_pos + e) > __ldg(p.kv_pos + e + 1);
+                bad |= ld_int(p.kv_pos + e) > ld_int(p.kv_pos + e + 1);
             }
             if (bad) atomicMax(kp.status, (int32_t)FEDATTN_ERR_ORDER);
         }
@@ -1120,7 +1120,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 #pragma unroll
                 for (int c = 0; c < kChunks; ++c) {
                     const int key = j * kKeys + 32 * c + lane;
-                    kpos[c] = it.kvp ? __ldg(it.kvp + min(key, T - 1)) : key;
+                    kpos[c] = it.kvp ? ld_int(it.kvp + min(key, T - 1)) : key;
                 }
             };
             if (pairs) {
@@ -1132,7 +1132,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                 // every (query, key) pair on its own positions
                 n_full = it.b;
                 const int row = sub.q_row0 + min(r, sub.n_valid - 1);
-                p_row = p.q_pos ? __ldg(p.q_pos + row) : row;
+                p_row = p.q_pos ? ld_int(p.q_pos + row) : row;
             } else {
                 if (p.sync && p.remote_only) {
                     c_row = it.a;                               // the same for every row of the segment
@@ -1142,7 +1142,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
                     // that can tell these rows apart (more only if positions repeat: then each lane searches).
                     const int T = (int)p.total_kv, p0 = sub.q_row0 + (r & ~31);
                     const int cw = count_le_warp(it.kvp, T, p0 - 1, lane);
-                    const int wv = cw + lane < T ? __ldg(it.kvp + cw + lane) : INT32_MAX;
+                    const int wv = cw + lane < T ? ld_int(it.kvp + cw + lane) : INT32_MAX;
                     int cnt = 0;
 #pragma unroll
                     for (int jj = 0; jj < 32; ++jj) cnt += __shfl_sync(0xffffffffu, wv, jj) <= p0 + lane;
@@ -1207,7 +1207,7 @@ prefill_sm100_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 #pragma unroll 4
                             for (int i = 0; i < 32; ++i) {
                                 const int key = cb + i;
-                                const int kpos = it.kvp ? __ldg(it.kvp + min(key, T - 1)) : key;
+                                const int kpos = it.kvp ? ld_int(it.kvp + min(key, T - 1)) : key;
                                 if (key < T && kpos <= p_row) m |= 1u << i;
                             }
                             vm[c] = m;
@@ -1431,7 +1431,7 @@ __device__ __forceinline__ void tile_min_max(const int32_t *pos, int64_t n, int6
     for (int e = 0; e < 4; ++e) {
         const int64_t i = i0 + e;
         if (i < n) {
-            const int v = pos ? __ldg(pos + i) : (int)i;
+            const int v = pos ? ld_int(pos + i) : (int)i;
             mn = min(mn, v); mx = max(mx, v);
         }
     }
