@@ -10,6 +10,8 @@ from typing import Optional, Sequence
 
 import torch
 
+from .build import marshal_path
+
 _PKG = os.path.dirname(os.path.abspath(__file__))
 # FEDATTN_LIBRARY overrides the path of the shared library (e.g. an instrumented build).
 _LIB_PATH = os.environ.get("FEDATTN_LIBRARY") or os.path.join(_PKG, "lib", "libfedattn.so")
@@ -50,7 +52,7 @@ def library_path() -> str:
 
 def _load_marshal():
     """The native marshalling module (csrc/marshal.cpp), built beside the library."""
-    name, path = "_fedattn_marshal", os.path.join(_PKG, "lib", "_fedattn_marshal.so")
+    name, path = "_fedattn_marshal", marshal_path()
     if not os.path.exists(path):
         raise ImportError("FedAttn marshalling module missing: %s (run `python paper_2511_02647_b200/build.py` "
                           "or __graft_entry__.build()); there is no fallback path" % path)

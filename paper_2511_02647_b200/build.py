@@ -12,7 +12,6 @@ CSRC = os.path.join(_PKG, "csrc")
 LIB_DIR = os.path.join(_PKG, "lib")
 LIB_PATH = os.path.join(LIB_DIR, "libfedattn.so")
 MARSHAL_SRC = os.path.join(CSRC, "marshal.cpp")
-MARSHAL_PATH = os.path.join(LIB_DIR, "_fedattn_marshal.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC"]
@@ -30,22 +29,32 @@ def _stale() -> bool:
     return any(os.path.getmtime(p) > t for p in deps)
 
 
+def marshal_path() -> str:
+    """Where the marshalling module for the running interpreter and torch is.  It is compiled against the layouts in torch's
+    headers, which no symbol version guards: one built for another torch must not be found, let alone loaded."""
+    import sysconfig
+    import torch
+    tag = "%s-%s" % (torch.__version__, (torch.version.git_version or "")[:8])
+    return os.path.join(LIB_DIR, "_fedattn_marshal-torch%s%s" % (tag, sysconfig.get_config_var("EXT_SUFFIX")))
+
+
 def build_marshal(force: bool = False) -> str:
     """Compile the binding's native marshalling module (a CPython extension against torch's headers)."""
-    if not force and os.path.exists(MARSHAL_PATH) and os.path.getmtime(MARSHAL_PATH) >= os.path.getmtime(MARSHAL_SRC):
-        return MARSHAL_PATH
+    path = marshal_path()
+    if not force and os.path.exists(path) and os.path.getmtime(path) >= os.path.getmtime(MARSHAL_SRC):
+        return path
     import sysconfig
     import torch
     inc = os.path.join(os.path.dirname(torch.__file__), "include")
     lib = os.path.join(os.path.dirname(torch.__file__), "lib")
-    tmp = MARSHAL_PATH + ".tmp%d" % os.getpid()
+    tmp = path + ".tmp%d" % os.getpid()
     subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC",
                            "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
                            "-I", sysconfig.get_paths()["include"], "-I", inc,
                            "-I", os.path.join(inc, "torch", "csrc", "api", "include"), MARSHAL_SRC, "-o", tmp,
                            "-L", lib, "-ltorch_python", "-ltorch_cpu", "-lc10"])
-    os.replace(tmp, MARSHAL_PATH)
-    return MARSHAL_PATH
+    os.replace(tmp, path)
+    return path
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

@@ -1,12 +1,17 @@
 """Argument arrays of the binding: what the native module packs, and what it leaves to the general path."""
 import ctypes as C
+import os
 import struct
+import subprocess
+import sys
 
 import numpy as np
 import pytest
 import torch
 
 import paper_2511_02647_b200.binding as b
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def words(x, fmt):
@@ -41,3 +46,27 @@ def test_int32s(xs):
 
 def test_int32s_beyond_32_bits_wrap_as_ctypes_does():
     assert words(b._i32_array([2 ** 32 + 5, 1]), "i") == words(bytes((C.c_int32 * 2)(2 ** 32 + 5, 1)), "i")
+
+
+def in_a_process(code, **env):
+    return subprocess.run([sys.executable, "-c", code], cwd=ROOT, env={**os.environ, **env}, capture_output=True, text=True)
+
+
+LOADED = "any('_fedattn_marshal' in x for x in open('/proc/self/maps'))"
+
+
+@pytest.mark.parametrize("change,loaded", [("", True), ("torch.__version__ = torch.__version__ + '.1'", False),
+                                           ("torch.version.git_version = '0' * 40", False),
+                                           ("import sysconfig; sysconfig.get_config_vars()['EXT_SUFFIX'] = '.cpython-399.so'", False)])
+def test_module_of_another_torch_or_python_is_not_loaded(change, loaded):
+    """The module reads torch's own layouts: the one in the tree is for one torch build and one interpreter."""
+    code = """
+import torch
+%s
+try:
+    import paper_2511_02647_b200
+except ImportError:
+    pass
+print(%s)
+"""
+    assert in_a_process(code % (change, LOADED)).stdout.strip() == str(loaded)
