@@ -6,6 +6,7 @@ import ctypes as C
 import importlib.machinery
 import importlib.util
 import os
+import warnings
 from typing import Optional, Sequence
 
 import torch
@@ -50,16 +51,29 @@ def library_path() -> str:
     return _LIB_PATH
 
 
+class _AllThroughCtypes:
+    """What stands for the marshalling module where there is none: it takes nothing."""
+
+    @staticmethod
+    def pointer(_):
+        return None
+
+    pointers = int32s = pointer
+
+
 def _load_marshal():
-    """The native marshalling module (csrc/marshal.cpp), built beside the library."""
+    """The native marshalling module (csrc/marshal.cpp).  It only saves host time: without one for this torch and this
+    interpreter (a library from elsewhere, a tree built earlier, no Python headers) the same calls go through ctypes."""
     name, path = "_fedattn_marshal", marshal_path()
-    if not os.path.exists(path):
-        raise ImportError("FedAttn marshalling module missing: %s (run `python paper_2511_02647_b200/build.py` "
-                          "or __graft_entry__.build()); there is no fallback path" % path)
-    loader = importlib.machinery.ExtensionFileLoader(name, path)
-    module = importlib.util.module_from_spec(importlib.util.spec_from_loader(name, loader))
-    loader.exec_module(module)
-    return module
+    try:
+        loader = importlib.machinery.ExtensionFileLoader(name, path)
+        module = importlib.util.module_from_spec(importlib.util.spec_from_loader(name, loader))
+        loader.exec_module(module)
+        return module
+    except ImportError as e:
+        warnings.warn("FedAttn marshalling module not loaded (%s): arguments go through ctypes, 10 us more for an "
+                      "aggregation of 16 participants; `python paper_2511_02647_b200/build.py` builds it" % e, RuntimeWarning)
+        return _AllThroughCtypes
 
 
 def _load():

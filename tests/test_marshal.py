@@ -1,6 +1,7 @@
 """Argument arrays of the binding: what the native module packs, and what it leaves to the general path."""
 import ctypes as C
 import os
+import shutil
 import struct
 import subprocess
 import sys
@@ -70,3 +71,23 @@ except ImportError:
 print(%s)
 """
     assert in_a_process(code % (change, LOADED)).stdout.strip() == str(loaded)
+
+
+def test_package_without_the_module(tmp_path):
+    """A library named by FEDATTN_LIBRARY, a package folder without any build: it imports, says so, and packs the same."""
+    shutil.copytree(os.path.join(ROOT, "paper_2511_02647_b200"), tmp_path / "paper_2511_02647_b200", ignore=shutil.ignore_patterns("lib"))
+    code = """
+import sys, warnings
+sys.path.insert(0, %r)
+with warnings.catch_warnings(record=True) as caught:
+    warnings.simplefilter("always")
+    import paper_2511_02647_b200.binding as b
+import torch
+t = torch.empty(3)
+assert b.__file__.startswith(%r) and any("marshalling module" in str(w.message) for w in caught)
+assert bytes(b._i32_array([1, -2])) == bytes((b.C.c_int32 * 2)(1, -2))
+assert bytes(b._ptr_array([t, None])) == bytes((b.C.c_void_p * 2)(t.data_ptr(), None)) and b._ptr(t) == t.data_ptr()
+print(b.status_string(0))
+""" % (str(tmp_path), str(tmp_path))
+    res = in_a_process(code, FEDATTN_LIBRARY=b.library_path())
+    assert res.stdout.strip() == "ok", res.stderr
