@@ -38,6 +38,11 @@ def marshal_path() -> str:
     return os.path.join(LIB_DIR, "_fedattn_marshal-torch%s%s" % (tag, sysconfig.get_config_var("EXT_SUFFIX")))
 
 
+def missing() -> list:
+    """The files that build() makes and that are not there."""
+    return [p for p in (LIB_PATH, marshal_path()) if not os.path.exists(p)]
+
+
 def build_marshal(force: bool = False) -> str:
     """Compile the binding's native marshalling module (a CPython extension against torch's headers)."""
     path = marshal_path()

@@ -13,13 +13,13 @@ def pytest_configure(config):
 
 
 def pytest_sessionstart(session):
-    """Build the C-ABI library when it is missing (nvcc cross-compiles without a GPU).  The package
-    itself never builds or falls back: it raises when the library is absent."""
+    """Build what is missing of the C-ABI library and the marshalling module (nvcc cross-compiles without a GPU).
+    The package itself never builds: it raises when the library is absent."""
     import importlib.util
     spec = importlib.util.spec_from_file_location("_fedattn_build", os.path.join(ROOT, "paper_2511_02647_b200", "build.py"))
     mod = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(mod)
-    if not os.path.exists(mod.LIB_PATH):
+    if mod.missing():
         mod.build()
 
 

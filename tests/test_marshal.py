@@ -1,6 +1,7 @@
 """Argument arrays of the binding: what the native module packs, and what it leaves to the general path."""
 import ctypes as C
 import os
+import re
 import shutil
 import struct
 import subprocess
@@ -91,3 +92,18 @@ print(b.status_string(0))
 """ % (str(tmp_path), str(tmp_path))
     res = in_a_process(code, FEDATTN_LIBRARY=b.library_path())
     assert res.stdout.strip() == "ok", res.stderr
+
+
+@pytest.mark.parametrize("absent", ["LIB_PATH", "module"])
+def test_what_is_missing_is_built(absent, tmp_path, monkeypatch):
+    """The test session and smoke() build when either file is absent, not for the library alone."""
+    import paper_2511_02647_b200.build as build
+    lib, module = tmp_path / "libfedattn.so", tmp_path / "module.so"
+    (module if absent == "LIB_PATH" else lib).touch()
+    monkeypatch.setattr(build, "LIB_PATH", str(lib))
+    monkeypatch.setattr(build, "marshal_path", lambda: str(module))
+    assert build.missing() == [str(lib if absent == "LIB_PATH" else module)]
+    for path in ("tests/conftest.py", "__graft_entry__.py"):
+        with open(os.path.join(ROOT, path)) as f:
+            src = f.read()
+        assert re.search(r"if \S*\.missing\(\):\n +\S*build\(\)", src) and "path.exists" not in src, path
