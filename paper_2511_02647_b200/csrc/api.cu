@@ -63,8 +63,9 @@ cudaError_t launch_prefill(Context *c, const PrefillParams &p, int dtype, cudaSt
         max_kv = 0;
         for (int n = 0; n < p.n_seg; ++n) max_kv = p.cu[n + 1] - p.cu[n] > max_kv ? p.cu[n + 1] - p.cu[n] : max_kv;
     }
-    c->released = false;
-    return launch_attn_generic(generic_params(p), dtype, (int)max_kv, c->sm_count, s, &c->launches);
+    const cudaError_t err = launch_attn_generic(generic_params(p), dtype, (int)max_kv, c->sm_count, s, &c->launches);
+    if (err == cudaSuccess) front_note(c->device, s, false);
+    return err;
 }
 
 struct DeviceGuard {
@@ -139,7 +140,6 @@ fedattn_status fedattn_create(fedattn_ctx **out, int device, void *workspace, si
     c.tc_launches = 0;
     c.agg_seq = 0;
     c.agg_key = ~0ull;
-    c.released = false;
     c.encode_tiled = nullptr;
     if (prop.major == 10) {
         void *fn = nullptr;
@@ -253,9 +253,9 @@ fedattn_status fedattn_aggregate_kv(fedattn_ctx *ctx, const fedattn_shape *shape
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int hkv = shape->n_kv_heads, d = shape->head_dim, eb = elt_bytes(shape);
     cudaError_t err = cudaSuccess;
-    ctx->c.released = mode != FEDATTN_AGG_CONCAT;
     if (mode == FEDATTN_AGG_CONCAT) {
         err = launch_concat(pp, hkv, d, eb, k_agg, v_agg, kv_pos, cu_kv, s, ctx->c.sm_count, &ctx->c.launches);
+        if (err == cudaSuccess) front_note(ctx->c.device, s, false);
         return status_of(err);
     }
     if (mode == FEDATTN_AGG_TOPK_KNORM) {
@@ -336,9 +336,10 @@ fedattn_status fedattn_merge(fedattn_ctx *ctx, const fedattn_shape *shape, int64
     if (!aligned16(o_a) || !aligned16(o_b) || !aligned16(o)) return FEDATTN_ERR_INVALID_ARG;
     DeviceGuard g(ctx->c.device);
     if (g.err != cudaSuccess) return status_of(g.err);
-    ctx->c.released = false;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
     cudaError_t err = launch_merge(shape->dtype, n_rows, shape->n_q_heads, shape->head_dim, o_a, lse_a, o_b, lse_b, o, lse,
-                                   ctx->c.sm_count, static_cast<cudaStream_t>(stream), &ctx->c.launches);
+                                   ctx->c.sm_count, s, &ctx->c.launches);
+    if (err == cudaSuccess) front_note(ctx->c.device, s, false);
     return status_of(err);
 }
 
@@ -360,8 +361,7 @@ fedattn_status fedattn_decode(fedattn_ctx *ctx, const fedattn_shape *shape, int3
     cudaError_t err;
     const int N = shape->n_participants;
     const size_t need = decode_scratch_bytes(N, shape->n_q_heads, shape->head_dim, ctx->c.sm_count);
-    ctx->c.released = shape->dtype == FEDATTN_BF16 && shape->head_dim == 128 && need > 0;
-    if (ctx->c.released) {
+    if (shape->dtype == FEDATTN_BF16 && shape->head_dim == 128 && need > 0) {
         if (ctx->c.scratch_bytes < need) return FEDATTN_ERR_WORKSPACE;
         DecodeParams p;
         memset(&p, 0, sizeof(p));
@@ -382,6 +382,7 @@ fedattn_status fedattn_decode(fedattn_ctx *ctx, const fedattn_shape *shape, int3
         p.kv_head_stride = shape->head_dim;
         p.kv_len = kv_len; p.cache_stride = cache_stride;
         err = launch_attn_generic(p, shape->dtype, max_kv_len, ctx->c.sm_count, s, &ctx->c.launches);
+        if (err == cudaSuccess) front_note(ctx->c.device, s, false);
     }
     return status_of(err);
 }

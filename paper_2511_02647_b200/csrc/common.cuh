@@ -49,7 +49,6 @@ struct Context {
     int64_t tc_launches;   // launches of the tcgen05 attention kernel among them
     int64_t agg_seq;       // sequence number of the latest sparse aggregation call
     uint64_t agg_key;      // key of the stream that call ran on (early-start bookkeeping)
-    bool released;         // the latest call releases its dependents early (selection, gather, bf16 decode)
     void *encode_tiled;    // cuTensorMapEncodeTiled entry point (driver), or nullptr
 };
 
@@ -79,6 +78,11 @@ EarlyStart early_start(int device, cudaStream_t stream, const MemRange *in, int 
 // Behind the call's last launch, or where it ends without one; returns e.  A call that was not launched leaves no record of
 // the grids before it behind.  While the stream is being captured, notes the node that the last launch became.
 cudaError_t early_start_end(const EarlyStart &r, cudaError_t e);
+// Whether the latest kernel that this library put on the stream, by any context or none, releases its dependents early
+// (selection, gather, bf16 decode: early_start_end notes them; the others note themselves).  A hint for the form of a
+// launch, kept for a few streams; no order rests on it.
+bool front_releases(int device, cudaStream_t stream);
+void front_note(int device, cudaStream_t stream, bool releases);
 // The owner's sequence numbers are about to lose their meaning (its context is being destroyed).
 void early_start_forget(int device, const void *owner);
 

@@ -33,6 +33,7 @@
 //     also from those of other streams of the capture, whose buffers its record does not hold.  So a captured
 //     call waits first unless the stream's one dependency is the last kernel of its latest recorded call.
 //     (Behind any other kernel waiting costs nothing: what releases nothing early has ended by then.)
+#include <atomic>
 #include <memory>
 #include <mutex>
 
@@ -60,6 +61,14 @@ struct DeviceRecord {
 };
 std::unique_ptr<DeviceRecord> g_record[64];
 std::mutex g_record_mutex;
+
+// Streams whose latest kernel of this library releases early, oldest first.  Most programs have none most of the time: the
+// count spares the other calls the lock.
+struct Fronts {
+    cudaStream_t stream[kSlots];
+    std::atomic<int> n{0};
+};
+Fronts g_fronts[64];
 
 struct Range {
     uintptr_t lo, hi;
@@ -198,6 +207,34 @@ EarlyStart early_start(int device, cudaStream_t stream, const MemRange *in, int 
     return r;
 }
 
+bool front_releases(int device, cudaStream_t stream)
+{
+    Fronts &f = g_fronts[device & 63];
+    if (f.n.load(std::memory_order_relaxed) == 0) return false;
+    std::lock_guard<std::mutex> lock(g_record_mutex);
+    for (int i = 0; i < f.n; ++i)
+        if (f.stream[i] == stream) return true;
+    return false;
+}
+
+void front_note(int device, cudaStream_t stream, bool releases)
+{
+    Fronts &f = g_fronts[device & 63];
+    if (!releases && f.n.load(std::memory_order_relaxed) == 0) return;
+    std::lock_guard<std::mutex> lock(g_record_mutex);
+    int n = 0;
+    for (int i = 0; i < f.n; ++i)
+        if (f.stream[i] != stream) f.stream[n++] = f.stream[i];
+    if (releases) {
+        if (n == kSlots) {
+            for (int i = 1; i < n; ++i) f.stream[i - 1] = f.stream[i];
+            --n;
+        }
+        f.stream[n++] = stream;
+    }
+    f.n = n;
+}
+
 cudaError_t early_start_end(const EarlyStart &r, cudaError_t e)
 {
     if (e != cudaSuccess) {
@@ -206,6 +243,7 @@ cudaError_t early_start_end(const EarlyStart &r, cudaError_t e)
         if (DeviceRecord *dev = g_record[r.device & 63].get()) dev->n_slots = 0;
         return e;
     }
+    front_note(r.device, r.stream, true);
     if (!r.capturing) return e;
     const Capture cap = capture_of(r.stream);
     std::lock_guard<std::mutex> lock(g_record_mutex);

@@ -1730,18 +1730,19 @@ cudaError_t launch_prefill_sm100(Context *ctx, const PrefillParams &p, cudaStrea
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    // Set up while the preceding grid ends, but behind a call of this context that releases its dependents early launched as
-    // usual: there the CTAs would take whatever SMs that grid leaves one by one (sparse sync behind its selection 569 us, 577
-    // set up early; bidirectional local + remote behind theirs 115.5, 117.0).  Elsewhere the early set-up gains: ragged round
-    // with 64 channels 84.3 -> 80.2, local of 4 x 2048 154.2 -> 152.5, dense sync 523.8 -> 518.5.  (The barriers and the TMEM
-    // set up before the wait: 79.5, 155.7, 533.7.)
+    // Set up while the preceding grid ends, but behind a kernel that releases its dependents early launched as usual: there
+    // the CTAs would take whatever SMs that grid leaves one by one (sparse sync behind its selection 569 us, 577 set up
+    // early; bidirectional local + remote behind theirs 115.5, 117.0).  Elsewhere the early set-up gains where calls are short
+    // (ragged round with 64 channels 84.3 -> 80.2) and costs nothing where they are long.  (The barriers and the TMEM set up
+    // before the wait: 79.5, local of 4 x 2048 152.5 -> 155.7, dense sync 518.5 -> 533.7.)  In front of a call with explicit
+    // query positions stands the kernel of its tables.
     WaitFirstLaunch l(dim3((unsigned)blocks), dim3(kThreads), smem, s);
-    if (ctx->released) l.cfg.numAttrs = 0;
-    ctx->released = false;
+    if (!p.general && front_releases(ctx->device, s)) l.cfg.numAttrs = 0;
     cudaError_t e = cudaLaunchKernelEx(&l.cfg, kernels[which], mq, mk, mv, mo, kp);
     ++ctx->launches;
     ++ctx->tc_launches;
     if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess) front_note(ctx->device, s, false);
     if (e != cudaSuccess && getenv("FEDATTN_DEBUG")) fprintf(stderr, "prefill_sm100_kernel launch: %s\n", cudaGetErrorString(e));
     return e;
 }
