@@ -155,3 +155,112 @@ def test_captured_branches_that_join():
         assert ctx.poll() == 0 and ctx2.poll() == 0
         for a, b in zip((ks, vs, kg, vg, sel, o), want):
             assert torch.equal(a, b)
+
+
+def run_ragged(dtype, d, hq, hkv, seed, mode, n_ops=48):
+    """Random calls of two contexts over ragged segments (empty ones and one of a single token among them; the bf16
+    attention gets more items than there are SMs): explicit query positions, whose tables share the scratch with the
+    decode partials, both masks, remote-only attention, whole tokens, empty selections, no keys at all."""
+    m, lens = fa(), [0, 1, 700, 257, 1300, 0]
+    N, T = len(lens), sum(lens)
+    cu, keep = np.concatenate([[0], np.cumsum(lens)]).tolist(), [min(x, 90) for x in lens]
+    K, dt = sum(keep), torch.bfloat16 if dtype == "bf16" else torch.float32
+    shape, both = (m.Shape(N, hq, hkv, d, m.BF16 if dtype == "bf16" else m.F32, causal) for causal in (1, 0))
+    contexts = [m.Context(shape, T, T) for _ in range(2)]
+    g = torch.Generator(device="cuda").manual_seed(9)
+
+    def new(*s):
+        return torch.randn(s, generator=g, device="cuda").to(dt)
+
+    def ints(*s):
+        return torch.zeros(s, dtype=torch.int32, device="cuda")
+
+    q, k, v, k2, v2 = new(T, hq, d), new(T, hkv, d), new(T, hkv, d), new(T, hkv, d), new(T, hkv, d)
+    o, lse = [torch.zeros_like(q) for _ in range(3)], [torch.zeros(T, hq, device="cuda") for _ in range(3)]
+    od, od2, cap = torch.zeros(N, hq, d, dtype=dt, device="cuda"), torch.zeros(N, hq, d, dtype=dt, device="cuda"), T // N
+    kt, vt, post, sel, cut = *(torch.zeros(hkv, K, d, dtype=dt, device="cuda") for _ in range(2)), ints(hkv, K), ints(hkv, K), ints(N + 1)
+    kw, vw, posw, selw = *(torch.zeros(K, hkv, d, dtype=dt, device="cuda") for _ in range(2)), ints(K), ints(K)
+    q_pos = torch.randperm(T, generator=g, device="cuda").int()
+    kv_pos = torch.arange(T, dtype=torch.int32, device="cuda")
+    n_loc, n_all = torch.full((N,), cap, dtype=torch.int32, device="cuda"), torch.tensor([T], dtype=torch.int32, device="cuda")
+    none = ints(0)
+    state = [*o, *lse, od, od2, kt, vt, post, sel, cut, kw, vw, posw, selw, k2, v2]
+
+    def split(x):
+        return [x[cu[i]:cu[i + 1]] for i in range(N)]
+
+    calls = [
+        lambda c, s: m.fedattn_local(c, shape, q, k, v, cu, o[0], lse[0], stream=s),
+        lambda c, s: m.fedattn_local(c, both, q, k, v2, cu, o[1], lse[1], stream=s),
+        lambda c, s: m.fedattn_aggregate_kv(c, shape, m.AGG_CONCAT, split(k), split(v), lens, None, None, k2, v2, None, None, None, stream=s),
+        lambda c, s: m.fedattn_sync(c, shape, q, None, k2, v2, None, T, False, o[1], lse[1], stream=s),
+        lambda c, s: m.fedattn_sync(c, both, q, None, kw, vw, posw, K, False, o[2], lse[2], stream=s),
+        lambda c, s: m.fedattn_sync(c, shape, q, q_pos, k2, v2, kv_pos, T, False, o[0], lse[0], stream=s),
+        lambda c, s: m.fedattn_sync(c, shape, q, q_pos, kt, vt, post, K, True, o[1], lse[1], stream=s),
+        lambda c, s: m.fedattn_sync(c, shape, q, None, None, None, None, 0, False, o[2], lse[2], stream=s),
+        lambda c, s: m.fedattn_sync_remote(c, shape, q, cu, kt, vt, post, K, True, o[1], lse[1], stream=s),
+        lambda c, s: m.fedattn_sync_remote(c, both, q, cu, kw, vw, posw, K, False, o[2], lse[2], stream=s),
+        lambda c, s: m.fedattn_merge(c, shape, T, o[0], lse[0], o[1], lse[1], o[2], lse[2], stream=s),
+        lambda c, s: m.fedattn_merge(c, shape, T, o[2], lse[2], o[1], lse[1], o[1], lse[1], stream=s),
+        lambda c, s: m.fedattn_decode(c, shape, m.DECODE_LOCAL, o[2][:N], k2, v2, cap * hkv * d, n_loc, cap, od, stream=s),
+        lambda c, s: m.fedattn_decode(c, shape, m.DECODE_SYNC, od, k2, v2, 0, n_all, T, o[0][:N], stream=s),
+        lambda c, s: m.fedattn_decode(c, shape, m.DECODE_SYNC, o[1][:N], k2, v2, 0, n_all, 1 << 20, od2, stream=s),   # two launches
+        lambda c, s: m.fedattn_aggregate_kv(c, shape, m.AGG_TOPK_KNORM, split(k2), split(v2), lens, keep, None, kt, vt, post, cut, sel, stream=s),
+        lambda c, s: m.fedattn_aggregate_kv(c, shape, m.AGG_TOPK_TOKEN, split(k2), split(v), lens, keep, None, kw, vw, posw, cut, selw, stream=s),
+        lambda c, s: m.fedattn_aggregate_kv(c, shape, m.AGG_INDEXED, split(k), split(v2), lens, keep, sel, kt, vt, post, cut, None, stream=s),
+        lambda c, s: m.fedattn_aggregate_kv(c, shape, m.AGG_INDEXED, split(k2), split(v2), lens, [0] * N, none, stream=s),
+        lambda c, s: m.fedattn_aggregate_kv(c, shape, m.AGG_TOPK_KNORM, split(k2), split(v2), lens, [0] * N, None, None, None, None, cut, stream=s),
+    ]
+    if dtype == "bf16" and d == 128:
+        calls.append(lambda c, s: m.fedattn_decode_noalloc(shape, m.DECODE_SYNC, od2, k2, v2, 0, n_all, T, o[2][:N], stream=s))
+    for i in (15, 16, 0, 3):                                    # what a first call sets up, and selections to start from
+        calls[i](contexts[0], None)
+    r = np.random.default_rng(seed)
+    order, who = r.integers(0, len(calls), n_ops), r.integers(0, 2, n_ops)
+    snaps = [[torch.zeros_like(x) for x in (*o, od, kt)] for _ in range(n_ops // 8)]
+    start = [x.clone() for x in state]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+
+    def walk(two):
+        turn = r.integers(0, 2, n_ops)
+        for i, c in enumerate(order):
+            s = streams[turn[i] if two else 0]
+            if two:
+                s.wait_stream(streams[1 - turn[i]])
+            calls[c](contexts[who[i]], s)
+            if mode == "synchronised":
+                torch.cuda.synchronize()
+            if i % 8 == 7:
+                with torch.cuda.stream(s):
+                    for a, b in zip(snaps[i // 8], (*o, od, kt)):
+                        a.copy_(b)
+        if two:
+            streams[0].wait_stream(streams[1])
+
+    if mode.startswith("graph"):
+        for i in (5, 6, 8, 9, 10, 12, 13, 14, 17, len(calls) - 1):
+            calls[i](contexts[0], None)
+        for a, b in zip(state, start):
+            a.copy_(b)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=streams[0]):
+            if mode == "graph of two streams":
+                streams[1].wait_stream(streams[0])
+            walk(mode == "graph of two streams")
+        graph.replay()
+    else:
+        walk(mode == "two streams")
+    torch.cuda.synchronize()
+    assert all(c.poll() == 0 for c in contexts)
+    return [x for s in snaps for x in s] + state
+
+
+@pytest.mark.parametrize("dtype,d,hq,hkv", [("f32", 64, 4, 2), ("bf16", 64, 8, 4), ("bf16", 128, 32, 8)])
+@pytest.mark.parametrize("seed", range(3))
+def test_ragged_sequences_without_synchronisation(dtype, d, hq, hkv, seed):
+    want = run_ragged(dtype, d, hq, hkv, seed, "synchronised")
+    for mode in ("free", "graph", "two streams", "graph of two streams"):
+        for i, (a, b) in enumerate(zip(run_ragged(dtype, d, hq, hkv, seed, mode), want)):
+            assert torch.equal(a, b), (mode, i)
