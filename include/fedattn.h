@@ -16,7 +16,8 @@
  *   - Work is enqueued on the given stream (a cudaStream_t passed as void*; NULL = default
  *     stream) and the call returns without synchronising.
  *   - Errors are return codes.  Arguments are validated on the host before anything is
- *     launched; a rejected call launches nothing.  A device-side anomaly (a bounded wait that
+ *     launched; a rejected call launches nothing.  FEDATTN_ERR_CUDA leaves no error with the
+ *     runtime that a later call would find.  A device-side anomaly (a bounded wait that
  *     ran out, an out-of-range or unsorted index in INDEXED mode, positions in an order the call
  *     cannot handle) sets a status word in the workspace that fedattn_poll reads; the kernel still
  *     terminates and the context stays usable.  Outputs of the call that raised the status are
@@ -33,10 +34,17 @@
  *   - One context serves one stream at a time: calls that share a context and may overlap on
  *     the GPU race on its workspace.
  *   - Results are those of stream order: every call behaves as if it ran after all earlier work
- *     of its stream and before all later work.  fedattn_decode and the sparse modes of
- *     fedattn_aggregate_kv are launched with programmatic stream serialization and may touch
- *     their buffers before the preceding kernel of the stream has ended; the library tracks the
- *     buffers of such calls and holds a call back whenever that could be observed.  What the
+ *     of its stream and before all later work.  Kernels are launched with programmatic stream
+ *     serialization, in two ways.  fedattn_decode (bf16, head_dim 128), fedattn_decode_noalloc and
+ *     the sparse modes of fedattn_aggregate_kv may touch their buffers before the preceding kernel
+ *     of the stream has ended, and let the next one start before they end; the library tracks the
+ *     buffers of such calls and holds a call back whenever that could be observed.  All others
+ *     wait for everything before them before they touch anything, and let nothing start early.
+ *     Launched the ordinary way are the self-test, the kernel that prepares a bf16 head_dim 128
+ *     sync call with query positions, and bf16 attention directly behind a call of the first kind.
+ *     In a stream capture the programmatic launches get programmatic edges, from every kernel that
+ *     the stream then depends on; one of the first kind that does not directly follow another on
+ *     its own stream waits before it reads.  What the
  *     caller has to keep: a kernel of the caller's own that is launched with the programmatic
  *     attribute into the same stream executes griddepcontrol.wait before it ends (kernels
  *     launched the ordinary way need nothing), and buffers shared with work on OTHER streams are
@@ -151,7 +159,8 @@ fedattn_status fedattn_local(fedattn_ctx *ctx, const fedattn_shape *shape,
  *   of one packed buffer).  seqlens_host host int32 [N].  k_sel_host host int32 [N], 0 <= k_sel[n]
  *   <= L_n (ignored for CONCAT).  Both TOPK modes need L_n <= 4096 per participant (else
  *   UNSUPPORTED).
- *   kv_pos and cu_kv may be NULL when not wanted. */
+ *   kv_pos and cu_kv may be NULL when not wanted.  A sparse call that selects nothing (T = 0) and
+ *   has no cu_kv to write launches nothing. */
 typedef enum {
     FEDATTN_AGG_CONCAT = 0,
     FEDATTN_AGG_TOPK_KNORM = 1,

@@ -90,9 +90,14 @@ void early_start_forget(int device, const void *owner);
 // preceding grid of the stream ends, instead of behind its end, and it completes behind that grid like an ordinary launch.
 // It releases nothing early, so it needs no record below.  Bound by launches and the gaps between them, the fp32 round of
 // two 128-token participants (local, concatenation, sync) takes 24.6 us with ordinary launches and 19.7-20.6 with these; the
-// round of six ragged bf16 segments, 16 / 4 heads of 64, 84.4 -> 82.4; local + remote + merge of 2160 tokens 120.1 -> 117.7;
-// decode with a suffix 12.7 -> 11.7.  (Dependents released at the kernel's start: 21.9, 82.4, 116.8, 12.0, and every output
-// would need a record.)
+// round of six ragged bf16 segments, 16 / 4 heads of 64, 84.4 -> 82.4; local + remote + merge of 2160 tokens 120.1 -> 117.7.
+// (Dependents released at the kernel's start: 21.9, 82.4, 116.8, and every output would need a record.)
+// Concatenation, merge and SIMT attention are launched so behind kernels that release early too: us a pass in a loop,
+// ordinary -> this, fp32 4 x 128 tokens, 8 / 2 heads of 64: selection, sync 24.7 -> 22.3; gather, sync 20.5 -> 18.3;
+// selection, local, remote, merge 43.6 -> 37.1; selection, concatenation 12.8 -> 11.3.  4 x 512, 128 channels: 113.1 -> 112.6,
+// 104.6 -> 102.5, 224.6 -> 218.5, 18.5 -> 16.9.  8 x 1024, 8 / 8 heads of 64: 535.7 -> 534.2, 527.1 -> 520.1, 804.5 -> 791.9,
+// 26.7 -> 25.2.  bf16 decode of 8 x 4096, local, shared and their merge 59.7 -> 58.8.  (As graphs: 0 to 7 us less; 0.4 us more
+// in one, selection, sync at 4 x 512, where the runs differ by 0.2.)
 struct WaitFirstLaunch {
     cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg;
